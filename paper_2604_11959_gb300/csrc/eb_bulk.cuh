@@ -38,8 +38,15 @@
 // tcgen05.ld, 32x32b shapes: TMEM lane = the thread's lane).  The double
 // path keeps them in registers.
 // Every field is read from HBM once per level (halo re-reads hit L2) and
-// written once.  Advective face fluxes carry a factor 6 that the divergence
-// removes with 1/(6 dx).
+// written once.  Advective face fluxes carry a factor 6 (12 on the face
+// grids) that the divergence removes with 1/(6 dx).
+//
+// What bounds it: instruction issue on the float path, FP64 instructions on
+// the double path (an SM starts two per clock, 1/64 of the FP32 rate).  The
+// double path therefore spends integer instructions where it can (selects
+// before the flux arithmetic, the finite test) and three FP64 instructions
+// per reciprocal: 256x256x128 hill, one FP64 step 4.80 -> 3.12 ms, 32x32x16
+// ridge 510 -> 337 us, the mixed hill step 224 -> 218 us.
 #pragma once
 
 #include "eb_step.cuh"
@@ -154,7 +161,21 @@ __device__ inline float2 psub(float2 a, float2 b) { return __ffma2_rn(b, make_fl
 __device__ inline double2 psub(double2 a, double2 b) { return make_double2(__dsub_rn(a.x, b.x), __dsub_rn(a.y, b.y)); }
 // elementwise reciprocal: the fast approximate one on the float path
 __device__ inline float2 prcp(float2 a) { return make_float2(__fdividef(1.f, a.x), __fdividef(1.f, a.y)); }
-__device__ inline double2 prcp(double2 a) { return make_double2(1.0 / a.x, 1.0 / a.y); }
+// FP64 instructions are what bounds the double path (two per clock and SM),
+// so the reciprocal is formed with three: r0 = 1/a (1 - e) from the
+// hardware's approximate double reciprocal (|e| about 2^-20), then 1/a = r0
+// (1 + e + e^2 + ...) cut after e^2, which leaves an error of |e|^3 = 2^-60
+// before the one rounding of the last operation; outside the range where r0
+// and its product are normal numbers the plain division runs.
+__device__ inline double rcp_fma(double a) {
+  const unsigned ex = (unsigned)__double2hiint(a) & 0x7ff00000u;
+  if (ex - 0x00300000u > 0x7f900000u) return 1.0 / a;   // zero, subnormal, near the range's ends, Inf, NaN
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
+  const double e = __fma_rn(-a, r, 1.0);
+  return __fma_rn(r, __fma_rn(e, e, e), r);
+}
+__device__ inline double2 prcp(double2 a) { return make_double2(rcp_fma(a.x), rcp_fma(a.y)); }
 template <typename P>
 __device__ inline P psel_pos(P m, P a, P b) {   // a where m > 0, else b
   return mk(m.x > 0 ? a.x : b.x, m.y > 0 ? a.y : b.y);
@@ -169,13 +190,37 @@ __device__ inline void st2(double *p, double2 v) { *reinterpret_cast<double2 *>(
 // c with far values a (low side) and d (high side): m > 0 takes
 // (5b + 2c - a), m < 0 takes (5c + 2b - d), or the centred 3(b + c) when the
 // far high CV does not exist (Sec. 4.1).
-template <typename P>
-__device__ inline P flux6(P m, P a, P b, P c, P d, bool has_d = true) {
-  using T = decltype(m.x);
-  const P two = splat(T(2)), five = splat(T(5)), mone = splat(T(-1));
-  const P vp = pfma(b, five, pfma(a, mone, pmul(c, two)));
-  const P vn = has_d ? pfma(c, five, pfma(d, mone, pmul(b, two))) : pmul(padd(b, c), splat(T(3)));
+__device__ inline float2 flux6(float2 m, float2 a, float2 b, float2 c, float2 d, bool has_d = true) {
+  const float2 two = splat(2.f), five = splat(5.f), mone = splat(-1.f);
+  const float2 vp = pfma(b, five, pfma(a, mone, pmul(c, two)));
+  const float2 vn = has_d ? pfma(c, five, pfma(d, mone, pmul(b, two))) : pmul(padd(b, c), splat(3.f));
   return pmul(m, psel_pos(m, vp, vn));
+}
+// The double path picks the upwind, downwind and far values before the
+// arithmetic, by the sign bit of m and integer selects: three FP64
+// instructions per face instead of eight, with the same bits (2c and 2b are
+// exact).
+__device__ inline double flux6_one(double m, double a, double b, double c, double d, bool has_d) {
+  const bool pos = __double2hiint(m) > 0;
+  if (!has_d && !pos) return m * ((b + c) * 3.0);
+  const double up = pos ? b : c, down = pos ? c : b, far = pos ? a : d;
+  return __dmul_rn(m, __fma_rn(up, 5.0, __fma_rn(down, 2.0, -far)));
+}
+__device__ inline double2 flux6(double2 m, double2 a, double2 b, double2 c, double2 d, bool has_d = true) {
+  return make_double2(flux6_one(m.x, a.x, b.x, c.x, d.x, has_d), flux6_one(m.y, a.y, b.y, c.y, d.y, has_d));
+}
+
+// bad turns non-finite once a written value is: a packed multiply by zero on
+// the float path, the largest exponent word (integer instructions) on the
+// double path
+__device__ inline void note_bad(float &bad, float o) { bad = fmaf(o, 0.f, bad); }
+__device__ inline void note_bad(double &bad, double o) {
+  bad = __hiloint2double(max(__double2hiint(bad), __double2hiint(o) & 0x7fffffff), 0);
+}
+__device__ inline void note_bad(float2 &bad, float2 o) { bad = pfma(o, splat(0.f), bad); }
+__device__ inline void note_bad(double2 &bad, double2 o) {
+  note_bad(bad.x, o.x);
+  note_bad(bad.y, o.y);
 }
 
 // Tile of the bulk march: TX x TY columns (TY = 16, or 14 so that a 256-row
@@ -276,7 +321,9 @@ __device__ __forceinline__ void bulk_march(const StepArgs<T> &A, const int4 sg, 
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * NPX + tx;
   const int tiles_x = (D.nx + TX - 1) / TX;
   const T idx = T(D.idx), idy = T(D.idy), idz = T(D.idz);
-  const T idx6 = T(D.idx / 6.0), idy6 = T(D.idy / 6.0), idz6 = T(D.idz / 6.0);
+  // minus the factors of the face flux differences: 1 / (6 dx) on the c grid,
+  // half of it on the face grids
+  const T nx6 = -T(D.idx / 6.0), ny6 = -T(D.idy / 6.0), nz6 = -T(D.idz / 6.0);
   const P half = splat(T(0.5)), zero = splat(T(0));
   const bool same_base = A.base[0] != nullptr && A.base[0] == A.src.f[0] && A.base[1] == A.src.f[1] &&
                          A.base[2] == A.src.f[2] && A.base[3] == A.src.f[3] && A.base[4] == A.src.f[4];
@@ -327,9 +374,11 @@ __device__ __forceinline__ void bulk_march(const StepArgs<T> &A, const int4 sg, 
     qraw[r] = q < TL::NQP ? TL::ri(2 * (q % (QX / 2)) - 2, q / (QX / 2) - 2) : -1;
   }
 
-  // face fluxes (x 6) through the low x and y faces of the column pair at
-  // even tile x, row y of level p, all four grids: each momentum and
-  // primitive value is read from shared memory once
+  // face fluxes (x 6, and x 12 on the face grids, whose masses are sums of
+  // two momenta: the half of the mean is left to the divergence's factor)
+  // through the low x and y faces of the column pair at even tile x, row y of
+  // level p, all four grids: each momentum and primitive value is read from
+  // shared memory once
   auto faces = [&](const T *Rk, const T *Rkm, int x, int y, T ru, T rv, T rum, T rvm, P fxo[4], P fyo[4]) {
     const int c = TL::ri(x, y);
     const T *U = Rk + 2 * NP, *Vv = Rk + 3 * NP;
@@ -338,8 +387,8 @@ __device__ __forceinline__ void bulk_march(const StepArgs<T> &A, const int4 sg, 
             ub = padd(ld2(Rkm + 2 * NP + c), splat(rum));
     const P vc = padd(ld2(Vv + c), prv), vl = padd(ld2(Vv + c - 2), prv), vd = padd(ld2(Vv + c - PX), prv),
             vkm = padd(ld2(Rkm + 3 * NP + c), splat(rvm));
-    const P mx[4] = {uc, pmul(padd(mk(ul.y, uc.x), uc), half), pmul(padd(ud, uc), half), pmul(padd(ub, uc), half)};
-    const P my[4] = {vc, pmul(padd(mk(vl.y, vc.x), vc), half), pmul(padd(vd, vc), half), pmul(padd(vkm, vc), half)};
+    const P mx[4] = {uc, padd(mk(ul.y, uc.x), uc), padd(ud, uc), padd(ub, uc)};
+    const P my[4] = {vc, padd(mk(vl.y, vc.x), vc), padd(vd, vc), padd(vkm, vc)};
 #pragma unroll
     for (int G = 0; G < 4; ++G) {
       const T *Q = prim + G * NQ + TL::qi(x, y);
@@ -384,7 +433,8 @@ __device__ __forceinline__ void bulk_march(const StepArgs<T> &A, const int4 sg, 
     // ---- phase 1: primitive plane of level p
     if (p < nz) {
       const T *R = RAWP(p), *Rm = RAWP(p - 1);
-      const P rrp = splat(rr_p);
+      const P rrp = splat(rr_p), rrz = splat(T(0.5) * (rr_m + rr_p));
+      const P hbu = splat(T(-0.5) * bu_p), hbv = splat(T(-0.5) * bv_p);
 #pragma unroll
       for (int r = 0; r < TL::QR; ++r) {
         const int c = qraw[r];
@@ -395,14 +445,14 @@ __device__ __forceinline__ void bulk_march(const StepArgs<T> &A, const int4 sg, 
         // rhobar') / rhobar, all from stored perturbations, so the
         // rounding scales with the deviation; w has no background
         const P rp = ld2(R + c);
-        const P rho = padd(rp, rrp);
-        const P rbx = pmul(padd(mk(R[c - 1], rp.x), rp), half);
-        const P rby = pmul(padd(ld2(R + c - PX), rp), half);
-        const P rhob = padd(ld2(Rm + c), splat(rr_m));
-        st2(Q, pmul(pfma(splat(-bt_p), rp, ld2(R + NP + c)), prcp(rho)));
-        st2(Q + NQ, pmul(pfma(splat(-bu_p), rbx, ld2(R + 2 * NP + c)), prcp(padd(rbx, rrp))));
-        st2(Q + 2 * NQ, pmul(pfma(splat(-bv_p), rby, ld2(R + 3 * NP + c)), prcp(padd(rby, rrp))));
-        st2(Q + 3 * NQ, pmul(ld2(R + 4 * NP + c), prcp(pmul(padd(rhob, rho), half))));
+        // (rbx, rby, rbz: twice the mean rho')
+        const P rbx = padd(mk(R[c - 1], rp.x), rp);
+        const P rby = padd(ld2(R + c - PX), rp);
+        const P rbz = padd(ld2(Rm + c), rp);
+        st2(Q, pmul(pfma(splat(-bt_p), rp, ld2(R + NP + c)), prcp(padd(rp, rrp))));
+        st2(Q + NQ, pmul(pfma(hbu, rbx, ld2(R + 2 * NP + c)), prcp(pfma(rbx, half, rrp))));
+        st2(Q + 2 * NQ, pmul(pfma(hbv, rby, ld2(R + 3 * NP + c)), prcp(pfma(rby, half, rrp))));
+        st2(Q + 3 * NQ, pmul(ld2(R + 4 * NP + c), prcp(pfma(rbz, half, rrz))));
       }
     }
     __syncthreads();
@@ -457,9 +507,8 @@ __device__ __forceinline__ void bulk_march(const StepArgs<T> &A, const int4 sg, 
         const T *Vv = Rk + 3 * NP;
         const P prv = splat(rv_p);
         const P vc = padd(ld2(Vv + c), prv);
-        const P mA = ty ? pmul(padd(padd(ld2(Vv + c - PX), prv), vc), half) : vc;
-        const P mB =
-            pmul(padd(ty ? padd(ld2(Rkm + 3 * NP + c), splat(rv_m)) : mk(Vv[c - 1] + rv_p, vc.x), vc), half);
+        const P mA = ty ? padd(padd(ld2(Vv + c - PX), prv), vc) : vc;
+        const P mB = padd(ty ? padd(ld2(Rkm + 3 * NP + c), splat(rv_m)) : mk(Vv[c - 1] + rv_p, vc.x), vc);
         const T *Q = prim + G0 * NQ + TL::qi(2 * tx, TY);
         const P fA = flux6(mA, ld2(Q - 2 * QX), ld2(Q - QX), ld2(Q), ld2(Q + QX));
         Q += NQ;
@@ -471,8 +520,8 @@ __device__ __forceinline__ void bulk_march(const StepArgs<T> &A, const int4 sg, 
         const int c = TL::ri(TX, tx);
         const T *U = Rk + 2 * NP;
         const T u0 = U[c] + ru_p;
-        const T mA = hi ? T(0.5) * ((U[c - PX] + ru_p) + u0) : u0;
-        const T mB = T(0.5) * ((hi ? Rkm[2 * NP + c] + ru_m : U[c - 1] + ru_p) + u0);
+        const T mA = hi ? (U[c - PX] + ru_p) + u0 : u0;
+        const T mB = (hi ? Rkm[2 * NP + c] + ru_m : U[c - 1] + ru_p) + u0;
         const T *Q = prim + G0 * NQ + TL::qi(TX, tx);
         FX[G0 * TL::NFX + tx * TL::FXW + NPX] =
             flux6(splat(mA), splat(Q[-2]), splat(Q[-1]), splat(Q[0]), splat(Q[1])).x;
@@ -484,12 +533,12 @@ __device__ __forceinline__ void bulk_march(const StepArgs<T> &A, const int4 sg, 
     copy_wait<1>();   // raw p + 1 landed (this thread's copies)
     __syncthreads();
 
-    // ---- phase 2b: x / y divergence of level p; z flux and update of level k
+    // ---- phase 2b: minus the x / y divergence of level p; z flux and update of level k
     P sxy[4];
     if (face_level) {
-      const P ix = splat(idx6), iy = splat(idy6);
 #pragma unroll
       for (int G = 0; G < 4; ++G) {
+        const P ix = splat(G ? T(0.5) * nx6 : nx6), iy = splat(G ? T(0.5) * ny6 : ny6);
         const P dfx = psub(mk(fx[G].y, FX[G * TL::NFX + ty * TL::FXW + tx + 1]), fx[G]);
         const P dfy = psub(ld2(FY + G * TL::NFY + (ty + 1) * TX + 2 * tx), fy[G]);
         sxy[G] = pfma(dfx, ix, pmul(dfy, iy));
@@ -511,9 +560,9 @@ __device__ __forceinline__ void bulk_march(const StepArgs<T> &A, const int4 sg, 
         const P mu = pfma(psub(u1, um), hx, pmul(psub(padd(vul, vu), padd(vl, v0)), hy));
         // v grid: x faces at edges (means along y of rho*u), y faces at cell centres
         const P mv = pfma(psub(padd(ud1, u1), padd(ud0, u0)), hx, pmul(psub(vu, vd), hy));
-        sxy[0] = pfma(splat(bt_p), mc, sxy[0]);
-        sxy[1] = pfma(splat(bu_p), mu, sxy[1]);
-        sxy[2] = pfma(splat(bv_p), mv, sxy[2]);
+        sxy[0] = pfma(splat(-bt_p), mc, sxy[0]);
+        sxy[1] = pfma(splat(-bu_p), mu, sxy[1]);
+        sxy[2] = pfma(splat(-bv_p), mv, sxy[2]);
       }
     } else {
 #pragma unroll
@@ -526,9 +575,9 @@ __device__ __forceinline__ void bulk_march(const StepArgs<T> &A, const int4 sg, 
       const T *Rk = RAWP(k);
       const T *W1 = RAWP(k + 1) + 4 * NP;
       const P m = has1 ? ld2(W1 + self) : zero;
-      const P mu = has1 ? pmul(padd(mk(W1[self - 1], m.x), m), half) : zero;
-      const P mv = has1 ? pmul(padd(ld2(W1 + self - PX), m), half) : zero;
-      const P mw = pmul(padd(ld2(Rk + 4 * NP + self), m), half);
+      const P mu = has1 ? padd(mk(W1[self - 1], m.x), m) : zero;
+      const P mv = has1 ? padd(ld2(W1 + self - PX), m) : zero;
+      const P mw = padd(ld2(Rk + 4 * NP + self), m);
       const P fzc = flux6(m, th[0], th[1], th[2], th[3], has2);
       const P fzu = flux6(mu, uu[0], uu[1], uu[2], uu[3], has2);
       const P fzv = flux6(mv, vv[0], vv[1], vv[2], vv[3], has2);
@@ -538,13 +587,13 @@ __device__ __forceinline__ void bulk_march(const StepArgs<T> &A, const int4 sg, 
         const P uc = ld2(U + self);
         const P dmx = psub(mk(uc.y, U[self + 2]), uc);
         const P dmy = psub(ld2(Vv + self + PX), ld2(Vv + self));
-        const P iz6 = splat(-idz6);
+        const P izc = splat(nz6), izf = splat(T(0.5) * nz6);
         P d[5];
         d[0] = pfma(dmx, splat(-idx), pfma(dmy, splat(-idy), pmul(psub(m, zc_m), splat(-idz))));
-        d[1] = pfma(psub(fzc, zc_t), iz6, pmul(q0[0], splat(T(-1))));
-        d[2] = pfma(psub(fzu, zu), iz6, pmul(q0[1], splat(T(-1))));
-        d[3] = pfma(psub(fzv, zv), iz6, pmul(q0[2], splat(T(-1))));
-        d[4] = pfma(psub(fzw, zw), iz6, pmul(q0[3], splat(T(-1))));
+        d[1] = pfma(psub(fzc, zc_t), izc, q0[0]);
+        d[2] = pfma(psub(fzu, zu), izf, q0[1]);
+        d[3] = pfma(psub(fzv, zv), izf, q0[2]);
+        d[4] = pfma(psub(fzw, zw), izf, q0[3]);
         const bool both = k >= kfx && k >= kfy;
         const P dtp = splat(A.dtT);
 #pragma unroll
@@ -565,13 +614,13 @@ __device__ __forceinline__ void bulk_march(const StepArgs<T> &A, const int4 sg, 
               dst[0] = o.x;
               dst[1] = o.y;
             }
-            bad = pfma(o, zero, bad);
+            note_bad(bad, o);
           } else if (k >= kfx) {
             dst[0] = o.x;
-            bad.x = fma(o.x, T(0), bad.x);
+            note_bad(bad.x, o.x);
           } else {
             dst[1] = o.y;
-            bad.y = fma(o.y, T(0), bad.y);
+            note_bad(bad.y, o.y);
           }
         }
       }
