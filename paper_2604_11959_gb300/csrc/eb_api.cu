@@ -21,7 +21,9 @@ std::string &eb_error_slot() { return g_last_error; }
 
 eb_status eb_replan_bulk(eb_geom g, int slab_levels) {
   std::vector<int> seg, off;
-  CUDA_TRY(bulk_plan(g->D, g->kfast_host.data(), g->prec == EB_F64, slab_levels, g->tile_rows, seg, off),
+  int rows = g->tile_rows;
+  CUDA_TRY(bulk_plan(g->D, g->kfast_host.data(), g->prec == EB_F64, slab_levels, g->tile_rows, !g->in_ensemble, seg,
+                     off, rows),
            "bulk work split");
   // the split arrays are small: the old ones are released right away
   for (void *p : {(void *)g->bseg, (void *)g->boff}) {
@@ -36,6 +38,7 @@ eb_status eb_replan_bulk(eb_geom g, int slab_levels) {
   g->bseg = nullptr;
   g->boff = nullptr;
   g->slab_levels = slab_levels;
+  g->plan_rows = rows;
   g->bctas = (int)off.size() - 1;
   ++g->plan_gen;
   CUDA_TRY(g->alloc(&g->bseg, std::max<long long>(1, (long long)seg.size() / 4)), "alloc bulk split");

@@ -223,12 +223,12 @@ __device__ inline void note_bad(double2 &bad, double2 o) {
   note_bad(bad.y, o.y);
 }
 
-// Tile of the bulk march: TX x TY columns (TY = 16, or 14 so that a 256-row
+// Tile of the bulk march: TX x TY columns (32 x 16; 32 x 14 so that a 256-row
 // domain cuts into 19 tile rows and two slabs of 152 tiles fill every SM
-// with two CTAs).
-template <typename T, int TY_ = 16>
+// with two CTAs; 16 x 8 for domains whose 32 x 16 tiles leave SMs idle).
+template <typename T, int TY_ = 16, int TX_ = 32>
 struct BulkTile {
-  static constexpr int TX = 32, TY = TY_;    // columns and rows of a tile
+  static constexpr int TX = TX_, TY = TY_;   // columns and rows of a tile
   static constexpr int NPX = TX / 2;         // column pairs per row (threads per row)
   static constexpr int NT = NPX * TY;        // threads
   static constexpr int HX = 4;               // raw halo in x on both sides (16-byte aligned rows)
@@ -246,6 +246,7 @@ struct BulkTile {
   static constexpr int PRIM = 4 * NQ;
   static constexpr size_t BYTES = sizeof(T) * (size_t)(RAW + PRIM + 4 * NFX + 4 * NFY);
   static constexpr int QR = (NQP + NT - 1) / NT;   // primitive pairs per thread
+  static constexpr unsigned TMC = 64u * ((NT + 127) / 128);   // tensor-memory columns (float path)
   __device__ static constexpr int ri(int x, int y) { return (y + 3) * PX + (x + HX); }
   __device__ static constexpr int qi(int x, int y) { return (y + 2) * QX + (x + 2); }
 };
@@ -263,15 +264,15 @@ __host__ __device__ constexpr bool bulk_tmem_default() {
   return sizeof(T) == sizeof(float);
 }
 
-// Tensor memory of a CTA for the carried state: 128 columns allocated by
+// Tensor memory of a CTA for the carried state: NC columns allocated by
 // warp 0; returns this thread's base address (lane = the thread's lane in
 // its warp's quarter, 64 columns per warp).  Without TM nothing is
 // allocated.
-template <typename T, bool TM = bulk_tmem_default<T>()>
+template <typename T, bool TM = bulk_tmem_default<T>(), unsigned NC = 128u>
 __device__ inline unsigned bulk_tmem_begin(unsigned *slot) {
   if constexpr (TM) {
-    const int tid = threadIdx.y * BulkTile<T>::NPX + threadIdx.x;
-    if (tid < 32) tm_alloc(slot, 128u);
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+    if (tid < 32) tm_alloc(slot, NC);
     tm_fence_before();
     __syncthreads();
     tm_fence_after();
@@ -282,27 +283,27 @@ __device__ inline unsigned bulk_tmem_begin(unsigned *slot) {
 }
 
 // Releases what bulk_tmem_begin allocated (every thread of the CTA calls it).
-template <typename T, bool TM = bulk_tmem_default<T>()>
+template <typename T, bool TM = bulk_tmem_default<T>(), unsigned NC = 128u>
 __device__ inline void bulk_tmem_end(unsigned *slot) {
   if constexpr (TM) {
-    const int tid = threadIdx.y * BulkTile<T>::NPX + threadIdx.x;
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
     tm_wait_st();
     tm_fence_before();
     __syncthreads();
     tm_fence_after();
-    if (tid < 32) tm_dealloc(*slot, 128u);
+    if (tid < 32) tm_dealloc(*slot, NC);
   }
 }
 
 // One march of the CTA over the levels [sg.y, sg.z) of tile sg.x (tiles of
-// TYV rows).  smem_bytes holds BulkTile<T, TYV>::BYTES of dynamic shared
-// memory, tbase is this thread's
+// TXV columns and TYV rows).  smem_bytes holds BulkTile<T, TYV, TXV>::BYTES of
+// dynamic shared memory, tbase is this thread's
 // tensor-memory base (bulk_tmem_begin), and bad turns NaN when a written
 // value is not finite.  Every thread of the CTA calls it.
-template <typename T, int V, bool TM = bulk_tmem_default<T>(), int TYV = 16>
+template <typename T, int V, bool TM = bulk_tmem_default<T>(), int TYV = 16, int TXV = 32>
 __device__ __forceinline__ void bulk_march(const StepArgs<T> &A, const int4 sg, unsigned char *smem_bytes,
                                            const unsigned tbase, typename PairOf<T>::type &bad) {
-  using TL = BulkTile<T, TYV>;
+  using TL = BulkTile<T, TYV, TXV>;
   using P = typename PairOf<T>::type;
   constexpr int TX = TL::TX, TY = TL::TY, NPX = TL::NPX, NT = TL::NT, PX = TL::PX, NP = TL::NP, QX = TL::QX,
                 NQ = TL::NQ;

@@ -127,7 +127,9 @@ eb_status build_tables(eb_ensemble e, EnsembleArgs<T> E[2]) {
   for (int q = 0; q < n; ++q) {
     eb_geom g = e->m[q];
     std::vector<int> seg, off;
-    CUDA_TRY(bulk_plan(g->D, g->kfast_host.data(), g->prec == EB_F64, g->slab_levels, 16, seg, off), "work split");
+    int rows = 16;
+    CUDA_TRY(bulk_plan(g->D, g->kfast_host.data(), g->prec == EB_F64, g->slab_levels, 16, false, seg, off, rows),
+             "work split");
     if ((int)off.size() - 1 != g->bctas)
       return fail(EB_ERR_STATE, "a member's work split changed outside the ensemble; tune it again");
     for (int u = 0; u + 1 < (int)off.size(); ++u) {
@@ -265,8 +267,9 @@ eb_status eb_ensemble_create(const eb_geom *members, int n, eb_ensemble *out) {
   }
   // the persistent kernel marches tiles of 16 rows: members keep that height
   for (int q = 0; q < n; ++q)
-    if (members[q]->tile_rows != 16) {
+    if (members[q]->tile_rows != 16 || !members[q]->in_ensemble) {
       members[q]->tile_rows = 16;
+      members[q]->in_ensemble = true;
       const eb_status st = eb_replan_bulk(members[q], members[q]->slab_levels);
       if (st != EB_OK) return st;
     }

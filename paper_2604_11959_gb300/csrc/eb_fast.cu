@@ -4,6 +4,7 @@
 #include "eb_bulk.cuh"
 
 #include <algorithm>
+#include <functional>
 #include <vector>
 
 namespace {
@@ -18,17 +19,18 @@ using namespace bulk;
 #ifndef EB_BULK_MAXNREG
 #define EB_BULK_MAXNREG 96
 #endif
-template <typename T, int V, int TYV>
-__global__ void __launch_bounds__(BulkTile<T, TYV>::NT, (sizeof(T) == 4 ? 2 : 1))
+template <typename T, int V, int TYV, int TXV>
+__global__ void __launch_bounds__(BulkTile<T, TYV, TXV>::NT, (sizeof(T) == 4 ? 2 : 1))
     __maxnreg__(sizeof(T) == 4 ? EB_BULK_MAXNREG : 255) k_fast_tiled(StepArgs<T> A) {
   using P = typename PairOf<T>::type;
   extern __shared__ __align__(16) unsigned char smem_bytes[];
   __shared__ unsigned tm_slot;
-  const unsigned tbase = bulk_tmem_begin<T>(&tm_slot);
+  constexpr unsigned NC = BulkTile<T, TYV, TXV>::TMC;
+  const unsigned tbase = bulk_tmem_begin<T, bulk_tmem_default<T>(), NC>(&tm_slot);
   P bad = splat(T(0));   // becomes NaN once any written value is not finite
   for (int sgi = A.boff[blockIdx.x]; sgi < A.boff[blockIdx.x + 1]; ++sgi)
-    bulk_march<T, V, bulk_tmem_default<T>(), TYV>(A, A.bseg[sgi], smem_bytes, tbase, bad);
-  bulk_tmem_end<T>(&tm_slot);
+    bulk_march<T, V, bulk_tmem_default<T>(), TYV, TXV>(A, A.bseg[sgi], smem_bytes, tbase, bad);
+  bulk_tmem_end<T, bulk_tmem_default<T>(), NC>(&tm_slot);
   if (!(isfinite(bad.x) && isfinite(bad.y))) atomicOr(A.status, EB_DEV_NUMERIC);
 }
 
@@ -67,31 +69,34 @@ __global__ void k_static(StepArgs<T> A, StaticBlocks SB) {
   }
 }
 
-template <typename T, int V, int TYV>
+template <typename T, int V, int TYV, int TXV>
 void set_smem_attr() {
   static unsigned long long done = 0;
-  ebk_smem_limit(k_fast_tiled<T, V, TYV>, (int)BulkTile<T, TYV>::BYTES, done);
+  ebk_smem_limit(k_fast_tiled<T, V, TYV, TXV>, (int)BulkTile<T, TYV, TXV>::BYTES, done);
 }
 
-template <typename T, int V, int TYV>
+template <typename T, int V, int TYV, int TXV = 32>
 void launch_bulk(const StepArgs<T> &A, cudaStream_t s) {
-  using TL = BulkTile<T, TYV>;
+  using TL = BulkTile<T, TYV, TXV>;
   if (A.bctas < 1) return;
-  set_smem_attr<T, V, TYV>();
-  k_fast_tiled<T, V, TYV><<<A.bctas, dim3(TL::NPX, TL::TY, 1), TL::BYTES, s>>>(A);
+  set_smem_attr<T, V, TYV, TXV>();
+  k_fast_tiled<T, V, TYV, TXV><<<A.bctas, dim3(TL::NPX, TL::TY, 1), TL::BYTES, s>>>(A);
 }
 
 template <typename T>
 int resident_ctas_per_sm() {
   constexpr int V = 16 / sizeof(T);
-  set_smem_attr<T, V, 16>();   // every variant set here, outside any graph capture
-  set_smem_attr<T, 1, 16>();
+  set_smem_attr<T, V, 16, 32>();   // every variant set here, outside any graph capture
+  set_smem_attr<T, 1, 16, 32>();
   if constexpr (sizeof(T) == sizeof(float)) {
-    set_smem_attr<T, V, 14>();
-    set_smem_attr<T, 1, 14>();
+    set_smem_attr<T, V, 14, 32>();
+    set_smem_attr<T, 1, 14, 32>();
+  } else {
+    set_smem_attr<T, V, 8, 16>();
+    set_smem_attr<T, 1, 8, 16>();
   }
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fast_tiled<T, V, 16>, BulkTile<T>::NT,
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fast_tiled<T, V, 16, 32>, BulkTile<T>::NT,
                                                     BulkTile<T>::BYTES) != cudaSuccess ||
       n < 1)
     n = 1;
@@ -100,19 +105,59 @@ int resident_ctas_per_sm() {
 
 }  // namespace
 
-cudaError_t bulk_plan(const Dims &D, const int *kfast_host, bool f64, int slab_levels, int tile_rows,
-                      std::vector<int> &seg, std::vector<int> &off) {
-  const int TX = BulkTile<float>::TX, TY = tile_rows;
+namespace {
+
+// Lockstep slabs: every tile is cut at the same levels, and the pieces are
+// launched slab by slab from the top, so CTAs of neighbouring tiles march
+// the same levels at the same time and read each other's halo from L2; the
+// short pieces of the lowest slabs come last.  piece(tile, first, end).
+template <typename F>
+void for_pieces(const Dims &D, const std::vector<int> &kb, long long Lc, F &&piece) {
+  const int nslab = (int)((D.nz + Lc - 1) / Lc);
+  for (int sl = nslab - 1; sl >= 0; --sl) {
+    const int za = (int)(sl * Lc), zb = (int)std::min<long long>(D.nz, (sl + 1) * Lc);
+    for (size_t t = 0; t < kb.size(); ++t) {
+      const int a = std::max(za, kb[t]);
+      if (a < zb) piece((int)t, a, zb);
+    }
+  }
+}
+
+// lowest kfast of every tile of TX x TY columns
+std::vector<int> tile_bottoms(const Dims &D, const int *kfast, int TX, int TY) {
   const int tx = (D.nx + TX - 1) / TX, ty = (D.ny + TY - 1) / TY;
-  const long long ntile = (long long)tx * ty;
-  std::vector<int> kb(ntile, D.nz);
+  std::vector<int> kb((size_t)tx * ty, D.nz);
   for (int j = 0; j < D.ny; ++j)
     for (int i = 0; i < D.nx; ++i) {
-      int &v = kb[(i / TX) + (long long)tx * (j / TY)];
-      v = std::min(v, kfast_host[i + (long long)D.nx * j]);
+      int &v = kb[(i / TX) + (size_t)tx * (j / TY)];
+      v = std::min(v, kfast[i + (long long)D.nx * j]);
     }
+  return kb;
+}
+
+// Time of a split on the double path when the pieces start in order on
+// `slots` SMs: a piece costs `start` (its two prologue levels, copies and
+// fill) plus `level` per level.
+double split_time(const Dims &D, const std::vector<int> &kb, long long Lc, int slots, double start, double level) {
+  std::vector<double> heap((size_t)slots, 0.0);   // min-heap of the slots' finishing times
+  double end = 0.0;
+  for_pieces(D, kb, Lc, [&](int, int a, int b) {
+    std::pop_heap(heap.begin(), heap.end(), std::greater<double>());
+    heap.back() += start + level * (b - a);
+    end = std::max(end, heap.back());
+    std::push_heap(heap.begin(), heap.end(), std::greater<double>());
+  });
+  return end;
+}
+
+}  // namespace
+
+cudaError_t bulk_plan(const Dims &D, const int *kfast_host, bool f64, int slab_levels, int tile_rows, bool alone,
+                      std::vector<int> &seg, std::vector<int> &off, int &plan_rows) {
+  plan_rows = tile_rows;
+  std::vector<int> kb = tile_bottoms(D, kfast_host, 32, tile_rows);
   long long W = 0;
-  for (long long t = 0; t < ntile; ++t) W += std::max(0, D.nz - kb[t]);
+  for (int k : kb) W += std::max(0, D.nz - k);
   seg.clear();
   off.assign(1, 0);
   if (W == 0) return cudaSuccess;
@@ -121,27 +166,40 @@ cudaError_t bulk_plan(const Dims &D, const int *kfast_host, bool f64, int slab_l
   if (e != cudaSuccess) return e;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  const long long slots = (long long)std::max(sms, 1) * (f64 ? resident_ctas_per_sm<double>()
-                                                              : resident_ctas_per_sm<float>());
-  // Lockstep slabs: every tile is cut at the same levels, and the pieces are
-  // launched slab by slab from the top, so CTAs of neighbouring tiles march
-  // the same levels at the same time and read each other's halo from L2.
+  sms = std::max(sms, 1);
+  const long long slots = (long long)sms * (f64 ? resident_ctas_per_sm<double>() : resident_ctas_per_sm<float>());
   // Slabs of slab_levels levels, or (0) of at least 16 levels sized for
-  // about three waves of CTAs; the short pieces of the lowest slabs come last.
-  const long long Lc = slab_levels > 0 ? (long long)slab_levels : std::max(16LL, (W + 3 * slots - 1) / (3 * slots));
-  const int nslab = (int)((D.nz + Lc - 1) / Lc);
-  for (int sl = nslab - 1; sl >= 0; --sl) {
-    const int za = (int)(sl * Lc), zb = (int)std::min<long long>(D.nz, (sl + 1) * Lc);
-    for (long long t = 0; t < ntile; ++t) {
-      const int a = std::max(za, kb[t]);
-      if (a >= zb) continue;
-      seg.push_back((int)t);
-      seg.push_back(a);
-      seg.push_back(zb);
-      seg.push_back(0);
-      off.push_back((int)(seg.size() / 4));
+  // about three waves of CTAs.
+  long long Lc = slab_levels > 0 ? (long long)slab_levels : std::max(16LL, (W + 3 * slots - 1) / (3 * slots));
+  if (slab_levels == 0 && f64 && alone) {
+    // Double path alone on the GPU: the height (and for small domains the
+    // 16 x 8 tile) of the shortest estimated time, in microseconds as
+    // measured for one CTA per SM: 39 + 23.7 per level for a 32 x 16 tile; 28
+    // + 13.7 per level for a 16 x 8 tile (four of them per 32 x 16 tile,
+    // each cheaper in time but not in FP64 instructions: more halo), which
+    // is taken only while every piece has an SM of its own.  32x32x16 ridge:
+    // 337 us with one slab of 32 x 16 tiles, 63 with one level per piece, 42
+    // with 16 x 8 tiles; 64x64x32: 407 -> 87; 256x256x128: 3084 -> 2816
+    // (slabs of 35 and 16 levels).
+    double best = split_time(D, kb, Lc, sms, 39.0, 23.7);
+    const std::vector<int> ks = tile_bottoms(D, kfast_host, 16, 8);
+    for (long long L : {1, 2, 3, 4, 6, 8, 12, 16, 24, 32}) {
+      if (L > D.nz) break;
+      const double t = split_time(D, kb, L, sms, 39.0, 23.7);
+      if (t < best) best = t, Lc = L, plan_rows = tile_rows;
+      long long pieces = 0;
+      for_pieces(D, ks, L, [&](int, int, int) { ++pieces; });
+      if (pieces <= sms && 28.0 + 13.7 * L < best) best = 28.0 + 13.7 * L, Lc = L, plan_rows = 8;
     }
+    if (plan_rows == 8) kb = ks;
   }
+  for_pieces(D, kb, Lc, [&](int t, int a, int zb) {
+    seg.push_back(t);
+    seg.push_back(a);
+    seg.push_back(zb);
+    seg.push_back(0);
+    off.push_back((int)(seg.size() / 4));
+  });
   return cudaGetLastError();
 }
 
@@ -182,6 +240,12 @@ void launch_flux_bulk(const StepArgs<T> &A, cudaStream_t s) {
     if (A.tile_rows == 14) {
       if (vec) launch_bulk<T, V, 14>(A, s);
       else launch_bulk<T, 1, 14>(A, s);
+      return;
+    }
+  } else {   // 16 x 8 tiles on the double path only
+    if (A.tile_rows == 8) {
+      if (vec) launch_bulk<T, V, 8, 16>(A, s);
+      else launch_bulk<T, 1, 8, 16>(A, s);
       return;
     }
   }
