@@ -328,6 +328,8 @@ __device__ __forceinline__ void bulk_march(const StepArgs<T> &A, const int4 sg, 
   const P half = splat(T(0.5)), zero = splat(T(0));
   const bool same_base = A.base[0] != nullptr && A.base[0] == A.src.f[0] && A.base[1] == A.src.f[1] &&
                          A.base[2] == A.src.f[2] && A.base[3] == A.src.f[3] && A.base[4] == A.src.f[4];
+  const bool base_ahead = A.base[0] != nullptr && !same_base;
+  constexpr int SECT = 32 / (2 * (int)sizeof(T));   // threads (column pairs) per 32-byte sector
   const int self = TL::ri(2 * tx, ty);
 
   auto RAWP = [&](int L) -> const T * { return raw + (L % TL::SLOTS) * 5 * NP; };
@@ -458,6 +460,14 @@ __device__ __forceinline__ void bulk_march(const StepArgs<T> &A, const int4 sg, 
     }
     __syncthreads();
     request(p + 2 <= p1 ? p + 2 : -1);
+    // stages whose base is another state than the source: the base values of
+    // the level updated two levels on start their way from HBM to L2 now
+    // (one thread per 32-byte sector; cidx is this thread's position on level k)
+    if (base_ahead && (tx & (SECT - 1)) == 0 && jin && i < D.nx && k + 2 >= kbeg && k + 2 < kend) {
+      const long long c2 = cidx + 2 * D.nxy;
+#pragma unroll
+      for (int f = 0; f < 5; ++f) asm volatile("prefetch.global.L2 [%0];" ::"l"(A.base[f] + c2));
+    }
 
     // ---- phase 2a: own window; x / y faces of level p
     // (on the tensor-memory path the own values of level p stay in registers
@@ -597,17 +607,22 @@ __device__ __forceinline__ void bulk_march(const StepArgs<T> &A, const int4 sg, 
         d[4] = pfma(psub(fzw, zw), izf, q0[3]);
         const bool both = k >= kfx && k >= kfy;
         const P dtp = splat(A.dtT);
+        if (same_base) {
+#pragma unroll
+          for (int f = 0; f < 5; ++f) d[f] = pfma(d[f], dtp, ld2(Rk + f * NP + self));
+        } else if (A.base[0]) {
+          P b[5];   // every load before the stores, which might alias them for all the compiler knows
+#pragma unroll
+          for (int f = 0; f < 5; ++f) {
+            const T *bp = A.base[f] + cidx;   // element-wise: the pair may end past the last column
+            b[f] = PAIRIO ? ld2(bp) : mk(k >= kfx ? bp[0] : T(0), k >= kfy ? bp[1] : T(0));
+          }
+#pragma unroll
+          for (int f = 0; f < 5; ++f) d[f] = pfma(d[f], dtp, b[f]);
+        }
 #pragma unroll
         for (int f = 0; f < 5; ++f) {
-          P o;
-          if (same_base) {
-            o = pfma(d[f], dtp, ld2(Rk + f * NP + self));
-          } else if (A.base[0]) {
-            const T *b = A.base[f] + cidx;   // element-wise: the pair may end past the last column
-            o = pfma(d[f], dtp, PAIRIO ? ld2(b) : mk(k >= kfx ? b[0] : T(0), k >= kfy ? b[1] : T(0)));
-          } else {
-            o = d[f];
-          }
+          const P o = d[f];
           T *dst = A.out[f] + cidx;
           if (both) {
             if (PAIRIO) st2(dst, o);
