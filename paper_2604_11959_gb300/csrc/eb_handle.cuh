@@ -129,7 +129,7 @@ struct eb_geom_s {
   int src_flags = 0;
   double *src_d[2] = {nullptr, nullptr};
   float *src_f[2] = {nullptr, nullptr};
-  void *src_pp = nullptr;   // p' of every cell, scratch of the source pass
+  void *src_pp = nullptr;   // p' of every cell, scratch of the source pass (double path)
   ProjWork pw;
 
   template <typename P>

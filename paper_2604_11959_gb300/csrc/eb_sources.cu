@@ -15,23 +15,26 @@
 //   p' = p0(k) * expm1(gamma * log1p((rho theta)' / (rho0 theta0)(k)))
 // (the deviation form of p - p0: the float path rounds p', not p ~ 1e5 Pa);
 // p0(k) and 1 / (rho0 theta0)(k) are per-level tables built in double when
-// the sources are switched on.  A first pass writes p' of every fluid cell
-// (k_pressure), the second forms the sources (k_sources).
+// the sources are switched on.
 #include "eb_step.cuh"
+
+#include <algorithm>
 
 namespace {
 
 template <typename T>
 struct SourceArgs {
   Dims D;
+  const int *kfast;          // from here up a column's cells, and theirs to the low sides, hold fluid
   const uint8_t *cflag;      // dense flags of the c grid (bit 0: holds fluid)
   const uint8_t *gflag[3];   // of the u, v, w grids
   const T *rho, *rt;         // rho', (rho theta)' of the stage's source state
   T *out[3];                 // rho*u, rho*v, rho*w of the stage's output
   const T *p0, *irt0;        // per level: p0, 1 / (rho0 theta0)
-  T *pp;                     // p' of every fluid cell (written by k_pressure)
+  T *pp;                     // double path: p' of every fluid cell (written by k_pressure)
   T dt, gamma, grav, inv[3];
   int pressure, buoyancy;
+  int strips, tiles, slabs;  // y strips, x tiles and z slabs of k_sources
   unsigned *status;
 };
 
@@ -40,60 +43,118 @@ __device__ inline double log1p_t(double x) { return log1p(x); }
 __device__ inline float expm1_t(float x) { return expm1f(x); }
 __device__ inline double expm1_t(double x) { return expm1(x); }
 
-// p' of every cell that holds fluid, once per stage (the source pass reads
-// each cell's value for up to six faces)
+template <typename T>
+__device__ inline T p_prime(const SourceArgs<T> &S, long long c, int k) {
+  return S.p0[k] * expm1_t(S.gamma * log1p_t(S.rt[c] * S.irt0[k]));
+}
+
+// double path: p' of every cell that holds fluid, once per stage (FP64
+// logarithms and exponentials are what this costs, so none is formed twice)
 template <typename T>
 __global__ void k_pressure(const __grid_constant__ SourceArgs<T> S) {
   const Dims &D = S.D;
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (t >= D.nxy * (long long)D.nz) return;
   if (!(S.cflag[t] & 1)) return;
-  const int k = (int)D.fnxy.div((unsigned)t);
-  S.pp[t] = S.p0[k] * expm1_t(S.gamma * log1p_t(S.rt[t] * S.irt0[k]));
+  S.pp[t] = p_prime(S, t, (int)D.fnxy.div((unsigned)t));
 }
 
-// one thread per (i, j, k) position: the u and v CVs of level k (k < nz) and
-// the w CV of face level k (0 < k < nz)
-template <typename T>
-__global__ void k_sources(const __grid_constant__ SourceArgs<T> S) {
+// The sources of the u and v CVs of levels 0 .. nz - 1 and the w CVs of face
+// levels 1 .. nz - 1.  HBM bounds it (rho', (rho theta)' and the three momenta
+// read, the momenta written: 32 bytes per cell in float), so one pass does
+// all: a block marches a tile of 32 x SR columns up a slab of levels, one
+// column per thread.  Each level's p' is formed once per cell into a shared
+// plane (two planes, one barrier per level) with the cells beside the tile's
+// low x and y sides; the level below stays in registers.  From a column's
+// kfast up no flag is read.  Every load of a level precedes its stores, which
+// might alias them for all the compiler knows.  256x256x128, float: 80 us (a
+// pass that stored p' and one that read it took 40 + 126); the logarithms and
+// exponentials keep it from the 40 us of its 268 MB.
+constexpr int SR = 8;
+
+template <typename T, bool STORED>
+__global__ void __launch_bounds__(32 * SR) k_sources(const __grid_constant__ SourceArgs<T> S) {
   const Dims &D = S.D;
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= D.nxy * (long long)(D.nz + 1)) return;
-  int i, j, k;
-  split_index(D, (unsigned)t, i, j, k);   // below 2^32 (checked when the handle is built)
-  auto pprime = [&](long long c, int) -> T { return S.pp[c]; };
-  const bool own = k < D.nz && (S.cflag[t] & 1);
-  T p_own = T(0);
-  if (own && S.pressure) p_own = pprime(t, k);
-  bool bad = false;
+  __shared__ T sp[2][SR + 1][33];   // p' at (row, column) = (ty + 1, tx + 1)
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  int w = blockIdx.x;
+  const int slab = w / (S.tiles * S.strips);
+  w -= slab * S.tiles * S.strips;
+  const int strip = w / S.tiles, i0 = (w - strip * S.tiles) * 32, j0 = strip * SR;
+  const int k0 = (int)((long long)D.nz * slab / S.slabs), k1 = (int)((long long)D.nz * (slab + 1) / S.slabs);
+  const bool in = i0 + tx < D.nx && j0 + ty < D.ny;
+  const int i = min(i0 + tx, D.nx - 1), j = min(j0 + ty, D.ny - 1);
+  const int col = i + D.nx * j;
+  const int cl = i == 0 ? col + D.nx - 1 : col - 1, cd = j == 0 ? col + D.nx * (D.ny - 1) : col - D.nx;
+  const int kf = S.kfast[col];
+  // cells beside the tile: row ty == 0 forms those below it, row ty == 1 (its first SR lanes) those left of it
+  int hc = -1, hy = 0, hx = 0, hkf = 0;
+  if (ty == 0) {
+    hc = cd;
+    hx = tx + 1;
+  } else if (ty == 1 && tx < SR) {
+    hc = (i0 == 0 ? D.nx - 1 : i0 - 1) + D.nx * min(j0 + tx, D.ny - 1);
+    hy = tx + 1;
+  }
+  if (hc >= 0) hkf = S.kfast[hc];
+
+  auto value = [&](long long c, int k) -> T {
+    if constexpr (STORED) return S.pp[c];
+    else return p_prime(S, c, k);
+  };
+  T pz = T(0), rz = T(0);
+  bool fz = false, bad = false;
+  if (k0 > 0) {
+    const long long c = col + D.nxy * (long long)(k0 - 1);
+    fz = k0 - 1 >= kf || (S.cflag[c] & 1);
+    if (fz && S.pressure) pz = value(c, k0 - 1);
+    rz = S.rho[c];
+  }
+  for (int k = k0; k < k1; ++k) {
+    const long long b = D.nxy * (long long)k, t = col + b;
+    const bool all = k >= kf;   // the cells and CVs this column's sources read hold fluid
+    const bool own = all || (S.cflag[t] & 1);
+    T m[3];
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    if (d < 2 ? k >= D.nz : (k == 0 || k >= D.nz)) continue;
-    if (!(S.gflag[d][t] & 1)) continue;
-    long long a;
-    int ka = k;
-    if (d == 0) a = (i == 0 ? D.nx - 1 : i - 1) + (long long)D.nx * j + D.nxy * k;
-    else if (d == 1) a = i + (long long)D.nx * (j == 0 ? D.ny - 1 : j - 1) + D.nxy * k;
-    else {
-      a = t - D.nxy;
-      ka = k - 1;
-    }
-    const bool fa = S.cflag[a] & 1;
-    if (!fa && !own) continue;
-    T s = T(0);
+    for (int d = 0; d < 3; ++d) m[d] = S.out[d][t];
+    const T rho = S.rho[t];
+    T p = T(0);
+    T(*P)[33] = sp[k & 1];
     if (S.pressure) {
-      T pa = fa ? pprime(a, ka) : p_own;
-      const T pb = own ? p_own : pa;
-      s -= (pb - pa) * S.inv[d];
+      if (own) p = value(t, k);
+      P[ty + 1][tx + 1] = p;
+      if (hc >= 0 && (k >= hkf || (S.cflag[hc + b] & 1))) P[hy][hx] = value(hc + b, k);
+      __syncthreads();
     }
-    if (S.buoyancy && d == 2) {
-      T ra = fa ? S.rho[a] : S.rho[t];
-      const T rb = own ? S.rho[t] : ra;
-      s -= S.grav * T(0.5) * (ra + rb);
+    if (in) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        if (d == 2 && k == 0) continue;
+        bool fa = true;
+        if (!all) {
+          fa = d == 2 ? fz : S.cflag[(d == 0 ? cl : cd) + b] & 1;
+          if (!(S.gflag[d][t] & 1) || (!fa && !own)) continue;
+        }
+        T s = T(0);
+        if (S.pressure) {
+          T pa = d == 0 ? P[ty + 1][tx] : d == 1 ? P[ty][tx + 1] : pz;
+          if (!fa) pa = p;
+          const T pb = own ? p : pa;
+          s -= (pb - pa) * S.inv[d];
+        }
+        if (S.buoyancy && d == 2) {
+          const T ra = fa ? rz : rho;
+          const T rb = own ? rho : ra;
+          s -= S.grav * T(0.5) * (ra + rb);
+        }
+        const T v = m[d] + S.dt * s;
+        S.out[d][t] = v;
+        bad = bad || !isfinite(v);
+      }
     }
-    const T v = S.out[d][t] + S.dt * s;
-    S.out[d][t] = v;
-    bad = bad || !isfinite(v);
+    pz = p;
+    rz = rho;
+    fz = own;
   }
   if (bad) atomicOr(S.status, EB_DEV_NUMERIC);
 }
@@ -104,6 +165,7 @@ template <typename T>
 void launch_sources(const StepArgs<T> &A, int flags, const T *p0, const T *irt0, T *pp, cudaStream_t s) {
   SourceArgs<T> S;
   S.D = A.D;
+  S.kfast = A.kfast;
   S.cflag = A.G[0].dflag;
   for (int d = 0; d < 3; ++d) {
     S.gflag[d] = A.G[d + 1].dflag;
@@ -123,12 +185,19 @@ void launch_sources(const StepArgs<T> &A, int flags, const T *p0, const T *irt0,
   S.pressure = (flags & EB_SOURCE_PRESSURE) ? 1 : 0;
   S.buoyancy = (flags & EB_SOURCE_BUOYANCY) ? 1 : 0;
   S.status = A.status;
-  if (S.pressure) {
+  constexpr bool STORED = sizeof(T) == sizeof(double);
+  if (STORED && S.pressure) {
     const long long nc = A.D.nxy * (long long)A.D.nz;
     k_pressure<T><<<(unsigned)((nc + 255) / 256), 256, 0, s>>>(S);
   }
-  const long long n = A.D.nxy * (long long)(A.D.nz + 1);
-  k_sources<T><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(S);
+  // slabs of at least four levels (each re-forms the level below its first),
+  // enough of them for about SOURCE_BLOCKS blocks per SM
+  constexpr long long SOURCE_BLOCKS = 16;
+  S.tiles = (A.D.nx + 31) / 32;
+  S.strips = (A.D.ny + SR - 1) / SR;
+  const long long cols = (long long)S.tiles * S.strips;
+  S.slabs = (int)std::max(1LL, std::min<long long>(A.D.nz / 4, (SOURCE_BLOCKS * ebk_sm_count() + cols - 1) / cols));
+  k_sources<T, STORED><<<(unsigned)(cols * S.slabs), dim3(32, SR, 1), 0, s>>>(S);
 }
 
 template void launch_sources<float>(const StepArgs<float> &, int, const float *, const float *, float *,
