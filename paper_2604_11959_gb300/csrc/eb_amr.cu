@@ -24,6 +24,8 @@
 // CV centre along each axis, and a fine unit is half a coarse one.
 #include "eb_handle.cuh"
 
+#include <algorithm>
+
 using namespace ebh;
 
 namespace {
@@ -61,18 +63,6 @@ __device__ inline int fine_cell(const FineC &F, int i, int j, int k, double v[20
     v[16] = F.G.aeb[r];
   }
   return F.G.flag[r];
-}
-
-// the volume fraction (q = 0) or the low q-1 face fraction (q = 1..3) of
-// fine cell (i, j, k) alone: 0 outside the domain or covered, 1 regular
-__device__ inline double fine_frac(const FineC &F, int i, int j, int k, int q) {
-  if (k < 0 || k >= F.D.nz) return 0.0;
-  const int col = wrapi(i, F.D.nx) + F.D.nx * wrapi(j, F.D.ny);
-  const int kc = F.G.kcov[col], kx = F.G.kxt[col];
-  if (k < kc) return 0.0;
-  if (k >= kx) return 1.0;
-  const long long r = F.G.roff[col] + (k - kc);
-  return q == 0 ? F.G.alpha[r] : F.G.beta[(q - 1) * F.G.nrec + r];
 }
 
 // open fraction of the low d-face of fine cell (i, j, k); the lid above the
@@ -230,55 +220,140 @@ struct RestrictArgs {
   int fx0, nxg, I0, ncols;
 };
 
-template <typename T>
-__global__ void k_restrict(const __grid_constant__ RestrictArgs<T> R, int f) {
-  const Dims &Dc = R.Dc;
-  const int g = f <= 1 ? 0 : f - 1;
-  const long long plane = (long long)R.ncols * Dc.ny;
-  const long long n = plane * nzg_of(Dc, g);
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  const int K = (int)(t / plane);
-  const long long c2 = t - (long long)K * plane;
-  const int J = (int)(c2 / R.ncols), It = (int)(c2 - (long long)J * R.ncols);
-  const int I = wrapi(R.I0 + It, Dc.nx);
-  const long long tc = I + (long long)Dc.nx * J + Dc.nxy * K;
-  const Dims &Df = R.F.D;
-  auto local = [&](int gx) { return wrapi(gx - R.fx0, R.nxg); };   // fine global column -> the handle's column
-  double w = 0.0, s = 0.0, sp = 0.0;
-  if (g == 0) {
-    for (int c = 0; c < 2; ++c)
-      for (int b = 0; b < 2; ++b)
-        for (int a = 0; a < 2; ++a) {
-          const int i = local(2 * I + a), j = 2 * J + b, k = 2 * K + c;
-          const double al = fine_frac(R.F, i, j, k, 0);
-          const long long q = i + (long long)Df.nx * j + Df.nxy * k;
-          w += al;
-          s += al * (double)R.uf[f][q];
-          if (R.pf[f]) sp += al * R.pf[f][k];
-        }
-  } else {
-    const int d = g - 1;
-    for (int y = 0; y < 2; ++y)
-      for (int x = 0; x < 2; ++x) {
-        int p[3] = {2 * I, 2 * J, 2 * K};
-        const int t1 = d == 0 ? 1 : 0, t2 = d == 2 ? 1 : 2;
-        p[t1] += x;
-        p[t2] += y;
-        if (p[2] >= Df.nz) continue;   // the lid above the top: a wall of w
-        p[0] = local(p[0]);
-        const double be = fine_frac(R.F, p[0], p[1], p[2], 1 + d);
-        const long long q = p[0] + (long long)Df.nx * p[1] + Df.nxy * p[2];
-        w += be;
-        s += be * (double)R.uf[f][q];
-        if (R.pf[f]) sp += be * R.pf[f][p[2]];
-      }
+// s + e = a + b exactly (float; Knuth's branch-free two-sum)
+__device__ inline void two_sum(float a, float b, float &s, float &e) {
+  s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+
+// the sum of N values and a level constant (hi, lo), scaled by an exact power
+// of two: in double, or for floats as an unevaluated pair (48 bits; rounded
+// to float once), since FP64 instructions would bound both kernels
+template <int N>
+__device__ inline double mean_plus(const double (&v)[N], double hi, double) {
+  double s = v[0];
+#pragma unroll
+  for (int q = 1; q < N; ++q) s += v[q];
+  return s * (1.0 / N) + hi;
+}
+template <int N>
+__device__ inline float mean_plus(const float (&v)[N], float hi, float lo) {
+  float s = v[0], c = 0.f;
+#pragma unroll
+  for (int q = 1; q < N; ++q) {
+    float e;
+    two_sum(s, v[q], s, e);
+    c = __fadd_rn(c, e);
   }
-  if (w > 0.0) {
-    double val = s / w;
-    if (R.pf[f]) val += sp / w;
-    if (R.pc[f]) val -= R.pc[f][K];
-    R.uc[f][tc] = (T)val;
+  constexpr float inv = 1.f / N;   // exact: N is 1, 2, 4 or 8
+  float t, e;
+  two_sum(__fmul_rn(s, inv), hi, t, e);
+  return __fadd_rn(t, __fadd_rn(e, __fmaf_rn(c, inv, lo)));
+}
+// a double constant as (hi, lo) of type T
+__device__ inline void split_const(double d, double &hi, double &lo) { hi = d, lo = 0.0; }
+__device__ inline void split_const(double d, float &hi, float &lo) { hi = (float)d, lo = (float)(d - (double)hi); }
+
+// The coarse CVs at (I, J, K) of all five fields where fine cells are cut or
+// covered: the eight fine cells' fractions are looked up once (one chain of
+// column, offset and record loads), then weight every field in double.
+template <typename T>
+__device__ inline void restrict_cut(const RestrictArgs<T> &R, const int cols[4], long long b0, int K, long long tc) {
+  const FineC &F = R.F;
+  const Dims &Df = F.D;
+  const int *kv = F.G.kcov;
+  if (min(min(kv[cols[0]], kv[cols[1]]), min(kv[cols[2]], kv[cols[3]])) > 2 * K + 1) return;   // all covered
+  double w[4][8];   // volume fraction, low x, y, z face fractions of fine cell a + 2 b + 4 c
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int col = cols[q], kc = F.G.kcov[col], kx = F.G.kxt[col];
+    const long long ro = F.G.roff[col];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int k = 2 * K + c, e = q + 4 * c;
+      const bool rec = k >= kc && k < kx;
+      const long long r = ro + (k - kc);
+#pragma unroll
+      for (int m = 0; m < 4; ++m)
+        w[m][e] = rec ? (m ? F.G.beta[(m - 1) * F.G.nrec + r] : F.G.alpha[r]) : (k < kc ? 0.0 : 1.0);
+    }
+  }
+#pragma unroll
+  for (int f = 0; f < 5; ++f) {
+    const int m = f <= 1 ? 0 : f - 1;
+    double ws = 0.0, s = 0.0, sp = 0.0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      if (m && ((e >> (m - 1)) & 1)) continue;   // a face field: the four cells on the coarse low face
+      const double we = w[m][e];
+      ws += we;
+      s += we * (double)R.uf[f][b0 + cols[e & 3] + (e >> 2) * Df.nxy];
+      if (R.pf[f]) sp += we * R.pf[f][2 * K + (e >> 2)];
+    }
+    if (ws > 0.0) {
+      double val = s / ws;
+      if (R.pf[f]) val += sp / ws;
+      if (R.pc[f]) val -= R.pc[f][K];
+      R.uc[f][tc] = (T)val;
+    }
+  }
+}
+
+// All five fields of one coarse level per blockIdx.y (the lid face above the
+// top level keeps its value).  HBM bounds it: where the four fine columns are
+// regular, every value is a plain mean of 8 (4) fine ones plus a constant of
+// the level, formed without FP64 on the float path.  64 x 256 x 128 fine cells
+// onto 32 x 128 x 64: 37 us, the FP64 sums over the cut cells most of it
+// (130 us for one launch per field with double sums over looked-up fractions).
+template <typename T>
+__global__ void __launch_bounds__(256) k_restrict(const __grid_constant__ RestrictArgs<T> R) {
+  const Dims &Dc = R.Dc, &Df = R.F.D;
+  __shared__ T chi[4], clo[4];   // per field: mean fine profile minus the coarse one
+  const unsigned n = (unsigned)R.ncols * (unsigned)Dc.ny;
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int J = (int)(t / (unsigned)R.ncols), It = (int)(t - (unsigned)J * (unsigned)R.ncols);
+  const int I = wrapi(R.I0 + It, Dc.nx);
+  for (int K = blockIdx.y; K < Dc.nz; K += gridDim.y) {
+    __syncthreads();
+    if (threadIdx.x < 4) {
+      const int f = threadIdx.x;
+      double d = 0.0;
+      if (R.pf[f]) d += 0.5 * (R.pf[f][2 * K] + R.pf[f][2 * K + 1]);
+      if (R.pc[f]) d -= R.pc[f][K];
+      split_const(d, chi[f], clo[f]);
+    }
+    __syncthreads();
+    if (t >= n) continue;
+    const long long tc = I + (long long)Dc.nx * J + Dc.nxy * K;
+    const int x0 = wrapi(2 * I - R.fx0, R.nxg), x1 = wrapi(2 * I + 1 - R.fx0, R.nxg);
+    const int c00 = x0 + Df.nx * (2 * J), c10 = x1 + Df.nx * (2 * J), c01 = c00 + Df.nx, c11 = c10 + Df.nx;
+    const int *kx = R.F.G.kxt;
+    if (max(max(kx[c00], kx[c10]), max(kx[c01], kx[c11])) > 2 * K) {
+      const int cols[4] = {c00, c10, c01, c11};
+      restrict_cut(R, cols, Df.nxy * (2LL * K), K, tc);
+      continue;
+    }
+    const long long b0 = Df.nxy * (2LL * K), b1 = b0 + Df.nxy;
+    T o[5];
+#pragma unroll
+    for (int f = 0; f < 2; ++f) {
+      const T *u = R.uf[f];
+      const T v[8] = {u[b0 + c00], u[b0 + c10], u[b0 + c01], u[b0 + c11],
+                      u[b1 + c00], u[b1 + c10], u[b1 + c01], u[b1 + c11]};
+      o[f] = mean_plus<8>(v, chi[f], clo[f]);
+    }
+    {
+      const T *u = R.uf[2], *v = R.uf[3], *w = R.uf[4];
+      const T vu[4] = {u[b0 + c00], u[b0 + c01], u[b1 + c00], u[b1 + c01]};
+      const T vv[4] = {v[b0 + c00], v[b0 + c10], v[b1 + c00], v[b1 + c10]};
+      const T vw[4] = {w[b0 + c00], w[b0 + c10], w[b0 + c01], w[b0 + c11]};
+      o[2] = mean_plus<4>(vu, chi[2], clo[2]);
+      o[3] = mean_plus<4>(vv, chi[3], clo[3]);
+      o[4] = mean_plus<4>(vw, T(0), T(0));
+    }
+#pragma unroll
+    for (int f = 0; f < 5; ++f) R.uc[f][tc] = o[f];
   }
 }
 
@@ -296,36 +371,57 @@ struct ProlongArgs {
   int fx0, nxg, lo, hi;
 };
 
+// One fine level per blockIdx.y, all five fields of the columns outside [lo,
+// hi) (the level above the top holds rho*w only).  HBM bounds it; a value
+// costs one addition of the level's profile difference (as on the
+// restriction's float path, without FP64).  24 of 88 columns x 256 x 128: 16
+// us (127 us for one launch per field over all columns).
 template <typename T>
-__global__ void k_prolong(const __grid_constant__ ProlongArgs<T> P, int f) {
+__global__ void __launch_bounds__(256) k_prolong(const __grid_constant__ ProlongArgs<T> P) {
   const Dims &Df = P.Df, &Dc = P.Dc;
-  const int g = f <= 1 ? 0 : f - 1;
-  const long long n = Df.nxy * (long long)nzg_of(Df, g);
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  int i, j, k;
-  split_index(Df, (unsigned)t, i, j, k);
-  if (i >= P.lo && i < P.hi) return;   // an owned column
+  __shared__ T chi[4], clo[4];   // per field: coarse profile minus the fine one
+  const unsigned cols = (unsigned)(Df.nx - (P.hi - P.lo));
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = (int)(t / cols);
+  int i = (int)(t - (unsigned)j * cols);
+  if (i >= P.lo) i += P.hi - P.lo;   // the owned columns are left out
   const int gi = wrapi(P.fx0 + i, P.nxg);
-  int c[3] = {gi / 2, j / 2, k / 2};
-  const int fc[3] = {gi, j, k};
-  auto full = [&](int I, int J, int K) -> double {
-    const double u = (double)P.uc[f][I + (long long)Dc.nx * J + Dc.nxy * K];
-    return P.pc[f] ? u + P.pc[f][K] : u;
-  };
-  double val;
-  const int d = g - 1;
-  if (g == 0 || fc[d] % 2 == 0) {
-    val = full(c[0], c[1], c[2]);
-  } else {
-    int e[3] = {c[0], c[1], c[2]};
-    e[d] += 1;
-    if (d == 0) e[0] = wrapi(e[0], Dc.nx);
-    if (d == 1) e[1] = wrapi(e[1], Dc.ny);
-    val = 0.5 * (full(c[0], c[1], c[2]) + full(e[0], e[1], e[2]));
+  const int I = gi / 2, J = j / 2;
+  for (int k = blockIdx.y; k <= Df.nz; k += gridDim.y) {
+    const int K = k / 2;
+    __syncthreads();
+    if (threadIdx.x < 4 && k < Df.nz) {
+      const int f = threadIdx.x;
+      double d = 0.0;
+      if (P.pc[f]) d += P.pc[f][K];
+      if (P.pf[f]) d -= P.pf[f][k];
+      split_const(d, chi[f], clo[f]);
+    }
+    __syncthreads();
+    if (t >= cols * (unsigned)Df.ny) continue;
+    const long long c = I + (long long)Dc.nx * J + Dc.nxy * K;
+    const long long q = i + (long long)Df.nx * j + Df.nxy * k;
+    // one value, or the mean of the two coarse faces around an odd fine face
+    auto mean = [&](int f, bool odd, long long c2, T hi, T lo) -> T {
+      const T v[2] = {P.uc[f][c], odd ? P.uc[f][c2] : T(0)};
+      if (odd) return mean_plus<2>(v, hi, lo);
+      const T one[1] = {v[0]};
+      return mean_plus<1>(one, hi, lo);
+    };
+    T o[5];
+    if (k < Df.nz) {
+#pragma unroll
+      for (int f = 0; f < 2; ++f) o[f] = mean(f, false, c, chi[f], clo[f]);
+      o[2] = mean(2, gi & 1, c - I + wrapi(I + 1, Dc.nx), chi[2], clo[2]);
+      o[3] = mean(3, j & 1, c + (long long)Dc.nx * (wrapi(J + 1, Dc.ny) - J), chi[3], clo[3]);
+    }
+    o[4] = mean(4, k & 1, c + Dc.nxy, T(0), T(0));
+    if (k < Df.nz) {
+#pragma unroll
+      for (int f = 0; f < 4; ++f) P.uf[f][q] = o[f];
+    }
+    P.uf[4][q] = o[4];
   }
-  if (P.pf[f]) val -= P.pf[f][k];
-  P.uf[f][t] = (T)val;
 }
 
 }  // namespace
@@ -364,11 +460,9 @@ static void restrict_t(eb_geom fine, eb_geom coarse, const eb_state *Uf, eb_stat
     R.pf[f] = f <= 3 ? fine->ref_d[f] : nullptr;
     R.pc[f] = f <= 3 ? coarse->ref_d[f] : nullptr;
   }
-  for (int f = 0; f < 5; ++f) {
-    const int g = f <= 1 ? 0 : f - 1;
-    const long long n = (long long)R.ncols * coarse->D.ny * nzg_of(coarse->D, g);
-    if (n > 0) k_restrict<T><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(R, f);
-  }
+  const long long n = (long long)R.ncols * coarse->D.ny;
+  const unsigned gy = (unsigned)std::min(coarse->D.nz, 65535);
+  if (n > 0) k_restrict<T><<<dim3((unsigned)((n + 255) / 256), gy, 1), 256, 0, s>>>(R);
 }
 
 template <typename T>
@@ -388,11 +482,9 @@ static void prolong_t(eb_geom coarse, const eb_state *Uc, eb_geom fine, eb_state
     P.pf[f] = f <= 3 ? fine->ref_d[f] : nullptr;
     P.pc[f] = f <= 3 ? coarse->ref_d[f] : nullptr;
   }
-  for (int f = 0; f < 5; ++f) {
-    const int g = f <= 1 ? 0 : f - 1;
-    const long long n = fine->D.nxy * (long long)nzg_of(fine->D, g);
-    k_prolong<T><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(P, f);
-  }
+  const long long n = (long long)(fine->D.nx - (hi - lo)) * fine->D.ny;
+  const unsigned gy = (unsigned)std::min(fine->D.nz + 1, 65535);
+  if (n > 0) k_prolong<T><<<dim3((unsigned)((n + 255) / 256), gy, 1), 256, 0, s>>>(P);
 }
 
 // the fine handle is the coarse level's fine level over fine columns fx0 ..
