@@ -47,7 +47,9 @@ struct MgLevel {
   Dims D;
   float ix2 = 0, iy2 = 0, iz2 = 0;
   float *bx = nullptr, *by = nullptr, *bz = nullptr;   // low-face open fractions
-  float *x = nullptr, *t = nullptr, *b = nullptr;      // correction, sweep target, right-hand side (coarse levels)
+  float *x = nullptr, *t = nullptr, *b = nullptr;      // correction, sweep target, right-hand side
+  float *wi = nullptr;                                 // Jacobi weight over the diagonal
+  int *kreg = nullptr;                                 // per column: every face within two columns open from here up
   int nb = 0;                                          // blocks of its kernels
 };
 constexpr int kMgMaxLevels = 16;
@@ -65,6 +67,8 @@ struct ProjWork {
   double *id = nullptr;        // its reciprocal (0 off the active cells): the Jacobi preconditioner
   double *rhs = nullptr, *r = nullptr, *z = nullptr, *p = nullptr, *q = nullptr, *x = nullptr;
   double *part = nullptr;      // partial sums, 8 slots of nb
+  int nrz = 0;                 // multigrid: partial sums of r.z, and their two slots
+  double *part_rz = nullptr;
   int *conv = nullptr;         // iteration count at convergence (0 = not yet)
   double *alpha = nullptr;     // c-cell volume fractions (warm-start input), on first use
   float *nin = nullptr, *nout = nullptr;   // network input (2 channels) and output, on first use

@@ -22,6 +22,8 @@
 
 #include <math.h>
 
+#include <algorithm>
+
 using namespace ebh;
 
 namespace {
@@ -35,16 +37,17 @@ __device__ inline double warp_sum(double v) {
   return v;
 }
 
-// Sum over the block; thread 0 writes it to part[blockIdx.x].
+// Sum over the block (PB threads in any shape); one thread writes it to part[blockIdx.x].
 __device__ inline void block_partial(double v, double *part) {
   __shared__ double s[PB / 32];
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
   v = warp_sum(v);
-  if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
+  if ((tid & 31) == 0) s[tid >> 5] = v;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    double a = threadIdx.x < PB / 32 ? s[threadIdx.x] : 0.0;
+  if (tid < 32) {
+    double a = tid < PB / 32 ? s[tid] : 0.0;
     a = warp_sum(a);
-    if (threadIdx.x == 0) part[blockIdx.x] = a;
+    if (tid == 0) part[blockIdx.x] = a;
   }
 }
 
@@ -167,8 +170,8 @@ __global__ void k_center(Op O, double *rhs, const double *psum, const double *pc
 }
 
 // r = -rhs - A x, z = r / d, p = z
-__global__ void k_init(Op O, const double *x, const double *rhs, double *r, double *z, double *p, double *prz,
-                       double *prr) {
+__global__ void k_init(Op O, const double *x, const double *rhs, double *r, float *rf, double *z, double *p,
+                       double *prz, double *prr) {
   const Dims &D = O.D;
   const long long N = D.nxy * D.nz;
   double rz = 0.0, rr = 0.0;
@@ -179,6 +182,7 @@ __global__ void k_init(Op O, const double *x, const double *rhs, double *r, doub
       zv = rv * O.id[c];
     }
     r[c] = rv;
+    if (rf) rf[c] = (float)rv;   // the V-cycle's right-hand side
     z[c] = zv;
     p[c] = zv;
     rz += rv * zv;
@@ -207,18 +211,20 @@ __global__ void k_apply(Op O, const double *p, double *q, double *ppq, const int
 // alpha = rz / pq; x += alpha p; r -= alpha q; z = r / d (Jacobi; the
 // multigrid preconditioner forms z and r.z afterwards)
 template <bool JAC>
-__global__ void k_update(Op O, double *x, const double *p, const double *q, double *r, double *z, const double *ppq,
-                         const double *prz, double *prz_next, double *prr, int nb, const int *conv) {
+__global__ void k_update(Op O, double *x, const double *p, const double *q, double *r, float *rf, double *z,
+                         const double *ppq, const double *prz, int nrz, double *prz_next, double *prr, int nb,
+                         const int *conv) {
   if (*conv) return;
   const Dims &D = O.D;
   const long long N = D.nxy * D.nz;
-  const double alpha = total(prz, nb) / total(ppq, nb);
+  const double alpha = total(prz, nrz) / total(ppq, nb);
   double rz = 0.0, rr = 0.0;
   for (long long c = blockIdx.x * (long long)PB + threadIdx.x; c < N; c += (long long)gridDim.x * PB) {
     if (O.d[c] > 0.0) {
       x[c] += alpha * p[c];
       const double rv = r[c] - alpha * q[c];
       r[c] = rv;
+      if (!JAC) rf[c] = (float)rv;
       if (JAC) {
         const double zv = rv * O.id[c];
         z[c] = zv;
@@ -236,7 +242,7 @@ __global__ void k_update(Op O, double *x, const double *p, const double *q, doub
 
 // convergence test; else p = z + (rz_next / rz) p
 __global__ void k_direction(Op O, double *p, const double *z, const double *prz, const double *prz_next,
-                            const double *prr, int nb, double thr2, int it, int *conv) {
+                            int nrz, const double *prr, int nb, double thr2, int it, int *conv) {
   if (*conv) return;
   const Dims &D = O.D;
   const long long N = D.nxy * D.nz;
@@ -245,7 +251,7 @@ __global__ void k_direction(Op O, double *p, const double *z, const double *prz,
     if (blockIdx.x == 0 && threadIdx.x == 0) *conv = it + 1;
     return;
   }
-  const double beta = total(prz_next, nb) / total(prz, nb);
+  const double beta = total(prz_next, nrz) / total(prz, nrz);
   for (long long c = blockIdx.x * (long long)PB + threadIdx.x; c < N; c += (long long)gridDim.x * PB)
     p[c] = z[c] + beta * p[c];
 }
@@ -287,12 +293,16 @@ constexpr float MG_OMEGA = 0.9f;
 // outer iterations, and fewer sweeps cost less (16: 7.6 ms, 64: 8.0 ms).
 constexpr int MG_COARSE_SWEEPS = 16;
 
-// the operator of one level: S = sum_f a_f x_nb (off-diagonal part) and the
-// diagonal d = sum_f a_f, from the six face coefficients of cell c
+// The operator of one level.  From kreg[column] up, every face of the cells
+// within two columns is fully open (the terrain lies below), so there, away
+// from the floor and the lid, the kernels read no coefficient at all.
 struct Op32 {
   Dims D;
-  const float *bx, *by, *bz;
+  const float *bx, *by, *bz;   // low-face open fractions
+  const float *wi;             // MG_OMEGA / diagonal (0 off the active cells)
+  const int *kreg;
   float ix2, iy2, iz2;
+  // off-diagonal sum and diagonal of cell c (grid-stride form; coarsest grids and set-up)
   __device__ inline void parts(const float *x, long long c, float &S, float &d) const {
     const Nbr n = neighbours(D, c);
     const float axl = bx[c] * ix2, axh = bx[n.xp] * ix2, ayl = by[c] * iy2, ayh = by[n.yp] * iy2;
@@ -308,6 +318,38 @@ struct Op32 {
     return (bx[c] + bx[n.xp]) * ix2 + (by[c] + by[n.yp]) * iy2 + bz[c] * iz2 + azh;
   }
 };
+
+__global__ void k_mg_winv(Op32 L, float *wi) {
+  const long long N = L.D.nxy * L.D.nz;
+  for (long long c = blockIdx.x * (long long)PB + threadIdx.x; c < N; c += (long long)gridDim.x * PB) {
+    const float d = L.diag(c);
+    wi[c] = d > 0.f ? MG_OMEGA / d : 0.f;
+  }
+}
+
+// top[col]: the level from which every low face of the column's cells is
+// fully open (the floor's z face apart)
+template <typename F>
+__global__ void k_open_top(Dims D, const F *bx, const F *by, const F *bz, int *top) {
+  const int col = blockIdx.x * blockDim.x + threadIdx.x;
+  if (col >= D.nxy) return;
+  int k = D.nz;
+  while (k > 0) {
+    const long long c = col + D.nxy * (long long)(k - 1);
+    if (bx[c] != F(1) || by[c] != F(1) || (k > 1 && bz[c] != F(1))) break;
+    --k;
+  }
+  top[col] = k;
+}
+__global__ void k_open_box(Dims D, const int *top, int *kreg) {
+  const int col = blockIdx.x * blockDim.x + threadIdx.x;
+  if (col >= D.nxy) return;
+  const int i = col % D.nx, j = col / D.nx;
+  int k = 0;
+  for (int dj = -2; dj <= 2; ++dj)
+    for (int di = -2; di <= 2; ++di) k = max(k, top[wrapmod(i + di, D.nx) + D.nx * wrapmod(j + dj, D.ny)]);
+  kreg[col] = k;
+}
 
 // level 0: float copies of the open fractions
 __global__ void k_mg_copy(long long N, const double *bx, const double *by, const double *bz, float *fx, float *fy,
@@ -333,177 +375,410 @@ __global__ void k_mg_coarsen(Op32 F, Dims C, float *bx, float *by, float *bz) {
   }
 }
 
-// one damped Jacobi sweep, xout = (1 - w) xin + w (b + S(xin)) / d (xin = 0
-// when first); B is the right-hand side's type (the FP64 residual on level
-// 0).  FINAL: the finest level's last sweep, which writes the FP64 z and the
-// block partials of r.z.
-template <typename B, bool FINAL>
-__global__ void k_mg_sweep(Op32 L, const float *xin, float *xout, double *zout, const B *b, int first, double *prz,
-                           const int *conv) {
-  if (*conv) return;
-  const long long N = L.D.nxy * L.D.nz;
-  double rz = 0.0;
-  for (long long c = blockIdx.x * (long long)PB + threadIdx.x; c < N; c += (long long)gridDim.x * PB) {
-    float v = 0.f;
-    if (first) {
-      const float d = L.diag(c);
-      if (d > 0.f) v = MG_OMEGA * (float)b[c] / d;
-    } else {
-      float S, d;
-      L.parts(xin, c, S, d);
-      if (d > 0.f) v = (1.f - MG_OMEGA) * xin[c] + MG_OMEGA * ((float)b[c] + S) / d;
-    }
-    if (FINAL) {
-      zout[c] = (double)v;
-      rz += (double)b[c] * (double)v;
-    } else {
-      xout[c] = v;
-    }
+// V adjacent values of a row
+template <int V>
+struct Vec {
+  float v[V];
+};
+template <int V>
+__device__ inline Vec<V> ldv(const float *p) {
+  Vec<V> o;
+  if constexpr (V == 4) {
+    const float4 t = *reinterpret_cast<const float4 *>(p);
+    o.v[0] = t.x, o.v[1] = t.y, o.v[2] = t.z, o.v[3] = t.w;
+  } else if constexpr (V == 2) {
+    const float2 t = *reinterpret_cast<const float2 *>(p);
+    o.v[0] = t.x, o.v[1] = t.y;
+  } else {
+    o.v[0] = p[0];
   }
-  if (FINAL) block_partial(rz, prz);
+  return o;
+}
+template <int V>
+__device__ inline void stv(float *p, const Vec<V> &a) {
+  if constexpr (V == 4) *reinterpret_cast<float4 *>(p) = make_float4(a.v[0], a.v[1], a.v[2], a.v[3]);
+  else if constexpr (V == 2) *reinterpret_cast<float2 *>(p) = make_float2(a.v[0], a.v[1]);
+  else p[0] = a.v[0];
 }
 
-// coarse right-hand side: the mean of the eight children's residuals b - A x
-template <typename B>
-__global__ void k_mg_restrict(Op32 F, const float *x, const B *b, Dims C, float *bc, const int *conv) {
-  if (*conv) return;
-  const long long N = C.nxy * C.nz;
-  const long long sy = F.D.nx, sz = F.D.nxy;
-  for (long long c = blockIdx.x * (long long)PB + threadIdx.x; c < N; c += (long long)gridDim.x * PB) {
-    int I, J, K;
-    split_index(C, (unsigned)c, I, J, K);
-    const long long f0 = 2LL * I + sy * 2LL * J + sz * 2LL * K;
-    float sum = 0.f;
-    for (int q = 0; q < 8; ++q) {
-      const long long f = f0 + (q & 1) + ((q >> 1) & 1) * sy + (q >> 2) * sz;
-      float S, d;
-      F.parts(x, f, S, d);
-      if (d > 0.f) sum += (float)b[f] - d * x[f] + S;
-    }
-    bc[c] = 0.125f * sum;
-  }
+// Work split of the marching kernels: a thread owns V adjacent columns of one
+// row and walks a slab of levels; a block is MBX x MBY threads.
+constexpr int MBX = 16, MBY = 16;
+static_assert(MBX * MBY == PB, "block sums take PB threads");
+struct Slabs {
+  int nbx, nby, nz;   // blocks along x and y, slabs
+  int blocks() const { return nbx * nby * nz; }
+};
+// enough slabs for about 1536 threads per SM, down to one level each on the
+// small grids, where latency is all that counts
+inline Slabs slabs_of(const Dims &D, int V, int sms) {
+  Slabs S;
+  S.nbx = (D.nx / V + MBX - 1) / MBX;
+  S.nby = (D.ny + MBY - 1) / MBY;
+  const int plane = S.nbx * S.nby;
+  S.nz = std::max(1, std::min(D.nz, (6 * sms + plane - 1) / plane));
+  return S;
+}
+// a thread's columns: offsets within a plane of its own row, the rows beside
+// it and the cells left and right of its V
+struct Cols {
+  int i, j, c, ym, yp, xl, xr, k0, k1;
+  bool in;
+};
+template <int V>
+__device__ inline Cols cols_of(const Dims &D, const Slabs &S) {
+  Cols q;
+  const int sl = blockIdx.x / (S.nbx * S.nby), b = blockIdx.x - sl * S.nbx * S.nby;
+  const int by = b / S.nbx, bx = b - by * S.nbx;
+  q.i = V * (bx * MBX + (int)threadIdx.x);
+  q.j = by * MBY + (int)threadIdx.y;
+  q.in = q.i < D.nx && q.j < D.ny;
+  if (!q.in) q.i = q.j = 0;
+  const int row = D.nx * q.j;
+  q.c = q.i + row;
+  q.ym = q.i + (q.j == 0 ? D.nx * (D.ny - 1) : row - D.nx);
+  q.yp = q.i + (q.j == D.ny - 1 ? 0 : row + D.nx);
+  q.xl = row + (q.i == 0 ? D.nx - 1 : q.i - 1);
+  q.xr = row + (q.i + V == D.nx ? 0 : q.i + V);
+  q.k0 = (int)((long long)D.nz * sl / S.nz);
+  q.k1 = (int)((long long)D.nz * (sl + 1) / S.nz);
+  return q;
 }
 
-// x += the parent's coarse correction (injection), on active cells
-__global__ void k_mg_prolong(Op32 F, Dims C, const float *xc, float *x, const int *conv) {
+// One damped Jacobi sweep, xout = (1 - w) x + w (b + S(x)) / d, of
+//   FIRST    x = w b / d, the sweep from zero (so two sweeps in one pass),
+//   PLAIN    x = xin,
+//   PROLONG  x = xin + the parent's coarse correction (injection; inactive
+//            cells are never read with a nonzero coefficient).
+// FINAL: the finest level's last sweep, which writes the FP64 z and the block
+// partials of r.z.
+// L2 bandwidth bounds it (16 bytes per cell; the level's arrays stay in the
+// 129 MB L2): V = 4 columns per thread with 16-byte accesses, the z
+// neighbours carried in registers, no coefficients above the terrain.
+// 192x192x96: 11 us (PLAIN), 18 (FIRST, two sweeps), 16 (PROLONG); one cell
+// per thread with index splits and six coefficient loads took 29 per sweep
+// and 12 for the prolongation.
+enum { FIRST = 0, PLAIN = 1, PROLONG = 2 };
+template <int V, int MODE, bool FINAL>
+__global__ void __launch_bounds__(MBX * MBY) k_mg_sweep(const __grid_constant__ Op32 L,
+                                                        const __grid_constant__ Slabs SL,
+                                                        const float *__restrict__ xin, const float *__restrict__ xc,
+                                                        const __grid_constant__ Dims C, float *__restrict__ xout,
+                                                        double *__restrict__ zout, const double *__restrict__ r,
+                                                        const float *__restrict__ b, double *prz, const int *conv) {
   if (*conv) return;
-  const long long N = F.D.nxy * F.D.nz;
-  for (long long c = blockIdx.x * (long long)PB + threadIdx.x; c < N; c += (long long)gridDim.x * PB) {
-    if (F.diag(c) > 0.f) {
-      int i, j, k;
-      split_index(F.D, (unsigned)c, i, j, k);
-      x[c] += xc[(i >> 1) + (long long)C.nx * ((j >> 1) + (long long)C.ny * (k >> 1))];
-    }
-  }
-}
-
-// the coarsest grid (at most MG_SMEM_CELLS cells): MG_COARSE_SWEEPS Jacobi
-// sweeps from zero in one block, the grid held in shared memory
-constexpr int MG_SMEM_CELLS = 1024;
-__global__ void k_mg_coarsest_smem(Op32 L, const float *b, float *x, const int *conv) {
-  if (*conv) return;
-  __shared__ float sbx[MG_SMEM_CELLS], sby[MG_SMEM_CELLS], sbz[MG_SMEM_CELLS], sb[MG_SMEM_CELLS];
-  __shared__ float sx[MG_SMEM_CELLS], st[MG_SMEM_CELLS];
-  const int N = (int)(L.D.nxy * L.D.nz);
-  for (int c = threadIdx.x; c < N; c += blockDim.x) {
-    sbx[c] = L.bx[c];
-    sby[c] = L.by[c];
-    sbz[c] = L.bz[c];
-    sb[c] = b[c];
-  }
-  __syncthreads();
-  Op32 S = L;
-  S.bx = sbx;
-  S.by = sby;
-  S.bz = sbz;
-  for (int sw = 0; sw < MG_COARSE_SWEEPS; ++sw) {
-    const float *in = (sw & 1) ? st : sx;
-    float *out = (sw & 1) ? sx : st;
-    for (int c = threadIdx.x; c < N; c += blockDim.x) {
-      float v = 0.f;
-      if (sw == 0) {
-        const float d = S.diag(c);
-        if (d > 0.f) v = MG_OMEGA * sb[c] / d;
+  const Dims &D = L.D;
+  const Cols q = cols_of<V>(D, SL);
+  const float wreg = MG_OMEGA / (2.f * (L.ix2 + L.iy2 + L.iz2));
+  int kr = 0;
+#pragma unroll
+  for (int e = 0; e < V; ++e) kr = max(kr, L.kreg[q.c + e]);
+  // plane offset of the parent of plane offset o in row j (PROLONG)
+  auto parent = [&](int i, int j) { return (i >> 1) + C.nx * (j >> 1); };
+  const int pc = parent(q.i, q.j), pym = parent(q.i, q.j == 0 ? D.ny - 1 : q.j - 1),
+            pyp = parent(q.i, q.j == D.ny - 1 ? 0 : q.j + 1), pxl = parent(q.i == 0 ? D.nx - 1 : q.i - 1, q.j),
+            pxr = parent(q.i + V == D.nx ? 0 : q.i + V, q.j);
+  // x of V cells at plane offset o (parents from po) / of one cell
+  auto vec = [&](int k, int o, int po, bool reg) -> Vec<V> {
+    const long long t = D.nxy * (long long)k + o;
+    Vec<V> a;
+    if constexpr (MODE == FIRST) {
+      a = ldv<V>(b + t);
+      if (reg) {
+#pragma unroll
+        for (int e = 0; e < V; ++e) a.v[e] *= wreg;
       } else {
-        float Sv, d;
-        S.parts(in, c, Sv, d);
-        if (d > 0.f) v = (1.f - MG_OMEGA) * in[c] + MG_OMEGA * (sb[c] + Sv) / d;
+        const Vec<V> w = ldv<V>(L.wi + t);
+#pragma unroll
+        for (int e = 0; e < V; ++e) a.v[e] *= w.v[e];
       }
-      out[c] = v;
+    } else {
+      a = ldv<V>(xin + t);
+      if constexpr (MODE == PROLONG) {
+        const float *p = xc + C.nxy * (long long)(k >> 1) + po;
+#pragma unroll
+        for (int e = 0; e < V; ++e) a.v[e] += p[e >> 1];
+      }
     }
-    __syncthreads();
+    return a;
+  };
+  auto one = [&](int k, int o, int po, bool reg) -> float {
+    const long long t = D.nxy * (long long)k + o;
+    if constexpr (MODE == FIRST) return b[t] * (reg ? wreg : L.wi[t]);
+    else if constexpr (MODE == PROLONG) return xin[t] + xc[C.nxy * (long long)(k >> 1) + po];
+    else return xin[t];
+  };
+  double rz = 0.0;
+  if (q.in) {
+    Vec<V> xm, x0, xp;
+#pragma unroll
+    for (int e = 0; e < V; ++e) xm.v[e] = xp.v[e] = 0.f;
+    if (q.k0 > 0) xm = vec(q.k0 - 1, q.c, pc, false);
+    x0 = vec(q.k0, q.c, pc, false);
+#pragma unroll 2
+    for (int k = q.k0; k < q.k1; ++k) {   // two levels' loads in flight
+      const bool reg = k > kr && k < D.nz - 2;   // open faces in this cell and in its neighbours
+      const long long t = D.nxy * (long long)k;
+      if (k + 1 < D.nz) xp = vec(k + 1, q.c, pc, reg);
+      const Vec<V> ym = vec(k, q.ym, pym, reg), yp = vec(k, q.yp, pyp, reg);
+      const float xl = one(k, q.xl, pxl, reg), xr = one(k, q.xr, pxr, reg);
+      const Vec<V> bv = ldv<V>(b + t + q.c);
+      Vec<V> o;
+      if (reg) {
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+          const float S = L.ix2 * ((e ? x0.v[e ? e - 1 : 0] : xl) + (e + 1 < V ? x0.v[e + 1 < V ? e + 1 : 0] : xr)) +
+                          L.iy2 * (ym.v[e] + yp.v[e]) + L.iz2 * (xm.v[e] + xp.v[e]);
+          o.v[e] = (1.f - MG_OMEGA) * x0.v[e] + wreg * (bv.v[e] + S);
+        }
+      } else {
+        const Vec<V> bx = ldv<V>(L.bx + t + q.c), yl = ldv<V>(L.by + t + q.c), yh = ldv<V>(L.by + t + q.yp),
+                     zl = ldv<V>(L.bz + t + q.c), wi = ldv<V>(L.wi + t + q.c);
+        Vec<V> zh;
+#pragma unroll
+        for (int e = 0; e < V; ++e) zh.v[e] = 0.f;
+        if (k + 1 < D.nz) zh = ldv<V>(L.bz + t + D.nxy + q.c);
+        const float bxr = L.bx[t + q.xr];
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+          const float S = L.ix2 * (bx.v[e] * (e ? x0.v[e ? e - 1 : 0] : xl) +
+                                   (e + 1 < V ? bx.v[e + 1 < V ? e + 1 : 0] * x0.v[e + 1 < V ? e + 1 : 0] : bxr * xr)) +
+                          L.iy2 * (yl.v[e] * ym.v[e] + yh.v[e] * yp.v[e]) +
+                          L.iz2 * (zl.v[e] * xm.v[e] + zh.v[e] * xp.v[e]);
+          o.v[e] = wi.v[e] > 0.f ? (1.f - MG_OMEGA) * x0.v[e] + wi.v[e] * (bv.v[e] + S) : 0.f;
+        }
+      }
+      if constexpr (FINAL) {
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+          const double z = (double)o.v[e];
+          zout[t + q.c + e] = z;
+          rz += r[t + q.c + e] * z;
+        }
+      } else {
+        stv<V>(xout + t + q.c, o);
+      }
+      xm = x0;
+      x0 = xp;
+    }
   }
-  for (int c = threadIdx.x; c < N; c += blockDim.x) x[c] = sx[c];
+  if constexpr (FINAL) block_partial(rz, prz);
+}
+
+// Coarse right-hand side: the mean of the eight children's residuals b - A x.
+// A thread forms V / 2 coarse cells per coarse level from V columns x 2 rows.
+// 192x192x96: 11 us (one coarse cell per thread: 25).
+template <int V>
+__global__ void __launch_bounds__(MBX * MBY) k_mg_restrict(const __grid_constant__ Op32 F, const float *x,
+                                                           const float *b, const __grid_constant__ Dims C,
+                                                           float *bc, int kper, const int *conv) {
+  if (*conv) return;
+  const Dims &D = F.D;
+  const int g = D.nx / V;   // groups of V columns per row
+  const long long t = blockIdx.x * (long long)(MBX * MBY) + threadIdx.y * MBX + threadIdx.x;
+  const long long plane = (long long)g * C.ny;
+  const int sl = (int)(t / plane), u = (int)(t - sl * plane);
+  const int J = u / g, i = V * (u - J * g);
+  const float dreg = 2.f * (F.ix2 + F.iy2 + F.iz2);
+  const int K0 = sl * kper, K1 = min(C.nz, K0 + kper);
+  if (K0 >= C.nz) return;
+  int kr = 0;
+#pragma unroll
+  for (int e = 0; e < V; ++e) kr = max(kr, max(F.kreg[i + e + D.nx * (2 * J)], F.kreg[i + e + D.nx * (2 * J + 1)]));
+  for (int K = K0; K < K1; ++K) {
+    float sum[V / 2];
+#pragma unroll
+    for (int e = 0; e < V / 2; ++e) sum[e] = 0.f;
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const int k = 2 * K + (h >> 1), j = 2 * J + (h & 1);
+      const int row = D.nx * j, o = i + row;
+      const int om = i + (j == 0 ? D.nx * (D.ny - 1) : row - D.nx), op = i + (j == D.ny - 1 ? 0 : row + D.nx);
+      const int ol = row + (i == 0 ? D.nx - 1 : i - 1), orr = row + (i + V == D.nx ? 0 : i + V);
+      const long long pl = D.nxy * (long long)k;
+      const Vec<V> x0 = ldv<V>(x + pl + o), ym = ldv<V>(x + pl + om), yp = ldv<V>(x + pl + op), bv = ldv<V>(b + pl + o);
+      Vec<V> xm, xp;
+#pragma unroll
+      for (int e = 0; e < V; ++e) xm.v[e] = xp.v[e] = 0.f;
+      if (k > 0) xm = ldv<V>(x + pl - D.nxy + o);
+      if (k + 1 < D.nz) xp = ldv<V>(x + pl + D.nxy + o);
+      const float xl = x[pl + ol], xr = x[pl + orr];
+      if (k >= kr && k > 0 && k < D.nz - 1) {
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+          const float S = F.ix2 * ((e ? x0.v[e ? e - 1 : 0] : xl) + (e + 1 < V ? x0.v[e + 1 < V ? e + 1 : 0] : xr)) +
+                          F.iy2 * (ym.v[e] + yp.v[e]) + F.iz2 * (xm.v[e] + xp.v[e]);
+          sum[e / 2] += bv.v[e] - dreg * x0.v[e] + S;
+        }
+      } else {
+        const Vec<V> bx = ldv<V>(F.bx + pl + o), yl = ldv<V>(F.by + pl + o), yh = ldv<V>(F.by + pl + op),
+                     zl = ldv<V>(F.bz + pl + o);
+        Vec<V> zh;
+#pragma unroll
+        for (int e = 0; e < V; ++e) zh.v[e] = 0.f;
+        if (k + 1 < D.nz) zh = ldv<V>(F.bz + pl + D.nxy + o);
+        const float bxr = F.bx[pl + orr];
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+          const float axl = F.ix2 * bx.v[e], axh = F.ix2 * (e + 1 < V ? bx.v[e + 1 < V ? e + 1 : 0] : bxr);
+          const float ayl = F.iy2 * yl.v[e], ayh = F.iy2 * yh.v[e], azl = F.iz2 * zl.v[e], azh = F.iz2 * zh.v[e];
+          const float d = axl + axh + ayl + ayh + azl + azh;
+          const float S = axl * (e ? x0.v[e ? e - 1 : 0] : xl) + axh * (e + 1 < V ? x0.v[e + 1 < V ? e + 1 : 0] : xr) +
+                          ayl * ym.v[e] + ayh * yp.v[e] + azl * xm.v[e] + azh * xp.v[e];
+          if (d > 0.f) sum[e / 2] += bv.v[e] - d * x0.v[e] + S;
+        }
+      }
+    }
+    float *dst = bc + C.nxy * (long long)K + (long long)C.nx * J + (i >> 1);
+#pragma unroll
+    for (int e = 0; e < V / 2; ++e) dst[e] = 0.125f * sum[e];
+  }
 }
 
 // The lower part of the V-cycle (every level from lt down, each at most
-// MG_LOWER_CELLS cells) in one block: the same sweeps, restrictions, coarsest
-// sweeps and prolongations as the multi-block kernels, separated by block
-// barriers instead of launches (these levels are launch-bound otherwise).
-constexpr long long MG_LOWER_CELLS = 8192;
+// MG_LOWER_CELLS cells) in one block, which holds the levels' fractions,
+// diagonals, right-hand sides and corrections in shared memory: the same
+// sweeps, restrictions, coarsest sweeps and prolongations as the multi-block
+// kernels, separated by block barriers instead of launches.  A serial chain
+// of about 30 block-wide passes bounds it, so a pass costs little: a thread
+// walks up whole columns with the z neighbours in registers and its row
+// offsets formed once.  Shared memory: seven floats per cell, at most
+// MG_LOWER_CELLS (1 + 1/8 + ...) cells.  Only a coarsest grid that cannot be
+// coarsened to MG_LOWER_CELLS runs from global memory (SMEM false).
+// 24x24x12 and below: 34 us (48 from global memory, a cell per thread).
+constexpr long long MG_LOWER_CELLS = 7000;
+constexpr int MG_LOWER_SMEM = (int)(MG_LOWER_CELLS * 8 / 7 + 8) * 28;
 struct MgLower {
   Op32 L[kMgMaxLevels];
   float *x[kMgMaxLevels], *t[kMgMaxLevels], *b[kMgMaxLevels];
   int lt, top;
 };
 
-__device__ inline void lower_sweep(const Op32 &L, const float *xin, float *xout, const float *b, bool first) {
-  const long long N = L.D.nxy * L.D.nz;
-  for (long long c = threadIdx.x; c < N; c += blockDim.x) {
-    float v = 0.f;
-    if (first) {
-      const float d = L.diag(c);
-      if (d > 0.f) v = MG_OMEGA * b[c] / d;
-    } else {
-      float S, d;
-      L.parts(xin, c, S, d);
-      if (d > 0.f) v = (1.f - MG_OMEGA) * xin[c] + MG_OMEGA * (b[c] + S) / d;
+// One level as the block sees it.  On the SMEM path the pointers are built
+// from the shared array itself, so that every access compiles to a
+// shared-memory one.
+struct LowerLevel {
+  int nx, ny, nz, n;
+  FastDiv fnx, fnxy;
+  float ix2, iy2, iz2;
+  float *bx, *by, *bz, *wi, *x, *t, *b;
+};
+template <bool SMEM>
+__device__ __forceinline__ LowerLevel lower_level(const MgLower &M, int l, float *smem) {
+  LowerLevel V;
+  const Op32 &L = M.L[l];
+  V.nx = L.D.nx, V.ny = L.D.ny, V.nz = L.D.nz, V.n = (int)(L.D.nxy * L.D.nz);
+  V.fnx = L.D.fnx, V.fnxy = L.D.fnxy;
+  V.ix2 = L.ix2, V.iy2 = L.iy2, V.iz2 = L.iz2;
+  if constexpr (SMEM) {
+    int o = 0;
+    for (int q = M.lt; q < l; ++q) o += 7 * (int)(M.L[q].D.nxy * M.L[q].D.nz);
+    float *q = smem + o;
+    V.bx = q, V.by = q + V.n, V.bz = q + 2 * V.n, V.wi = q + 3 * V.n;
+    V.x = q + 4 * V.n, V.t = q + 5 * V.n, V.b = q + 6 * V.n;
+  } else {
+    V.bx = const_cast<float *>(L.bx), V.by = const_cast<float *>(L.by), V.bz = const_cast<float *>(L.bz);
+    V.wi = const_cast<float *>(L.wi);
+    V.x = M.x[l], V.t = M.t[l], V.b = M.b[l];
+  }
+  return V;
+}
+
+// out = one sweep of xin, or (RES) the residual b - A xin.  A thread takes a
+// column, or a run of levels of it where the block has threads for more.
+template <bool RES>
+__device__ __forceinline__ void lower_pass(const LowerLevel &L, const float *__restrict__ xin,
+                                           float *__restrict__ out) {
+  const int nx = L.nx, ny = L.ny, nz = L.nz, nxy = nx * ny;
+  const float *__restrict__ bx = L.bx, *__restrict__ by = L.by, *__restrict__ bz = L.bz, *__restrict__ wi = L.wi,
+                            *__restrict__ b = L.b;
+  const int per = nxy >= (int)blockDim.x ? nz : max(1, (nz * nxy + (int)blockDim.x - 1) / (int)blockDim.x);
+  for (int u = threadIdx.x; u < nxy * ((nz + per - 1) / per); u += blockDim.x) {
+    const int seg = (int)L.fnxy.div((unsigned)u), col = u - seg * nxy, k0 = seg * per, k1 = min(nz, k0 + per);
+    const int j = (int)L.fnx.div((unsigned)col), i = col - j * nx;
+    const int xl = i == 0 ? nx - 1 : -1, xr = i == nx - 1 ? 1 - nx : 1;
+    const int ym = j == 0 ? nx * (ny - 1) : -nx, yp = j == ny - 1 ? -nx * (ny - 1) : nx;
+    int c = col + nxy * k0;
+    float xm = k0 > 0 ? xin[c - nxy] : 0.f, x0 = xin[c], zl = bz[c];
+#pragma unroll 3
+    for (int k = k0; k < k1; ++k, c += nxy) {
+      const bool up = k + 1 < nz;
+      const float zh = up ? bz[c + nxy] : 0.f, xp = up ? xin[c + nxy] : 0.f;
+      const float bxl = bx[c], bxr = bx[c + xr], byl = by[c], byr = by[c + yp], w = wi[c];
+      const float S = L.ix2 * (bxl * xin[c + xl] + bxr * xin[c + xr]) + L.iy2 * (byl * xin[c + ym] + byr * xin[c + yp]) +
+                      L.iz2 * (zl * xm + zh * xp);
+      float v;
+      if (RES) v = b[c] - (L.ix2 * (bxl + bxr) + L.iy2 * (byl + byr) + L.iz2 * (zl + zh)) * x0 + S;
+      else v = (1.f - MG_OMEGA) * x0 + w * (b[c] + S);
+      out[c] = w > 0.f ? v : 0.f;
+      xm = x0;
+      x0 = xp;
+      zl = zh;
     }
-    xout[c] = v;
   }
   __syncthreads();
 }
+// the sweep from zero
+__device__ __forceinline__ void lower_first(const LowerLevel &L, float *__restrict__ out) {
+  const float *__restrict__ wi = L.wi, *__restrict__ b = L.b;
+#pragma unroll 4
+  for (int c = threadIdx.x; c < L.n; c += blockDim.x) out[c] = wi[c] * b[c];
+  __syncthreads();
+}
 
-__global__ void k_mg_lower(const __grid_constant__ MgLower M, const int *conv) {
+template <bool SMEM>
+__global__ void __launch_bounds__(1024) k_mg_lower(const __grid_constant__ MgLower M, const int *conv) {
   if (*conv) return;
-  for (int l = M.lt; l < M.top; ++l) {
-    const Op32 &F = M.L[l];
-    lower_sweep(F, nullptr, M.t[l], M.b[l], true);
-    lower_sweep(F, M.t[l], M.x[l], M.b[l], false);
-    const Dims &C = M.L[l + 1].D;
-    const long long N = C.nxy * C.nz, sy = F.D.nx, sz = F.D.nxy;
-    for (long long c = threadIdx.x; c < N; c += blockDim.x) {   // as k_mg_restrict
-      int I, J, K;
-      split_index(C, (unsigned)c, I, J, K);
-      const long long f0 = 2LL * I + sy * 2LL * J + sz * 2LL * K;
-      float sum = 0.f;
-      for (int q = 0; q < 8; ++q) {
-        const long long f = f0 + (q & 1) + ((q >> 1) & 1) * sy + (q >> 2) * sz;
-        float S, d;
-        F.parts(M.x[l], f, S, d);
-        if (d > 0.f) sum += M.b[l][f] - d * M.x[l][f] + S;
+  extern __shared__ float lower_smem[];
+  const int lt = M.lt, top = M.top;
+  if constexpr (SMEM) {
+    for (int l = lt; l <= top; ++l) {
+      const LowerLevel V = lower_level<true>(M, l, lower_smem);
+      const float *__restrict__ gx = M.L[l].bx, *__restrict__ gy = M.L[l].by, *__restrict__ gz = M.L[l].bz,
+                                *__restrict__ gw = M.L[l].wi, *__restrict__ gb = M.b[l];
+#pragma unroll 4
+      for (int c = threadIdx.x; c < V.n; c += blockDim.x) {
+        const float a0 = gx[c], a1 = gy[c], a2 = gz[c], a3 = gw[c], a4 = l == lt ? gb[c] : 0.f;
+        V.bx[c] = a0, V.by[c] = a1, V.bz[c] = a2, V.wi[c] = a3, V.b[c] = a4;
       }
-      M.b[l + 1][c] = 0.125f * sum;
     }
     __syncthreads();
   }
-  const int top = M.top;
-  for (int sw = 0; sw < MG_COARSE_SWEEPS; ++sw)   // coarsest sweeps; the result ends in x
-    lower_sweep(M.L[top], (sw & 1) ? M.t[top] : M.x[top], (sw & 1) ? M.x[top] : M.t[top], M.b[top], sw == 0);
-  for (int l = top - 1; l >= M.lt; --l) {
-    const Op32 &F = M.L[l];
-    const Dims &C = M.L[l + 1].D;
-    const long long N = F.D.nxy * F.D.nz;
-    for (long long c = threadIdx.x; c < N; c += blockDim.x) {   // as k_mg_prolong
-      if (F.diag(c) > 0.f) {
-        int i, j, k;
-        split_index(F.D, (unsigned)c, i, j, k);
-        M.x[l][c] += M.x[l + 1][(i >> 1) + (long long)C.nx * ((j >> 1) + (long long)C.ny * (k >> 1))];
-      }
+  for (int l = lt; l < top; ++l) {
+    const LowerLevel V = lower_level<SMEM>(M, l, lower_smem), W = lower_level<SMEM>(M, l + 1, lower_smem);
+    lower_first(V, V.t);
+    lower_pass<false>(V, V.t, V.x);
+    lower_pass<true>(V, V.x, V.t);
+    const int sy = V.nx, sz = V.nx * V.ny;
+    for (int c = threadIdx.x; c < W.n; c += blockDim.x) {   // the children's mean, as k_mg_restrict
+      const int K = (int)W.fnxy.div((unsigned)c), col = c - K * W.nx * W.ny;
+      const int J = (int)W.fnx.div((unsigned)col), I = col - J * W.nx;
+      const float *f = V.t + 2 * I + sy * 2 * J + sz * 2 * K;
+      W.b[c] = 0.125f * (((f[0] + f[1]) + (f[sy] + f[sy + 1])) +
+                         ((f[sz] + f[sz + 1]) + (f[sz + sy] + f[sz + sy + 1])));
     }
     __syncthreads();
-    lower_sweep(F, M.x[l], M.t[l], M.b[l], false);
-    lower_sweep(F, M.t[l], M.x[l], M.b[l], false);
+  }
+  {
+    const LowerLevel V = lower_level<SMEM>(M, top, lower_smem);
+    lower_first(V, V.t);
+    for (int sw = 1; sw < MG_COARSE_SWEEPS; ++sw)   // coarsest sweeps; the result ends in x
+      lower_pass<false>(V, (sw & 1) ? V.t : V.x, (sw & 1) ? V.x : V.t);
+  }
+  for (int l = top - 1; l >= lt; --l) {
+    const LowerLevel V = lower_level<SMEM>(M, l, lower_smem), W = lower_level<SMEM>(M, l + 1, lower_smem);
+    for (int c = threadIdx.x; c < V.n; c += blockDim.x) {   // the parent's correction, as PROLONG
+      const int k = (int)V.fnxy.div((unsigned)c), col = c - k * V.nx * V.ny;
+      const int j = (int)V.fnx.div((unsigned)col), i = col - j * V.nx;
+      V.x[c] += W.x[(i >> 1) + W.nx * ((j >> 1) + W.ny * (k >> 1))];
+    }
+    __syncthreads();
+    lower_pass<false>(V, V.x, V.t);
+    lower_pass<false>(V, V.t, V.x);
+  }
+  if constexpr (SMEM) {
+    const LowerLevel V = lower_level<true>(M, lt, lower_smem);
+    for (int c = threadIdx.x; c < V.n; c += blockDim.x) M.x[lt][c] = V.x[c];
   }
 }
 
@@ -513,6 +788,8 @@ Op32 level_op(const MgLevel &L) {
   O.bx = L.bx;
   O.by = L.by;
   O.bz = L.bz;
+  O.wi = L.wi;
+  O.kreg = L.kreg;
   O.ix2 = L.ix2;
   O.iy2 = L.iy2;
   O.iz2 = L.iz2;
@@ -583,6 +860,8 @@ eb_status setup(eb_geom g, cudaStream_t s) {
   return EB_OK;
 }
 
+int final_blocks(eb_geom g);
+
 // the multigrid hierarchy, on the first projection that uses it
 eb_status mg_setup(eb_geom g, cudaStream_t s) {
   ProjWork &w = g->pw;
@@ -595,8 +874,24 @@ eb_status mg_setup(eb_geom g, cudaStream_t s) {
   L0.ix2 = (float)O0.ix2, L0.iy2 = (float)O0.iy2, L0.iz2 = (float)O0.iz2;
   L0.nb = w.nb;
   const long long N0 = g->D.nxy * g->D.nz;
-  for (float **a : {&L0.bx, &L0.by, &L0.bz, &L0.x, &L0.t}) CUDA_TRY(g->alloc(a, N0), "alloc multigrid level");
+  for (float **a : {&L0.bx, &L0.by, &L0.bz, &L0.x, &L0.t, &L0.b, &L0.wi})
+    CUDA_TRY(g->alloc(a, N0), "alloc multigrid level");
   k_mg_copy<<<L0.nb, PB, 0, s>>>(N0, w.bx, w.by, w.bz, L0.bx, L0.by, L0.bz);
+  // MG_OMEGA / diagonal and the open levels of a level whose fractions are set
+  auto finish = [&](MgLevel &L) -> cudaError_t {
+    cudaError_t e = g->alloc(&L.kreg, L.D.nxy);
+    int *top = nullptr;
+    if (e == cudaSuccess) e = cudaMalloc(&top, sizeof(int) * (size_t)L.D.nxy);
+    if (e != cudaSuccess) return e;
+    const unsigned nb = (unsigned)((L.D.nxy + 127) / 128);
+    k_mg_winv<<<L.nb, PB, 0, s>>>(level_op(L), L.wi);
+    k_open_top<float><<<nb, 128, 0, s>>>(L.D, L.bx, L.by, L.bz, top);
+    k_open_box<<<nb, 128, 0, s>>>(L.D, top, L.kreg);
+    e = cudaStreamSynchronize(s);
+    cudaFree(top);
+    return e;
+  };
+  CUDA_TRY(finish(L0), "multigrid set-up");
   for (int l = 1; l < nlev; ++l) {
     MgLevel &L = w.lev[l];
     const MgLevel &F = w.lev[l - 1];
@@ -612,15 +907,58 @@ eb_status mg_setup(eb_geom g, cudaStream_t s) {
     L.ix2 = 0.25f * F.ix2, L.iy2 = 0.25f * F.iy2, L.iz2 = 0.25f * F.iz2;
     const long long N = C.nxy * C.nz;
     L.nb = (int)std::max(1LL, std::min<long long>(w.nb, (N + PB - 1) / PB));
-    for (float **a : {&L.bx, &L.by, &L.bz, &L.x, &L.t, &L.b}) CUDA_TRY(g->alloc(a, N), "alloc multigrid level");
+    for (float **a : {&L.bx, &L.by, &L.bz, &L.x, &L.t, &L.b, &L.wi})
+      CUDA_TRY(g->alloc(a, N), "alloc multigrid level");
     k_mg_coarsen<<<L.nb, PB, 0, s>>>(level_op(F), C, L.bx, L.by, L.bz);
+    CUDA_TRY(finish(L), "multigrid set-up");
   }
+  w.nrz = final_blocks(g);
+  CUDA_TRY(g->alloc(&w.part_rz, 2LL * w.nrz), "alloc projection work space");
   CUDA_TRY(cudaGetLastError(), "multigrid set-up");
   w.nlev = nlev;
   return EB_OK;
 }
 
-// z = V(r) (FP64 in and out) and the partial sums of r.z into prz
+// columns per thread of a level's marching kernels
+inline int level_v(const MgLevel &L) {
+  if (L.D.nxy * L.D.nz < 4LL * MBX * MBY * ebk_sm_count()) return 1;   // too few threads otherwise
+  return L.D.nx % 4 == 0 ? 4 : L.D.nx % 2 == 0 ? 2 : 1;
+}
+
+template <int MODE, bool FINAL>
+void sweep(const MgLevel &L, const float *xin, const MgLevel *coarse, float *xout, double *zout, const double *r,
+           double *prz, const int *conv, cudaStream_t s) {
+  const int V = level_v(L);
+  const Slabs S = slabs_of(L.D, V, ebk_sm_count());
+  const Op32 O = level_op(L);
+  const Dims C = coarse ? coarse->D : L.D;
+  const float *xc = coarse ? coarse->x : nullptr;
+  const dim3 blk(MBX, MBY, 1);
+  if (V == 4) k_mg_sweep<4, MODE, FINAL><<<S.blocks(), blk, 0, s>>>(O, S, xin, xc, C, xout, zout, r, L.b, prz, conv);
+  else if (V == 2) k_mg_sweep<2, MODE, FINAL><<<S.blocks(), blk, 0, s>>>(O, S, xin, xc, C, xout, zout, r, L.b, prz, conv);
+  else k_mg_sweep<1, MODE, FINAL><<<S.blocks(), blk, 0, s>>>(O, S, xin, xc, C, xout, zout, r, L.b, prz, conv);
+}
+
+// from a level with an even number of columns (it is coarsened)
+void restrict_residual(const MgLevel &F, const float *x, const MgLevel &C, const int *conv, cudaStream_t s) {
+  const int V = F.D.nx % 4 == 0 ? 4 : 2;
+  const long long plane = (long long)(F.D.nx / V) * C.D.ny;
+  // two coarse levels per thread where that leaves about a wave of threads
+  const int kper = plane * C.D.nz >= 2LL * 2048 * ebk_sm_count() ? 2 : 1;
+  const long long n = plane * ((C.D.nz + kper - 1) / kper);
+  const unsigned nb = (unsigned)((n + MBX * MBY - 1) / (MBX * MBY));
+  if (V == 4) k_mg_restrict<4><<<nb, dim3(MBX, MBY, 1), 0, s>>>(level_op(F), x, F.b, C.D, C.b, kper, conv);
+  else k_mg_restrict<2><<<nb, dim3(MBX, MBY, 1), 0, s>>>(level_op(F), x, F.b, C.D, C.b, kper, conv);
+}
+
+// blocks of the sweep that forms r.z (its partial sums)
+int final_blocks(eb_geom g) {
+  const MgLevel &L = g->pw.lev[0];
+  return slabs_of(L.D, level_v(L), ebk_sm_count()).blocks();
+}
+
+// z = V(r) (r in FP64 and, as the finest level's right-hand side, in float)
+// and the partial sums of r.z into prz
 void vcycle(eb_geom g, const double *r, double *z, double *prz, cudaStream_t s) {
   ProjWork &w = g->pw;
   const MgLevel *L = w.lev;
@@ -628,23 +966,15 @@ void vcycle(eb_geom g, const double *r, double *z, double *prz, cudaStream_t s) 
   // levels lt .. top (at most MG_LOWER_CELLS cells each) run in one block; level 0 never does
   int lt = top;
   while (lt > 1 && L[lt - 1].D.nxy * L[lt - 1].D.nz <= MG_LOWER_CELLS) --lt;
-  // level 0: right-hand side r (FP64)
-  {
-    const Op32 O = level_op(L[0]);
-    k_mg_sweep<double, false><<<L[0].nb, PB, 0, s>>>(O, nullptr, L[0].x, nullptr, r, 1, nullptr, w.conv);
-    k_mg_sweep<double, false><<<L[0].nb, PB, 0, s>>>(O, L[0].x, L[0].t, nullptr, r, 0, nullptr, w.conv);
-    k_mg_sweep<double, false><<<L[0].nb, PB, 0, s>>>(O, L[0].t, L[0].x, nullptr, r, 0, nullptr, w.conv);
-    k_mg_restrict<double><<<L[1].nb, PB, 0, s>>>(O, L[0].x, r, L[1].D, L[1].b, w.conv);
-  }
+  // sweeps before and after the coarse correction: three on the finest level, two below
+  sweep<FIRST, false>(L[0], nullptr, nullptr, L[0].t, nullptr, nullptr, nullptr, w.conv, s);
+  sweep<PLAIN, false>(L[0], L[0].t, nullptr, L[0].x, nullptr, nullptr, nullptr, w.conv, s);
+  restrict_residual(L[0], L[0].x, L[1], w.conv, s);
   for (int l = 1; l < lt; ++l) {
-    const Op32 O = level_op(L[l]);
-    k_mg_sweep<float, false><<<L[l].nb, PB, 0, s>>>(O, nullptr, L[l].t, nullptr, L[l].b, 1, nullptr, w.conv);
-    k_mg_sweep<float, false><<<L[l].nb, PB, 0, s>>>(O, L[l].t, L[l].x, nullptr, L[l].b, 0, nullptr, w.conv);
-    k_mg_restrict<float><<<L[l + 1].nb, PB, 0, s>>>(O, L[l].x, L[l].b, L[l + 1].D, L[l + 1].b, w.conv);
+    sweep<FIRST, false>(L[l], nullptr, nullptr, L[l].x, nullptr, nullptr, nullptr, w.conv, s);
+    restrict_residual(L[l], L[l].x, L[l + 1], w.conv, s);
   }
-  if (lt == top && L[top].D.nxy * L[top].D.nz <= MG_SMEM_CELLS) {
-    k_mg_coarsest_smem<<<1, 1024, 0, s>>>(level_op(L[top]), L[top].b, L[top].x, w.conv);
-  } else {
+  {
     MgLower M;
     for (int l = lt; l <= top; ++l) {
       M.L[l] = level_op(L[l]);
@@ -654,21 +984,18 @@ void vcycle(eb_geom g, const double *r, double *z, double *prz, cudaStream_t s) 
     }
     M.lt = lt;
     M.top = top;
-    k_mg_lower<<<1, 1024, 0, s>>>(M, w.conv);
+    static unsigned long long attr = 0;
+    ebk_smem_limit(k_mg_lower<true>, MG_LOWER_SMEM, attr);
+    if (L[lt].D.nxy * L[lt].D.nz <= MG_LOWER_CELLS) k_mg_lower<true><<<1, 1024, MG_LOWER_SMEM, s>>>(M, w.conv);
+    else k_mg_lower<false><<<1, 1024, 0, s>>>(M, w.conv);
   }
   for (int l = lt - 1; l >= 1; --l) {
-    const Op32 O = level_op(L[l]);
-    k_mg_prolong<<<L[l].nb, PB, 0, s>>>(O, L[l + 1].D, L[l + 1].x, L[l].x, w.conv);
-    k_mg_sweep<float, false><<<L[l].nb, PB, 0, s>>>(O, L[l].x, L[l].t, nullptr, L[l].b, 0, nullptr, w.conv);
-    k_mg_sweep<float, false><<<L[l].nb, PB, 0, s>>>(O, L[l].t, L[l].x, nullptr, L[l].b, 0, nullptr, w.conv);
+    sweep<PROLONG, false>(L[l], L[l].x, &L[l + 1], L[l].t, nullptr, nullptr, nullptr, w.conv, s);
+    sweep<PLAIN, false>(L[l], L[l].t, nullptr, L[l].x, nullptr, nullptr, nullptr, w.conv, s);
   }
-  {
-    const Op32 O = level_op(L[0]);
-    k_mg_prolong<<<L[0].nb, PB, 0, s>>>(O, L[1].D, L[1].x, L[0].x, w.conv);
-    k_mg_sweep<double, false><<<L[0].nb, PB, 0, s>>>(O, L[0].x, L[0].t, nullptr, r, 0, nullptr, w.conv);
-    k_mg_sweep<double, false><<<L[0].nb, PB, 0, s>>>(O, L[0].t, L[0].x, nullptr, r, 0, nullptr, w.conv);
-    k_mg_sweep<double, true><<<L[0].nb, PB, 0, s>>>(O, L[0].x, nullptr, z, r, 0, prz, w.conv);
-  }
+  sweep<PROLONG, false>(L[0], L[0].x, &L[1], L[0].t, nullptr, nullptr, nullptr, w.conv, s);
+  sweep<PLAIN, false>(L[0], L[0].t, nullptr, L[0].x, nullptr, nullptr, nullptr, w.conv, s);
+  sweep<PLAIN, true>(L[0], L[0].x, nullptr, nullptr, z, r, prz, w.conv, s);
 }
 
 double host_total(eb_geom g, int slot, cudaStream_t s, cudaError_t &e) {
@@ -737,9 +1064,13 @@ eb_status eb_project_impl(eb_geom g, void *const mom[3], double dt, double rtol,
     if (st != EB_OK) return st;
   }
   CUDA_TRY(cudaMemsetAsync(w.conv, 0, sizeof(int), s), "reset");
-  k_init<<<w.nb, PB, 0, s>>>(O, w.x, w.rhs, w.r, w.z, w.p, w.part + S_RZ0 * w.nb, w.part + S_RR * w.nb);
+  double *const part_rz[2] = {w.part + S_RZ0 * w.nb, w.part + S_RZ1 * w.nb};
+  double *const rz_of[2] = {mg ? w.part_rz : part_rz[0], mg ? w.part_rz + w.nrz : part_rz[1]};
+  const int nrz = mg ? w.nrz : w.nb;   // partial sums of r.z
+  float *rf = mg ? w.lev[0].b : nullptr;
+  k_init<<<w.nb, PB, 0, s>>>(O, w.x, w.rhs, w.r, rf, w.z, w.p, part_rz[0], w.part + S_RR * w.nb);
   if (mg) {   // z = V(r), p = z
-    vcycle(g, w.r, w.z, w.part + S_RZ0 * w.nb, s);
+    vcycle(g, w.r, w.z, rz_of[0], s);
     CUDA_TRY(cudaMemcpyAsync(w.p, w.z, sizeof(double) * N, cudaMemcpyDeviceToDevice, s), "search direction");
   }
   cudaError_t e = cudaSuccess;
@@ -753,18 +1084,18 @@ eb_status eb_project_impl(eb_geom g, void *const mom[3], double dt, double rtol,
   if (bb > 0.0 && rr0 > thr2) {
     int done = 0;
     for (it = 0; it < maxit; ++it) {
-      double *prz = w.part + (it % 2 ? S_RZ1 : S_RZ0) * w.nb;
-      double *prz_next = w.part + (it % 2 ? S_RZ0 : S_RZ1) * w.nb;
+      double *prz = rz_of[it % 2], *prz_next = rz_of[1 - it % 2];
       k_apply<<<w.nb, PB, 0, s>>>(O, w.p, w.q, w.part + S_PQ * w.nb, w.conv);
       if (mg) {
-        k_update<false><<<w.nb, PB, 0, s>>>(O, w.x, w.p, w.q, w.r, w.z, w.part + S_PQ * w.nb, prz, prz_next,
+        k_update<false><<<w.nb, PB, 0, s>>>(O, w.x, w.p, w.q, w.r, rf, w.z, w.part + S_PQ * w.nb, prz, nrz, prz_next,
                                             w.part + S_RR * w.nb, w.nb, w.conv);
         vcycle(g, w.r, w.z, prz_next, s);
       } else {
-        k_update<true><<<w.nb, PB, 0, s>>>(O, w.x, w.p, w.q, w.r, w.z, w.part + S_PQ * w.nb, prz, prz_next,
-                                           w.part + S_RR * w.nb, w.nb, w.conv);
+        k_update<true><<<w.nb, PB, 0, s>>>(O, w.x, w.p, w.q, w.r, nullptr, w.z, w.part + S_PQ * w.nb, prz, nrz,
+                                           prz_next, w.part + S_RR * w.nb, w.nb, w.conv);
       }
-      k_direction<<<w.nb, PB, 0, s>>>(O, w.p, w.z, prz, prz_next, w.part + S_RR * w.nb, w.nb, thr2, it, w.conv);
+      k_direction<<<w.nb, PB, 0, s>>>(O, w.p, w.z, prz, prz_next, nrz, w.part + S_RR * w.nb, w.nb, thr2, it,
+                                      w.conv);
       // the host reads the convergence flag every few iterations (a V-cycle
       // iteration costs far more than a Jacobi one, so it looks sooner)
       if ((it + 1) % (mg ? 4 : 32) == 0 || it + 1 == maxit) {
