@@ -59,20 +59,22 @@ struct ProjWork {
   int nlev = 0;                // levels of the multigrid hierarchy (0: not built yet)
   MgLevel lev[kMgMaxLevels];
   bool ready = false;
-  int nb = 0;                  // blocks of every projection kernel (fixed: deterministic sums)
+  int nb = 0;                  // blocks of the flat projection kernels (fixed: deterministic sums)
   long long nact = 0;          // cells in the solve (diagonal > 0)
   double *bx = nullptr, *by = nullptr, *bz = nullptr;   // low-face open fractions of the c-cells
   double *ax = nullptr, *ay = nullptr, *az = nullptr;   // the same times 1 / delta^2 (the operator's coefficients)
   double *d = nullptr;         // diagonal of -L
   double *id = nullptr;        // its reciprocal (0 off the active cells): the Jacobi preconditioner
   double *rhs = nullptr, *r = nullptr, *z = nullptr, *p = nullptr, *q = nullptr, *x = nullptr;
-  double *part = nullptr;      // partial sums, 8 slots of nb
-  int nrz = 0;                 // multigrid: partial sums of r.z, and their two slots
-  double *part_rz = nullptr;
+  int npart = 0, ncols = 1;    // partial sums per slot; columns per thread of the operator kernel
+  double *part = nullptr;      // partial sums of the solver's dot products, npart per slot
+  double *scal = nullptr;      // their totals, one per slot
+  unsigned *done = nullptr;    // blocks that have added theirs, per slot
+  int *kreg = nullptr;         // per column: every face within two columns open from here up
   int *conv = nullptr;         // iteration count at convergence (0 = not yet)
   double *alpha = nullptr;     // c-cell volume fractions (warm-start input), on first use
   float *nin = nullptr, *nout = nullptr;   // network input (2 channels) and output, on first use
-  double *host = nullptr;      // pinned copy of one slot of partial sums
+  double *host = nullptr;      // pinned copies of the totals and of the convergence flag
 };
 
 struct eb_geom_s {

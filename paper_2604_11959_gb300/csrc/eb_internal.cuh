@@ -43,6 +43,30 @@ inline int ebk_sm_count() {
   return c;
 }
 
+// Chains of short kernels: a kernel launched with launch_chained may be
+// placed on the GPU while the kernel before it on the stream still runs, and
+// waits in chain_begin for that kernel's end (and its memory) before it
+// touches anything.  The 2-4 us between dependent launches shrink to about
+// one.  A chained kernel calls chain_begin first, in every thread.
+__device__ inline void chain_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename... P, typename... A>
+inline void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 #define EBK_COVERED 0
 #define EBK_REGULAR 1
 #define EBK_CUT 2

@@ -13,11 +13,22 @@
 // and -L phi = -rhs is solved by Jacobi-preconditioned conjugate gradients
 // in FP64 to a relative residual.
 //
-// Every kernel runs on a fixed grid of nb blocks with grid-stride loops and
-// writes one partial sum per block; a consumer block adds the nb partials in
-// a fixed order, so the solve is deterministic.  Convergence is detected on
-// the device (the kernels of later iterations return at once) and read by
-// the host every 32 iterations (every 4 with the multigrid preconditioner).
+// Every kernel that forms a dot product writes one partial sum per block; the
+// block that finishes last adds them in a fixed order, so the solve is
+// deterministic and the next kernel reads one number.  Convergence is
+// detected on the device (the kernels of later iterations return at once)
+// and read by the host every 32 iterations (every 4 with the multigrid
+// preconditioner).
+//
+// What bounds an iteration of the outer conjugate gradients is FP64 (two
+// instructions per clock and SM): nine per cell in the operator and its dot
+// product, two each in the update and the direction, conversions from and to
+// float counted like arithmetic.  So the operator's constant rows above the
+// terrain are formed from sums of opposite neighbours, x is updated with the
+// direction (p is read once), floats are widened by integer instructions, and
+// nothing is computed for the mask of inactive cells (their r, p and q are
+// zero).  192x192x96: operator 63 -> 51 us, update 47 -> 24, direction (with x) 24
+// -> 31, right-hand side 116 -> 39, correction 114 -> 51.
 #include "eb_handle.cuh"
 
 #include <math.h>
@@ -30,40 +41,69 @@ namespace {
 
 constexpr int PB = 256;   // threads per block of every projection kernel
 
-enum { S_SUM = 0, S_BB = 1, S_PQ = 2, S_RR = 3, S_RZ0 = 4, S_RZ1 = 5, S_CNT = 6, S_TMP = 7 };
+// slots of the scalars (w.scal), their partial sums (w.part) and counters
+enum { S_SUM = 0, S_BB = 1, S_PQ = 2, S_RR = 3, S_RZ0 = 4, S_RZ1 = 5, S_CNT = 6, S_SLOTS = 7 };
 
 __device__ inline double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
-// Sum over the block (PB threads in any shape); one thread writes it to part[blockIdx.x].
-__device__ inline void block_partial(double v, double *part) {
+// Where a kernel's dot product goes: partial sums (one per block), the total
+// and the count of finished blocks (zero before and after).
+struct Sum {
+  double *part, *total;
+  unsigned *done;
+};
+
+// sum over the block (PB threads in any shape), in every thread of its first warp
+__device__ inline double block_sum(double v) {
   __shared__ double s[PB / 32];
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
   v = warp_sum(v);
+  __syncthreads();
   if ((tid & 31) == 0) s[tid >> 5] = v;
   __syncthreads();
+  double a = 0.0;
   if (tid < 32) {
-    double a = tid < PB / 32 ? s[tid] : 0.0;
+    a = tid < PB / 32 ? s[tid] : 0.0;
     a = warp_sum(a);
-    if (tid == 0) part[blockIdx.x] = a;
+  }
+  return a;
+}
+
+// Adds v over the grid into *S.total: the last block to finish sums every
+// block's partial in the same order whichever block it is.  Every thread of
+// every block calls it, once per Sum and launch.
+__device__ inline void grid_sum(double v, const Sum &S) {
+  __shared__ bool last;
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  const double a = block_sum(v);
+  if (tid == 0) {
+    S.part[blockIdx.x] = a;
+    __threadfence();
+    last = atomicAdd(S.done, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double t = 0.0;
+  for (unsigned q = tid; q < gridDim.x; q += PB) t += __ldcg(S.part + q);
+  t = block_sum(t);
+  if (tid == 0) {
+    *S.total = t;
+    *S.done = 0;
   }
 }
 
-// Total of nb partial sums, the same bits in every block.
-__device__ inline double total(const double *part, int nb) {
-  __shared__ double t;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double a = 0.0;
-    for (int q = threadIdx.x; q < nb; q += 32) a += part[q];
-    a = warp_sum(a);
-    if (threadIdx.x == 0) t = a;
-  }
-  __syncthreads();
-  return t;
+// a float as a double, by integer instructions (FP64 conversions run at the
+// FP64 rate); subnormals, infinities and NaN take the conversion
+__device__ inline double widen(float f) {
+  const unsigned u = __float_as_uint(f), e = u & 0x7f800000u;
+  if (e - 0x00800000u >= 0x7f000000u) return (u << 1) ? (double)f : __hiloint2double((int)u, 0);
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
 }
+__device__ inline double widen(double f) { return f; }
 
 struct Nbr {
   long long xm, xp, ym, yp;
@@ -86,6 +126,7 @@ struct Op {
   Dims D;
   const double *bx, *by, *bz, *d, *id;
   const double *ax, *ay, *az;   // open fractions times 1 / delta^2 (set-up)
+  const int *kreg;        // per column: every face within two columns open from here up
   double ix2, iy2, iz2;   // 1 / delta^2
   // (-L p)_c for an active cell: one product and six fused multiply-adds
   // (FP64 arithmetic, not HBM, bounds this on the GPU)
@@ -117,155 +158,338 @@ __global__ void k_wall(Dims D, double *bz) {
   if (c < D.nxy) bz[c] = 0.0;   // z = 0 carries no flux
 }
 
-__global__ void k_diag(Op O, double *d, double *part) {
+__global__ void k_diag(Op O, double *d, Sum cnt) {
   const Dims &D = O.D;
   const long long N = D.nxy * D.nz;
-  double cnt = 0.0;
+  double n_act = 0.0;
   for (long long c = blockIdx.x * (long long)PB + threadIdx.x; c < N; c += (long long)gridDim.x * PB) {
     const Nbr n = neighbours(D, c);
     const double bzh = n.k + 1 < D.nz ? O.bz[c + D.nxy] : 0.0;
     const double v = (O.bx[c] + O.bx[n.xp]) * O.ix2 + (O.by[c] + O.by[n.yp]) * O.iy2 + (O.bz[c] + bzh) * O.iz2;
     d[c] = v;
-    cnt += v > 0.0 ? 1.0 : 0.0;
+    n_act += v > 0.0 ? 1.0 : 0.0;
   }
-  block_partial(cnt, part);
+  grid_sum(n_act, cnt);
 }
 
-// rhs = D(m) / dt on the active cells
-template <typename T>
-__global__ void k_rhs(Op O, const T *mu, const T *mv, const T *mw, double idt, double *rhs, double *part) {
-  const Dims &D = O.D;
-  const long long N = D.nxy * D.nz;
-  double sum = 0.0;
-  for (long long c = blockIdx.x * (long long)PB + threadIdx.x; c < N; c += (long long)gridDim.x * PB) {
-    double v = 0.0;
-    if (O.d[c] > 0.0) {
-      const Nbr n = neighbours(D, c);
-      const double bzh = n.k + 1 < D.nz ? O.bz[c + D.nxy] : 0.0;
-      const double dx = O.bx[n.xp] * (double)mu[n.xp] - O.bx[c] * (double)mu[c];
-      const double dy = O.by[n.yp] * (double)mv[n.yp] - O.by[c] * (double)mv[c];
-      const double dz = bzh * (double)mw[c + D.nxy] - O.bz[c] * (double)mw[c];
-      v = (dx * D.idx + dy * D.idy + dz * D.idz) * idt;
-    }
-    rhs[c] = v;
-    sum += v;
+// top[col]: the level from which every low face of the column's cells is
+// fully open (the floor's z face apart)
+template <typename F>
+__global__ void k_open_top(Dims D, const F *bx, const F *by, const F *bz, int *top) {
+  const int col = blockIdx.x * blockDim.x + threadIdx.x;
+  if (col >= D.nxy) return;
+  int k = D.nz;
+  while (k > 0) {
+    const long long c = col + D.nxy * (long long)(k - 1);
+    if (bx[c] != F(1) || by[c] != F(1) || (k > 1 && bz[c] != F(1))) break;
+    --k;
   }
-  block_partial(sum, part);
+  top[col] = k;
+}
+__global__ void k_open_box(Dims D, const int *top, int *kreg) {
+  const int col = blockIdx.x * blockDim.x + threadIdx.x;
+  if (col >= D.nxy) return;
+  const int i = col % D.nx, j = col / D.nx;
+  int k = 0;
+  for (int dj = -2; dj <= 2; ++dj)
+    for (int di = -2; di <= 2; ++di) k = max(k, top[wrapmod(i + di, D.nx) + D.nx * wrapmod(j + dj, D.ny)]);
+  kreg[col] = k;
+}
+
+// Work split of the marching kernels: a thread owns V adjacent columns of one
+// row and walks a slab of levels; a block is MBX x MBY threads.
+constexpr int MBX = 16, MBY = 16;
+static_assert(MBX * MBY == PB, "block sums take PB threads");
+struct Slabs {
+  int nbx, nby, nz;   // blocks along x and y, slabs
+  int blocks() const { return nbx * nby * nz; }
+};
+// enough slabs for about 1536 threads per SM, down to one level each on the
+// small grids, where latency is all that counts
+inline Slabs slabs_of(const Dims &D, int V, int sms) {
+  Slabs S;
+  S.nbx = (D.nx / V + MBX - 1) / MBX;
+  S.nby = (D.ny + MBY - 1) / MBY;
+  const int plane = S.nbx * S.nby;
+  S.nz = std::max(1, std::min(D.nz, (6 * sms + plane - 1) / plane));
+  return S;
+}
+// a thread's columns: offsets within a plane of its own row, the rows beside
+// it and the cells left and right of its V
+struct Cols {
+  int i, j, c, ym, yp, xl, xr, k0, k1;
+  bool in;
+};
+template <int V>
+__device__ inline Cols cols_of(const Dims &D, const Slabs &S) {
+  Cols q;
+  const int sl = blockIdx.x / (S.nbx * S.nby), b = blockIdx.x - sl * S.nbx * S.nby;
+  const int by = b / S.nbx, bx = b - by * S.nbx;
+  q.i = V * (bx * MBX + (int)threadIdx.x);
+  q.j = by * MBY + (int)threadIdx.y;
+  q.in = q.i < D.nx && q.j < D.ny;
+  if (!q.in) q.i = q.j = 0;
+  const int row = D.nx * q.j;
+  q.c = q.i + row;
+  q.ym = q.i + (q.j == 0 ? D.nx * (D.ny - 1) : row - D.nx);
+  q.yp = q.i + (q.j == D.ny - 1 ? 0 : row + D.nx);
+  q.xl = row + (q.i == 0 ? D.nx - 1 : q.i - 1);
+  q.xr = row + (q.i + V == D.nx ? 0 : q.i + V);
+  q.k0 = (int)((long long)D.nz * sl / S.nz);
+  q.k1 = (int)((long long)D.nz * (sl + 1) / S.nz);
+  return q;
+}
+
+// rhs = D(m) / dt on the active cells; cx, cy, cz = 1 / (delta dt)
+template <typename T>
+__global__ void __launch_bounds__(PB) k_rhs(const __grid_constant__ Op O, const __grid_constant__ Slabs SL,
+                                            const T *__restrict__ mu, const T *__restrict__ mv,
+                                            const T *__restrict__ mw, double cx, double cy, double cz,
+                                            double *__restrict__ rhs, Sum total) {
+  const Dims &D = O.D;
+  const Cols q = cols_of<1>(D, SL);
+  double sum = 0.0;
+  if (q.in) {
+    const int kr = O.kreg[q.c];
+    double wl = widen(mw[D.nxy * (long long)q.k0 + q.c]);
+#pragma unroll 2
+    for (int k = q.k0; k < q.k1; ++k) {
+      const long long t = D.nxy * (long long)k, c = t + q.c;
+      const double wh = widen(mw[c + D.nxy]);   // rho*w has nz + 1 levels
+      const double ul = widen(mu[c]), uh = widen(mu[t + q.xr]), vl = widen(mv[c]), vh = widen(mv[t + q.yp]);
+      double v = 0.0;
+      if (k >= kr && k > 0 && k < D.nz - 1) {
+        v = fma(uh - ul, cx, fma(vh - vl, cy, (wh - wl) * cz));
+      } else if (O.d[c] > 0.0) {
+        const double bzh = k + 1 < D.nz ? O.bz[c + D.nxy] : 0.0;
+        const double bxl = O.bx[c], bxh = O.bx[t + q.xr], byl = O.by[c], byh = O.by[t + q.yp], bzl = O.bz[c];
+        const double dx = bxh * uh - bxl * ul, dy = byh * vh - byl * vl, dz = bzh * wh - bzl * wl;
+        v = fma(dx, cx, fma(dy, cy, dz * cz));
+      }
+      rhs[c] = v;
+      sum += v;
+      wl = wh;
+    }
+  }
+  grid_sum(sum, total);
 }
 
 // remove the mean of the right-hand side over the active cells
-__global__ void k_center(Op O, double *rhs, const double *psum, const double *pcnt, int nb, double *pbb) {
+__global__ void __launch_bounds__(PB) k_center(const __grid_constant__ Op O, double *rhs, const double *sum,
+                                               const double *cnt, Sum bb) {
   const Dims &D = O.D;
   const long long N = D.nxy * D.nz;
-  const double mean = total(psum, nb) / fmax(1.0, total(pcnt, nb));
-  double bb = 0.0;
+  const double mean = *sum / fmax(1.0, *cnt);
+  double a = 0.0;
   for (long long c = blockIdx.x * (long long)PB + threadIdx.x; c < N; c += (long long)gridDim.x * PB) {
-    if (O.d[c] > 0.0) {
+    const int k = (int)D.fnxy.div((unsigned)c);
+    if (k >= O.kreg[c - D.nxy * (long long)k] || O.d[c] > 0.0) {
       const double v = rhs[c] - mean;
       rhs[c] = v;
-      bb += v * v;
+      a = fma(v, v, a);
     }
   }
-  block_partial(bb, pbb);
+  grid_sum(a, bb);
 }
 
-// r = -rhs - A x, z = r / d, p = z
-__global__ void k_init(Op O, const double *x, const double *rhs, double *r, float *rf, double *z, double *p,
-                       double *prz, double *prr) {
+// r = -rhs - A x (x = nullptr: zero) with r.r, and Jacobi: p = z = r / d with r.z
+__global__ void __launch_bounds__(PB) k_init(const __grid_constant__ Op O, const double *x, const double *rhs,
+                                             double *r, float *rf, double *p, Sum srz, Sum srr) {
   const Dims &D = O.D;
   const long long N = D.nxy * D.nz;
   double rz = 0.0, rr = 0.0;
   for (long long c = blockIdx.x * (long long)PB + threadIdx.x; c < N; c += (long long)gridDim.x * PB) {
-    double rv = 0.0, zv = 0.0;
-    if (O.d[c] > 0.0) {
-      rv = -rhs[c] - O.apply(x, c, neighbours(D, c));
-      zv = rv * O.id[c];
-    }
+    double rv = -rhs[c];   // zero on the inactive cells
+    if (x) rv = O.d[c] > 0.0 ? rv - O.apply(x, c, neighbours(D, c)) : 0.0;
     r[c] = rv;
-    if (rf) rf[c] = (float)rv;   // the V-cycle's right-hand side
-    z[c] = zv;
-    p[c] = zv;
-    rz += rv * zv;
-    rr += rv * rv;
+    if (rf) {
+      rf[c] = (float)rv;   // the V-cycle's right-hand side
+    } else {
+      const double zv = rv * O.id[c];
+      p[c] = zv;
+      rz = fma(rv, zv, rz);
+    }
+    rr = fma(rv, rv, rr);
   }
-  block_partial(rz, prz);
-  __syncthreads();
-  block_partial(rr, prr);
+  if (!rf) grid_sum(rz, srz);
+  grid_sum(rr, srr);
 }
 
-// q = A p
-__global__ void k_apply(Op O, const double *p, double *q, double *ppq, const int *conv) {
-  if (*conv) return;
+// iteration `it` has nothing left to do when an earlier one converged
+// (*conv = number of iterations then)
+__device__ inline bool finished(const int *conv, int it) {
+  const int c = *conv;
+  return c != 0 && c <= it;
+}
+
+// q = A p and p.q; V = 2 columns per thread where rows hold whole pairs
+template <int V>
+__global__ void __launch_bounds__(PB) k_apply(const __grid_constant__ Op O, const __grid_constant__ Slabs SL,
+                                              const double *__restrict__ p, double *__restrict__ qo, Sum spq,
+                                              const int *conv, int it) {
+  chain_begin();
+  if (finished(conv, it)) return;
   const Dims &D = O.D;
-  const long long N = D.nxy * D.nz;
+  const Cols q = cols_of<V>(D, SL);
+  const double dreg = 2.0 * (O.ix2 + O.iy2 + O.iz2);
   double pq = 0.0;
-  for (long long c = blockIdx.x * (long long)PB + threadIdx.x; c < N; c += (long long)gridDim.x * PB) {
-    double v = 0.0;
-    if (O.d[c] > 0.0) v = O.apply(p, c, neighbours(D, c));
-    q[c] = v;
-    pq += p[c] * v;
-  }
-  block_partial(pq, ppq);
-}
-
-// alpha = rz / pq; x += alpha p; r -= alpha q; z = r / d (Jacobi; the
-// multigrid preconditioner forms z and r.z afterwards)
-template <bool JAC>
-__global__ void k_update(Op O, double *x, const double *p, const double *q, double *r, float *rf, double *z,
-                         const double *ppq, const double *prz, int nrz, double *prz_next, double *prr, int nb,
-                         const int *conv) {
-  if (*conv) return;
-  const Dims &D = O.D;
-  const long long N = D.nxy * D.nz;
-  const double alpha = total(prz, nrz) / total(ppq, nb);
-  double rz = 0.0, rr = 0.0;
-  for (long long c = blockIdx.x * (long long)PB + threadIdx.x; c < N; c += (long long)gridDim.x * PB) {
-    if (O.d[c] > 0.0) {
-      x[c] += alpha * p[c];
-      const double rv = r[c] - alpha * q[c];
-      r[c] = rv;
-      if (!JAC) rf[c] = (float)rv;
-      if (JAC) {
-        const double zv = rv * O.id[c];
-        z[c] = zv;
-        rz += rv * zv;
+  auto ld = [&](const double *s, double (&v)[V]) {
+    if constexpr (V == 2) {
+      const double2 t = *reinterpret_cast<const double2 *>(s);
+      v[0] = t.x, v[1] = t.y;
+    } else {
+      v[0] = *s;
+    }
+  };
+  if (q.in) {
+    int kr = 0;
+#pragma unroll
+    for (int e = 0; e < V; ++e) kr = max(kr, O.kreg[q.c + e]);
+    double xm[V], x0[V], xp[V];
+#pragma unroll
+    for (int e = 0; e < V; ++e) xm[e] = xp[e] = 0.0;
+    if (q.k0 > 0) ld(p + D.nxy * (long long)(q.k0 - 1) + q.c, xm);
+    ld(p + D.nxy * (long long)q.k0 + q.c, x0);
+#pragma unroll 2
+    for (int k = q.k0; k < q.k1; ++k) {
+      const long long t = D.nxy * (long long)k, c = t + q.c;
+      if (k + 1 < D.nz) ld(p + c + D.nxy, xp);
+      double ym[V], yp[V], o[V];
+      ld(p + t + q.ym, ym);
+      ld(p + t + q.yp, yp);
+      const double xl = p[t + q.xl], xr = p[t + q.xr];
+      if (k >= kr && k > 0 && k < D.nz - 1) {
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+          const double sx = (e ? x0[0] : xl) + (e + 1 < V ? x0[V - 1] : xr);
+          o[e] = fma(-O.ix2, sx, fma(-O.iy2, ym[e] + yp[e], fma(-O.iz2, xm[e] + xp[e], dreg * x0[e])));
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+          const long long ce = c + e;
+          const double dd = O.d[ce];
+          o[e] = 0.0;
+          if (dd > 0.0) {
+            const double azl = O.az[ce], azh = k + 1 < D.nz ? O.az[ce + D.nxy] : 0.0;
+            double v = dd * x0[e];
+            v = fma(-O.ax[ce], e ? x0[0] : xl, v);
+            v = fma(-O.ax[e + 1 < V ? ce + 1 : t + q.xr], e + 1 < V ? x0[V - 1] : xr, v);
+            v = fma(-O.ay[ce], ym[e], v);
+            v = fma(-O.ay[t + q.yp + e], yp[e], v);
+            if (azl > 0.0) v = fma(-azl, xm[e], v);
+            if (azh > 0.0) v = fma(-azh, xp[e], v);
+            o[e] = v;
+          }
+        }
       }
-      rr += rv * rv;
+      if constexpr (V == 2) *reinterpret_cast<double2 *>(qo + c) = make_double2(o[0], o[1]);
+      else qo[c] = o[0];
+#pragma unroll
+      for (int e = 0; e < V; ++e) {
+        pq = fma(x0[e], o[e], pq);
+        xm[e] = x0[e];
+        x0[e] = xp[e];
+      }
     }
   }
-  if (JAC) {
-    block_partial(rz, prz_next);
-    __syncthreads();
-  }
-  block_partial(rr, prr);
+  grid_sum(pq, spq);
 }
 
-// convergence test; else p = z + (rz_next / rz) p
-__global__ void k_direction(Op O, double *p, const double *z, const double *prz, const double *prz_next,
-                            int nrz, const double *prr, int nb, double thr2, int it, int *conv) {
-  if (*conv) return;
-  const Dims &D = O.D;
-  const long long N = D.nxy * D.nz;
-  const double rr = total(prr, nb);
-  if (rr <= thr2) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) *conv = it + 1;
-    return;
+// alpha = rz / pq; r -= alpha q, r.r; Jacobi: r.z with z = r / d (the
+// multigrid preconditioner forms z and r.z afterwards, from the float copy)
+template <bool JAC>
+__global__ void __launch_bounds__(PB) k_update(const __grid_constant__ Op O, const double *__restrict__ q,
+                                               double *__restrict__ r, float *__restrict__ rf, const double *rz,
+                                               const double *pq, Sum srz, Sum srr, const int *conv, int it) {
+  chain_begin();
+  if (finished(conv, it)) return;
+  const long long N = O.D.nxy * O.D.nz, N2 = N & ~1LL;
+  const double alpha = *rz / *pq;
+  double az = 0.0, rr = 0.0;
+  auto one = [&](long long c, double rv, double qv) -> double {
+    rv = fma(-alpha, qv, rv);
+    if (JAC) az = fma(rv, rv * O.id[c], az);
+    rr = fma(rv, rv, rr);
+    return rv;
+  };
+  const long long t0 = 2 * (blockIdx.x * (long long)PB + threadIdx.x), dt = 2LL * gridDim.x * PB;
+#pragma unroll 2
+  for (long long c = t0; c < N2; c += dt) {
+    double2 v = *reinterpret_cast<const double2 *>(r + c);
+    const double2 qv = *reinterpret_cast<const double2 *>(q + c);
+    v.x = one(c, v.x, qv.x);
+    v.y = one(c + 1, v.y, qv.y);
+    *reinterpret_cast<double2 *>(r + c) = v;
+    if (!JAC) *reinterpret_cast<float2 *>(rf + c) = make_float2((float)v.x, (float)v.y);
   }
-  const double beta = total(prz_next, nrz) / total(prz, nrz);
-  for (long long c = blockIdx.x * (long long)PB + threadIdx.x; c < N; c += (long long)gridDim.x * PB)
-    p[c] = z[c] + beta * p[c];
+  if (t0 == 0 && N2 < N) {   // an odd last cell
+    const double v = one(N2, r[N2], q[N2]);
+    r[N2] = v;
+    if (!JAC) rf[N2] = (float)v;
+  }
+  if (JAC) grid_sum(az, srz);
+  grid_sum(rr, srr);
 }
 
-// m -= dt G(x) on the open faces
+// x += alpha p; then, unless r.r meets the threshold (conv is set), p = z +
+// (rz_next / rz) p with Jacobi's z = r / d
+template <bool JAC>
+__global__ void __launch_bounds__(PB) k_direction(const __grid_constant__ Op O, double *__restrict__ x,
+                                                  double *__restrict__ p, const double *__restrict__ zr,
+                                                  const double *rz, const double *rz_next, const double *pq,
+                                                  const double *rr, double thr2, int it, int *conv) {
+  chain_begin();
+  if (finished(conv, it)) return;
+  const long long N = O.D.nxy * O.D.nz, N2 = N & ~1LL;
+  const double alpha = *rz / *pq;
+  const bool stop = *rr <= thr2;
+  if (stop && blockIdx.x == 0 && threadIdx.x == 0) *conv = it + 1;
+  const double beta = *rz_next / *rz;
+  const long long t0 = 2 * (blockIdx.x * (long long)PB + threadIdx.x), dt = 2LL * gridDim.x * PB;
+#pragma unroll 2
+  for (long long c = t0; c < N2; c += dt) {
+    double2 pv = *reinterpret_cast<const double2 *>(p + c), xv = *reinterpret_cast<const double2 *>(x + c);
+    xv.x = fma(alpha, pv.x, xv.x);
+    xv.y = fma(alpha, pv.y, xv.y);
+    *reinterpret_cast<double2 *>(x + c) = xv;
+    if (!stop) {
+      double2 z = *reinterpret_cast<const double2 *>(zr + c);
+      if (JAC) {
+        const double2 i = *reinterpret_cast<const double2 *>(O.id + c);
+        z.x *= i.x, z.y *= i.y;
+      }
+      pv.x = fma(beta, pv.x, z.x);
+      pv.y = fma(beta, pv.y, z.y);
+      *reinterpret_cast<double2 *>(p + c) = pv;
+    }
+  }
+  if (t0 == 0 && N2 < N) {
+    x[N2] = fma(alpha, p[N2], x[N2]);
+    if (!stop) p[N2] = fma(beta, p[N2], JAC ? zr[N2] * O.id[N2] : zr[N2]);
+  }
+}
+
+// m -= dt G(x) on the open faces; cx, cy, cz = dt / delta
 template <typename T>
-__global__ void k_correct(Op O, const double *x, double dt, T *mu, T *mv, T *mw) {
+__global__ void __launch_bounds__(PB) k_correct(const __grid_constant__ Op O, const __grid_constant__ Slabs SL,
+                                                const double *__restrict__ x, double cx, double cy, double cz,
+                                                T *__restrict__ mu, T *__restrict__ mv, T *__restrict__ mw) {
   const Dims &D = O.D;
-  const long long N = D.nxy * D.nz;
-  for (long long c = blockIdx.x * (long long)PB + threadIdx.x; c < N; c += (long long)gridDim.x * PB) {
-    const Nbr n = neighbours(D, c);
-    if (O.bx[c] > 0.0) mu[c] = (T)((double)mu[c] - dt * (x[c] - x[n.xm]) * D.idx);
-    if (O.by[c] > 0.0) mv[c] = (T)((double)mv[c] - dt * (x[c] - x[n.ym]) * D.idy);
-    if (n.k >= 1 && O.bz[c] > 0.0) mw[c] = (T)((double)mw[c] - dt * (x[c] - x[c - D.nxy]) * D.idz);
+  const Cols q = cols_of<1>(D, SL);
+  if (!q.in) return;
+  const int kr = O.kreg[q.c];
+  double xm = q.k0 > 0 ? x[D.nxy * (long long)(q.k0 - 1) + q.c] : 0.0;
+#pragma unroll 2
+  for (int k = q.k0; k < q.k1; ++k) {
+    const long long t = D.nxy * (long long)k, c = t + q.c;
+    const double x0 = x[c];
+    const bool open = k >= kr;
+    const T u = mu[c], v = mv[c], w = mw[c];
+    if (open || O.bx[c] > 0.0) mu[c] = (T)fma(-cx, x0 - x[t + q.xl], widen(u));
+    if (open || O.by[c] > 0.0) mv[c] = (T)fma(-cy, x0 - x[t + q.ym], widen(v));
+    if (k >= 1 && (open || O.bz[c] > 0.0)) mw[c] = (T)fma(-cz, x0 - xm, widen(w));
+    xm = x0;
   }
 }
 
@@ -302,16 +526,6 @@ struct Op32 {
   const float *wi;             // MG_OMEGA / diagonal (0 off the active cells)
   const int *kreg;
   float ix2, iy2, iz2;
-  // off-diagonal sum and diagonal of cell c (grid-stride form; coarsest grids and set-up)
-  __device__ inline void parts(const float *x, long long c, float &S, float &d) const {
-    const Nbr n = neighbours(D, c);
-    const float axl = bx[c] * ix2, axh = bx[n.xp] * ix2, ayl = by[c] * iy2, ayh = by[n.yp] * iy2;
-    const float azl = bz[c] * iz2, azh = n.k + 1 < D.nz ? bz[c + D.nxy] * iz2 : 0.f;
-    d = axl + axh + ayl + ayh + azl + azh;
-    S = axl * x[n.xm] + axh * x[n.xp] + ayl * x[n.ym] + ayh * x[n.yp];
-    if (azl > 0.f) S += azl * x[c - D.nxy];
-    if (azh > 0.f) S += azh * x[c + D.nxy];
-  }
   __device__ inline float diag(long long c) const {
     const Nbr n = neighbours(D, c);
     const float azh = n.k + 1 < D.nz ? bz[c + D.nxy] * iz2 : 0.f;
@@ -325,30 +539,6 @@ __global__ void k_mg_winv(Op32 L, float *wi) {
     const float d = L.diag(c);
     wi[c] = d > 0.f ? MG_OMEGA / d : 0.f;
   }
-}
-
-// top[col]: the level from which every low face of the column's cells is
-// fully open (the floor's z face apart)
-template <typename F>
-__global__ void k_open_top(Dims D, const F *bx, const F *by, const F *bz, int *top) {
-  const int col = blockIdx.x * blockDim.x + threadIdx.x;
-  if (col >= D.nxy) return;
-  int k = D.nz;
-  while (k > 0) {
-    const long long c = col + D.nxy * (long long)(k - 1);
-    if (bx[c] != F(1) || by[c] != F(1) || (k > 1 && bz[c] != F(1))) break;
-    --k;
-  }
-  top[col] = k;
-}
-__global__ void k_open_box(Dims D, const int *top, int *kreg) {
-  const int col = blockIdx.x * blockDim.x + threadIdx.x;
-  if (col >= D.nxy) return;
-  const int i = col % D.nx, j = col / D.nx;
-  int k = 0;
-  for (int dj = -2; dj <= 2; ++dj)
-    for (int di = -2; di <= 2; ++di) k = max(k, top[wrapmod(i + di, D.nx) + D.nx * wrapmod(j + dj, D.ny)]);
-  kreg[col] = k;
 }
 
 // level 0: float copies of the open fractions
@@ -401,57 +591,12 @@ __device__ inline void stv(float *p, const Vec<V> &a) {
   else p[0] = a.v[0];
 }
 
-// Work split of the marching kernels: a thread owns V adjacent columns of one
-// row and walks a slab of levels; a block is MBX x MBY threads.
-constexpr int MBX = 16, MBY = 16;
-static_assert(MBX * MBY == PB, "block sums take PB threads");
-struct Slabs {
-  int nbx, nby, nz;   // blocks along x and y, slabs
-  int blocks() const { return nbx * nby * nz; }
-};
-// enough slabs for about 1536 threads per SM, down to one level each on the
-// small grids, where latency is all that counts
-inline Slabs slabs_of(const Dims &D, int V, int sms) {
-  Slabs S;
-  S.nbx = (D.nx / V + MBX - 1) / MBX;
-  S.nby = (D.ny + MBY - 1) / MBY;
-  const int plane = S.nbx * S.nby;
-  S.nz = std::max(1, std::min(D.nz, (6 * sms + plane - 1) / plane));
-  return S;
-}
-// a thread's columns: offsets within a plane of its own row, the rows beside
-// it and the cells left and right of its V
-struct Cols {
-  int i, j, c, ym, yp, xl, xr, k0, k1;
-  bool in;
-};
-template <int V>
-__device__ inline Cols cols_of(const Dims &D, const Slabs &S) {
-  Cols q;
-  const int sl = blockIdx.x / (S.nbx * S.nby), b = blockIdx.x - sl * S.nbx * S.nby;
-  const int by = b / S.nbx, bx = b - by * S.nbx;
-  q.i = V * (bx * MBX + (int)threadIdx.x);
-  q.j = by * MBY + (int)threadIdx.y;
-  q.in = q.i < D.nx && q.j < D.ny;
-  if (!q.in) q.i = q.j = 0;
-  const int row = D.nx * q.j;
-  q.c = q.i + row;
-  q.ym = q.i + (q.j == 0 ? D.nx * (D.ny - 1) : row - D.nx);
-  q.yp = q.i + (q.j == D.ny - 1 ? 0 : row + D.nx);
-  q.xl = row + (q.i == 0 ? D.nx - 1 : q.i - 1);
-  q.xr = row + (q.i + V == D.nx ? 0 : q.i + V);
-  q.k0 = (int)((long long)D.nz * sl / S.nz);
-  q.k1 = (int)((long long)D.nz * (sl + 1) / S.nz);
-  return q;
-}
-
 // One damped Jacobi sweep, xout = (1 - w) x + w (b + S(x)) / d, of
 //   FIRST    x = w b / d, the sweep from zero (so two sweeps in one pass),
 //   PLAIN    x = xin,
 //   PROLONG  x = xin + the parent's coarse correction (injection; inactive
 //            cells are never read with a nonzero coefficient).
-// FINAL: the finest level's last sweep, which writes the FP64 z and the block
-// partials of r.z.
+// FINAL: the finest level's last sweep, which writes the FP64 z and sums r.z.
 // L2 bandwidth bounds it (16 bytes per cell; the level's arrays stay in the
 // 129 MB L2): V = 4 columns per thread with 16-byte accesses, the z
 // neighbours carried in registers, no coefficients above the terrain.
@@ -465,7 +610,8 @@ __global__ void __launch_bounds__(MBX * MBY) k_mg_sweep(const __grid_constant__ 
                                                         const float *__restrict__ xin, const float *__restrict__ xc,
                                                         const __grid_constant__ Dims C, float *__restrict__ xout,
                                                         double *__restrict__ zout, const double *__restrict__ r,
-                                                        const float *__restrict__ b, double *prz, const int *conv) {
+                                                        const float *__restrict__ b, Sum srz, const int *conv) {
+  chain_begin();
   if (*conv) return;
   const Dims &D = L.D;
   const Cols q = cols_of<V>(D, SL);
@@ -551,9 +697,9 @@ __global__ void __launch_bounds__(MBX * MBY) k_mg_sweep(const __grid_constant__ 
       if constexpr (FINAL) {
 #pragma unroll
         for (int e = 0; e < V; ++e) {
-          const double z = (double)o.v[e];
+          const double z = widen(o.v[e]);
           zout[t + q.c + e] = z;
-          rz += r[t + q.c + e] * z;
+          rz = fma(r[t + q.c + e], z, rz);
         }
       } else {
         stv<V>(xout + t + q.c, o);
@@ -562,7 +708,7 @@ __global__ void __launch_bounds__(MBX * MBY) k_mg_sweep(const __grid_constant__ 
       x0 = xp;
     }
   }
-  if constexpr (FINAL) block_partial(rz, prz);
+  if constexpr (FINAL) grid_sum(rz, srz);
 }
 
 // Coarse right-hand side: the mean of the eight children's residuals b - A x.
@@ -572,6 +718,7 @@ template <int V>
 __global__ void __launch_bounds__(MBX * MBY) k_mg_restrict(const __grid_constant__ Op32 F, const float *x,
                                                            const float *b, const __grid_constant__ Dims C,
                                                            float *bc, int kper, const int *conv) {
+  chain_begin();
   if (*conv) return;
   const Dims &D = F.D;
   const int g = D.nx / V;   // groups of V columns per row
@@ -728,6 +875,7 @@ __device__ __forceinline__ void lower_first(const LowerLevel &L, float *__restri
 
 template <bool SMEM>
 __global__ void __launch_bounds__(1024) k_mg_lower(const __grid_constant__ MgLower M, const int *conv) {
+  chain_begin();
   if (*conv) return;
   extern __shared__ float lower_smem[];
   const int lt = M.lt, top = M.top;
@@ -820,10 +968,16 @@ Op make_op(eb_geom g) {
   O.ax = g->pw.ax;
   O.ay = g->pw.ay;
   O.az = g->pw.az;
+  O.kreg = g->pw.kreg;
   O.ix2 = g->D.idx * g->D.idx;
   O.iy2 = g->D.idy * g->D.idy;
   O.iz2 = g->D.idz * g->D.idz;
   return O;
+}
+
+Sum sum_of(eb_geom g, int slot) {
+  ProjWork &w = g->pw;
+  return Sum{w.part + (long long)slot * w.npart, w.scal + slot, w.done + slot};
 }
 
 // work space and the fixed part of the operator, on the first call
@@ -838,9 +992,15 @@ eb_status setup(eb_geom g, cudaStream_t s) {
   w.nb = (int)std::max(1LL, std::min<long long>(4LL * std::max(sms, 1), (N + PB - 1) / PB));
   for (double **a : {&w.bx, &w.by, &w.bz, &w.ax, &w.ay, &w.az, &w.d, &w.id, &w.rhs, &w.r, &w.z, &w.p, &w.q, &w.x})
     CUDA_TRY(g->alloc(a, N), "alloc projection work space");
-  CUDA_TRY(g->alloc(&w.part, 8LL * w.nb), "alloc projection work space");
+  w.ncols = D.nx % 2 == 0 ? 2 : 1;
+  w.npart = std::max({w.nb, slabs_of(D, 1, sms).blocks(), slabs_of(D, 2, sms).blocks(), slabs_of(D, 4, sms).blocks()});
+  CUDA_TRY(g->alloc(&w.part, (long long)S_SLOTS * w.npart), "alloc projection work space");
+  CUDA_TRY(g->alloc(&w.scal, S_SLOTS), "alloc projection work space");
+  CUDA_TRY(g->alloc(&w.done, S_SLOTS), "alloc projection work space");
+  CUDA_TRY(cudaMemsetAsync(w.done, 0, sizeof(unsigned) * S_SLOTS, s), "projection work space");
+  CUDA_TRY(g->alloc(&w.kreg, D.nxy), "alloc projection work space");
   CUDA_TRY(g->alloc(&w.conv, 1), "alloc projection work space");
-  CUDA_TRY(cudaMallocHost(&w.host, sizeof(double) * (size_t)w.nb), "alloc pinned scratch");
+  CUDA_TRY(cudaMallocHost(&w.host, sizeof(double) * (S_SLOTS + 1)), "alloc pinned scratch");
   launch_export_geometry(g->h, D, 0, g->G[0], EB_X_BETA_X, w.bx, s);
   launch_export_geometry(g->h, D, 0, g->G[0], EB_X_BETA_Y, w.by, s);
   launch_export_geometry(g->h, D, 0, g->G[0], EB_X_BETA_Z, w.bz, s);
@@ -848,19 +1008,23 @@ eb_status setup(eb_geom g, cudaStream_t s) {
   k_scale<<<w.nb, PB, 0, s>>>(N, w.bx, D.idx * D.idx, w.ax);
   k_scale<<<w.nb, PB, 0, s>>>(N, w.by, D.idy * D.idy, w.ay);
   k_scale<<<w.nb, PB, 0, s>>>(N, w.bz, D.idz * D.idz, w.az);
-  k_diag<<<w.nb, PB, 0, s>>>(make_op(g), w.d, w.part + S_CNT * w.nb);
+  k_diag<<<w.nb, PB, 0, s>>>(make_op(g), w.d, sum_of(g, S_CNT));
   k_recip<<<w.nb, PB, 0, s>>>(N, w.d, w.id);
-  CUDA_TRY(cudaMemcpyAsync(w.host, w.part + S_CNT * w.nb, sizeof(double) * w.nb, cudaMemcpyDeviceToHost, s),
-           "count active cells");
-  CUDA_TRY(cudaStreamSynchronize(s), "count active cells");
-  double cnt = 0.0;
-  for (int q = 0; q < w.nb; ++q) cnt += w.host[q];
-  w.nact = (long long)cnt;
+  {
+    int *top = nullptr;
+    CUDA_TRY(cudaMalloc(&top, sizeof(int) * (size_t)D.nxy), "open levels");
+    const unsigned nc = (unsigned)((D.nxy + 127) / 128);
+    k_open_top<double><<<nc, 128, 0, s>>>(D, w.bx, w.by, w.bz, top);
+    k_open_box<<<nc, 128, 0, s>>>(D, top, w.kreg);
+    cudaError_t e = cudaMemcpyAsync(w.host, w.scal + S_CNT, sizeof(double), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaFree(top);
+    CUDA_TRY(e, "count active cells");
+  }
+  w.nact = (long long)w.host[0];
   w.ready = true;
   return EB_OK;
 }
-
-int final_blocks(eb_geom g);
 
 // the multigrid hierarchy, on the first projection that uses it
 eb_status mg_setup(eb_geom g, cudaStream_t s) {
@@ -912,8 +1076,6 @@ eb_status mg_setup(eb_geom g, cudaStream_t s) {
     k_mg_coarsen<<<L.nb, PB, 0, s>>>(level_op(F), C, L.bx, L.by, L.bz);
     CUDA_TRY(finish(L), "multigrid set-up");
   }
-  w.nrz = final_blocks(g);
-  CUDA_TRY(g->alloc(&w.part_rz, 2LL * w.nrz), "alloc projection work space");
   CUDA_TRY(cudaGetLastError(), "multigrid set-up");
   w.nlev = nlev;
   return EB_OK;
@@ -927,16 +1089,16 @@ inline int level_v(const MgLevel &L) {
 
 template <int MODE, bool FINAL>
 void sweep(const MgLevel &L, const float *xin, const MgLevel *coarse, float *xout, double *zout, const double *r,
-           double *prz, const int *conv, cudaStream_t s) {
+           const Sum &rz, const int *conv, cudaStream_t s) {
   const int V = level_v(L);
   const Slabs S = slabs_of(L.D, V, ebk_sm_count());
   const Op32 O = level_op(L);
   const Dims C = coarse ? coarse->D : L.D;
   const float *xc = coarse ? coarse->x : nullptr;
   const dim3 blk(MBX, MBY, 1);
-  if (V == 4) k_mg_sweep<4, MODE, FINAL><<<S.blocks(), blk, 0, s>>>(O, S, xin, xc, C, xout, zout, r, L.b, prz, conv);
-  else if (V == 2) k_mg_sweep<2, MODE, FINAL><<<S.blocks(), blk, 0, s>>>(O, S, xin, xc, C, xout, zout, r, L.b, prz, conv);
-  else k_mg_sweep<1, MODE, FINAL><<<S.blocks(), blk, 0, s>>>(O, S, xin, xc, C, xout, zout, r, L.b, prz, conv);
+  if (V == 4) launch_chained(k_mg_sweep<4, MODE, FINAL>, S.blocks(), blk, 0, s, O, S, xin, xc, C, xout, zout, r, L.b, rz, conv);
+  else if (V == 2) launch_chained(k_mg_sweep<2, MODE, FINAL>, S.blocks(), blk, 0, s, O, S, xin, xc, C, xout, zout, r, L.b, rz, conv);
+  else launch_chained(k_mg_sweep<1, MODE, FINAL>, S.blocks(), blk, 0, s, O, S, xin, xc, C, xout, zout, r, L.b, rz, conv);
 }
 
 // from a level with an even number of columns (it is coarsened)
@@ -947,19 +1109,14 @@ void restrict_residual(const MgLevel &F, const float *x, const MgLevel &C, const
   const int kper = plane * C.D.nz >= 2LL * 2048 * ebk_sm_count() ? 2 : 1;
   const long long n = plane * ((C.D.nz + kper - 1) / kper);
   const unsigned nb = (unsigned)((n + MBX * MBY - 1) / (MBX * MBY));
-  if (V == 4) k_mg_restrict<4><<<nb, dim3(MBX, MBY, 1), 0, s>>>(level_op(F), x, F.b, C.D, C.b, kper, conv);
-  else k_mg_restrict<2><<<nb, dim3(MBX, MBY, 1), 0, s>>>(level_op(F), x, F.b, C.D, C.b, kper, conv);
-}
-
-// blocks of the sweep that forms r.z (its partial sums)
-int final_blocks(eb_geom g) {
-  const MgLevel &L = g->pw.lev[0];
-  return slabs_of(L.D, level_v(L), ebk_sm_count()).blocks();
+  if (V == 4) launch_chained(k_mg_restrict<4>, nb, dim3(MBX, MBY, 1), 0, s, level_op(F), x, F.b, C.D, C.b, kper, conv);
+  else launch_chained(k_mg_restrict<2>, nb, dim3(MBX, MBY, 1), 0, s, level_op(F), x, F.b, C.D, C.b, kper, conv);
 }
 
 // z = V(r) (r in FP64 and, as the finest level's right-hand side, in float)
-// and the partial sums of r.z into prz
-void vcycle(eb_geom g, const double *r, double *z, double *prz, cudaStream_t s) {
+// and r.z into the slot rz
+void vcycle(eb_geom g, const double *r, double *z, int rz, cudaStream_t s) {
+  const Sum none{nullptr, nullptr, nullptr};
   ProjWork &w = g->pw;
   const MgLevel *L = w.lev;
   const int top = w.nlev - 1;
@@ -967,11 +1124,11 @@ void vcycle(eb_geom g, const double *r, double *z, double *prz, cudaStream_t s) 
   int lt = top;
   while (lt > 1 && L[lt - 1].D.nxy * L[lt - 1].D.nz <= MG_LOWER_CELLS) --lt;
   // sweeps before and after the coarse correction: three on the finest level, two below
-  sweep<FIRST, false>(L[0], nullptr, nullptr, L[0].t, nullptr, nullptr, nullptr, w.conv, s);
-  sweep<PLAIN, false>(L[0], L[0].t, nullptr, L[0].x, nullptr, nullptr, nullptr, w.conv, s);
+  sweep<FIRST, false>(L[0], nullptr, nullptr, L[0].t, nullptr, nullptr, none, w.conv, s);
+  sweep<PLAIN, false>(L[0], L[0].t, nullptr, L[0].x, nullptr, nullptr, none, w.conv, s);
   restrict_residual(L[0], L[0].x, L[1], w.conv, s);
   for (int l = 1; l < lt; ++l) {
-    sweep<FIRST, false>(L[l], nullptr, nullptr, L[l].x, nullptr, nullptr, nullptr, w.conv, s);
+    sweep<FIRST, false>(L[l], nullptr, nullptr, L[l].x, nullptr, nullptr, none, w.conv, s);
     restrict_residual(L[l], L[l].x, L[l + 1], w.conv, s);
   }
   {
@@ -986,38 +1143,55 @@ void vcycle(eb_geom g, const double *r, double *z, double *prz, cudaStream_t s) 
     M.top = top;
     static unsigned long long attr = 0;
     ebk_smem_limit(k_mg_lower<true>, MG_LOWER_SMEM, attr);
-    if (L[lt].D.nxy * L[lt].D.nz <= MG_LOWER_CELLS) k_mg_lower<true><<<1, 1024, MG_LOWER_SMEM, s>>>(M, w.conv);
-    else k_mg_lower<false><<<1, 1024, 0, s>>>(M, w.conv);
+    if (L[lt].D.nxy * L[lt].D.nz <= MG_LOWER_CELLS) launch_chained(k_mg_lower<true>, 1, 1024, MG_LOWER_SMEM, s, M, w.conv);
+    else launch_chained(k_mg_lower<false>, 1, 1024, 0, s, M, w.conv);
   }
   for (int l = lt - 1; l >= 1; --l) {
-    sweep<PROLONG, false>(L[l], L[l].x, &L[l + 1], L[l].t, nullptr, nullptr, nullptr, w.conv, s);
-    sweep<PLAIN, false>(L[l], L[l].t, nullptr, L[l].x, nullptr, nullptr, nullptr, w.conv, s);
+    sweep<PROLONG, false>(L[l], L[l].x, &L[l + 1], L[l].t, nullptr, nullptr, none, w.conv, s);
+    sweep<PLAIN, false>(L[l], L[l].t, nullptr, L[l].x, nullptr, nullptr, none, w.conv, s);
   }
-  sweep<PROLONG, false>(L[0], L[0].x, &L[1], L[0].t, nullptr, nullptr, nullptr, w.conv, s);
-  sweep<PLAIN, false>(L[0], L[0].t, nullptr, L[0].x, nullptr, nullptr, nullptr, w.conv, s);
-  sweep<PLAIN, true>(L[0], L[0].x, nullptr, nullptr, z, r, prz, w.conv, s);
+  sweep<PROLONG, false>(L[0], L[0].x, &L[1], L[0].t, nullptr, nullptr, none, w.conv, s);
+  sweep<PLAIN, false>(L[0], L[0].t, nullptr, L[0].x, nullptr, nullptr, none, w.conv, s);
+  sweep<PLAIN, true>(L[0], L[0].x, nullptr, nullptr, z, r, sum_of(g, rz), w.conv, s);
 }
 
-double host_total(eb_geom g, int slot, cudaStream_t s, cudaError_t &e) {
+// the scalars of slots first .. last on the host (synchronises the stream)
+cudaError_t host_scalars(eb_geom g, int first, int last, double *out, cudaStream_t s) {
   ProjWork &w = g->pw;
-  e = cudaMemcpyAsync(w.host, w.part + slot * w.nb, sizeof(double) * w.nb, cudaMemcpyDeviceToHost, s);
+  const size_t n = sizeof(double) * (size_t)(last - first + 1);
+  cudaError_t e = cudaMemcpyAsync(w.host, w.scal + first, n, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  double t = 0.0;
-  for (int q = 0; q < w.nb; ++q) t += w.host[q];
-  return t;
+  for (int q = 0; q <= last - first; ++q) out[q] = w.host[q];
+  return e;
 }
 
+// the mean-free right-hand side of the momenta and its square norm (S_BB)
 template <typename T>
 void launch_rhs(eb_geom g, void *const mom[3], double dt, cudaStream_t s) {
   ProjWork &w = g->pw;
-  k_rhs<T><<<w.nb, PB, 0, s>>>(make_op(g), (const T *)mom[0], (const T *)mom[1], (const T *)mom[2], 1.0 / dt, w.rhs,
-                               w.part + S_SUM * w.nb);
+  const Dims &D = g->D;
+  const Slabs S = slabs_of(D, 1, ebk_sm_count());
+  k_rhs<T><<<S.blocks(), dim3(MBX, MBY, 1), 0, s>>>(make_op(g), S, (const T *)mom[0], (const T *)mom[1],
+                                                   (const T *)mom[2], D.idx / dt, D.idy / dt, D.idz / dt, w.rhs,
+                                                   sum_of(g, S_SUM));
+  k_center<<<w.nb, PB, 0, s>>>(make_op(g), w.rhs, w.scal + S_SUM, w.scal + S_CNT, sum_of(g, S_BB));
 }
 
 template <typename T>
 void launch_correct(eb_geom g, void *const mom[3], double dt, cudaStream_t s) {
   ProjWork &w = g->pw;
-  k_correct<T><<<w.nb, PB, 0, s>>>(make_op(g), w.x, dt, (T *)mom[0], (T *)mom[1], (T *)mom[2]);
+  const Dims &D = g->D;
+  const Slabs S = slabs_of(D, 1, ebk_sm_count());
+  k_correct<T><<<S.blocks(), dim3(MBX, MBY, 1), 0, s>>>(make_op(g), S, w.x, dt * D.idx, dt * D.idy, dt * D.idz,
+                                                       (T *)mom[0], (T *)mom[1], (T *)mom[2]);
+}
+
+void launch_apply(eb_geom g, const double *p, double *q, int it, cudaStream_t s) {
+  ProjWork &w = g->pw;
+  const Slabs S = slabs_of(g->D, w.ncols, ebk_sm_count());
+  const dim3 blk(MBX, MBY, 1);
+  if (w.ncols == 2) launch_chained(k_apply<2>, S.blocks(), blk, 0, s, make_op(g), S, p, q, sum_of(g, S_PQ), w.conv, it);
+  else launch_chained(k_apply<1>, S.blocks(), blk, 0, s, make_op(g), S, p, q, sum_of(g, S_PQ), w.conv, it);
 }
 
 }  // namespace
@@ -1032,11 +1206,8 @@ eb_status eb_project_rhs(eb_geom g, void *const mom[3], double dt, double *rms, 
   ProjWork &w = g->pw;
   if (g->prec == EB_F64) launch_rhs<double>(g, mom, dt, s);
   else launch_rhs<float>(g, mom, dt, s);
-  k_center<<<w.nb, PB, 0, s>>>(make_op(g), w.rhs, w.part + S_SUM * w.nb, w.part + S_CNT * w.nb, w.nb,
-                               w.part + S_BB * w.nb);
-  cudaError_t e = cudaSuccess;
-  const double bb = host_total(g, S_BB, s, e);
-  CUDA_TRY(e, "right-hand side");
+  double bb = 0.0;
+  CUDA_TRY(host_scalars(g, S_BB, S_BB, &bb, s), "right-hand side");
   if (rms) *rms = w.nact > 0 ? sqrt(bb / (double)w.nact) : 0.0;
   return EB_OK;
 }
@@ -1055,7 +1226,6 @@ eb_status eb_project_impl(eb_geom g, void *const mom[3], double dt, double rtol,
   const Op O = make_op(g);
   if (g->prec == EB_F64) launch_rhs<double>(g, mom, dt, s);
   else launch_rhs<float>(g, mom, dt, s);
-  k_center<<<w.nb, PB, 0, s>>>(O, w.rhs, w.part + S_SUM * w.nb, w.part + S_CNT * w.nb, w.nb, w.part + S_BB * w.nb);
   if (phi0) CUDA_TRY(cudaMemcpyAsync(w.x, phi0, sizeof(double) * N, cudaMemcpyDeviceToDevice, s), "initial guess");
   else CUDA_TRY(cudaMemsetAsync(w.x, 0, sizeof(double) * N, s), "initial guess");
   const bool mg = w.precond == EB_PRECOND_MG;
@@ -1064,49 +1234,44 @@ eb_status eb_project_impl(eb_geom g, void *const mom[3], double dt, double rtol,
     if (st != EB_OK) return st;
   }
   CUDA_TRY(cudaMemsetAsync(w.conv, 0, sizeof(int), s), "reset");
-  double *const part_rz[2] = {w.part + S_RZ0 * w.nb, w.part + S_RZ1 * w.nb};
-  double *const rz_of[2] = {mg ? w.part_rz : part_rz[0], mg ? w.part_rz + w.nrz : part_rz[1]};
-  const int nrz = mg ? w.nrz : w.nb;   // partial sums of r.z
   float *rf = mg ? w.lev[0].b : nullptr;
-  k_init<<<w.nb, PB, 0, s>>>(O, w.x, w.rhs, w.r, rf, w.z, w.p, part_rz[0], w.part + S_RR * w.nb);
-  if (mg) {   // z = V(r), p = z
-    vcycle(g, w.r, w.z, rz_of[0], s);
-    CUDA_TRY(cudaMemcpyAsync(w.p, w.z, sizeof(double) * N, cudaMemcpyDeviceToDevice, s), "search direction");
-  }
-  cudaError_t e = cudaSuccess;
-  const double bb = host_total(g, S_BB, s, e);
-  CUDA_TRY(e, "residual norm");
-  const double rr0 = host_total(g, S_RR, s, e);
-  CUDA_TRY(e, "residual norm");
+  k_init<<<w.nb, PB, 0, s>>>(O, phi0 ? w.x : nullptr, w.rhs, w.r, rf, w.p, sum_of(g, S_RZ0), sum_of(g, S_RR));
+  if (mg) vcycle(g, w.r, w.p, S_RZ0, s);   // p = z = V(r)
+  double h[3] = {0.0, 0.0, 0.0};   // S_BB, S_PQ (not yet formed), S_RR
+  CUDA_TRY(host_scalars(g, S_BB, S_RR, h, s), "residual norm");
+  const double bb = h[0], rr0 = h[2];
   const double thr2 = rtol * rtol * bb;
   int it = 0;
   double rr = rr0;
   if (bb > 0.0 && rr0 > thr2) {
     int done = 0;
     for (it = 0; it < maxit; ++it) {
-      double *prz = rz_of[it % 2], *prz_next = rz_of[1 - it % 2];
-      k_apply<<<w.nb, PB, 0, s>>>(O, w.p, w.q, w.part + S_PQ * w.nb, w.conv);
+      const int rz = it % 2 ? S_RZ1 : S_RZ0, rz_next = it % 2 ? S_RZ0 : S_RZ1;
+      launch_apply(g, w.p, w.q, it, s);
       if (mg) {
-        k_update<false><<<w.nb, PB, 0, s>>>(O, w.x, w.p, w.q, w.r, rf, w.z, w.part + S_PQ * w.nb, prz, nrz, prz_next,
-                                            w.part + S_RR * w.nb, w.nb, w.conv);
-        vcycle(g, w.r, w.z, prz_next, s);
+        launch_chained(k_update<false>, w.nb, PB, 0, s, O, w.q, w.r, rf, w.scal + rz, w.scal + S_PQ, sum_of(g, rz_next),
+                                            sum_of(g, S_RR), w.conv, it);
+        vcycle(g, w.r, w.z, rz_next, s);
+        launch_chained(k_direction<false>, w.nb, PB, 0, s, O, w.x, w.p, w.z, w.scal + rz, w.scal + rz_next, w.scal + S_PQ,
+                                               w.scal + S_RR, thr2, it, w.conv);
       } else {
-        k_update<true><<<w.nb, PB, 0, s>>>(O, w.x, w.p, w.q, w.r, nullptr, w.z, w.part + S_PQ * w.nb, prz, nrz,
-                                           prz_next, w.part + S_RR * w.nb, w.nb, w.conv);
+        launch_chained(k_update<true>, w.nb, PB, 0, s, O, w.q, w.r, nullptr, w.scal + rz, w.scal + S_PQ, sum_of(g, rz_next),
+                                           sum_of(g, S_RR), w.conv, it);
+        launch_chained(k_direction<true>, w.nb, PB, 0, s, O, w.x, w.p, w.r, w.scal + rz, w.scal + rz_next, w.scal + S_PQ,
+                                              w.scal + S_RR, thr2, it, w.conv);
       }
-      k_direction<<<w.nb, PB, 0, s>>>(O, w.p, w.z, prz, prz_next, nrz, w.part + S_RR * w.nb, w.nb, thr2, it,
-                                      w.conv);
       // the host reads the convergence flag every few iterations (a V-cycle
       // iteration costs far more than a Jacobi one, so it looks sooner)
       if ((it + 1) % (mg ? 4 : 32) == 0 || it + 1 == maxit) {
-        CUDA_TRY(cudaMemcpyAsync(&done, w.conv, sizeof(int), cudaMemcpyDeviceToHost, s), "convergence flag");
+        int *flag = reinterpret_cast<int *>(w.host + S_SLOTS);
+        CUDA_TRY(cudaMemcpyAsync(flag, w.conv, sizeof(int), cudaMemcpyDeviceToHost, s), "convergence flag");
         CUDA_TRY(cudaStreamSynchronize(s), "convergence flag");
+        done = *flag;
         if (done) break;
       }
     }
     it = done ? done : maxit;
-    rr = host_total(g, S_RR, s, e);
-    CUDA_TRY(e, "residual norm");
+    CUDA_TRY(host_scalars(g, S_RR, S_RR, &rr, s), "residual norm");
   }
   if (correct) {
     if (g->prec == EB_F64) launch_correct<double>(g, mom, dt, s);
