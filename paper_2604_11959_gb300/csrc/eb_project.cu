@@ -370,15 +370,15 @@ __global__ void __launch_bounds__(PB) k_apply(const __grid_constant__ Op O, cons
           const long long ce = c + e;
           const double dd = O.d[ce];
           o[e] = 0.0;
-          if (dd > 0.0) {
+          if (__double2hiint(dd) > 0) {   // tests of non-negative doubles by their high words
             const double azl = O.az[ce], azh = k + 1 < D.nz ? O.az[ce + D.nxy] : 0.0;
             double v = dd * x0[e];
             v = fma(-O.ax[ce], e ? x0[0] : xl, v);
             v = fma(-O.ax[e + 1 < V ? ce + 1 : t + q.xr], e + 1 < V ? x0[V - 1] : xr, v);
             v = fma(-O.ay[ce], ym[e], v);
             v = fma(-O.ay[t + q.yp + e], yp[e], v);
-            if (azl > 0.0) v = fma(-azl, xm[e], v);
-            if (azh > 0.0) v = fma(-azh, xp[e], v);
+            if (__double2hiint(azl) > 0) v = fma(-azl, xm[e], v);
+            if (__double2hiint(azh) > 0) v = fma(-azh, xp[e], v);
             o[e] = v;
           }
         }
@@ -496,26 +496,43 @@ __global__ void __launch_bounds__(PB) k_correct(const __grid_constant__ Op O, co
 // ---------------------------------------------------------------------------
 // Multigrid preconditioner (EB_PRECOND_MG): z = V(r), one V-cycle in FP32
 // (FP64 arithmetic is scarce on this GPU; the outer conjugate gradients stay
-// in FP64).  Damped Jacobi with the same weight and the same number of
-// sweeps before and after the coarse correction (three on the finest grid,
-// where they cut 18 iterations to 16 at rtol 1e-10 on the 192x192x96 random
-// terrain for a shorter solve; two on the coarser grids), restriction = 1/8
-// of the transpose of the injection
-// prolongation, and a fixed number of Jacobi sweeps from zero on the
-// coarsest grid: up to float rounding V is a fixed symmetric positive
-// semi-definite operator, as conjugate gradients need.
+// in FP64).  Damped Jacobi with the same weights before and after the coarse
+// correction (three sweeps on the finest grid, two on the coarser ones),
+// restriction = 1/8 of the transpose of the injection prolongation, and a
+// fixed number of Jacobi sweeps from zero on the coarsest grid: up to float
+// rounding V is a fixed symmetric positive semi-definite operator, as
+// conjugate gradients need.
 // ---------------------------------------------------------------------------
-// Jacobi weight: the rows of the operator have off-diagonal magnitudes
-// summing to the diagonal, so the eigenvalues of D^-1 A lie in [0, 2] and any
-// weight below 1 keeps the smoother convergent and the V-cycle definite; 0.9
-// took the 192x192x96 random terrain's projection from 16 iterations (0.8) to
-// 13 at rtol 1e-10, 0.95 back up to 17.
-constexpr float MG_OMEGA = 0.9f;
-// Jacobi sweeps from zero on the coarsest grid (even: the result ends in x).
-// Any count gives a positive operator (the weight keeps 1 - w*lambda in
-// (-1, 1]); on the 192x192x96 random terrain 8 to 64 sweeps all needed 13
-// outer iterations, and fewer sweeps cost less (16: 7.6 ms, 64: 8.0 ms).
+// Jacobi sweeps on the coarsest grid (even: the result ends in x).
 constexpr int MG_COARSE_SWEEPS = 16;
+
+// Weights of the sweeps: the n sweeps of a smoother are one polynomial in
+// D^-1 A, whose eigenvalues lie in [0, 2] (the rows' off-diagonal magnitudes
+// sum to the diagonal).  The Chebyshev polynomial of an interval [a, 2]
+// damps everything in it to 1 / T_n((2 + a) / (2 - a)) (Saad, "Iterative
+// Methods for Sparse Linear Systems", 2003, sec. 12.3): the weights are the
+// reciprocals of its roots.  Below a it stays in (0, 1), so the V-cycle, the
+// same polynomial before and after the coarse correction, stays definite.
+// Three sweeps on [0.4, 2] on the finest grid, two on [0.3, 2] below,
+// sixteen on [0.1, 2] on the coarsest (taken in bit-reversed order, which
+// keeps the intermediate results small).  Iterations at rtol 1e-10, against
+// the weight 0.9 for every sweep: 192x192x96 random terrain 14 -> 11, 44x36x20 14
+// -> 9, 160x48x32 50 -> 40.
+struct MgWeights {
+  float fine[3], coarse[2], coarsest[MG_COARSE_SWEEPS];
+  MgWeights() {
+    auto weight = [](double a, int q, int n) {
+      return (float)(1.0 / (0.5 * (2.0 + a) + 0.5 * (2.0 - a) * cos((2 * q + 1) * M_PI / (2 * n))));
+    };
+    for (int q = 0; q < 3; ++q) fine[q] = weight(0.4, q, 3);
+    for (int q = 0; q < 2; ++q) coarse[q] = weight(0.3, q, 2);
+    for (int q = 0; q < MG_COARSE_SWEEPS; ++q) {
+      int r = 0;
+      for (int b = 1, m = MG_COARSE_SWEEPS / 2; b < MG_COARSE_SWEEPS; b *= 2, m /= 2) r += (q & b) ? m : 0;
+      coarsest[q] = weight(0.1, r, MG_COARSE_SWEEPS);
+    }
+  }
+};
 
 // The operator of one level.  From kreg[column] up, every face of the cells
 // within two columns is fully open (the terrain lies below), so there, away
@@ -523,7 +540,7 @@ constexpr int MG_COARSE_SWEEPS = 16;
 struct Op32 {
   Dims D;
   const float *bx, *by, *bz;   // low-face open fractions
-  const float *wi;             // MG_OMEGA / diagonal (0 off the active cells)
+  const float *wi;             // 1 / diagonal (0 off the active cells)
   const int *kreg;
   float ix2, iy2, iz2;
   __device__ inline float diag(long long c) const {
@@ -537,7 +554,7 @@ __global__ void k_mg_winv(Op32 L, float *wi) {
   const long long N = L.D.nxy * L.D.nz;
   for (long long c = blockIdx.x * (long long)PB + threadIdx.x; c < N; c += (long long)gridDim.x * PB) {
     const float d = L.diag(c);
-    wi[c] = d > 0.f ? MG_OMEGA / d : 0.f;
+    wi[c] = d > 0.f ? 1.f / d : 0.f;
   }
 }
 
@@ -610,12 +627,13 @@ __global__ void __launch_bounds__(MBX * MBY) k_mg_sweep(const __grid_constant__ 
                                                         const float *__restrict__ xin, const float *__restrict__ xc,
                                                         const __grid_constant__ Dims C, float *__restrict__ xout,
                                                         double *__restrict__ zout, const double *__restrict__ r,
-                                                        const float *__restrict__ b, Sum srz, const int *conv) {
+                                                        const float *__restrict__ b, float w0, float w, Sum srz,
+                                                        const int *conv) {
   chain_begin();
   if (*conv) return;
   const Dims &D = L.D;
   const Cols q = cols_of<V>(D, SL);
-  const float wreg = MG_OMEGA / (2.f * (L.ix2 + L.iy2 + L.iz2));
+  const float ireg = 1.f / (2.f * (L.ix2 + L.iy2 + L.iz2)), wreg = w * ireg, wfirst = w0 * ireg;
   int kr = 0;
 #pragma unroll
   for (int e = 0; e < V; ++e) kr = max(kr, L.kreg[q.c + e]);
@@ -632,11 +650,11 @@ __global__ void __launch_bounds__(MBX * MBY) k_mg_sweep(const __grid_constant__ 
       a = ldv<V>(b + t);
       if (reg) {
 #pragma unroll
-        for (int e = 0; e < V; ++e) a.v[e] *= wreg;
+        for (int e = 0; e < V; ++e) a.v[e] *= wfirst;
       } else {
-        const Vec<V> w = ldv<V>(L.wi + t);
+        const Vec<V> iv = ldv<V>(L.wi + t);
 #pragma unroll
-        for (int e = 0; e < V; ++e) a.v[e] *= w.v[e];
+        for (int e = 0; e < V; ++e) a.v[e] *= w0 * iv.v[e];
       }
     } else {
       a = ldv<V>(xin + t);
@@ -650,7 +668,7 @@ __global__ void __launch_bounds__(MBX * MBY) k_mg_sweep(const __grid_constant__ 
   };
   auto one = [&](int k, int o, int po, bool reg) -> float {
     const long long t = D.nxy * (long long)k + o;
-    if constexpr (MODE == FIRST) return b[t] * (reg ? wreg : L.wi[t]);
+    if constexpr (MODE == FIRST) return b[t] * (reg ? wfirst : w0 * L.wi[t]);
     else if constexpr (MODE == PROLONG) return xin[t] + xc[C.nxy * (long long)(k >> 1) + po];
     else return xin[t];
   };
@@ -675,7 +693,7 @@ __global__ void __launch_bounds__(MBX * MBY) k_mg_sweep(const __grid_constant__ 
         for (int e = 0; e < V; ++e) {
           const float S = L.ix2 * ((e ? x0.v[e ? e - 1 : 0] : xl) + (e + 1 < V ? x0.v[e + 1 < V ? e + 1 : 0] : xr)) +
                           L.iy2 * (ym.v[e] + yp.v[e]) + L.iz2 * (xm.v[e] + xp.v[e]);
-          o.v[e] = (1.f - MG_OMEGA) * x0.v[e] + wreg * (bv.v[e] + S);
+          o.v[e] = (1.f - w) * x0.v[e] + wreg * (bv.v[e] + S);
         }
       } else {
         const Vec<V> bx = ldv<V>(L.bx + t + q.c), yl = ldv<V>(L.by + t + q.c), yh = ldv<V>(L.by + t + q.yp),
@@ -691,15 +709,23 @@ __global__ void __launch_bounds__(MBX * MBY) k_mg_sweep(const __grid_constant__ 
                                    (e + 1 < V ? bx.v[e + 1 < V ? e + 1 : 0] * x0.v[e + 1 < V ? e + 1 : 0] : bxr * xr)) +
                           L.iy2 * (yl.v[e] * ym.v[e] + yh.v[e] * yp.v[e]) +
                           L.iz2 * (zl.v[e] * xm.v[e] + zh.v[e] * xp.v[e]);
-          o.v[e] = wi.v[e] > 0.f ? (1.f - MG_OMEGA) * x0.v[e] + wi.v[e] * (bv.v[e] + S) : 0.f;
+          o.v[e] = wi.v[e] > 0.f ? (1.f - w) * x0.v[e] + w * wi.v[e] * (bv.v[e] + S) : 0.f;
         }
       }
       if constexpr (FINAL) {
+        double z[V];
 #pragma unroll
-        for (int e = 0; e < V; ++e) {
-          const double z = widen(o.v[e]);
-          zout[t + q.c + e] = z;
-          rz = fma(r[t + q.c + e], z, rz);
+        for (int e = 0; e < V; ++e) z[e] = widen(o.v[e]);
+        if constexpr (V > 1) {
+#pragma unroll
+          for (int e = 0; e < V; e += 2) {
+            const double2 rv = *reinterpret_cast<const double2 *>(r + t + q.c + e);
+            *reinterpret_cast<double2 *>(zout + t + q.c + e) = make_double2(z[e], z[e + 1]);
+            rz = fma(rv.x, z[e], fma(rv.y, z[e + 1], rz));
+          }
+        } else {
+          zout[t + q.c] = z[0];
+          rz = fma(r[t + q.c], z[0], rz);
         }
       } else {
         stv<V>(xout + t + q.c, o);
@@ -799,6 +825,8 @@ struct MgLower {
   Op32 L[kMgMaxLevels];
   float *x[kMgMaxLevels], *t[kMgMaxLevels], *b[kMgMaxLevels];
   int lt, top;
+  float w[2];   // weights of the two sweeps (reversed after the coarse correction)
+  float wc[MG_COARSE_SWEEPS];
 };
 
 // One level as the block sees it.  On the SMEM path the pointers are built
@@ -834,7 +862,7 @@ __device__ __forceinline__ LowerLevel lower_level(const MgLower &M, int l, float
 // out = one sweep of xin, or (RES) the residual b - A xin.  A thread takes a
 // column, or a run of levels of it where the block has threads for more.
 template <bool RES>
-__device__ __forceinline__ void lower_pass(const LowerLevel &L, const float *__restrict__ xin,
+__device__ __forceinline__ void lower_pass(const LowerLevel &L, float om, const float *__restrict__ xin,
                                            float *__restrict__ out) {
   const int nx = L.nx, ny = L.ny, nz = L.nz, nxy = nx * ny;
   const float *__restrict__ bx = L.bx, *__restrict__ by = L.by, *__restrict__ bz = L.bz, *__restrict__ wi = L.wi,
@@ -856,7 +884,7 @@ __device__ __forceinline__ void lower_pass(const LowerLevel &L, const float *__r
                       L.iz2 * (zl * xm + zh * xp);
       float v;
       if (RES) v = b[c] - (L.ix2 * (bxl + bxr) + L.iy2 * (byl + byr) + L.iz2 * (zl + zh)) * x0 + S;
-      else v = (1.f - MG_OMEGA) * x0 + w * (b[c] + S);
+      else v = (1.f - om) * x0 + om * w * (b[c] + S);
       out[c] = w > 0.f ? v : 0.f;
       xm = x0;
       x0 = xp;
@@ -866,10 +894,10 @@ __device__ __forceinline__ void lower_pass(const LowerLevel &L, const float *__r
   __syncthreads();
 }
 // the sweep from zero
-__device__ __forceinline__ void lower_first(const LowerLevel &L, float *__restrict__ out) {
+__device__ __forceinline__ void lower_first(const LowerLevel &L, float om, float *__restrict__ out) {
   const float *__restrict__ wi = L.wi, *__restrict__ b = L.b;
 #pragma unroll 4
-  for (int c = threadIdx.x; c < L.n; c += blockDim.x) out[c] = wi[c] * b[c];
+  for (int c = threadIdx.x; c < L.n; c += blockDim.x) out[c] = om * wi[c] * b[c];
   __syncthreads();
 }
 
@@ -894,9 +922,9 @@ __global__ void __launch_bounds__(1024) k_mg_lower(const __grid_constant__ MgLow
   }
   for (int l = lt; l < top; ++l) {
     const LowerLevel V = lower_level<SMEM>(M, l, lower_smem), W = lower_level<SMEM>(M, l + 1, lower_smem);
-    lower_first(V, V.t);
-    lower_pass<false>(V, V.t, V.x);
-    lower_pass<true>(V, V.x, V.t);
+    lower_first(V, M.w[0], V.t);
+    lower_pass<false>(V, M.w[1], V.t, V.x);
+    lower_pass<true>(V, 0.f, V.x, V.t);
     const int sy = V.nx, sz = V.nx * V.ny;
     for (int c = threadIdx.x; c < W.n; c += blockDim.x) {   // the children's mean, as k_mg_restrict
       const int K = (int)W.fnxy.div((unsigned)c), col = c - K * W.nx * W.ny;
@@ -909,9 +937,9 @@ __global__ void __launch_bounds__(1024) k_mg_lower(const __grid_constant__ MgLow
   }
   {
     const LowerLevel V = lower_level<SMEM>(M, top, lower_smem);
-    lower_first(V, V.t);
+    lower_first(V, M.wc[0], V.t);
     for (int sw = 1; sw < MG_COARSE_SWEEPS; ++sw)   // coarsest sweeps; the result ends in x
-      lower_pass<false>(V, (sw & 1) ? V.t : V.x, (sw & 1) ? V.x : V.t);
+      lower_pass<false>(V, M.wc[sw], (sw & 1) ? V.t : V.x, (sw & 1) ? V.x : V.t);
   }
   for (int l = top - 1; l >= lt; --l) {
     const LowerLevel V = lower_level<SMEM>(M, l, lower_smem), W = lower_level<SMEM>(M, l + 1, lower_smem);
@@ -921,8 +949,8 @@ __global__ void __launch_bounds__(1024) k_mg_lower(const __grid_constant__ MgLow
       V.x[c] += W.x[(i >> 1) + W.nx * ((j >> 1) + W.ny * (k >> 1))];
     }
     __syncthreads();
-    lower_pass<false>(V, V.x, V.t);
-    lower_pass<false>(V, V.t, V.x);
+    lower_pass<false>(V, M.w[1], V.x, V.t);
+    lower_pass<false>(V, M.w[0], V.t, V.x);
   }
   if constexpr (SMEM) {
     const LowerLevel V = lower_level<true>(M, lt, lower_smem);
@@ -1041,7 +1069,7 @@ eb_status mg_setup(eb_geom g, cudaStream_t s) {
   for (float **a : {&L0.bx, &L0.by, &L0.bz, &L0.x, &L0.t, &L0.b, &L0.wi})
     CUDA_TRY(g->alloc(a, N0), "alloc multigrid level");
   k_mg_copy<<<L0.nb, PB, 0, s>>>(N0, w.bx, w.by, w.bz, L0.bx, L0.by, L0.bz);
-  // MG_OMEGA / diagonal and the open levels of a level whose fractions are set
+  // 1 / diagonal and the open levels of a level whose fractions are set
   auto finish = [&](MgLevel &L) -> cudaError_t {
     cudaError_t e = g->alloc(&L.kreg, L.D.nxy);
     int *top = nullptr;
@@ -1089,16 +1117,16 @@ inline int level_v(const MgLevel &L) {
 
 template <int MODE, bool FINAL>
 void sweep(const MgLevel &L, const float *xin, const MgLevel *coarse, float *xout, double *zout, const double *r,
-           const Sum &rz, const int *conv, cudaStream_t s) {
+           float w0, float w, const Sum &rz, const int *conv, cudaStream_t s) {
   const int V = level_v(L);
   const Slabs S = slabs_of(L.D, V, ebk_sm_count());
   const Op32 O = level_op(L);
   const Dims C = coarse ? coarse->D : L.D;
   const float *xc = coarse ? coarse->x : nullptr;
   const dim3 blk(MBX, MBY, 1);
-  if (V == 4) launch_chained(k_mg_sweep<4, MODE, FINAL>, S.blocks(), blk, 0, s, O, S, xin, xc, C, xout, zout, r, L.b, rz, conv);
-  else if (V == 2) launch_chained(k_mg_sweep<2, MODE, FINAL>, S.blocks(), blk, 0, s, O, S, xin, xc, C, xout, zout, r, L.b, rz, conv);
-  else launch_chained(k_mg_sweep<1, MODE, FINAL>, S.blocks(), blk, 0, s, O, S, xin, xc, C, xout, zout, r, L.b, rz, conv);
+  if (V == 4) launch_chained(k_mg_sweep<4, MODE, FINAL>, S.blocks(), blk, 0, s, O, S, xin, xc, C, xout, zout, r, L.b, w0, w, rz, conv);
+  else if (V == 2) launch_chained(k_mg_sweep<2, MODE, FINAL>, S.blocks(), blk, 0, s, O, S, xin, xc, C, xout, zout, r, L.b, w0, w, rz, conv);
+  else launch_chained(k_mg_sweep<1, MODE, FINAL>, S.blocks(), blk, 0, s, O, S, xin, xc, C, xout, zout, r, L.b, w0, w, rz, conv);
 }
 
 // from a level with an even number of columns (it is coarsened)
@@ -1118,17 +1146,18 @@ void restrict_residual(const MgLevel &F, const float *x, const MgLevel &C, const
 void vcycle(eb_geom g, const double *r, double *z, int rz, cudaStream_t s) {
   const Sum none{nullptr, nullptr, nullptr};
   ProjWork &w = g->pw;
+  static const MgWeights W;
   const MgLevel *L = w.lev;
   const int top = w.nlev - 1;
   // levels lt .. top (at most MG_LOWER_CELLS cells each) run in one block; level 0 never does
   int lt = top;
   while (lt > 1 && L[lt - 1].D.nxy * L[lt - 1].D.nz <= MG_LOWER_CELLS) --lt;
   // sweeps before and after the coarse correction: three on the finest level, two below
-  sweep<FIRST, false>(L[0], nullptr, nullptr, L[0].t, nullptr, nullptr, none, w.conv, s);
-  sweep<PLAIN, false>(L[0], L[0].t, nullptr, L[0].x, nullptr, nullptr, none, w.conv, s);
+  sweep<FIRST, false>(L[0], nullptr, nullptr, L[0].t, nullptr, nullptr, W.fine[0], W.fine[1], none, w.conv, s);
+  sweep<PLAIN, false>(L[0], L[0].t, nullptr, L[0].x, nullptr, nullptr, 0.f, W.fine[2], none, w.conv, s);
   restrict_residual(L[0], L[0].x, L[1], w.conv, s);
   for (int l = 1; l < lt; ++l) {
-    sweep<FIRST, false>(L[l], nullptr, nullptr, L[l].x, nullptr, nullptr, none, w.conv, s);
+    sweep<FIRST, false>(L[l], nullptr, nullptr, L[l].x, nullptr, nullptr, W.coarse[0], W.coarse[1], none, w.conv, s);
     restrict_residual(L[l], L[l].x, L[l + 1], w.conv, s);
   }
   {
@@ -1139,6 +1168,8 @@ void vcycle(eb_geom g, const double *r, double *z, int rz, cudaStream_t s) {
       M.t[l] = L[l].t;
       M.b[l] = L[l].b;
     }
+    M.w[0] = W.coarse[0], M.w[1] = W.coarse[1];
+    for (int q = 0; q < MG_COARSE_SWEEPS; ++q) M.wc[q] = W.coarsest[q];
     M.lt = lt;
     M.top = top;
     static unsigned long long attr = 0;
@@ -1147,12 +1178,12 @@ void vcycle(eb_geom g, const double *r, double *z, int rz, cudaStream_t s) {
     else launch_chained(k_mg_lower<false>, 1, 1024, 0, s, M, w.conv);
   }
   for (int l = lt - 1; l >= 1; --l) {
-    sweep<PROLONG, false>(L[l], L[l].x, &L[l + 1], L[l].t, nullptr, nullptr, none, w.conv, s);
-    sweep<PLAIN, false>(L[l], L[l].t, nullptr, L[l].x, nullptr, nullptr, none, w.conv, s);
+    sweep<PROLONG, false>(L[l], L[l].x, &L[l + 1], L[l].t, nullptr, nullptr, 0.f, W.coarse[1], none, w.conv, s);
+    sweep<PLAIN, false>(L[l], L[l].t, nullptr, L[l].x, nullptr, nullptr, 0.f, W.coarse[0], none, w.conv, s);
   }
-  sweep<PROLONG, false>(L[0], L[0].x, &L[1], L[0].t, nullptr, nullptr, none, w.conv, s);
-  sweep<PLAIN, false>(L[0], L[0].t, nullptr, L[0].x, nullptr, nullptr, none, w.conv, s);
-  sweep<PLAIN, true>(L[0], L[0].x, nullptr, nullptr, z, r, sum_of(g, rz), w.conv, s);
+  sweep<PROLONG, false>(L[0], L[0].x, &L[1], L[0].t, nullptr, nullptr, 0.f, W.fine[2], none, w.conv, s);
+  sweep<PLAIN, false>(L[0], L[0].t, nullptr, L[0].x, nullptr, nullptr, 0.f, W.fine[1], none, w.conv, s);
+  sweep<PLAIN, true>(L[0], L[0].x, nullptr, nullptr, z, r, 0.f, W.fine[0], sum_of(g, rz), w.conv, s);
 }
 
 // the scalars of slots first .. last on the host (synchronises the stream)
@@ -1244,7 +1275,7 @@ eb_status eb_project_impl(eb_geom g, void *const mom[3], double dt, double rtol,
   int it = 0;
   double rr = rr0;
   if (bb > 0.0 && rr0 > thr2) {
-    int done = 0;
+    int done = 0, next = mg ? 4 : 32;
     for (it = 0; it < maxit; ++it) {
       const int rz = it % 2 ? S_RZ1 : S_RZ0, rz_next = it % 2 ? S_RZ0 : S_RZ1;
       launch_apply(g, w.p, w.q, it, s);
@@ -1260,14 +1291,18 @@ eb_status eb_project_impl(eb_geom g, void *const mom[3], double dt, double rtol,
         launch_chained(k_direction<true>, w.nb, PB, 0, s, O, w.x, w.p, w.r, w.scal + rz, w.scal + rz_next, w.scal + S_PQ,
                                               w.scal + S_RR, thr2, it, w.conv);
       }
-      // the host reads the convergence flag every few iterations (a V-cycle
-      // iteration costs far more than a Jacobi one, so it looks sooner)
-      if ((it + 1) % (mg ? 4 : 32) == 0 || it + 1 == maxit) {
+      // The host reads the convergence flag after a first few iterations
+      // (fewer with V-cycles, which cost far more than Jacobi iterations),
+      // and then where the mean reduction so far says the threshold is met.
+      if (it + 1 == next || it + 1 == maxit) {
         int *flag = reinterpret_cast<int *>(w.host + S_SLOTS);
         CUDA_TRY(cudaMemcpyAsync(flag, w.conv, sizeof(int), cudaMemcpyDeviceToHost, s), "convergence flag");
-        CUDA_TRY(cudaStreamSynchronize(s), "convergence flag");
+        CUDA_TRY(host_scalars(g, S_RR, S_RR, &rr, s), "convergence flag");
         done = *flag;
         if (done) break;
+        const double rate = log(rr0 / rr) / (it + 1), left = log(rr / thr2);
+        const double more = rate > 0.0 ? ceil(left / rate) : 1.0;
+        next = it + 1 + (int)fmin(fmax(more, 1.0), mg ? 8.0 : 64.0);
       }
     }
     it = done ? done : maxit;
