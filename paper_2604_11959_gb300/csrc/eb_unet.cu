@@ -80,6 +80,29 @@ struct ConvTile {
   static_assert(TZ % 2 == 0 && COLS <= 256, "two warp quads share the z-levels; two CTAs per SM share TMEM");
 };
 
+// The input of a convolution: plain (cup = 0: channels of a), or the
+// concatenation of cup channels of the half-resolution tensor a, upsampled
+// by nearest neighbours, and the full-resolution channels of b.  The loads
+// read the parts where they lie (a concatenated copy of the 192x192x96
+// network's finest level took 0.3 ms to write and read); cup is a multiple
+// of the 16 channels of a chunk, so a chunk has one source.
+struct ConvIn {
+  const float *a, *b;
+  int cup;
+};
+
+// Where a convolution's output goes: channels below split to a, the others
+// to b (split a multiple of 16); with head set (the last layer, 16 channels)
+// the 1x1 head of the network is applied in the epilogue as well, y = hb + sum
+// of hw[c] times channel c, and a may be NULL (inference needs no more).
+struct ConvOut {
+  float *a, *b;
+  int split;
+  const __nv_bfloat16 *hw;
+  const float *hb;
+  float *y;
+};
+
 constexpr long long kWaitCycles = 2000000000LL;   // about one second at the maximum SM clock
 
 __device__ __forceinline__ uint32_t pack_bf16(__nv_bfloat16 a, __nv_bfloat16 b) {
@@ -87,8 +110,8 @@ __device__ __forceinline__ uint32_t pack_bf16(__nv_bfloat16 a, __nv_bfloat16 b) 
 }
 
 template <int NP, int TZ, bool MASK>
-__global__ void __launch_bounds__(256, 2) k_conv3_umma(const float *in, int cin, const __nv_bfloat16 *Wp,
-                                                       const float *bias, float *out, int cout, Vol V, int relu,
+__global__ void __launch_bounds__(256, 2) k_conv3_umma(ConvIn in, int cin, const __nv_bfloat16 *Wp,
+                                                       const float *bias, ConvOut out, int cout, Vol V, int relu,
                                                        const float *mask, int *err, int skip_commit) {
   using G = ConvTile<NP, TZ>;
   extern __shared__ __align__(16) unsigned char cv_smem[];
@@ -118,6 +141,10 @@ __global__ void __launch_bounds__(256, 2) k_conv3_umma(const float *in, int cin,
   auto load_step = [&](int i) {
     const int tile = tile_of(i), c0 = (i % nch) * 16;
     const int x0 = (tile % ntx) * 8, y0 = ((tile / ntx) % nty) * 16, z0 = (tile / (ntx * nty)) * TZ;
+    const bool up = c0 < in.cup;
+    const float *base = up ? in.a + (long long)c0 * (N / 8)
+                           : (in.cup ? in.b + (long long)(c0 - in.cup) * N : in.a + (long long)c0 * N);
+    const long long cs = up ? N / 8 : N;   // channel stride
 #pragma unroll
     for (int k = 0; k < IS; ++k) {
       const int q = tid + 256 * k;
@@ -125,11 +152,12 @@ __global__ void __launch_bounds__(256, 2) k_conv3_umma(const float *in, int cin,
       const int hx = h % G::HX, hy = (h / G::HX) % G::HY, hz = h / (G::HX * G::HY);
       const int x = x0 + hx - 1, y = y0 + hy - 1, z = z0 + hz - 1;
       const bool inside = q < ITEMS && x >= 0 && x < V.nx && y >= 0 && y < V.ny && z >= 0 && z < V.nz;
-      const float *src = in + ((long long)z * V.ny + y) * V.nx + x;
+      const float *src = base + (up ? ((long long)(z >> 1) * (V.ny / 2) + (y >> 1)) * (V.nx / 2) + (x >> 1)
+                                    : ((long long)z * V.ny + y) * V.nx + x);
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        const int c = c0 + kg * 8 + j;
-        pv[k][j] = inside && c < cin ? src[(long long)c * N] : 0.f;
+        const int c = kg * 8 + j;
+        pv[k][j] = inside && c0 + c < cin ? src[c * cs] : 0.f;
       }
     }
   };
@@ -174,6 +202,8 @@ __global__ void __launch_bounds__(256, 2) k_conv3_umma(const float *in, int cin,
         float v[16];
         umma::ld16(tm + ((uint32_t)(32 * quad) << 16) + (uint32_t)(rz * NP + cc), v);
         if (live) {
+          float *dst = cc < out.split ? out.a + (long long)cc * N : out.b + (long long)(cc - out.split) * N;
+          float y = out.y ? out.hb[0] : 0.f;
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
             const int co = cc + j;
@@ -181,9 +211,11 @@ __global__ void __launch_bounds__(256, 2) k_conv3_umma(const float *in, int cin,
               float o = v[j] + (bias ? bias[co] : 0.f);
               if (relu) o = fmaxf(o, 0.f);
               if (MASK && !(mk[j] > 0.f)) o = 0.f;   // ReLU backward of the input
-              out[(long long)co * N + vox] = o;
+              if (out.y) y = fmaf(__bfloat162float(out.hw[co]), o, y);
+              if (out.a) dst[(long long)j * N + vox] = o;
             }
           }
+          if (out.y) out.y[vox] = y;
         }
       }
     }
@@ -248,15 +280,6 @@ __global__ void __launch_bounds__(256, 2) k_conv3_umma(const float *in, int cin,
   umma::fence_before();
   __syncthreads();
   if (warp == 0) umma::dealloc(tm, G::TCOLS);
-}
-
-// 1x1 head: out[v] = b + sum_ci W[ci] in[ci][v]
-__global__ void k_head(const float *in, int cin, const __nv_bfloat16 *W, const float *bias, float *out, long long N) {
-  const long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (v >= N) return;
-  float a = bias[0];
-  for (int c = 0; c < cin; ++c) a = fmaf(__bfloat162float(W[c]), in[c * N + v], a);
-  out[v] = a;
 }
 
 // head backward: dIn[ci][v] = W[ci] dy[v] where the head's (ReLU) input post[ci][v] > 0, else 0
@@ -355,7 +378,7 @@ struct WgTile {
 };
 
 template <int NP>
-__global__ void __launch_bounds__(256, 2) k_conv3_wgrad_umma(const float *in, int cin, const float *dout, int cout,
+__global__ void __launch_bounds__(256, 2) k_conv3_wgrad_umma(ConvIn in, int cin, const float *dout, int cout,
                                                              Vol V, float *dW, float *dB, int *err, int vec) {
   using G = WgTile<NP>;
   extern __shared__ __align__(16) unsigned char wg_smem[];
@@ -385,6 +408,7 @@ __global__ void __launch_bounds__(256, 2) k_conv3_wgrad_umma(const float *in, in
   float pin[IS][10], pdo[DS][8], bsum[DS];
 #pragma unroll
   for (int k = 0; k < DS; ++k) bsum[k] = 0.f;
+  const bool up = c0 < in.cup;   // the chunk's channels are upsampled ones
   auto load_tile = [&](int tile) {
     const int x0 = (tile % ntx) * G::TX, y0 = ((tile / ntx) % nty) * G::TY, z0 = (tile / (ntx * nty)) * G::TZ;
 #pragma unroll
@@ -393,8 +417,18 @@ __global__ void __launch_bounds__(256, 2) k_conv3_wgrad_umma(const float *in, in
       const int ci = q % G::CI, hy = (q / G::CI) % G::HY, hz = q / (G::CI * G::HY);
       const int y = y0 + hy - 1, z = z0 + hz - 1, c = c0 + ci;
       const bool row = q < IT && c < cin && y >= 0 && y < V.ny && z >= 0 && z < V.nz;
-      const float *src = in + (long long)c * N + ((long long)z * V.ny + y) * V.nx;
-      if (vec) {   // rows of a multiple of 4 values, 16-byte aligned: x0 - 4 ... x0 + 11 in four float4
+      const float *src = up ? in.a + (long long)c * (N / 8) + ((long long)(z >> 1) * (V.ny / 2) + (y >> 1)) * (V.nx / 2)
+                            : (in.cup ? in.b + (long long)(c - in.cup) * N : in.a + (long long)c * N) +
+                                  ((long long)z * V.ny + y) * V.nx;
+      if (up) {   // the half-resolution row: x0 / 2 - 1 ... x0 / 2 + 4, each value twice
+        const int hx0 = x0 / 2, hn = V.nx / 2;
+        float h[6];
+        h[0] = row && hx0 >= 1 ? src[hx0 - 1] : 0.f;
+#pragma unroll
+        for (int e = 0; e < 5; ++e) h[e + 1] = row && hx0 + e < hn ? src[hx0 + e] : 0.f;
+#pragma unroll
+        for (int e = 0; e < 10; ++e) pin[k][e] = h[(e + 1) / 2];
+      } else if (vec) {   // rows of a multiple of 4 values, 16-byte aligned: x0 - 4 ... x0 + 11 in four float4
         const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
         const float4 *s4 = reinterpret_cast<const float4 *>(src + x0);
         const float4 a = row && x0 >= 4 ? __ldg(s4 - 1) : z4;
@@ -589,16 +623,6 @@ __global__ void k_pool_bwd_add(const float *dout, Vol V, const float *post, floa
   din[q] = post[q] > 0.f ? g : 0.f;
 }
 
-// out (C, V) = nearest upsampling of in (C, V/2)
-__global__ void k_up(const float *in, Vol V, float *out) {
-  const unsigned n = (unsigned)V.nx * V.ny * V.nz;
-  const unsigned r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= n) return;
-  const unsigned x = r % V.nx, t = r / V.nx, y = t % V.ny, z = t / V.ny;
-  const unsigned hx = V.nx / 2, hy = V.ny / 2, hn = hx * hy * (unsigned)(V.nz / 2);
-  out[(size_t)blockIdx.y * n + r] = in[(size_t)blockIdx.y * hn + ((z / 2) * hy + y / 2) * hx + x / 2];
-}
-
 // din (C, V/2) = upsampling backward of dout (C, V): sum of the 8 children,
 // zeroed where post (C, V/2) (the ReLU output upsampled) is not positive
 __global__ void k_up_bwd(const float *dout, Vol V, const float *post, float *din) {
@@ -670,7 +694,7 @@ struct eb_unet_s {
   long long wp_off[10][2];                       // packed weights: forward, input gradient
   long long off_w[11], off_b[11];
   // activations (forward) and their gradients
-  float *e1a, *e1, *p1, *e2a, *e2, *p2, *ba, *bt, *c2, *d2a, *d2, *c1, *d1a, *d1, *y;
+  float *e1a, *e1, *p1, *e2a, *e2, *p2, *ba, *bt, *d2a, *d2, *d1a, *d1, *y;
   float *ge1a, *ge1, *gp1, *ge2a, *ge2, *gp2, *gba, *gbt, *gc2, *gd2a, *gd2, *gc1, *gd1a, *gd1, *gy;
   float *loss = nullptr;
   bool grads = false;
@@ -694,8 +718,8 @@ namespace {
 long long packed_size(int cin, int cout) { return (long long)((cin + 15) / 16) * 27 * 2 * ((cout + 15) / 16 * 16) * 8; }
 
 template <int NP, int TZ, bool MASK>
-void conv3_umma_launch(const float *in, int cin, const __nv_bfloat16 *Wp, const float *bias, float *out, int cout,
-                       const Vol &V, bool relu, const float *mask, int *err, int skip_commit, cudaStream_t s) {
+void conv3_umma_launch(const ConvIn &in, int cin, const __nv_bfloat16 *Wp, const float *bias, const ConvOut &out,
+                       int cout, const Vol &V, bool relu, const float *mask, int *err, int skip_commit, cudaStream_t s) {
   using G = ConvTile<NP, TZ>;
   static unsigned long long attr = 0;
   ebk_smem_limit(k_conv3_umma<NP, TZ, MASK>, G::SMEM, attr);
@@ -710,8 +734,8 @@ void conv3_umma_launch(const float *in, int cin, const __nv_bfloat16 *Wp, const 
 // own, or its transposed and flipped ones for an input gradient); mask:
 // where not NULL, out is zeroed wherever mask (cout, V) is not positive (the
 // ReLU backward of the layer below)
-void conv3_tc(eb_unet u, const float *in, int cin, const __nv_bfloat16 *Wp, const float *bias, float *out, int cout,
-              const Vol &V, bool relu, const float *mask, cudaStream_t s) {
+void conv3_tc(eb_unet u, const ConvIn &in, int cin, const __nv_bfloat16 *Wp, const float *bias, const ConvOut &out,
+              int cout, const Vol &V, bool relu, const float *mask, cudaStream_t s) {
   const int NP = (cout + 15) / 16 * 16;
   const int skip = u->fault;   // the failure test: one launch never signals its products' completion
   u->fault = 0;
@@ -734,7 +758,10 @@ void conv3_tc(eb_unet u, const float *in, int cin, const __nv_bfloat16 *Wp, cons
   }
 }
 
-void conv3(eb_unet u, int l, const float *in, float *out, const Vol &V, bool relu, cudaStream_t s) {
+ConvIn plain(const float *a) { return ConvIn{a, nullptr, 0}; }
+ConvOut whole(float *a) { return ConvOut{a, nullptr, 1 << 20, nullptr, nullptr, nullptr}; }
+
+void conv3(eb_unet u, int l, const ConvIn &in, const ConvOut &out, const Vol &V, bool relu, cudaStream_t s) {
   const LayerSpec &L = kLayers[l];
   conv3_tc(u, in, L.cin, u->wp + u->wp_off[l][0], u->p + u->off_b[l], out, L.cout, V, relu, nullptr, s);
 }
@@ -747,9 +774,10 @@ static_assert(kLayers[1].cin == 16 && kLayers[3].cin == 32 && kLayers[5].cin == 
 
 // input gradient of layer l: din = conv of dout with flipped, transposed W,
 // zeroed where mask (the layer's ReLU input, when there is one) is not positive
-void conv3_dgrad(eb_unet u, int l, const float *dout, float *din, const float *mask, const Vol &V, cudaStream_t s) {
+void conv3_dgrad(eb_unet u, int l, const float *dout, const ConvOut &din, const float *mask, const Vol &V,
+                 cudaStream_t s) {
   const LayerSpec &L = kLayers[l];
-  conv3_tc(u, dout, L.cout, u->wp + u->wp_off[l][1], nullptr, din, L.cin, V, false, mask, s);
+  conv3_tc(u, plain(dout), L.cout, u->wp + u->wp_off[l][1], nullptr, din, L.cin, V, false, mask, s);
 }
 
 // every convolution's packed weights from the BF16 working weights
@@ -771,7 +799,7 @@ void pack_weights(eb_unet u, cudaStream_t s) {
 }
 
 template <int NP>
-void conv3_wgrad_launch(const float *in, int cin, const float *dout, int cout, const Vol &V, float *dW, float *dB,
+void conv3_wgrad_launch(const ConvIn &in, int cin, const float *dout, int cout, const Vol &V, float *dW, float *dB,
                         int *err, cudaStream_t s) {
   using G = WgTile<NP>;
   static unsigned long long attr = 0;
@@ -781,11 +809,11 @@ void conv3_wgrad_launch(const float *in, int cin, const float *dout, int cout, c
   const int gy = 3 / G::DZN, gz = (cin + G::CI - 1) / G::CI;
   const int gx = std::max(1, std::min(ntiles, 2 * sms / (gy * gz)));   // two CTAs per SM, each over many tiles
   // float4 loads where every row starts on a 16-byte boundary
-  const int vec = V.nx % 4 == 0 && (uintptr_t)in % 16 == 0 && (uintptr_t)dout % 16 == 0;
+  const int vec = V.nx % 4 == 0 && (uintptr_t)in.a % 16 == 0 && (uintptr_t)in.b % 16 == 0 && (uintptr_t)dout % 16 == 0;
   k_conv3_wgrad_umma<NP><<<dim3(gx, gy, gz), 256, G::SMEM, s>>>(in, cin, dout, cout, V, dW, dB, err, vec);
 }
 
-void conv3_wgrad(eb_unet u, int l, const float *in, const float *dout, const Vol &V, cudaStream_t s) {
+void conv3_wgrad(eb_unet u, int l, const ConvIn &in, const float *dout, const Vol &V, cudaStream_t s) {
   const LayerSpec &L = kLayers[l];
   float *dW = u->g + u->off_w[l], *dB = u->g + u->off_b[l];   // the bias gradient rides along
   if (L.cout <= 16) conv3_wgrad_launch<16>(in, L.cin, dout, L.cout, V, dW, dB, u->err, s);
@@ -793,25 +821,26 @@ void conv3_wgrad(eb_unet u, int l, const float *in, const float *dout, const Vol
   else conv3_wgrad_launch<64>(in, L.cin, dout, L.cout, V, dW, dB, u->err, s);
 }
 
-void forward(eb_unet u, const float *x, cudaStream_t s) {
+// inputs of the two layers after the skips: upsampled channels, then the skip's
+ConvIn cat2(eb_unet u) { return ConvIn{u->bt, u->e2, 64}; }
+ConvIn cat1(eb_unet u) { return ConvIn{u->d2, u->e1, 32}; }
+
+// the network's output into y; keep: the last layer's activations stay for a backward pass
+void forward(eb_unet u, const float *x, float *y, bool keep, cudaStream_t s) {
   const Vol &V0 = u->V[0], &V1 = u->V[1], &V2 = u->V[2];
-  conv3(u, 0, x, u->e1a, V0, true, s);
-  conv3(u, 1, u->e1a, u->e1, V0, true, s);
+  conv3(u, 0, plain(x), whole(u->e1a), V0, true, s);
+  conv3(u, 1, plain(u->e1a), whole(u->e1), V0, true, s);
   k_pool<<<dim3(nblk(V1.n()), 16), 256, 0, s>>>(u->e1, V0, u->p1);
-  conv3(u, 2, u->p1, u->e2a, V1, true, s);
-  conv3(u, 3, u->e2a, u->e2, V1, true, s);
+  conv3(u, 2, plain(u->p1), whole(u->e2a), V1, true, s);
+  conv3(u, 3, plain(u->e2a), whole(u->e2), V1, true, s);
   k_pool<<<dim3(nblk(V2.n()), 32), 256, 0, s>>>(u->e2, V1, u->p2);
-  conv3(u, 4, u->p2, u->ba, V2, true, s);
-  conv3(u, 5, u->ba, u->bt, V2, true, s);
-  k_up<<<dim3(nblk(V1.n()), 64), 256, 0, s>>>(u->bt, V1, u->c2);
-  cudaMemcpyAsync(u->c2 + 64 * V1.n(), u->e2, sizeof(float) * 32 * V1.n(), cudaMemcpyDeviceToDevice, s);
-  conv3(u, 6, u->c2, u->d2a, V1, true, s);
-  conv3(u, 7, u->d2a, u->d2, V1, true, s);
-  k_up<<<dim3(nblk(V0.n()), 32), 256, 0, s>>>(u->d2, V0, u->c1);
-  cudaMemcpyAsync(u->c1 + 32 * V0.n(), u->e1, sizeof(float) * 16 * V0.n(), cudaMemcpyDeviceToDevice, s);
-  conv3(u, 8, u->c1, u->d1a, V0, true, s);
-  conv3(u, 9, u->d1a, u->d1, V0, true, s);
-  k_head<<<nblk(V0.n()), 256, 0, s>>>(u->d1, 16, u->pb + u->off_w[10], u->p + u->off_b[10], u->y, V0.n());
+  conv3(u, 4, plain(u->p2), whole(u->ba), V2, true, s);
+  conv3(u, 5, plain(u->ba), whole(u->bt), V2, true, s);
+  conv3(u, 6, cat2(u), whole(u->d2a), V1, true, s);
+  conv3(u, 7, plain(u->d2a), whole(u->d2), V1, true, s);
+  conv3(u, 8, cat1(u), whole(u->d1a), V0, true, s);
+  const ConvOut last{keep ? u->d1 : nullptr, nullptr, 1 << 20, u->pb + u->off_w[10], u->p + u->off_b[10], y};
+  conv3(u, 9, plain(u->d1a), last, V0, true, s);
 }
 
 // gradient of the masked loss into u->g (zeroed first); loss into u->loss
@@ -823,31 +852,33 @@ void backward(eb_unet u, const float *x, cudaStream_t s) {
   k_chan_dot<<<dim3(64, 16), 256, 0, s>>>(u->d1, u->gy, 16, n0, u->g + u->off_w[10]);
   k_chan_dot<<<dim3(64, 1), 256, 0, s>>>(u->gy, nullptr, 1, n0, u->g + u->off_b[10]);
   k_head_bwd<<<nblk(n0), 256, 0, s>>>(u->gy, u->pb + u->off_w[10], 16, u->d1, u->gd1, n0);
-  conv3_wgrad(u, 9, u->d1a, u->gd1, V0, s);
-  conv3_dgrad(u, 9, u->gd1, u->gd1a, u->d1a, V0, s);
-  conv3_wgrad(u, 8, u->c1, u->gd1a, V0, s);
-  conv3_dgrad(u, 8, u->gd1a, u->gc1, nullptr, V0, s);
+  conv3_wgrad(u, 9, plain(u->d1a), u->gd1, V0, s);
+  conv3_dgrad(u, 9, u->gd1, whole(u->gd1a), u->d1a, V0, s);
+  conv3_wgrad(u, 8, cat1(u), u->gd1a, V0, s);
+  ConvOut split1 = whole(u->gc1);   // the upsampled channels' gradient and the skip's
+  split1.b = u->ge1, split1.split = 32;
+  conv3_dgrad(u, 8, u->gd1a, split1, nullptr, V0, s);
   k_up_bwd<<<dim3(nblk(n1), 32), 256, 0, s>>>(u->gc1, V0, u->d2, u->gd2);
-  cudaMemcpyAsync(u->ge1, u->gc1 + 32 * n0, sizeof(float) * 16 * n0, cudaMemcpyDeviceToDevice, s);
-  conv3_wgrad(u, 7, u->d2a, u->gd2, V1, s);
-  conv3_dgrad(u, 7, u->gd2, u->gd2a, u->d2a, V1, s);
-  conv3_wgrad(u, 6, u->c2, u->gd2a, V1, s);
-  conv3_dgrad(u, 6, u->gd2a, u->gc2, nullptr, V1, s);
+  conv3_wgrad(u, 7, plain(u->d2a), u->gd2, V1, s);
+  conv3_dgrad(u, 7, u->gd2, whole(u->gd2a), u->d2a, V1, s);
+  conv3_wgrad(u, 6, cat2(u), u->gd2a, V1, s);
+  ConvOut split2 = whole(u->gc2);
+  split2.b = u->ge2, split2.split = 64;
+  conv3_dgrad(u, 6, u->gd2a, split2, nullptr, V1, s);
   k_up_bwd<<<dim3(nblk(n2), 64), 256, 0, s>>>(u->gc2, V1, u->bt, u->gbt);
-  cudaMemcpyAsync(u->ge2, u->gc2 + 64 * n1, sizeof(float) * 32 * n1, cudaMemcpyDeviceToDevice, s);
-  conv3_wgrad(u, 5, u->ba, u->gbt, V2, s);
-  conv3_dgrad(u, 5, u->gbt, u->gba, u->ba, V2, s);
-  conv3_wgrad(u, 4, u->p2, u->gba, V2, s);
-  conv3_dgrad(u, 4, u->gba, u->gp2, nullptr, V2, s);
+  conv3_wgrad(u, 5, plain(u->ba), u->gbt, V2, s);
+  conv3_dgrad(u, 5, u->gbt, whole(u->gba), u->ba, V2, s);
+  conv3_wgrad(u, 4, plain(u->p2), u->gba, V2, s);
+  conv3_dgrad(u, 4, u->gba, whole(u->gp2), nullptr, V2, s);
   k_pool_bwd_add<<<dim3(nblk(n1), 32), 256, 0, s>>>(u->gp2, V1, u->e2, u->ge2);
-  conv3_wgrad(u, 3, u->e2a, u->ge2, V1, s);
-  conv3_dgrad(u, 3, u->ge2, u->ge2a, u->e2a, V1, s);
-  conv3_wgrad(u, 2, u->p1, u->ge2a, V1, s);
-  conv3_dgrad(u, 2, u->ge2a, u->gp1, nullptr, V1, s);
+  conv3_wgrad(u, 3, plain(u->e2a), u->ge2, V1, s);
+  conv3_dgrad(u, 3, u->ge2, whole(u->ge2a), u->e2a, V1, s);
+  conv3_wgrad(u, 2, plain(u->p1), u->ge2a, V1, s);
+  conv3_dgrad(u, 2, u->ge2a, whole(u->gp1), nullptr, V1, s);
   k_pool_bwd_add<<<dim3(nblk(n0), 16), 256, 0, s>>>(u->gp1, V0, u->e1, u->ge1);
-  conv3_wgrad(u, 1, u->e1a, u->ge1, V0, s);
-  conv3_dgrad(u, 1, u->ge1, u->ge1a, u->e1a, V0, s);
-  conv3_wgrad(u, 0, x, u->ge1a, V0, s);
+  conv3_wgrad(u, 1, plain(u->e1a), u->ge1, V0, s);
+  conv3_dgrad(u, 1, u->ge1, whole(u->ge1a), u->e1a, V0, s);
+  conv3_wgrad(u, 0, plain(x), u->ge1a, V0, s);
 }
 
 eb_status ensure_grads(eb_unet u) {
@@ -857,8 +888,8 @@ eb_status ensure_grads(eb_unet u) {
     float **q;
     long long n;
   } b[] = {{&u->ge1a, 16 * n0}, {&u->ge1, 16 * n0}, {&u->gp1, 16 * n1}, {&u->ge2a, 32 * n1}, {&u->ge2, 32 * n1},
-           {&u->gp2, 32 * n2},  {&u->gba, 64 * n2},  {&u->gbt, 64 * n2}, {&u->gc2, 96 * n1},  {&u->gd2a, 32 * n1},
-           {&u->gd2, 32 * n1},  {&u->gc1, 48 * n0},  {&u->gd1a, 16 * n0}, {&u->gd1, 16 * n0}, {&u->gy, n0}};
+           {&u->gp2, 32 * n2},  {&u->gba, 64 * n2},  {&u->gbt, 64 * n2}, {&u->gc2, 64 * n1},  {&u->gd2a, 32 * n1},
+           {&u->gd2, 32 * n1},  {&u->gc1, 32 * n0},  {&u->gd1a, 16 * n0}, {&u->gd1, 16 * n0}, {&u->gy, n0}};
   for (auto &e : b) CUDA_TRY(u->alloc(e.q, e.n), "alloc network gradients");
   CUDA_TRY(u->alloc(&u->g, u->np), "alloc network gradients");
   CUDA_TRY(u->alloc(&u->m, u->np), "alloc optimiser state");
@@ -875,7 +906,7 @@ eb_status loss_and_backward(eb_unet u, const float *x, const float *target, cons
   eb_status st = ensure_grads(u);
   if (st != EB_OK) return st;
   const long long n0 = u->V[0].n();
-  forward(u, x, s);
+  forward(u, x, u->y, true, s);
   CUDA_TRY(cudaMemsetAsync(u->loss, 0, 2 * sizeof(float), s), "loss");
   k_chan_dot<<<dim3(64, 1), 256, 0, s>>>(mask, nullptr, 1, n0, u->loss + 1);   // voxels the mask selects
   k_loss<<<256, 256, 0, s>>>(u->y, target, mask, n0, u->loss + 1, u->gy, u->loss);
@@ -945,8 +976,8 @@ eb_status eb_unet_create(int nx, int ny, int nz, eb_unet *out) {
     float **q;
     long long n;
   } b[] = {{&u->e1a, 16 * n0}, {&u->e1, 16 * n0}, {&u->p1, 16 * n1}, {&u->e2a, 32 * n1}, {&u->e2, 32 * n1},
-           {&u->p2, 32 * n2},  {&u->ba, 64 * n2},  {&u->bt, 64 * n2}, {&u->c2, 96 * n1},  {&u->d2a, 32 * n1},
-           {&u->d2, 32 * n1},  {&u->c1, 48 * n0},  {&u->d1a, 16 * n0}, {&u->d1, 16 * n0}, {&u->y, n0}};
+           {&u->p2, 32 * n2},  {&u->ba, 64 * n2},  {&u->bt, 64 * n2},  {&u->d2a, 32 * n1},
+           {&u->d2, 32 * n1},   {&u->d1a, 16 * n0}, {&u->d1, 16 * n0}, {&u->y, n0}};
   cudaError_t e = cudaSuccess;
   for (auto &x : b)
     if (e == cudaSuccess) e = u->alloc(x.q, x.n);
@@ -1001,8 +1032,7 @@ eb_status eb_unet_get_params(eb_unet u, float *host, int64_t n) {
 eb_status eb_unet_forward(eb_unet u, const float *in, float *out, void *stream) {
   if (!u || !in || !out) return fail(EB_ERR_INVALID_ARG, "NULL argument");
   cudaStream_t s = as_stream(stream);
-  forward(u, in, s);
-  CUDA_TRY(cudaMemcpyAsync(out, u->y, sizeof(float) * u->V[0].n(), cudaMemcpyDeviceToDevice, s), "output");
+  forward(u, in, out, false, s);
   CUDA_TRY(cudaGetLastError(), "network forward");
   return EB_OK;
 }
@@ -1155,7 +1185,7 @@ eb_status eb_project_warm(eb_geom geom, eb_unet net, eb_state *U, double dt, dou
   const double *phi0 = nullptr;
   if (rms > 0.0) {
     k_net_input<<<nblk(N), 256, 0, s>>>(w.rhs, w.alpha, w.d, 1.0 / rms, N, w.nin, nullptr);
-    forward(net, w.nin, s);
+    forward(net, w.nin, net->y, false, s);
     k_net_phi0<<<nblk(N), 256, 0, s>>>(net->y, w.d, rms * D.dx * D.dx * scale, N, w.z);
     phi0 = w.z;   // copied into the solution vector before the solver touches z
   }
