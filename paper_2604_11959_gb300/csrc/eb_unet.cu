@@ -282,6 +282,219 @@ __global__ void __launch_bounds__(256, 2) k_conv3_umma(ConvIn in, int cin, const
   if (warp == 0) umma::dealloc(tm, G::TCOLS);
 }
 
+// The same convolution for up to 48 output channels, where a product of the
+// kernel above spends its time reading the 4 KB A operand for 16 columns.
+// The three dz taps of one halo plane become one product: plane hz feeds the
+// output levels hz - 2, hz - 1 and hz (dz = 2, 1, 0), whose accumulators lie
+// side by side in tensor memory, so with the three taps' weights stacked
+// along N one product of N = 3 NP columns serves all three (2 NP or NP at
+// the tile's ends).  An A operand is read 9 (TZ + 2) times instead of 27 TZ.
+// The first product into a level's accumulator overwrites it and is issued
+// for that level alone.  Weights: [chunk][tap (dy, dx)][channel group][3 NP
+// rows: dz = 2, 1, 0][8 channels].
+// One CTA of 512 threads per SM with two operand buffers and two sets of
+// accumulators: while the tensor core works on step i, the threads load step
+// i + 1, write out the tile that step i - 1 finished and convert step i + 1
+// into the other buffer.  192x192x96, 16 -> 16 channels: 360 us per chunk of
+// 16 input channels with the kernel above.
+template <int NP, int TZ>
+struct PipeTile {
+  static constexpr int HX = 10, HY = 18, HZ = TZ + 2;
+  static constexpr int HV = HX * HY * HZ;
+  static constexpr int PLANE = HV * 16;         // bytes of one 8-channel group
+  static constexpr int ACT = 2 * PLANE;         // hi (or lo) of a 16-channel chunk
+  static constexpr int WB = 27 * 2 * NP * 16;   // the chunk's weights
+  static constexpr int BUF = 2 * ACT + WB;
+  static constexpr int SMEM = 2 * BUF;
+  static constexpr int COLS = TZ * NP;          // accumulator columns of a tile
+  static constexpr uint32_t TCOLS = 2 * COLS <= 64 ? 64 : 2 * COLS <= 128 ? 128 : 2 * COLS <= 256 ? 256 : 512;
+  static constexpr int NT = 512;
+  static_assert(NP % 16 == 0 && 3 * NP <= 256 && 2 * COLS <= 512 && TZ >= 2, "product and tensor-memory limits");
+  static_assert(SMEM <= 227 * 1024, "two operand buffers in shared memory");
+};
+
+template <int NP, int TZ, bool MASK>
+__global__ void __launch_bounds__(512, 1) k_conv3_pipe(ConvIn in, int cin, const __nv_bfloat16 *Wp, const float *bias,
+                                                       ConvOut out, int cout, Vol V, int relu, const float *mask,
+                                                       int *err, int skip_commit) {
+  using G = PipeTile<NP, TZ>;
+  extern __shared__ __align__(16) unsigned char pp_smem[];
+  __shared__ uint32_t tbase;
+  __shared__ __align__(8) uint64_t mbar[2];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ntx = (V.nx + 7) / 8, nty = (V.ny + 15) / 16, ntz = (V.nz + TZ - 1) / TZ;
+  const int ntiles = ntx * nty * ntz, nch = (cin + 15) / 16;
+  const long long N = V.n();
+  if (warp == 0) umma::alloc(&tbase, G::TCOLS);
+  if (tid == 0) {
+    umma::bar_init(&mbar[0], 1);
+    umma::bar_init(&mbar[1], 1);
+  }
+  umma::fence_before();
+  __syncthreads();
+  umma::fence_after();
+  const uint32_t tm = tbase;
+  constexpr int ITEMS = 2 * G::HV, IS = (ITEMS + G::NT - 1) / G::NT;
+  const int mine = ((int)blockIdx.x < ntiles) ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+  const int nsteps = mine * nch;
+  auto tile_of = [&](int i) { return (int)blockIdx.x + (i / nch) * (int)gridDim.x; };
+  float pv[IS][8];
+  auto load_step = [&](int i) {
+    const int tile = tile_of(i), c0 = (i % nch) * 16;
+    const int x0 = (tile % ntx) * 8, y0 = ((tile / ntx) % nty) * 16, z0 = (tile / (ntx * nty)) * TZ;
+    const bool up = c0 < in.cup;
+    const float *base = up ? in.a + (long long)c0 * (N / 8)
+                           : (in.cup ? in.b + (long long)(c0 - in.cup) * N : in.a + (long long)c0 * N);
+    const long long cs = up ? N / 8 : N;   // channel stride
+#pragma unroll
+    for (int k = 0; k < IS; ++k) {
+      const int q = tid + G::NT * k;
+      const int kg = q / G::HV, h = q - kg * G::HV;
+      const int hx = h % G::HX, hy = (h / G::HX) % G::HY, hz = h / (G::HX * G::HY);
+      const int x = x0 + hx - 1, y = y0 + hy - 1, z = z0 + hz - 1;
+      const bool inside = q < ITEMS && x >= 0 && x < V.nx && y >= 0 && y < V.ny && z >= 0 && z < V.nz;
+      const float *src = base + (up ? ((long long)(z >> 1) * (V.ny / 2) + (y >> 1)) * (V.nx / 2) + (x >> 1)
+                                    : ((long long)z * V.ny + y) * V.nx + x);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int c = kg * 8 + j;
+        pv[k][j] = inside && c0 + c < cin ? src[c * cs] : 0.f;
+      }
+    }
+  };
+  auto store_step = [&](unsigned char *buf) {
+#pragma unroll
+    for (int k = 0; k < IS; ++k) {
+      const int q = tid + G::NT * k;
+      if (q >= ITEMS) break;
+      uint32_t hw[4], lw[4];
+#pragma unroll
+      for (int j = 0; j < 8; j += 2) {
+        const __nv_bfloat16 h0 = __float2bfloat16_rn(pv[k][j]), h1 = __float2bfloat16_rn(pv[k][j + 1]);
+        hw[j / 2] = pack_bf16(h0, h1);
+        lw[j / 2] = pack_bf16(__float2bfloat16_rn(pv[k][j] - __bfloat162float(h0)),
+                              __float2bfloat16_rn(pv[k][j + 1] - __bfloat162float(h1)));
+      }
+      // item q = group * HV + halo voxel: the two groups' planes follow each other
+      *reinterpret_cast<uint4 *>(buf + q * 16) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+      *reinterpret_cast<uint4 *>(buf + G::ACT + q * 16) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+    }
+  };
+  // one thread: the products of a step from buffer buf (weights at wb) into
+  // the accumulators at column d0; first: the tile's first chunk
+  auto issue = [&](unsigned char *buf, unsigned char *wb, uint32_t d0, bool first) {
+    const uint64_t ahi = umma::sdesc(umma::smem_u32(buf), G::PLANE, G::HX * 16);
+    const uint64_t alo = umma::sdesc(umma::smem_u32(buf + G::ACT), G::PLANE, G::HX * 16);
+    const uint64_t bw = umma::sdesc(umma::smem_u32(wb), 3 * NP * 16, 128);
+#pragma unroll
+    for (int hz = 0; hz < G::HZ; ++hz) {
+      const int lo = hz >= 2 ? hz - 2 : 0, hi = hz < TZ ? hz : TZ - 1;   // output levels fed by this plane
+      const uint32_t d = d0 + (uint32_t)(lo * NP);
+      const uint32_t full = umma::idesc_bf16(128, (hi - lo + 1) * NP);
+#pragma unroll
+      for (int t = 0; t < 9; ++t) {
+        const uint64_t off = (uint64_t)((hz * G::HY + t / 3) * G::HX + t % 3);          // 16-byte rows
+        const uint64_t bo = bw + (uint64_t)(t * 6 * NP + (lo - (hz - 2)) * NP);
+        if (t == 0 && hz < TZ) {   // level hz (the last of the stack) starts here
+          if (hi > lo) umma::mma_bf16(d, ahi + off, bo, umma::idesc_bf16(128, (hi - lo) * NP), 1u);
+          umma::mma_bf16(d0 + (uint32_t)(hz * NP), ahi + off, bw + (uint64_t)(t * 6 * NP + 2 * NP),
+                         umma::idesc_bf16(128, NP), first ? 0u : 1u);
+        } else {
+          umma::mma_bf16(d, ahi + off, bo, full, 1u);
+        }
+        umma::mma_bf16(d, alo + off, bo, full, 1u);
+      }
+    }
+  };
+  // a finished tile: warps w, w + 4, w + 8, w + 12 read TMEM lanes 32 (w % 4)
+  // ... (row m = this lane) and share the levels and channel blocks
+  auto epilogue = [&](int tile, uint32_t d0) {
+    const int x0 = (tile % ntx) * 8, y0 = ((tile / ntx) % nty) * 16, z0 = (tile / (ntx * nty)) * TZ;
+    const int quad = warp & 3;
+    const int m = 32 * quad + lane;
+    const int x = x0 + (m & 7), y = y0 + (m >> 3);
+    const bool xy = x < V.nx && y < V.ny;
+    for (int u = warp >> 2; u < TZ * (NP / 16); u += 4) {
+      const int rz = u / (NP / 16), cc = (u % (NP / 16)) * 16, z = z0 + rz;
+      const long long vox = ((long long)z * V.ny + y) * V.nx + x;
+      const bool live = xy && z < V.nz;
+      // the mask values first (all 16 loads in flight), then the accumulators
+      float mk[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j)
+        mk[j] = MASK && live && cc + j < cout ? __ldg(mask + (long long)(cc + j) * N + vox) : 1.f;
+      float v[16];
+      umma::ld16(tm + ((uint32_t)(32 * quad) << 16) + d0 + (uint32_t)(rz * NP + cc), v);
+      if (live) {
+        float *dst = cc < out.split ? out.a + (long long)cc * N : out.b + (long long)(cc - out.split) * N;
+        float yv = out.y ? out.hb[0] : 0.f;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          const int co = cc + j;
+          if (co < cout) {
+            float o = v[j] + (bias ? bias[co] : 0.f);
+            if (relu) o = fmaxf(o, 0.f);
+            if (MASK && !(mk[j] > 0.f)) o = 0.f;   // ReLU backward of the input
+            if (out.y) yv = fmaf(__bfloat162float(out.hw[co]), o, yv);
+            if (out.a) dst[(long long)j * N + vox] = o;
+          }
+        }
+        if (out.y) out.y[vox] = yv;
+      }
+    }
+  };
+  auto wait = [&](int i) {   // the products of step i, in every thread
+    const bool w = umma::bar_wait(&mbar[i & 1], (uint32_t)((i >> 1) & 1), kWaitCycles);
+    const bool all = __syncthreads_and(w) != 0;
+    umma::fence_after();
+    return all;
+  };
+  auto acc_of = [&](int i) { return (uint32_t)(((i / nch) & 1) * G::COLS); };
+  bool ok = true;
+  int i = 0;
+  if (nsteps > 0) load_step(0);
+  for (; i < nsteps; ++i) {
+    const int ch = i % nch;
+    unsigned char *buf = pp_smem + (i & 1) * G::BUF;
+    unsigned char *wb = nch > 1 ? buf + 2 * G::ACT : pp_smem + 2 * G::ACT;   // one chunk: its weights stay
+    if (i >= 2 && !(ok = wait(i - 2))) break;   // step i - 2's products read this buffer
+    store_step(buf);
+    if (nch > 1 || i == 0) {
+      const uint4 *wsrc = reinterpret_cast<const uint4 *>(Wp) + (long long)ch * (G::WB / 16);
+      for (int q = tid; q < G::WB / 16; q += G::NT) reinterpret_cast<uint4 *>(wb)[q] = wsrc[q];
+    }
+    umma::fence_async_smem();
+    umma::fence_before();
+    __syncthreads();
+    if (tid == 0) {
+      umma::fence_after();
+      issue(buf, wb, tm + acc_of(i), ch == 0);
+      if (!(skip_commit && i == 0)) umma::commit(&mbar[i & 1]);   // skipped only by the failure test
+    }
+    if (i + 1 < nsteps) load_step(i + 1);
+    if (i > 0 && ch == 0) {   // step i - 1 finished a tile
+      if (!(ok = wait(i - 1))) {
+        ++i;
+        break;
+      }
+      epilogue(tile_of(i - 1), acc_of(i - 1));
+    }
+  }
+  if (ok && nsteps > 0) {
+    ok = wait(nsteps - 1);
+    if (ok) epilogue(tile_of(nsteps - 1), acc_of(nsteps - 1));
+  }
+  if (!ok) {
+    // products may still be running: give the last two steps another bounded
+    // wait each before the tensor memory is released
+    for (int q = i > 2 ? i - 2 : 0; q < i; ++q) umma::bar_wait(&mbar[q & 1], (uint32_t)((q >> 1) & 1), kWaitCycles);
+    if (tid == 0) atomicExch(err, 1);
+  }
+  umma::fence_before();
+  __syncthreads();
+  if (warp == 0) umma::dealloc(tm, G::TCOLS);
+}
+
 // head backward: dIn[ci][v] = W[ci] dy[v] where the head's (ReLU) input post[ci][v] > 0, else 0
 __global__ void k_head_bwd(const float *dy, const __nv_bfloat16 *W, int cin, const float *post, float *din,
                            long long N) {
@@ -308,16 +521,29 @@ __global__ void k_chan_dot(const float *a, const float *b, int C, long long N, f
   }
 }
 
-// The weights of a convolution prepacked for k_conv3_umma: Wp[chunk][tap]
-// [group][n][j] = the weight from input channel 16 chunk + 8 group + j to
-// output channel n at that tap, zero beyond the channel counts.  flip = 0:
-// the layer itself (n = output channel, W[n][c][a]); flip = 1: its input
-// gradient, the convolution with transposed and flipped weights (n = the
-// layer's input channel, c its output channel: W[c][n][26 - a]).
+// The weights of a convolution prepacked: the weight from input channel 16
+// chunk + 8 group + j to output channel n at a tap, zero beyond the channel
+// counts, as Wp[chunk][tap][group][n][j] (k_conv3_umma) or, up to 48 output
+// channels, Wp[chunk][tap (dy, dx)][group][dz = 2, 1, 0][n][j] (k_conv3_pipe).
+// flip = 0: the layer itself (n = output channel, W[n][c][a]); flip = 1: its
+// input gradient, the convolution with transposed and flipped weights (n =
+// the layer's input channel, c its output channel: W[c][n][26 - a]).
+constexpr int kPipeMaxN = 48;
 __device__ inline void pack_elem(const __nv_bfloat16 *W, int cout, int cin, int flip, int NP, __nv_bfloat16 *Wp,
                                  long long q) {
-  const int j = (int)(q % 8), n = (int)((q / 8) % NP), kg = (int)((q / (8 * NP)) % 2);
-  const int a = (int)((q / (16LL * NP)) % 27), chunk = (int)(q / (16LL * NP * 27));
+  const int j = (int)(q % 8), chunk = (int)(q / (16LL * NP * 27));
+  const int r = (int)(q - chunk * (16LL * NP * 27));
+  int n, kg, a;
+  if (NP <= kPipeMaxN) {
+    const int n3 = (r / 8) % (3 * NP);
+    n = n3 % NP;
+    kg = (r / (24 * NP)) % 2;
+    a = (2 - n3 / NP) * 9 + r / (48 * NP);
+  } else {
+    n = (r / 8) % NP;
+    kg = (r / (8 * NP)) % 2;
+    a = r / (16 * NP);
+  }
   const int c = chunk * 16 + kg * 8 + j;
   __nv_bfloat16 w = __float2bfloat16_rn(0.f);
   if (!flip) {
@@ -730,6 +956,29 @@ void conv3_umma_launch(const ConvIn &in, int cin, const __nv_bfloat16 *Wp, const
                                                     skip_commit);
 }
 
+template <int NP, int TZ, bool MASK>
+void conv3_pipe_tiles(const ConvIn &in, int cin, const __nv_bfloat16 *Wp, const float *bias, const ConvOut &out,
+                      int cout, const Vol &V, bool relu, const float *mask, int *err, int skip_commit,
+                      cudaStream_t s) {
+  using G = PipeTile<NP, TZ>;
+  static unsigned long long attr = 0;
+  ebk_smem_limit(k_conv3_pipe<NP, TZ, MASK>, G::SMEM, attr);
+  const int tiles = ((V.nx + 7) / 8) * ((V.ny + 15) / 16) * ((V.nz + TZ - 1) / TZ);
+  const int grid = std::max(1, std::min(tiles, ebk_sm_count()));   // persistent: one CTA per SM walks the tiles
+  k_conv3_pipe<NP, TZ, MASK><<<grid, G::NT, G::SMEM, s>>>(in, cin, Wp, bias, out, cout, V, relu ? 1 : 0, mask, err,
+                                                         skip_commit);
+}
+// tiles of four levels (fewer halo planes and products per level) where they
+// still give every SM two or more, else of two
+template <int NP, bool MASK>
+void conv3_pipe(const ConvIn &in, int cin, const __nv_bfloat16 *Wp, const float *bias, const ConvOut &out, int cout,
+                const Vol &V, bool relu, const float *mask, int *err, int skip_commit, cudaStream_t s) {
+  const long long tiles4 = (long long)((V.nx + 7) / 8) * ((V.ny + 15) / 16) * ((V.nz + 3) / 4);
+  if (NP <= 32 && tiles4 >= 2 * ebk_sm_count())
+    conv3_pipe_tiles<NP, NP <= 32 ? 4 : 2, MASK>(in, cin, Wp, bias, out, cout, V, relu, mask, err, skip_commit, s);
+  else conv3_pipe_tiles<NP, 2, MASK>(in, cin, Wp, bias, out, cout, V, relu, mask, err, skip_commit, s);
+}
+
 // out (cout, V) = conv of in (cin, V) with the packed weights Wp (a layer's
 // own, or its transposed and flipped ones for an input gradient); mask:
 // where not NULL, out is zeroed wherever mask (cout, V) is not positive (the
@@ -743,15 +992,15 @@ void conv3_tc(eb_unet u, const ConvIn &in, int cin, const __nv_bfloat16 *Wp, con
   // gradients with one where a ReLU lies below the layer
   if (mask) {
     switch (NP) {
-      case 16: conv3_umma_launch<16, 2, true>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
-      case 32: conv3_umma_launch<32, 2, true>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
+      case 16: conv3_pipe<16, true>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
+      case 32: conv3_pipe<32, true>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
       default: conv3_umma_launch<64, 2, true>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
     }
   } else {
     switch (NP) {
-      case 16: conv3_umma_launch<16, 2, false>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
-      case 32: conv3_umma_launch<32, 2, false>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
-      case 48: conv3_umma_launch<48, 2, false>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
+      case 16: conv3_pipe<16, false>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
+      case 32: conv3_pipe<32, false>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
+      case 48: conv3_pipe<48, false>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
       case 64: conv3_umma_launch<64, 2, false>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
       default: conv3_umma_launch<96, 2, false>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
     }
