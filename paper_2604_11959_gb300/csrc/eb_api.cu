@@ -131,6 +131,34 @@ cudaError_t update_background(eb_geom g) {
   return cudaSuccess;
 }
 
+// Level differences of the profiles (device copies in g->ref_d) for the
+// redistribution, formed in double and kept in the state's precision.
+template <typename T>
+cudaError_t update_rdiff_t(eb_geom g) {
+  const int nz = g->D.nz;
+  for (int q = 0; q < 4; ++q) {
+    std::vector<double> r(nz);
+    cudaError_t e = cudaMemcpy(r.data(), g->ref_d[q], sizeof(double) * nz, cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return e;
+    std::vector<T> t((size_t)nz * WSRD_DK, T(0));
+    for (int k = 0; k < nz; ++k)
+      for (int d = 0; d < WSRD_DK; ++d) {
+        const int ka = k + d - WSRD_DK / 2;
+        if (ka >= 0 && ka < nz) t[(size_t)k * WSRD_DK + d] = (T)(r[ka] - r[k]);
+      }
+    if (!g->rdiff[q]) {
+      T *p = nullptr;
+      e = g->alloc(&p, (long long)t.size());
+      if (e != cudaSuccess) return e;
+      g->rdiff[q] = p;
+    }
+    e = cudaMemcpy(g->rdiff[q], t.data(), sizeof(T) * t.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+cudaError_t update_rdiff(eb_geom g) { return g->prec == EB_F64 ? update_rdiff_t<double>(g) : update_rdiff_t<float>(g); }
+
 // Builds the handle's geometry, tables and lists: from the nodal heights, or
 // (fine != nullptr) as the coarse level of the fine handle, merged from its
 // cells (eb_amr.cu; the heights then are every other fine node, kept as a
@@ -420,6 +448,11 @@ eb_status build_impl(eb_geom g, const double *h_nodes, const double *ref_rho, co
     CUDA_TRY(e, "redistribution reach");
     g->wsrd_side = far_h == 0 ? 1 : 0;
   }
+  // the step's tables; the set-up's arrays go
+  for (int q = 0; q < 4; ++q) {
+    CUDA_TRY(pack_wsrd(D, g->W[q], g->prec == EB_F64, g->WT[q], s), "redistribution tables");
+    free_wsrd(g->W[q]);
+  }
   CUDA_TRY(g->alloc((double **)&g->qhat, g->max_small), "alloc qhat");
   CUDA_TRY(g->alloc((double **)&g->sig, 3 * g->max_small), "alloc sig");
   CUDA_TRY(g->alloc((double **)&g->pval, g->max_small), "alloc pivot values");
@@ -445,6 +478,7 @@ eb_status build_impl(eb_geom g, const double *h_nodes, const double *ref_rho, co
     CUDA_TRY(alloc_profile(g, &g->bg_f[q]), "alloc background");
   }
   CUDA_TRY(update_background(g), "background");
+  CUDA_TRY(update_rdiff(g), "profile differences");
   CUDA_TRY(g->alloc(&g->status, 1), "alloc status");
   CUDA_TRY(cudaMemsetAsync(g->status, 0, sizeof(unsigned), s), "memset status");
   // host-side counts for eb_geom_info
@@ -578,9 +612,9 @@ void wsrd_field_scratch(eb_geom g, int field, T *u, char *scratch, cudaStream_t 
   const size_t one = round256((size_t)g->W[grid].nsmall * sizeof(T));
   WsrdArgs<T> R;
   R.D = g->D;
-  R.W = g->W[grid];
+  R.W = g->WT[grid];
   R.u = u;
-  R.refd = field <= 3 ? g->ref_d[field] : nullptr;
+  R.rdiff = field <= 3 ? (const T *)g->rdiff[field] : nullptr;
   R.dev = (T *)scratch;
   R.pval = (T *)(scratch + one);
   R.sig = (T *)(scratch + 2 * one);
@@ -910,6 +944,7 @@ eb_status eb_geom_set_wind_reference(eb_geom geom, const double *ref_rhou, const
   }
   geom->has_wind_ref = nonzero;
   CUDA_TRY(update_background(geom), "background");
+  CUDA_TRY(update_rdiff(geom), "profile differences");
   return EB_OK;
 }
 

@@ -145,11 +145,11 @@ eb_status build_tables(eb_ensemble e, EnsembleArgs<T> E[2]) {
   CUDA_TRY(cudaMalloc(&e->units, sizeof(int2) * std::max<size_t>(1, hu.size())), "ensemble units");
   if (!hu.empty())
     CUDA_TRY(cudaMemcpy(e->units, hu.data(), sizeof(int2) * hu.size(), cudaMemcpyHostToDevice), "ensemble units");
-  // prefix sums: staged CVs, faces, near-EB CVs, small CVs and affected CVs of the five fields
+  // prefix sums: staged CVs, faces, near-EB CVs, small CVs of the four grids, affected CVs of the five fields
   std::vector<long long> pre(5 * (n + 1), 0);
   for (int q = 0; q < n; ++q) {
     const EnsMember<T> &M = host[q];
-    long long c[5] = {0, 0, 0, M.S.off_small[5], M.S.off_aff[5]};
+    long long c[5] = {0, 0, 0, M.S.off_small[4], M.S.off_aff[5]};
     for (int g = 0; g < 4; ++g) {
       c[0] += M.A.G[g].nstage;
       c[2] += M.A.G[g].nband;

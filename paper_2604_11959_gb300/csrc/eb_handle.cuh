@@ -100,6 +100,8 @@ struct eb_geom_s {
   int kcov_max = 0;
   GridDev G[4];
   WsrdDev W[4];
+  WsrdTab WT[4];
+  void *rdiff[4] = {};    // per field with a profile: WsrdArgs::rdiff in the state's precision
   // per-level reference profiles (zeros where none was given): rho0,
   // rho0*theta0, and the background momenta of rho*u and rho*v; states hold
   // each field minus its profile
@@ -161,7 +163,10 @@ struct eb_geom_s {
     allocs.clear();
     if (pw.host) cudaFreeHost(pw.host);
     pw = ProjWork();
-    for (int g = 0; g < 4; ++g) free_wsrd(W[g]);
+    for (int g = 0; g < 4; ++g) {
+      free_wsrd(W[g]);
+      free_wsrd_tab(WT[g]);
+    }
   }
 };
 
@@ -236,9 +241,9 @@ void wsrd_field(eb_geom g, int field, T *u, cudaStream_t s) {
   const int grid = field <= 1 ? 0 : field - 1;
   WsrdArgs<T> R;
   R.D = g->D;
-  R.W = g->W[grid];
+  R.W = g->WT[grid];
   R.u = u;
-  R.refd = field <= 3 ? g->ref_d[field] : nullptr;
+  R.rdiff = field <= 3 ? (const T *)g->rdiff[field] : nullptr;
   R.dev = (T *)g->qhat;
   R.sig = (T *)g->sig;
   R.pval = (T *)g->pval;
@@ -286,25 +291,23 @@ void flux_update(eb_geom g, const StepArgs<T> &A, cudaStream_t s) {
 template <typename T>
 WsrdSet<T> wsrd_set(eb_geom g, void *const out[5]) {
   WsrdSet<T> S;
-  long long os = 0, oa = 0;
+  long long os = 0;
   for (int f = 0; f < 5; ++f) {
     const int grid = f <= 1 ? 0 : f - 1;
     WsrdArgs<T> &R = S.f[f];
     R.D = g->D;
-    R.W = g->W[grid];
+    R.W = g->WT[grid];
     R.u = (T *)out[f];
-    R.refd = f <= 3 ? g->ref_d[f] : nullptr;
+    R.rdiff = f <= 3 ? (const T *)g->rdiff[f] : nullptr;
     R.dev = (T *)g->qhat5 + os;
     R.pval = (T *)g->pval5 + os;
     R.sig = (T *)g->sig5 + 3 * os;
     R.status = g->status;
-    S.off_small[f] = os;
-    S.off_aff[f] = oa;
     os += g->W[grid].nsmall;
-    oa += g->W[grid].naff;
   }
-  S.off_small[5] = os;
-  S.off_aff[5] = oa;
+  S.off_small[0] = S.off_aff[0] = 0;
+  for (int q = 0; q < 4; ++q) S.off_small[q + 1] = S.off_small[q] + g->W[q].nsmall;
+  for (int f = 0; f < 5; ++f) S.off_aff[f + 1] = S.off_aff[f] + g->W[f <= 1 ? 0 : f - 1].naff;
   return S;
 }
 

@@ -6,7 +6,8 @@
 
 #include <vector>
 
-// Compact redistribution tables of one grid (Sec. 5.1), built once.
+// Compact redistribution tables of one grid (Sec. 5.1) as the set-up builds
+// them; only the counts outlive it (the step reads WsrdTab).
 struct WsrdDev {
   long long nsmall = 0, naff = 0, nlsq = 0, nw = 0;
   int *sid = nullptr;             // [nrec] small id of a record, -1 if not small
@@ -32,9 +33,35 @@ struct WsrdDev {
   int *w_sid = nullptr;           // [nw] small CV r whose neighbourhood holds the CV
   double *w_k = nullptr;          // [nw] kappa_r / N_i
   double *w_e = nullptr;          // [3 * nw] x_i - xhat_r (cell units, relative to r)
-  // float copies of the weight tables for the mixed-precision path
-  float *s_mw_f = nullptr, *s_me_f = nullptr, *l_c_f = nullptr, *a_eself_f = nullptr, *w_k_f = nullptr,
-        *w_e_f = nullptr;
+};
+
+// The same tables as the step reads them, weights in the state's precision
+// T, each component in an array of its own: entry e of small CV s at [e * ns +
+// s], the lists of uneven length one after another (several lanes share a
+// list, so a warp reads one contiguous run).  Indices are 32 bit (grids hold
+// fewer than 2^32 CVs).  A tag holds a small id + 1 (0: none) in its low 28
+// bits and a level difference + 8 in the upper 4, which replaces looking up
+// the reference profiles at both levels (see WsrdArgs::rdiff).
+struct WsrdTab {
+  long long ns = 0, na = 0;       // small, affected CVs
+  long long nl = 0, nw = 0;       // entries of the two lists
+  unsigned *plin = nullptr;       // [ns] state index of the pivot member
+  uint8_t *nmem = nullptr;        // [ns] members incl. itself (<= 8) | pivot member << 4
+  unsigned *mlin = nullptr;       // [8][ns] members' state indices
+  void *mw = nullptr;             // [8][ns] weights of Qhat
+  void *me = nullptr;             // [24][ns] limiter points: member q, direction d at [3 q + d]
+  long long *loff = nullptr;      // [ns + 1]
+  unsigned *lplin = nullptr;      // [nl] pivot state index of the stencil CV
+  unsigned *ltag = nullptr;       // [nl] its small id; level of lplin - level of the CV's own pivot
+  void *lc = nullptr;             // [3][nl] gradient coefficients
+  unsigned *alin = nullptr;       // [na] state index
+  unsigned *atag = nullptr;       // [na] own small id; level of its pivot - own level
+  void *es = nullptr;             // [3][na] own centroid - own xhat
+  long long *woff = nullptr;      // [na + 1]
+  unsigned *wtag = nullptr;       // [nw] small CV r whose neighbourhood holds the CV; level of r's pivot - level of
+                                  // the CV's (its own, when it is not small)
+  void *wk = nullptr;             // [nw] kappa_r / N_i
+  void *we = nullptr;             // [3][nw] x_i - xhat_r
 };
 
 // eb_geom.cu
@@ -92,7 +119,10 @@ void scan_exclusive(long long *data, long long n, long long *total, cudaStream_t
 struct SetupScratch;
 cudaError_t build_wsrd(const Dims &D, int g, GridDev &G, const GridDev *all, double vt, WsrdDev &W,
                        cudaStream_t s, long long *dev_tmp);
-void free_wsrd(WsrdDev &W);
+void free_wsrd(WsrdDev &W);   // the arrays; the counts stay
+// the step's tables from the set-up's (f64: weights in double, else float)
+cudaError_t pack_wsrd(const Dims &D, const WsrdDev &W, bool f64, WsrdTab &T, cudaStream_t s);
+void free_wsrd_tab(WsrdTab &T);
 // sets *far when a CV the redistribution of grid g reads or writes is not a
 // near-EB CV (see k_wsrd_reach)
 void launch_wsrd_reach(const Dims &D, int g, const WsrdDev &W, const int *kcov, const int *kfast, unsigned *far,

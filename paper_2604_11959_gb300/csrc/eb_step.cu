@@ -15,7 +15,7 @@
 //   weighted state redistribution (Sec. 5.1, Eqs. qhat_omega, qrecon,
 //   final_update_omega), on compact lists built at set-up:
 //     k_qhat  : neighbourhood averages of the small CVs;
-//     k_sigma : least-squares slopes and the limiter, 8 lanes per small CV;
+//     k_sigma : least-squares slopes and the limiter;
 //     k_final : the final update of every CV the redistribution changes.
 //
 // Every kernel writes a disjoint set of CVs, so no atomics are needed and
@@ -407,6 +407,7 @@ __device__ inline void face_one(const StepArgs<T> &A, long long t) {
 
 template <typename T>
 __global__ void k_face_flux(StepArgs<T> A) {
+  chain_begin();
   face_one(A, blockIdx.x * (long long)blockDim.x + threadIdx.x);
 }
 
@@ -615,7 +616,8 @@ __device__ inline void band_one(const StepArgs<T> &A, long long t) {
 }
 
 template <typename T>
-__global__ void k_band(StepArgs<T> A) {
+__global__ void k_band(const __grid_constant__ StepArgs<T> A) {
+  chain_begin();
   band_one(A, blockIdx.x * (long long)blockDim.x + threadIdx.x);
 }
 
@@ -631,40 +633,14 @@ __global__ void k_band(StepArgs<T> A) {
 // is reproduced exactly.
 // ---------------------------------------------------------------------------
 
-// Uhat_a - Uhat_b of two CVs of the field (state indices), with the
-// reference profile difference taken in double.
+// ref[kb + dk] - ref[kb] of the field's profile (0 without one)
 template <typename T>
-__device__ inline T vdiff(const WsrdArgs<T> &R, long long a, long long b) {
-  T d = R.u[a] - R.u[b];
-  if (R.refd) {
-    const unsigned ka = R.D.fnxy.div((unsigned)a), kb = R.D.fnxy.div((unsigned)b);
-    if (ka != kb) d += (T)(R.refd[ka] - R.refd[kb]);
-  }
-  return d;
+__device__ inline T ref_diff(const WsrdArgs<T> &R, int kb, int dk) {
+  return R.rdiff ? R.rdiff[kb * WSRD_DK + dk + WSRD_DK / 2] : T(0);
 }
-
-// The same difference from two values already read, located at a and b.
-template <typename T>
-__device__ inline T vdiff_vals(const WsrdArgs<T> &R, T va, long long a, T vb, long long b) {
-  T d = va - vb;
-  if (R.refd) {
-    const unsigned ka = R.D.fnxy.div((unsigned)a), kb = R.D.fnxy.div((unsigned)b);
-    if (ka != kb) d += (T)(R.refd[ka] - R.refd[kb]);
-  }
-  return d;
-}
-
-// A weight table in the state's precision (float copies on the mixed path).
-template <typename T>
-__device__ inline const T *tab(const double *d, const float *f);
-template <>
-__device__ inline const double *tab<double>(const double *d, const float *) {
-  return d;
-}
-template <>
-__device__ inline const float *tab<float>(const double *, const float *f) {
-  return f;
-}
+// small id (-1: none) and level difference of a tag
+__device__ inline int tag_sid(unsigned tag) { return (int)(tag & 0x0fffffffu) - 1; }
+__device__ inline int tag_dk(unsigned tag) { return (int)(tag >> 28) - 8; }
 
 // Kahan-compensated running sum in float; plain in double.
 template <typename T>
@@ -683,75 +659,150 @@ struct CompSum<double> {
   __device__ inline void add(double x) { s += x; }
 };
 
-template <typename T>
-__device__ inline void qhat_one(const WsrdArgs<T> &R, long long s) {
-  const int n = R.W.s_nmem[s], p = R.W.s_piv[s];
-  const long long lp = R.W.s_plin[s];
-  CompSum<T> acc;
+// The first two passes take the NF fields R[0 .. NF-1] of a small CV's grid
+// together (rho and rho*theta share the c grid's tables, whose entries are
+// most of what they read).
+template <typename T, int NF>
+__device__ inline void qhat_one(const WsrdArgs<T> *R, long long s) {
+  const WsrdTab &W = R[0].W;
+  const Dims &D = R[0].D;
+  const long long ns = W.ns;
+  const int n = W.nmem[s] & 15, p = W.nmem[s] >> 4;
+  const unsigned lp = W.plin[s];
+  const int kp = (int)D.fnxy.div(lp);
+  CompSum<T> acc[NF];
+  T up[NF];
+#pragma unroll
+  for (int f = 0; f < NF; ++f) up[f] = R[f].u[lp];
+#pragma unroll 2
   for (int q = 0; q < n; ++q) {
     if (q == p) continue;
-    acc.add(tab<T>(R.W.s_mw, R.W.s_mw_f)[8 * s + q] * vdiff(R, R.W.s_mlin[8 * s + q], lp));
+    const unsigned m = W.mlin[q * ns + s];
+    const T w = ((const T *)W.mw)[q * ns + s];
+    const int dk = (int)D.fnxy.div(m) - kp;
+#pragma unroll
+    for (int f = 0; f < NF; ++f) acc[f].add(w * ((R[f].u[m] - up[f]) + ref_diff(R[f], kp, dk)));
   }
-  R.dev[s] = acc.s;
-  R.pval[s] = R.u[lp];   // snapshot: the final update overwrites the field in place
+#pragma unroll
+  for (int f = 0; f < NF; ++f) {
+    R[f].dev[s] = acc[f].s;
+    R[f].pval[s] = up[f];   // snapshot: the final update overwrites the field in place
+  }
 }
 
-// One group of GS lanes per small CV (8 in the kernels: four CVs per warp):
-// lanes walk the stencil, shuffles reduce the slope and the stencil's range
-// of Qhat - Qhat_r; lane q evaluates the limiter at member q's centroid and a
-// min-reduction combines them.  A group without a CV (valid false) takes part
-// in the shuffles only.
-template <typename T, int GS>
-__device__ inline void sigma_one(const WsrdArgs<T> &R, long long s, int lane, bool valid) {
-  static_assert(GS == 8 || GS == 16 || GS == 32, "lane groups of 8, 16 or 32 lanes");
-  long long o0 = 0, o1 = 0, pr = 0;
-  T dr = T(0);
+// The least-squares slope and the limiter of small CV s, SIGMA_LANES
+// neighbouring lanes per CV: they take every fourth stencil entry (and
+// member), shuffles join the sums and bounds.  The table entries (20 bytes
+// each in float, 26 per CV, read once for the grid's fields) and the latency
+// of the gathers behind them bound it; four lanes cut that chain to seven
+// entries and read their list as one run.  512x512x256 random terrain (2.3M
+// field values): 480 us with eight lanes and one field per group, profile
+// differences in FP64.
+// A lane without a CV (valid false) takes part in the shuffles only.
+constexpr int SIGMA_LANES = 4;
+template <typename T, int NF>
+__device__ inline void sigma_one(const WsrdArgs<T> *R, long long s, int lane, bool valid) {
+  const WsrdTab &W = R[0].W;
+  int cnt = 0, kr = 0, n = 0;
+  long long base = 0;
+  T dr[NF], ur[NF], sx[NF], sy[NF], sz[NF], bmax[NF], bmin[NF];
+#pragma unroll
+  for (int f = 0; f < NF; ++f) dr[f] = ur[f] = sx[f] = sy[f] = sz[f] = bmax[f] = bmin[f] = T(0);
   if (valid) {
-    o0 = R.W.s_loff[s];
-    o1 = R.W.s_loff[s + 1];
-    pr = R.W.s_plin[s];
-    dr = R.dev[s];
+    base = W.loff[s];
+    cnt = (int)(W.loff[s + 1] - base);
+    n = W.nmem[s] & 15;
+    const unsigned pr = W.plin[s];
+    kr = (int)R[0].D.fnxy.div(pr);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      dr[f] = R[f].dev[s];
+      ur[f] = R[f].u[pr];
+    }
   }
-  T sx = T(0), sy = T(0), sz = T(0), bmax = T(0), bmin = T(0);
-#pragma unroll 2
-  for (long long o = o0 + lane; o < o1; o += GS) {
-    const int sid = R.W.l_sid[o];
-    const long long pm = R.W.l_plin[o];
-    const T dm = sid >= 0 ? R.dev[sid] : T(0);
-    const T b = vdiff(R, pm, pr) + (dm - dr);
-    const T *lc = tab<T>(R.W.l_c, R.W.l_c_f) + 3 * o;
-    sx += lc[0] * b;
-    sy += lc[1] * b;
-    sz += lc[2] * b;
-    bmax = b > bmax ? b : bmax;
-    bmin = b < bmin ? b : bmin;
+  // four entries at a time: their table loads, then their gathers are all in
+  // flight together (an entry beyond the list adds zeros)
+  const T *lc = (const T *)W.lc;
+  constexpr int B = 4;
+  for (int e0 = lane; e0 < cnt; e0 += B * SIGMA_LANES) {
+    unsigned pm[B], tag[B];
+    T c0[B], c1[B], c2[B], v[B][NF], dm[B][NF];
+#pragma unroll
+    for (int q = 0; q < B; ++q) {
+      const int e = e0 + q * SIGMA_LANES;
+      const bool ok = e < cnt;
+      const long long pos = base + (ok ? e : e0);
+      pm[q] = W.lplin[pos];
+      tag[q] = W.ltag[pos];
+      c0[q] = lc[pos];
+      c1[q] = lc[W.nl + pos];
+      c2[q] = lc[2 * W.nl + pos];
+    }
+#pragma unroll
+    for (int q = 0; q < B; ++q) {
+      const int sid = tag_sid(tag[q]);
+#pragma unroll
+      for (int f = 0; f < NF; ++f) {
+        v[q][f] = R[f].u[pm[q]];
+        dm[q][f] = sid >= 0 ? R[f].dev[sid] : T(0);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < B; ++q) {
+      const bool ok = e0 + q * SIGMA_LANES < cnt;
+      const int dk = tag_dk(tag[q]);
+#pragma unroll
+      for (int f = 0; f < NF; ++f) {
+        T b = ((v[q][f] - ur[f]) + ref_diff(R[f], kr, dk)) + (dm[q][f] - dr[f]);
+        b = ok ? b : T(0);
+        sx[f] = fma(c0[q], b, sx[f]);
+        sy[f] = fma(c1[q], b, sy[f]);
+        sz[f] = fma(c2[q], b, sz[f]);
+        bmax[f] = b > bmax[f] ? b : bmax[f];
+        bmin[f] = b < bmin[f] ? b : bmin[f];
+      }
+    }
   }
-  for (int off = GS / 2; off > 0; off >>= 1) {   // stays within the group
-    sx += __shfl_xor_sync(0xffffffffu, sx, off);
-    sy += __shfl_xor_sync(0xffffffffu, sy, off);
-    sz += __shfl_xor_sync(0xffffffffu, sz, off);
-    const T a = __shfl_xor_sync(0xffffffffu, bmax, off);
-    const T c = __shfl_xor_sync(0xffffffffu, bmin, off);
-    bmax = a > bmax ? a : bmax;
-    bmin = c < bmin ? c : bmin;
+  T phi[NF];
+#pragma unroll
+  for (int f = 0; f < NF; ++f) {
+    phi[f] = T(1);
+#pragma unroll
+    for (int o = SIGMA_LANES / 2; o > 0; o >>= 1) {
+      sx[f] += __shfl_xor_sync(0xffffffffu, sx[f], o);
+      sy[f] += __shfl_xor_sync(0xffffffffu, sy[f], o);
+      sz[f] += __shfl_xor_sync(0xffffffffu, sz[f], o);
+      const T a = __shfl_xor_sync(0xffffffffu, bmax[f], o), b = __shfl_xor_sync(0xffffffffu, bmin[f], o);
+      bmax[f] = a > bmax[f] ? a : bmax[f];
+      bmin[f] = b < bmin[f] ? b : bmin[f];
+    }
   }
-  T phi = T(1);
-  if (o1 > o0 && lane < R.W.s_nmem[s]) {   // o1 > o0 only for a valid group
-    const T *e = tab<T>(R.W.s_me, R.W.s_me_f) + 24 * s + 3 * lane;
-    const T del = sx * e[0] + sy * e[1] + sz * e[2];
-    T ph = T(1);
-    if (del > T(0)) ph = bmax / del;
-    else if (del < T(0)) ph = bmin / del;
-    phi = ph < T(1) ? ph : T(1);   // a value that is not below 1 (or NaN) leaves phi at 1
+  if (cnt > 0) {
+    const T *me = (const T *)W.me + s;
+#pragma unroll
+    for (int q0 = 0; q0 < 8; q0 += SIGMA_LANES) {
+      const int q = q0 + lane;
+      if (q >= n) continue;
+      const T e0 = me[(3 * q) * W.ns], e1 = me[(3 * q + 1) * W.ns], e2 = me[(3 * q + 2) * W.ns];
+#pragma unroll
+      for (int f = 0; f < NF; ++f) {
+        const T del = sx[f] * e0 + sy[f] * e1 + sz[f] * e2;
+        T ph = T(1);
+        if (del > T(0)) ph = bmax[f] / del;
+        else if (del < T(0)) ph = bmin[f] / del;
+        phi[f] = ph < phi[f] ? ph : phi[f];   // a value that is not below (or NaN) changes nothing
+      }
+    }
   }
-  for (int off = 4; off > 0; off >>= 1) {   // members are lanes 0 .. 7
-    const T o = __shfl_xor_sync(0xffffffffu, phi, off);
-    phi = o < phi ? o : phi;
+#pragma unroll
+  for (int f = 0; f < NF; ++f) {
+#pragma unroll
+    for (int o = SIGMA_LANES / 2; o > 0; o >>= 1) {
+      const T a = __shfl_xor_sync(0xffffffffu, phi[f], o);
+      phi[f] = a < phi[f] ? a : phi[f];
+    }
+    if (valid && lane < 3) R[f].sig[3 * s + lane] = (lane == 0 ? sx[f] : lane == 1 ? sy[f] : sz[f]) * phi[f];
   }
-  if (lane != 0 || !valid) return;
-  R.sig[3 * s] = sx * phi;
-  R.sig[3 * s + 1] = sy * phi;
-  R.sig[3 * s + 2] = sz * phi;
 }
 
 // U_i = P_i + sum_r (kappa_r / N_i) (q_r(x_i) - P_i), P_i = q_i(x_i) for a
@@ -759,93 +810,108 @@ __device__ inline void sigma_one(const WsrdArgs<T> &R, long long s, int lane, bo
 // as 1 - sum_r kappa_r / N_i.  Formed as an offset added to Uhat_i.
 template <typename T>
 __device__ inline void final_one(const WsrdArgs<T> &R, long long a) {
-  const long long c = R.W.a_lin[a];
-  const int sid = R.W.a_sid[a];
+  const WsrdTab &W = R.W;
+  const unsigned c = W.alin[a], atag = W.atag[a];
+  const int sid = tag_sid(atag), dkp = tag_dk(atag);   // own pivot's level - own level
+  const int kc = (int)R.D.fnxy.div(c), kp = kc + dkp;
+  const long long o0 = W.woff[a], o1 = W.woff[a + 1];
   // every value this thread reads besides its own CV comes from the
   // snapshots of k_qhat: other threads overwrite their CVs meanwhile
   const T ui = R.u[c];
   T si = T(0), di = T(0), pvi = ui;
-  long long pi = c;
   if (sid >= 0) {
-    const T *e = tab<T>(R.W.a_eself, R.W.a_eself_f) + 3 * a;
-    si = R.sig[3 * sid] * e[0] + R.sig[3 * sid + 1] * e[1] + R.sig[3 * sid + 2] * e[2];
-    pi = R.W.s_plin[sid];
+    const T *es = (const T *)W.es + a;
+    const T *sg = R.sig + 3 * (long long)sid;
+    si = sg[0] * es[0] + sg[1] * es[W.na] + sg[2] * es[2 * W.na];
     pvi = R.pval[sid];
     di = R.dev[sid];
   }
   CompSum<T> acc;
-  for (long long o = R.W.a_woff[a]; o < R.W.a_woff[a + 1]; ++o) {
-    const int r = R.W.w_sid[o];
-    const T *e = tab<T>(R.W.w_e, R.W.w_e_f) + 3 * o;
-    const long long pr = R.W.s_plin[r];
-    const T sr = R.sig[3 * r] * e[0] + R.sig[3 * r + 1] * e[1] + R.sig[3 * r + 2] * e[2];
-    const T diff = vdiff_vals(R, R.pval[r], pr, pvi, pi) + (R.dev[r] - di) + (sr - si);
-    acc.add(tab<T>(R.W.w_k, R.W.w_k_f)[o] * diff);
+  const T *we = (const T *)W.we, *wk = (const T *)W.wk;
+  for (long long pos = o0; pos < o1; ++pos) {
+    const unsigned tag = W.wtag[pos];
+    const long long r = tag_sid(tag);
+    const T *sg = R.sig + 3 * r;
+    const T sr = sg[0] * we[pos] + sg[1] * we[W.nw + pos] + sg[2] * we[2 * W.nw + pos];
+    const T diff = ((R.pval[r] - pvi) + ref_diff(R, kp, tag_dk(tag))) + (R.dev[r] - di) + (sr - si);
+    acc.add(wk[pos] * diff);
   }
   // a small CV's result is anchored at its pivot value: its own provisional
   // value can be huge (tiny cell after the flux update) and must not be added
   // and subtracted again
-  T v;
-  if (sid >= 0) {
-    T anchor = pvi;
-    if (R.refd) {
-      const unsigned kp = R.D.fnxy.div((unsigned)pi), kc = R.D.fnxy.div((unsigned)c);
-      if (kp != kc) anchor += (T)(R.refd[kp] - R.refd[kc]);
-    }
-    v = anchor + ((di + si) + acc.s);
-  } else {
-    v = ui + acc.s;
-  }
+  const T v = sid >= 0 ? (pvi + ref_diff(R, kc, dkp)) + ((di + si) + acc.s) : ui + acc.s;
   R.u[c] = v;
   if (!finite_val(v)) atomicOr(R.status, EB_DEV_NUMERIC);
 }
 
 // one field
 template <typename T>
-__global__ void k_qhat(WsrdArgs<T> R) {
+__global__ void k_qhat(const __grid_constant__ WsrdArgs<T> R) {
+  chain_begin();
   const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (s < R.W.nsmall) qhat_one(R, s);
+  if (s < R.W.ns) qhat_one<T, 1>(&R, s);
 }
 template <typename T>
-__global__ void k_sigma(WsrdArgs<T> R) {
-  const long long s = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 3;
-  sigma_one<T, 8>(R, s, threadIdx.x & 7, s < R.W.nsmall);
+__global__ void k_sigma(const __grid_constant__ WsrdArgs<T> R) {
+  chain_begin();
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x, s = t / SIGMA_LANES;
+  const bool valid = s < R.W.ns;
+  sigma_one<T, 1>(&R, valid ? s : 0, (int)(t % SIGMA_LANES), valid);
 }
 template <typename T>
-__global__ void k_final(WsrdArgs<T> R) {
+__global__ void k_final(const __grid_constant__ WsrdArgs<T> R) {
+  chain_begin();
   const long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (a < R.W.naff) final_one(R, a);
+  if (a < R.W.na) final_one(R, a);
 }
 
-// all five fields in one launch: work item t belongs to the field f with
-// off[f] <= t < off[f + 1]
-__device__ inline int field_of(const long long off[6], long long t) {
+// all five fields in one launch: small-CV item t belongs to the grid g with
+// off[g] <= t < off[g + 1]
+__device__ inline int grid_of(const long long off[5], long long t) {
+  int g = 0;
+  while (g < 3 && t >= off[g + 1]) ++g;
+  return g;
+}
+template <typename T>
+__device__ inline void qhat_item(const WsrdSet<T> &S, long long t) {
+  const int g = grid_of(S.off_small, t);
+  if (g == 0) qhat_one<T, 2>(S.f, t);
+  else qhat_one<T, 1>(S.f + g + 1, t - S.off_small[g]);
+}
+// (the shuffles want whole warps in one of the two: the grid of the warp's
+// first item decides which, and a warp astride the c grid's end runs both)
+template <typename T>
+__device__ inline void sigma_item(const WsrdSet<T> &S, long long t, int lane, bool valid) {
+  const int g = grid_of(S.off_small, t);
+  const bool c = valid && g == 0, o = valid && g > 0;
+  if (__any_sync(0xffffffffu, c)) sigma_one<T, 2>(S.f, c ? t : 0, lane, c);
+  if (__any_sync(0xffffffffu, o)) sigma_one<T, 1>(S.f + (o ? g + 1 : 2), o ? t - S.off_small[g] : 0, lane, o);
+}
+template <typename T>
+__device__ inline void final_item(const WsrdSet<T> &S, long long t) {
   int f = 0;
-  while (f < 4 && t >= off[f + 1]) ++f;
-  return f;
+  while (f < 4 && t >= S.off_aff[f + 1]) ++f;
+  final_one(S.f[f], t - S.off_aff[f]);
 }
 template <typename T>
 __global__ void k_qhat5(const __grid_constant__ WsrdSet<T> S) {
+  chain_begin();
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= S.off_small[5]) return;
-  const int f = field_of(S.off_small, t);
-  qhat_one(S.f[f], t - S.off_small[f]);
+  if (t < S.off_small[4]) qhat_item(S, t);
 }
 template <typename T>
-__global__ void k_sigma5(const __grid_constant__ WsrdSet<T> S) {
-  const long long t = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 3;
-  const bool valid = t < S.off_small[5];
-  const int f = valid ? field_of(S.off_small, t) : 0;
-  sigma_one<T, 8>(S.f[f], valid ? t - S.off_small[f] : 0, threadIdx.x & 7, valid);
+__global__ void __launch_bounds__(128) k_sigma5(const __grid_constant__ WsrdSet<T> S) {
+  chain_begin();
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x, s = t / SIGMA_LANES;
+  const bool valid = s < S.off_small[4];
+  sigma_item(S, valid ? s : 0, (int)(t % SIGMA_LANES), valid);
 }
 template <typename T>
 __global__ void k_final5(const __grid_constant__ WsrdSet<T> S) {
+  chain_begin();
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= S.off_aff[5]) return;
-  const int f = field_of(S.off_aff, t);
-  final_one(S.f[f], t - S.off_aff[f]);
+  if (t < S.off_aff[5]) final_item(S, t);
 }
-
 
 // ---------------------------------------------------------------------------
 // persistent ensemble step: every phase of one step of every member in one
@@ -982,33 +1048,25 @@ __global__ void __launch_bounds__(bulk::BulkTile<T>::NT, (sizeof(T) == 4 ? 2 : 1
   // phases 4-6: redistribution of all five fields of every member
   for (long long t = gtid; t < E.pre_small[nm]; t += nthreads) {
     const int q = member_of(E.pre_small, nm, t);
-    const WsrdSet<T> &S = E.m[q].S;
-    const long long ts = t - E.pre_small[q];
-    const int f = field_of(S.off_small, ts);
-    qhat_one(S.f[f], ts - S.off_small[f]);
+    qhat_item(E.m[q].S, t - E.pre_small[q]);
   }
   if (!ens_barrier(E)) return;
   {
-    // 8 lanes per small CV; every lane of a warp takes part in each round
-    const long long groups = E.pre_small[nm];
-    const long long wbase = (gtid >> 5) * 4, wstep = (nthreads >> 5) * 4;
-    for (long long b = wbase; b < groups; b += wstep) {
-      const long long g = b + ((tid & 31) >> 3);
-      const bool valid = g < groups;
-      const int q = valid ? member_of(E.pre_small, nm, g) : 0;
-      const WsrdSet<T> &S = E.m[q].S;
-      const long long ts = valid ? g - E.pre_small[q] : 0;
-      const int f = valid ? field_of(S.off_small, ts) : 0;
-      sigma_one<T, 8>(S.f[f], valid ? ts - S.off_small[f] : 0, tid & 7, valid);
+    // SIGMA_LANES lanes per small CV; every lane of a warp takes part in each
+    // round, and a warp stays with one member
+    const long long wb = (gtid >> 5) * (32 / SIGMA_LANES), ws = (nthreads >> 5) * (32 / SIGMA_LANES);
+    for (int q = 0; q < nm; ++q) {
+      const long long n = E.pre_small[q + 1] - E.pre_small[q];
+      for (long long b = wb; b < n; b += ws) {
+        const long long t = b + (tid & 31) / SIGMA_LANES;
+        sigma_item(E.m[q].S, t < n ? t : 0, tid % SIGMA_LANES, t < n);
+      }
     }
   }
   if (!ens_barrier(E)) return;
   for (long long t = gtid; t < E.pre_aff[nm]; t += nthreads) {
     const int q = member_of(E.pre_aff, nm, t);
-    const WsrdSet<T> &S = E.m[q].S;
-    const long long ta = t - E.pre_aff[q];
-    const int f = field_of(S.off_aff, ta);
-    final_one(S.f[f], ta - S.off_aff[f]);
+    final_item(E.m[q].S, t - E.pre_aff[q]);
   }
 }
 
@@ -1064,7 +1122,7 @@ void launch_flux_band(const StepArgs<T> &A, cudaStream_t s) {
   for (int g = 0; g < 4; ++g) ns += A.G[g].nstage;
   if (ns) k_stage<T><<<(unsigned)((ns + 255) / 256), 256, 0, s>>>(A);
   if (nf) k_face_flux<T><<<(unsigned)((nf + 255) / 256), 256, 0, s>>>(A);
-  if (nb + nr) k_band<T><<<(unsigned)((nb + nr + 255) / 256), 256, 0, s>>>(A);
+  if (nb + nr) launch_chained(k_band<T>, (unsigned)((nb + nr + 255) / 256), 256, 0, s, A);
 }
 
 template <typename T>
@@ -1075,20 +1133,22 @@ void launch_flux_update(const StepArgs<T> &A, cudaStream_t s) {
 
 template <typename T>
 void launch_wsrd(const WsrdArgs<T> &R, cudaStream_t s) {
-  if (R.W.nsmall) {
-    k_qhat<T><<<(unsigned)((R.W.nsmall + 127) / 128), 128, 0, s>>>(R);
-    k_sigma<T><<<(unsigned)((R.W.nsmall * 8 + 255) / 256), 256, 0, s>>>(R);
+  const unsigned ns = (unsigned)((R.W.ns + 127) / 128), na = (unsigned)((R.W.na + 127) / 128);
+  if (ns) {
+    k_qhat<T><<<ns, 128, 0, s>>>(R);
+    launch_chained(k_sigma<T>, (unsigned)((R.W.ns * SIGMA_LANES + 127) / 128), 128, 0, s, R);
   }
-  if (R.W.naff) k_final<T><<<(unsigned)((R.W.naff + 127) / 128), 128, 0, s>>>(R);
+  if (na) launch_chained(k_final<T>, na, 128, 0, s, R);
 }
 
 template <typename T>
 void launch_wsrd5(const WsrdSet<T> &S, cudaStream_t s) {
-  if (S.off_small[5]) {
-    k_qhat5<T><<<(unsigned)((S.off_small[5] + 127) / 128), 128, 0, s>>>(S);
-    k_sigma5<T><<<(unsigned)((S.off_small[5] * 8 + 255) / 256), 256, 0, s>>>(S);
+  const unsigned ns = (unsigned)((S.off_small[4] + 127) / 128), na = (unsigned)((S.off_aff[5] + 127) / 128);
+  if (ns) {
+    launch_chained(k_qhat5<T>, ns, 128, 0, s, S);
+    launch_chained(k_sigma5<T>, (unsigned)((S.off_small[4] * SIGMA_LANES + 127) / 128), 128, 0, s, S);
   }
-  if (S.off_aff[5]) k_final5<T><<<(unsigned)((S.off_aff[5] + 127) / 128), 128, 0, s>>>(S);
+  if (na) launch_chained(k_final5<T>, na, 128, 0, s, S);
 }
 
 void launch_band_rows(const Dims &D, const GridDev G[4], int g, bool fill, long long *cnt, cudaStream_t s) {

@@ -28,22 +28,28 @@ struct StepArgs {
 template <typename T>
 struct WsrdArgs {
   Dims D;
-  WsrdDev W;
+  WsrdTab W;
   T *u;                // field on its grid, redistributed in place
-  const double *refd;  // per-level reference profile of the field (stored values are u - refd) or nullptr
-  T *dev;              // [nsmall] deviation sums D of the neighbourhood averages
-  T *pval;             // [nsmall] field value at each neighbourhood's pivot
-  T *sig;              // [3 * nsmall] limited slopes
+  // profile differences of the field (stored values are u minus a per-level
+  // profile), (T)(ref[kb + dk] - ref[kb]) at [kb * WSRD_DK + dk + WSRD_DK / 2],
+  // formed in double at set-up, or nullptr: FP64 work per entry otherwise
+  const T *rdiff;
+  T *dev;              // [ns] deviation sums D of the neighbourhood averages
+  T *pval;             // [ns] field value at each neighbourhood's pivot
+  T *sig;              // [3 * ns] limited slopes
   unsigned *status;
 };
+constexpr int WSRD_DK = 17;   // level differences -8 .. 8 (tables reach 4 levels)
 
-// the redistribution of all five fields in one pass: f[q] is field q, and
-// its small CVs (affected CVs) are the work items off_small[q] .. off_small[q+1]-1
-// (off_aff[q] ..) of each fused launch
+// the redistribution of all five fields in one pass: f[q] is field q.  The
+// items off_small[g] .. off_small[g+1]-1 of a launch over the small CVs belong
+// to grid g and take every field of the grid (rho and rho*theta share the c
+// grid's tables); the items off_aff[f] .. of the launch over the affected CVs
+// belong to field f.
 template <typename T>
 struct WsrdSet {
   WsrdArgs<T> f[5];
-  long long off_small[6];
+  long long off_small[5];
   long long off_aff[6];
 };
 

@@ -468,9 +468,50 @@ __global__ void k_aff_fill(Dims D, int g, GridDev G, const long long *aff_id, Ws
   }
 }
 
-__global__ void k_to_float(const double *src, float *dst, long long n) {
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t < n) dst[t] = (float)src[t];
+// ---- the step's tables (WsrdTab) ------------------------------------------
+constexpr unsigned kMaxSmall = 1u << 28;   // a tag's room for small ids
+
+__device__ inline unsigned make_tag(long long sid, int dk) { return (unsigned)(sid + 1) | (unsigned)(dk + 8) << 28; }
+
+template <typename T>
+__global__ void k_pack_small(Dims D, WsrdDev W, WsrdTab P) {
+  const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x, ns = W.nsmall;
+  if (s >= ns) return;
+  const long long pl = W.s_plin[s];
+  P.plin[s] = (unsigned)pl;
+  P.nmem[s] = (uint8_t)(W.s_nmem[s] | W.s_piv[s] << 4);
+  for (int q = 0; q < 8; ++q) {
+    P.mlin[q * ns + s] = q < W.s_nmem[s] ? (unsigned)W.s_mlin[8 * s + q] : (unsigned)pl;
+    ((T *)P.mw)[q * ns + s] = (T)W.s_mw[8 * s + q];
+    for (int d = 0; d < 3; ++d) ((T *)P.me)[(3 * q + d) * ns + s] = (T)W.s_me[24 * s + 3 * q + d];
+  }
+  const int kp = (int)(pl / D.nxy);
+  const long long o0 = W.s_loff[s], o1 = W.s_loff[s + 1];
+  for (long long o = o0; o < o1; ++o) {
+    const long long pm = W.l_plin[o];
+    P.lplin[o] = (unsigned)pm;
+    P.ltag[o] = make_tag(W.l_sid[o], (int)(pm / D.nxy) - kp);
+    for (int d = 0; d < 3; ++d) ((T *)P.lc)[d * P.nl + o] = (T)W.l_c[3 * o + d];
+  }
+}
+
+template <typename T>
+__global__ void k_pack_aff(Dims D, WsrdDev W, WsrdTab P) {
+  const long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (a >= W.naff) return;
+  const long long c = W.a_lin[a];
+  const int sid = W.a_sid[a], kc = (int)(c / D.nxy);
+  const int kp = sid >= 0 ? (int)(W.s_plin[sid] / D.nxy) : kc;
+  P.alin[a] = (unsigned)c;
+  P.atag[a] = make_tag(sid, kp - kc);
+  for (int d = 0; d < 3; ++d) ((T *)P.es)[d * W.naff + a] = (T)W.a_eself[3 * a + d];
+  const long long o0 = W.a_woff[a], o1 = W.a_woff[a + 1];
+  for (long long o = o0; o < o1; ++o) {
+    const int r = W.w_sid[o];
+    P.wtag[o] = make_tag(r, (int)(W.s_plin[r] / D.nxy) - kp);
+    ((T *)P.wk)[o] = (T)W.w_k[o];
+    for (int d = 0; d < 3; ++d) ((T *)P.we)[d * P.nw + o] = (T)W.w_e[3 * o + d];
+  }
 }
 
 inline int cols_blocks(const Dims &D) { return (D.nx * D.ny + 127) / 128; }
@@ -579,18 +620,6 @@ cudaError_t build_wsrd(const Dims &D, int g, GridDev &G, const GridDev *all, dou
   CK(dalloc(&W.w_k, W.nw));
   CK(dalloc(&W.w_e, 3 * W.nw));
   k_aff_fill<<<cb, 128, 0, s>>>(D, g, G, aff_id, W);
-  // float copies of the weight tables (mixed-precision path)
-  const struct {
-    const double *src;
-    float **dst;
-    long long n;
-  } tabs[6] = {{W.s_mw, &W.s_mw_f, 8 * W.nsmall}, {W.s_me, &W.s_me_f, 24 * W.nsmall},
-               {W.l_c, &W.l_c_f, 3 * W.nlsq},     {W.a_eself, &W.a_eself_f, 3 * W.naff},
-               {W.w_k, &W.w_k_f, W.nw},           {W.w_e, &W.w_e_f, 3 * W.nw}};
-  for (const auto &t : tabs) {
-    CK(dalloc(t.dst, t.n));
-    if (t.n > 0) k_to_float<<<lin_blocks(t.n), 128, 0, s>>>(t.src, *t.dst, t.n);
-  }
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
   return cudaSuccess;
@@ -598,11 +627,61 @@ cudaError_t build_wsrd(const Dims &D, int g, GridDev &G, const GridDev *all, dou
 
 void free_wsrd(WsrdDev &W) {
   void *ptrs[] = {W.sid, W.s_lin, W.s_rec, W.s_nmem, W.s_piv, W.s_mlin, W.s_mw, W.s_me, W.s_loff, W.l_lin,
-                  W.l_sid, W.l_c, W.a_lin, W.a_sid, W.a_eself, W.a_woff, W.w_sid, W.w_k, W.w_e,
-                  W.s_mw_f, W.s_me_f, W.l_c_f, W.a_eself_f, W.w_k_f, W.w_e_f, W.s_plin, W.l_plin};
+                  W.l_sid, W.l_c, W.a_lin, W.a_sid, W.a_eself, W.a_woff, W.w_sid, W.w_k, W.w_e, W.s_plin, W.l_plin};
   for (void *p : ptrs)
     if (p) cudaFree(p);
-  W = WsrdDev();
+  WsrdDev none;
+  none.nsmall = W.nsmall;
+  none.naff = W.naff;
+  W = none;
+}
+
+namespace {
+
+template <typename T>
+cudaError_t pack_wsrd_t(const Dims &D, const WsrdDev &W, WsrdTab &P, cudaStream_t s) {
+  const long long ns = W.nsmall, na = W.naff;
+  P.ns = ns;
+  P.na = na;
+  P.nl = W.nlsq;
+  P.nw = W.nw;
+  CK(dalloc(&P.loff, ns + 1));
+  CK(dalloc(&P.woff, na + 1));
+  CK(cudaMemcpyAsync(P.loff, W.s_loff, sizeof(long long) * (size_t)(ns + 1), cudaMemcpyDeviceToDevice, s));
+  CK(cudaMemcpyAsync(P.woff, W.a_woff, sizeof(long long) * (size_t)(na + 1), cudaMemcpyDeviceToDevice, s));
+  CK(dalloc(&P.plin, ns));
+  CK(dalloc(&P.nmem, ns));
+  CK(dalloc(&P.mlin, 8 * ns));
+  CK(dalloc((T **)&P.mw, 8 * ns));
+  CK(dalloc((T **)&P.me, 24 * ns));
+  CK(dalloc(&P.lplin, P.nl));
+  CK(dalloc(&P.ltag, P.nl));
+  CK(dalloc((T **)&P.lc, 3 * P.nl));
+  CK(dalloc(&P.alin, na));
+  CK(dalloc(&P.atag, na));
+  CK(dalloc((T **)&P.es, 3 * na));
+  CK(dalloc(&P.wtag, P.nw));
+  CK(dalloc((T **)&P.wk, P.nw));
+  CK(dalloc((T **)&P.we, 3 * P.nw));
+  if (ns) k_pack_small<T><<<lin_blocks(ns), 128, 0, s>>>(D, W, P);
+  if (na) k_pack_aff<T><<<lin_blocks(na), 128, 0, s>>>(D, W, P);
+  CK(cudaGetLastError());
+  return cudaStreamSynchronize(s);
+}
+
+}  // namespace
+
+cudaError_t pack_wsrd(const Dims &D, const WsrdDev &W, bool f64, WsrdTab &P, cudaStream_t s) {
+  if (W.nsmall >= kMaxSmall - 1) return cudaErrorInvalidValue;
+  return f64 ? pack_wsrd_t<double>(D, W, P, s) : pack_wsrd_t<float>(D, W, P, s);
+}
+
+void free_wsrd_tab(WsrdTab &P) {
+  void *ptrs[] = {P.plin, P.nmem, P.mlin, P.mw, P.me, P.loff, P.lplin, P.ltag, P.lc, P.alin, P.atag, P.es,
+                  P.woff, P.wtag, P.wk, P.we};
+  for (void *p : ptrs)
+    if (p) cudaFree(p);
+  P = WsrdTab();
 }
 
 void launch_wsrd_reach(const Dims &D, int g, const WsrdDev &W, const int *kcov, const int *kfast, unsigned *far,
