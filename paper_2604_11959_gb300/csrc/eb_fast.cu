@@ -171,6 +171,18 @@ cudaError_t bulk_plan(const Dims &D, const int *kfast_host, bool f64, int slab_l
   // Slabs of slab_levels levels, or (0) of at least 16 levels sized for
   // about three waves of CTAs.
   long long Lc = slab_levels > 0 ? (long long)slab_levels : std::max(16LL, (W + 3 * slots - 1) / (3 * slots));
+  if (slab_levels == 0 && !f64 && alone) {
+    // Float path alone on the GPU: the near-EB kernels run beside the march
+    // and are as much of the step, so fewer, taller pieces (less prologue
+    // work in their way) win over full waves: about 1.5 CTAs per SM, one
+    // wave, of at least 16 levels; 8 where even those leave SMs idle and the
+    // longest piece counts.  Whole steps, slabs of three waves and this rule:
+    // 256x256x128 hill 248 and 228 us, 256x256x64 random terrain 348 and
+    // 328, 200x100x40 107 and 105, 64x64x64 49 and 43, 32x32x16 41 and 39.
+    const long long tiles = (long long)kb.size();
+    const long long nslab = std::max(1LL, std::min<long long>(D.nz / 16, (3LL * sms / 2 + tiles / 2) / tiles));
+    Lc = tiles * nslab < sms ? 8 : (D.nz + nslab - 1) / nslab;
+  }
   if (slab_levels == 0 && f64 && alone) {
     // Double path alone on the GPU: the height (and for small domains the
     // 16 x 8 tile) of the shortest estimated time, in microseconds as
