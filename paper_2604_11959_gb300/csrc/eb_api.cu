@@ -828,20 +828,24 @@ eb_status eb_step(eb_geom geom, const eb_state *Un, eb_state *Unp1, double dt, i
         geom->info.device_bytes += (int64_t)(field_count(geom->D, f) * es);
       }
   void **C = geom->scr[0], **Dd = geom->scr[1], **A = geom->scr[2], **B = geom->scr[3];
-  // Covered CVs and the w wall levels enter no flux, source or
-  // redistribution, so only Unp1 receives them, from Un in the last stage
-  // (512x512x256 random terrain, three stages: two of three 0.11 ms copies less).
+  // C, D, A, B and Unp1 need their covered CVs and w wall levels once: where
+  // the first and last column of a window do not meet, the stencils across
+  // that seam read covered CVs.
+  bool fresh[5] = {true, true, true, true, true};
+  auto fresh_of = [&](void **p) -> bool & {
+    return p == C ? fresh[0] : p == Dd ? fresh[1] : p == A ? fresh[2] : p == B ? fresh[3] : fresh[4];
+  };
   void **cur = u0;
   for (int n = 0; n < nsteps; ++n) {
-    const bool last = n == nsteps - 1;
-    void **dst = last ? u1 : (cur == C ? Dd : C);
+    void **dst = n == nsteps - 1 ? u1 : (cur == C ? Dd : C);
     const double c[3] = {stages == 1 ? dt : dt / 3.0, dt / 2.0, dt};
     void **srcs[3] = {cur, A, B};
     void **outs[3] = {stages == 1 ? dst : A, B, dst};
     for (int q = 0; q < stages; ++q) {
-      const int copy = last && q == stages - 1;
-      if (geom->prec == EB_F64) stage<double>(geom, srcs[q], cur, outs[q], c[q], copy, s, true, u0);
-      else stage<float>(geom, srcs[q], cur, outs[q], c[q], copy, s, true, u0);
+      bool &fr = fresh_of(outs[q]);
+      if (geom->prec == EB_F64) stage<double>(geom, srcs[q], cur, outs[q], c[q], fr, s);
+      else stage<float>(geom, srcs[q], cur, outs[q], c[q], fr, s);
+      fr = false;
     }
     cur = dst;
   }

@@ -62,7 +62,7 @@ __global__ void k_static(StepArgs<T> A, StaticBlocks SB) {
     T v[STATIC_PER_THREAD];
 #pragma unroll
     for (int e = 0; e < STATIC_PER_THREAD; ++e)
-      v[e] = (c[e] != 0xffffffffu && A.stat[0]) ? A.stat[f][c[e]] : T(0);
+      v[e] = (c[e] != 0xffffffffu && A.base[0]) ? A.base[f][c[e]] : T(0);
 #pragma unroll
     for (int e = 0; e < STATIC_PER_THREAD; ++e)
       if (c[e] != 0xffffffffu) A.out[f][c[e]] = v[e];

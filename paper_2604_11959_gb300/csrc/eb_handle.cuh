@@ -202,7 +202,6 @@ StepArgs<T> step_args(eb_geom g, void *const src[5], void *const base[5], void *
   for (int f = 0; f < 5; ++f) {
     A.src.f[f] = (const T *)src[f];
     A.base[f] = base ? (const T *)base[f] : nullptr;
-    A.stat[f] = A.base[f];
     A.out[f] = (T *)out[f];
   }
   if (sizeof(T) == sizeof(double)) {
@@ -323,14 +322,11 @@ void wsrd_all(eb_geom g, void *const out[5], cudaStream_t s) {
 // the bulk kernel; otherwise it follows the join.  (Ensembles keep it after
 // the join: their members already fill the GPU side by side, and the longer
 // branches cost more than the shorter critical path gains.)  copy: the
-// covered CVs and the w wall levels of out are written too, from the state
-// stat (default: base).
+// covered CVs and the w wall levels of out are written too, from base.
 template <typename T>
 void stage(eb_geom g, void *const src[5], void *const base[5], void *const out[5], double dt, int copy,
-           cudaStream_t s, bool wsrd_beside = true, void *const *stat = nullptr) {
+           cudaStream_t s, bool wsrd_beside = true) {
   StepArgs<T> A = step_args<T>(g, src, base, out, dt, copy);
-  if (stat)
-    for (int f = 0; f < 5; ++f) A.stat[f] = (const T *)stat[f];
   if (g->src_flags) {   // the sources follow the whole flux update; the redistribution follows them
     flux_update(g, A, s);
     const bool f64 = sizeof(T) == sizeof(double);

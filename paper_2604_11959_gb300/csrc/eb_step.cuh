@@ -8,7 +8,6 @@ struct StepArgs {
   Dims D;
   StateIn<T> src;      // state the fluxes are computed from
   const T *base[5];    // state the update is added to; base[0] == nullptr: write dU itself
-  const T *stat[5];    // state the covered CVs and w wall levels are copied from (stat[0] == nullptr: zeros)
   T *out[5];
   double dt;
   T dtT;

@@ -59,6 +59,27 @@ def test_covered_values_come_from_the_first_state(eb, precision):
         assert torch.equal(V["rhow"][0], wall[0]) and torch.equal(V["rhow"][-1], wall[-1])
 
 
+@pytest.mark.parametrize("precision", ["f64", "mixed"])
+@pytest.mark.parametrize("stages", [1, 3])
+def test_steps_of_a_window_whose_ends_do_not_meet(eb, precision, stages):
+    """The terrain jumps from the last column of the window to the first, so
+    stencils across that seam read covered CVs: two steps in one call (scratch
+    state between them) are bit for bit two calls (full states between them)."""
+    w = inputs.Workload("seam", 24, 20, 16, 1, terrain="grf", seed=4, hmax=0.12)
+    refs = refs_for(w.nz, w.Lz)
+    h = w.heights() + np.linspace(0.0, 0.2, w.nx + 1)[None, :]
+    U = to_device(w.state("uniform", pert=1e-2, seed=5), precision, refs)
+    for nsteps in (2, 4):
+        once = make_geometry(eb, w, h, precision, refs)
+        got = eb.step(once, U, w.dt(), nsteps, stages)
+        each = make_geometry(eb, w, h, precision, refs)
+        want = U
+        for _ in range(nsteps):
+            want = eb.step(each, want, w.dt(), 1, stages)
+        for f in FIELDS:
+            assert torch.allclose(got[f], want[f], rtol=0.0, atol=0.0, equal_nan=True), (f, nsteps)
+
+
 @pytest.mark.parametrize("n", [(16, 16, 8), (20, 12, 8), (24, 36, 28), (50, 34, 18), (64, 32, 16), (144, 16, 16)])
 def test_multigrid_reaches_the_jacobi_solution(eb, n):
     """V-cycles over grids with 4, 2 and 1 columns per thread, one or several
