@@ -339,6 +339,11 @@ eb_status build_impl(eb_geom g, const double *h_nodes, const double *ref_rho, co
         if (e == cudaSuccess) e = g->alloc((char **)&G.fh[d], (long long)(nfa * es));
         G.fhm[d] = nullptr;
         if (e == cudaSuccess && q == 0) e = g->alloc((char **)&G.fhm[d], (long long)(nfa * es));
+        // where a window's last and first columns do not meet, the high face of
+        // the one may be open and the low face of the other closed: the flux of
+        // such a face is never formed and reads 0
+        if (e == cudaSuccess) e = cudaMemsetAsync(G.fh[d], 0, (size_t)nfa * es, s);
+        if (e == cudaSuccess && q == 0) e = cudaMemsetAsync(G.fhm[d], 0, (size_t)nfa * es, s);
       }
     }
     if (e == cudaSuccess) {
