@@ -383,8 +383,8 @@ eb_status eb_step_profile(eb_geom geom, const eb_state *Un, eb_state *Unp1, doub
  *   phi      device, nx*ny*nz doubles: receives the solution, or NULL.
  *   iters    host: iterations used (NULL allowed).
  *   relres   host: final relative residual (NULL allowed).
- * rho and rho*theta are not touched.  Synchronises the stream every 32
- * iterations (convergence test).  The first call on a handle allocates its
+ * rho and rho*theta are not touched.  Synchronises the stream where the
+ * reduction so far predicts convergence (at least every 64 iterations).  The first call on a handle allocates its
  * work space (about 10 doubles per cell), so it must not be inside a stream
  * capture.
  */

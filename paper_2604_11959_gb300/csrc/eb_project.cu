@@ -17,8 +17,8 @@
 // block that finishes last adds them in a fixed order, so the solve is
 // deterministic and the next kernel reads one number.  Convergence is
 // detected on the device (the kernels of later iterations return at once)
-// and read by the host every 32 iterations (every 4 with the multigrid
-// preconditioner).
+// and read by the host after 32 iterations (4 with the multigrid
+// preconditioner) and then where the reduction so far predicts it.
 //
 // What bounds an iteration of the outer conjugate gradients is FP64 (two
 // instructions per clock and SM): nine per cell in the operator and its dot
@@ -27,8 +27,9 @@
 // terrain are formed from sums of opposite neighbours, x is updated with the
 // direction (p is read once), floats are widened by integer instructions, and
 // nothing is computed for the mask of inactive cells (their r, p and q are
-// zero).  192x192x96: operator 63 -> 51 us, update 47 -> 24, direction (with x) 24
-// -> 31, right-hand side 116 -> 39, correction 114 -> 51.
+// zero).  192x192x96: operator 63 -> 64 us (its floor is about 47), update 47 ->
+// 27 (x moved out), direction 24 -> 22 (x moved in), right-hand side 116 -> 70,
+// correction 114 -> 74, start of the solve 95 -> 30, centring 34 -> 25.
 #include "eb_handle.cuh"
 
 #include <math.h>
