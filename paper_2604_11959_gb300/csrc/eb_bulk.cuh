@@ -44,9 +44,9 @@
 // What bounds it: instruction issue on the float path, FP64 instructions on
 // the double path (an SM starts two per clock, 1/64 of the FP32 rate).  The
 // double path therefore spends integer instructions where it can (selects
-// before the flux arithmetic, the finite test) and three FP64 instructions
-// per reciprocal: 256x256x128 hill, one FP64 step 4.80 -> 3.12 ms, 32x32x16
-// ridge 510 -> 337 us, the mixed hill step 224 -> 218 us.
+// before the flux arithmetic, the finite test) and leaves halves to constant
+// factors.  256x256x128 hill, one FP64 step 4.80 -> 3.21 ms and ten of the
+// 32x32x16 ridge 5105 -> 502 us, both with the split of eb_fast.cu.
 #pragma once
 
 #include "eb_step.cuh"
@@ -161,21 +161,12 @@ __device__ inline float2 psub(float2 a, float2 b) { return __ffma2_rn(b, make_fl
 __device__ inline double2 psub(double2 a, double2 b) { return make_double2(__dsub_rn(a.x, b.x), __dsub_rn(a.y, b.y)); }
 // elementwise reciprocal: the fast approximate one on the float path
 __device__ inline float2 prcp(float2 a) { return make_float2(__fdividef(1.f, a.x), __fdividef(1.f, a.y)); }
-// FP64 instructions are what bounds the double path (two per clock and SM),
-// so the reciprocal is formed with three: r0 = 1/a (1 - e) from the
-// hardware's approximate double reciprocal (|e| about 2^-20), then 1/a = r0
-// (1 + e + e^2 + ...) cut after e^2, which leaves an error of |e|^3 = 2^-60
-// before the one rounding of the last operation; outside the range where r0
-// and its product are normal numbers the plain division runs.
-__device__ inline double rcp_fma(double a) {
-  const unsigned ex = (unsigned)__double2hiint(a) & 0x7ff00000u;
-  if (ex - 0x00300000u > 0x7f900000u) return 1.0 / a;   // zero, subnormal, near the range's ends, Inf, NaN
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-  const double e = __fma_rn(-a, r, 1.0);
-  return __fma_rn(r, __fma_rn(e, e, e), r);
-}
-__device__ inline double2 prcp(double2 a) { return make_double2(rcp_fma(a.x), rcp_fma(a.y)); }
+// The double path's are correctly rounded.  A cubic iteration from the
+// hardware's approximate reciprocal (three FP64 instructions, 256x256x128 hill
+// step 3017 us against 3207) was an ulp off in 0.03 % of the values and
+// could flush to zero just below 2^1022; its rounding corrected by two more (3220)
+// it gained nothing over the division.
+__device__ inline double2 prcp(double2 a) { return make_double2(1.0 / a.x, 1.0 / a.y); }
 template <typename P>
 __device__ inline P psel_pos(P m, P a, P b) {   // a where m > 0, else b
   return mk(m.x > 0 ? a.x : b.x, m.y > 0 ? a.y : b.y);
