@@ -227,33 +227,59 @@ __device__ inline void two_sum(float a, float b, float &s, float &e) {
   e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
 
-// the sum of N values and a level constant (hi, lo), scaled by an exact power
-// of two: in double, or for floats as an unevaluated pair (48 bits; rounded
-// to float once), since FP64 instructions would bound both kernels
-template <int N>
-__device__ inline double mean_plus(const double (&v)[N], double hi, double) {
-  double s = v[0];
+// A constant of a level: in double and, for the float path, as the nearest
+// float and the rest.
+struct LevelConst {
+  double d;
+  float hi, lo;
+};
+__device__ inline LevelConst level_const(double d) {
+  const float hi = (float)d;
+  return LevelConst{d, hi, (float)(d - (double)hi)};
+}
+
+// the mean of N values (a power of two) plus a level constant, in double
+template <int N, typename T>
+__device__ inline double mean_double(const T (&v)[N], const LevelConst &c) {
+  double s = (double)v[0];
 #pragma unroll
-  for (int q = 1; q < N; ++q) s += v[q];
-  return s * (1.0 / N) + hi;
+  for (int q = 1; q < N; ++q) s += (double)v[q];
+  return s * (1.0 / N) + c.d;
+}
+// The same rounded to the state's type.  FP64 instructions would bound both
+// kernels on the float path, so there N times the value is first formed as t +
+// rest, every addition's rounding error kept (the errors' own roundings, and
+// what two floats leave of the constant, are added up as a bound); where both
+// ends of rest +- bound round to the same float, that is the rounded value (the
+// rounding test of Ziv, ACM Trans. Math. Softw. 17, 1991; plain means, whose
+// bound is mostly zero, may then end on ties).  Otherwise, and where anything is
+// infinite, NaN or overflows (every such comparison is false) or the scaled
+// value could be subnormal, sure becomes false, and the caller forms its
+// values by mean_double: all of a thread's after one test, so that their loads
+// stay together.
+template <int N>
+__device__ inline double mean_plus(const double (&v)[N], const LevelConst &c, bool &) {
+  return mean_double(v, c);
 }
 template <int N>
-__device__ inline float mean_plus(const float (&v)[N], float hi, float lo) {
-  float s = v[0], c = 0.f;
+__device__ inline float mean_plus(const float (&v)[N], const LevelConst &c, bool &sure) {
+  float s = v[0], rest = 0.f, bound = 0.f, t, e, r;
 #pragma unroll
   for (int q = 1; q < N; ++q) {
-    float e;
     two_sum(s, v[q], s, e);
-    c = __fadd_rn(c, e);
+    two_sum(rest, e, rest, r);
+    bound = __fadd_ru(bound, fabsf(r));
   }
-  constexpr float inv = 1.f / N;   // exact: N is 1, 2, 4 or 8
-  float t, e;
-  two_sum(__fmul_rn(s, inv), hi, t, e);
-  return __fadd_rn(t, __fadd_rn(e, __fmaf_rn(c, inv, lo)));
+  two_sum(s, N * c.hi, t, e);   // (products with N are exact)
+  two_sum(rest, e, rest, r);
+  bound = __fadd_ru(bound, fabsf(r));
+  two_sum(rest, N * c.lo, rest, r);
+  bound = __fadd_ru(bound, fabsf(r));
+  bound = __fmaf_ru(fabsf(N * c.hi), 0x1p-47f, bound);
+  const float a = __fadd_rn(t, __fsub_rd(rest, bound)), b = __fadd_rn(t, __fadd_ru(rest, bound));
+  sure = sure && a == b && (fabsf(a) >= 0x1p-100f || a == 0.f);
+  return a * (1.f / N);
 }
-// a double constant as (hi, lo) of type T
-__device__ inline void split_const(double d, double &hi, double &lo) { hi = d, lo = 0.0; }
-__device__ inline void split_const(double d, float &hi, float &lo) { hi = (float)d, lo = (float)(d - (double)hi); }
 
 // The coarse CVs at (I, J, K) of all five fields where fine cells are cut or
 // covered: the eight fine cells' fractions are looked up once (one chain of
@@ -303,13 +329,14 @@ __device__ inline void restrict_cut(const RestrictArgs<T> &R, const int cols[4],
 // All five fields of one coarse level per blockIdx.y (the lid face above the
 // top level keeps its value).  HBM bounds it: where the four fine columns are
 // regular, every value is a plain mean of 8 (4) fine ones plus a constant of
-// the level, formed without FP64 on the float path.  64 x 256 x 128 fine cells
+// the level, formed almost without FP64 on the float path.  64 x 256 x 128 fine cells
 // onto 32 x 128 x 64: 37 us, the FP64 sums over the cut cells most of it
 // (130 us for one launch per field with double sums over looked-up fractions).
 template <typename T>
 __global__ void __launch_bounds__(256) k_restrict(const __grid_constant__ RestrictArgs<T> R) {
   const Dims &Dc = R.Dc, &Df = R.F.D;
-  __shared__ T chi[4], clo[4];   // per field: mean fine profile minus the coarse one
+  __shared__ LevelConst lc[4];   // per field: mean fine profile minus the coarse one
+  const LevelConst none{0.0, 0.f, 0.f};
   const unsigned n = (unsigned)R.ncols * (unsigned)Dc.ny;
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
   const int J = (int)(t / (unsigned)R.ncols), It = (int)(t - (unsigned)J * (unsigned)R.ncols);
@@ -321,7 +348,7 @@ __global__ void __launch_bounds__(256) k_restrict(const __grid_constant__ Restri
       double d = 0.0;
       if (R.pf[f]) d += 0.5 * (R.pf[f][2 * K] + R.pf[f][2 * K + 1]);
       if (R.pc[f]) d -= R.pc[f][K];
-      split_const(d, chi[f], clo[f]);
+      lc[f] = level_const(d);
     }
     __syncthreads();
     if (t >= n) continue;
@@ -335,22 +362,23 @@ __global__ void __launch_bounds__(256) k_restrict(const __grid_constant__ Restri
       continue;
     }
     const long long b0 = Df.nxy * (2LL * K), b1 = b0 + Df.nxy;
-    T o[5];
-#pragma unroll
-    for (int f = 0; f < 2; ++f) {
-      const T *u = R.uf[f];
-      const T v[8] = {u[b0 + c00], u[b0 + c10], u[b0 + c01], u[b0 + c11],
-                      u[b1 + c00], u[b1 + c10], u[b1 + c01], u[b1 + c11]};
-      o[f] = mean_plus<8>(v, chi[f], clo[f]);
-    }
-    {
-      const T *u = R.uf[2], *v = R.uf[3], *w = R.uf[4];
-      const T vu[4] = {u[b0 + c00], u[b0 + c01], u[b1 + c00], u[b1 + c01]};
-      const T vv[4] = {v[b0 + c00], v[b0 + c10], v[b1 + c00], v[b1 + c10]};
-      const T vw[4] = {w[b0 + c00], w[b0 + c10], w[b0 + c01], w[b0 + c11]};
-      o[2] = mean_plus<4>(vu, chi[2], clo[2]);
-      o[3] = mean_plus<4>(vv, chi[3], clo[3]);
-      o[4] = mean_plus<4>(vw, T(0), T(0));
+    const T *r = R.uf[0], *h = R.uf[1], *u = R.uf[2], *v = R.uf[3], *w = R.uf[4];
+    const T vr[8] = {r[b0 + c00], r[b0 + c10], r[b0 + c01], r[b0 + c11],
+                     r[b1 + c00], r[b1 + c10], r[b1 + c01], r[b1 + c11]};
+    const T vh[8] = {h[b0 + c00], h[b0 + c10], h[b0 + c01], h[b0 + c11],
+                     h[b1 + c00], h[b1 + c10], h[b1 + c01], h[b1 + c11]};
+    const T vu[4] = {u[b0 + c00], u[b0 + c01], u[b1 + c00], u[b1 + c01]};
+    const T vv[4] = {v[b0 + c00], v[b0 + c10], v[b1 + c00], v[b1 + c10]};
+    const T vw[4] = {w[b0 + c00], w[b0 + c10], w[b0 + c01], w[b0 + c11]};
+    bool sure = true;
+    T o[5] = {mean_plus(vr, lc[0], sure), mean_plus(vh, lc[1], sure), mean_plus(vu, lc[2], sure),
+              mean_plus(vv, lc[3], sure), mean_plus(vw, none, sure)};
+    if (!sure) {
+      o[0] = (T)mean_double(vr, lc[0]);
+      o[1] = (T)mean_double(vh, lc[1]);
+      o[2] = (T)mean_double(vu, lc[2]);
+      o[3] = (T)mean_double(vv, lc[3]);
+      o[4] = (T)mean_double(vw, none);
     }
 #pragma unroll
     for (int f = 0; f < 5; ++f) R.uc[f][tc] = o[f];
@@ -374,12 +402,13 @@ struct ProlongArgs {
 // One fine level per blockIdx.y, all five fields of the columns outside [lo,
 // hi) (the level above the top holds rho*w only).  HBM bounds it; a value
 // costs one addition of the level's profile difference (as on the
-// restriction's float path, without FP64).  24 of 88 columns x 256 x 128: 16
+// restriction's float path, almost without FP64).  24 of 88 columns x 256 x 128: 16
 // us (127 us for one launch per field over all columns).
 template <typename T>
 __global__ void __launch_bounds__(256) k_prolong(const __grid_constant__ ProlongArgs<T> P) {
   const Dims &Df = P.Df, &Dc = P.Dc;
-  __shared__ T chi[4], clo[4];   // per field: coarse profile minus the fine one
+  __shared__ LevelConst lc[4];   // per field: coarse profile minus the fine one
+  const LevelConst none{0.0, 0.f, 0.f};
   const unsigned cols = (unsigned)(Df.nx - (P.hi - P.lo));
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = (int)(t / cols);
@@ -395,27 +424,38 @@ __global__ void __launch_bounds__(256) k_prolong(const __grid_constant__ Prolong
       double d = 0.0;
       if (P.pc[f]) d += P.pc[f][K];
       if (P.pf[f]) d -= P.pf[f][k];
-      split_const(d, chi[f], clo[f]);
+      lc[f] = level_const(d);
     }
     __syncthreads();
     if (t >= cols * (unsigned)Df.ny) continue;
     const long long c = I + (long long)Dc.nx * J + Dc.nxy * K;
     const long long q = i + (long long)Df.nx * j + Df.nxy * k;
-    // one value, or the mean of the two coarse faces around an odd fine face
-    auto mean = [&](int f, bool odd, long long c2, T hi, T lo) -> T {
-      const T v[2] = {P.uc[f][c], odd ? P.uc[f][c2] : T(0)};
-      if (odd) return mean_plus<2>(v, hi, lo);
-      const T one[1] = {v[0]};
-      return mean_plus<1>(one, hi, lo);
-    };
-    T o[5];
-    if (k < Df.nz) {
+    // one coarse value (twice the same), or the two coarse faces around an odd fine face
+    const bool cell = k < Df.nz;
+    const bool odd[5] = {false, false, (gi & 1) != 0, (j & 1) != 0, (k & 1) != 0};
+    const long long c2[5] = {c, c, odd[2] ? c - I + wrapi(I + 1, Dc.nx) : c,
+                             odd[3] ? c + (long long)Dc.nx * (wrapi(J + 1, Dc.ny) - J) : c, odd[4] ? c + Dc.nxy : c};
+    T v[5][2], o[5];
 #pragma unroll
-      for (int f = 0; f < 2; ++f) o[f] = mean(f, false, c, chi[f], clo[f]);
-      o[2] = mean(2, gi & 1, c - I + wrapi(I + 1, Dc.nx), chi[2], clo[2]);
-      o[3] = mean(3, j & 1, c + (long long)Dc.nx * (wrapi(J + 1, Dc.ny) - J), chi[3], clo[3]);
+    for (int f = 0; f < 5; ++f) {
+      v[f][0] = cell || f == 4 ? P.uc[f][c] : T(0);
+      v[f][1] = f < 2 ? v[f][0] : cell || f == 4 ? P.uc[f][c2[f]] : T(0);
     }
-    o[4] = mean(4, k & 1, c + Dc.nxy, T(0), T(0));
+    bool sure = sizeof(T) == sizeof(float);
+    if (sure) {
+#pragma unroll
+      for (int f = 0; f < 5; ++f) {
+        const T (&two)[2] = v[f];
+        o[f] = mean_plus(two, f < 4 ? lc[f] : none, sure);
+      }
+    }
+    if (!sure) {
+#pragma unroll
+      for (int f = 0; f < 5; ++f) {
+        const T one[1] = {v[f][0]};
+        o[f] = (T)(odd[f] ? mean_double(v[f], f < 4 ? lc[f] : none) : mean_double(one, f < 4 ? lc[f] : none));
+      }
+    }
     if (k < Df.nz) {
 #pragma unroll
       for (int f = 0; f < 4; ++f) P.uf[f][q] = o[f];
