@@ -130,7 +130,9 @@ typedef struct {
                                is a near-EB CV, so eb_step runs it right after
                                the near-EB kernels, beside the bulk kernel
                                (ensembles keep it after the bulk kernel)      */
-  int64_t tile_rows;        /* rows of the bulk kernel's tiles (16, or 14)    */
+  int64_t tile_rows;        /* rows of the bulk kernel's tiles in use (16, 14
+                               on the mixed path, or 8 where the automatic
+                               split of an FP64 handle chose 16x8 tiles)      */
 } eb_geom_info_t;
 
 /*
@@ -610,7 +612,9 @@ eb_status eb_geom_set_bulk_priority(eb_geom geom, int high);
  * earlier.  Waits for the device to be idle (the old plan may be in use). */
 eb_status eb_geom_set_slab_levels(eb_geom geom, int slab_levels);
 
-/* Rows of the bulk kernel's tiles of 32 columns: 16 (default) or, on the
+/* Rows of the bulk kernel's tiles of 32 columns: 16 (default; until this is
+ * called, the automatic split of an FP64 handle may take tiles of 16 columns
+ * and 8 rows on small domains) or, on the
  * mixed path, 14 (a 256-row domain then cuts into 19 tile rows, and two slabs
  * of its 152 tiles fill every SM with two CTAs).  Scheduling only: every
  * cell's arithmetic is the same.  eb_geom_tune tries both on the mixed path;

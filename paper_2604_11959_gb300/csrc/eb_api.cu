@@ -22,8 +22,8 @@ std::string &eb_error_slot() { return g_last_error; }
 eb_status eb_replan_bulk(eb_geom g, int slab_levels) {
   std::vector<int> seg, off;
   int rows = g->tile_rows;
-  CUDA_TRY(bulk_plan(g->D, g->kfast_host.data(), g->prec == EB_F64, slab_levels, g->tile_rows, !g->in_ensemble, seg,
-                     off, rows),
+  CUDA_TRY(bulk_plan(g->D, g->kfast_host.data(), g->prec == EB_F64, slab_levels, g->tile_rows, !g->in_ensemble,
+                     !g->rows_set, seg, off, rows),
            "bulk work split");
   // the split arrays are small: the old ones are released right away
   for (void *p : {(void *)g->bseg, (void *)g->boff}) {
@@ -719,7 +719,7 @@ eb_status eb_geom_info(eb_geom geom, eb_geom_info_t *info) {
   info->slab_levels = geom->slab_levels;
   info->bulk_high_priority = geom->bulk_high;
   info->wsrd_beside_bulk = geom->wsrd_side;
-  info->tile_rows = geom->tile_rows;
+  info->tile_rows = geom->plan_rows;
   return EB_OK;
 }
 
@@ -908,6 +908,7 @@ eb_status eb_geom_set_tile_rows(eb_geom geom, int rows) {
   if (rows == 14 && geom->prec == EB_F64) return fail(EB_ERR_INVALID_ARG, "14-row tiles are for the mixed path");
   CUDA_TRY(cudaDeviceSynchronize(), "drain before re-planning");
   geom->tile_rows = rows;
+  geom->rows_set = true;
   return eb_replan_bulk(geom, geom->slab_levels);
 }
 

@@ -128,7 +128,7 @@ eb_status build_tables(eb_ensemble e, EnsembleArgs<T> E[2]) {
     eb_geom g = e->m[q];
     std::vector<int> seg, off;
     int rows = 16;
-    CUDA_TRY(bulk_plan(g->D, g->kfast_host.data(), g->prec == EB_F64, g->slab_levels, 16, false, seg, off, rows),
+    CUDA_TRY(bulk_plan(g->D, g->kfast_host.data(), g->prec == EB_F64, g->slab_levels, 16, false, false, seg, off, rows),
              "work split");
     if ((int)off.size() - 1 != g->bctas)
       return fail(EB_ERR_STATE, "a member's work split changed outside the ensemble; tune it again");

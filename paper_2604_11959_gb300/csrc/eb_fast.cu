@@ -153,7 +153,7 @@ double split_time(const Dims &D, const std::vector<int> &kb, long long Lc, int s
 }  // namespace
 
 cudaError_t bulk_plan(const Dims &D, const int *kfast_host, bool f64, int slab_levels, int tile_rows, bool alone,
-                      std::vector<int> &seg, std::vector<int> &off, int &plan_rows) {
+                      bool rows_free, std::vector<int> &seg, std::vector<int> &off, int &plan_rows) {
   plan_rows = tile_rows;
   std::vector<int> kb = tile_bottoms(D, kfast_host, 32, tile_rows);
   long long W = 0;
@@ -189,7 +189,8 @@ cudaError_t bulk_plan(const Dims &D, const int *kfast_host, bool f64, int slab_l
     // measured for one CTA per SM: 39 + 23.7 per level for a 32 x 16 tile; 28
     // + 13.7 per level for a 16 x 8 tile (four of them per 32 x 16 tile,
     // each cheaper in time but not in FP64 instructions: more halo), which
-    // is taken only while every piece has an SM of its own.  32x32x16 ridge:
+    // is taken only while every piece has an SM of its own, and not where the
+    // caller set the rows.  32x32x16 ridge:
     // 337 us with one slab of 32 x 16 tiles, 63 with one level per piece, 42
     // with 16 x 8 tiles; 64x64x32: 407 -> 87; 256x256x128: 3084 -> 2816
     // (slabs of 35 and 16 levels).
@@ -201,7 +202,7 @@ cudaError_t bulk_plan(const Dims &D, const int *kfast_host, bool f64, int slab_l
       if (t < best) best = t, Lc = L, plan_rows = tile_rows;
       long long pieces = 0;
       for_pieces(D, ks, L, [&](int, int, int) { ++pieces; });
-      if (pieces <= sms && 28.0 + 13.7 * L < best) best = 28.0 + 13.7 * L, Lc = L, plan_rows = 8;
+      if (rows_free && pieces <= sms && 28.0 + 13.7 * L < best) best = 28.0 + 13.7 * L, Lc = L, plan_rows = 8;
     }
     if (plan_rows == 8) kb = ks;
   }

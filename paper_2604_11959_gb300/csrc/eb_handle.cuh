@@ -93,6 +93,7 @@ struct eb_geom_s {
   int plan_gen = 0;       // incremented whenever the split is rebuilt (its arrays move)
   int bulk_high = 0;      // 1: the bulk kernel runs on the high-priority stream
   int tile_rows = 16;     // rows of the bulk kernel's tiles (16, or 14 on the float path)
+  bool rows_set = false;  // tile_rows was set by the caller: an automatic split keeps it
   int plan_rows = 16;     // rows of the tiles of the split in use (tile_rows, or 8: see bulk_plan)
   bool in_ensemble = false;   // a member of an ensemble shares the GPU: its split is not fitted to an empty one
   int wsrd_side = 0;      // 1: the redistribution runs on the side stream (see stage)
