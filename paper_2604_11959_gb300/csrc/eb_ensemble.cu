@@ -39,7 +39,13 @@ struct eb_ensemble_s {
   cudaEvent_t ev_root = nullptr;
   int ctas = 0;                 // CTAs of the persistent kernel (all resident at once)
   bool vec = true;              // every member's rows suit 16-byte copies
-  // device tables of the persistent kernel, rebuilt with the graphs
+  // the members' work splits in an ensemble's step: 16-row tiles, each member's
+  // slab height, not fitted to an empty GPU; the handles keep their own.  Their
+  // arrays, and the device tables of the persistent kernel, are rebuilt with
+  // the graphs
+  std::vector<BulkSplit> split;
+  int4 *seg = nullptr;
+  int *off = nullptr;
   void *dmem[2] = {nullptr, nullptr};   // EnsMember<T>[n] per step direction
   int2 *units = nullptr;
   long long *pre = nullptr;             // 5 prefix arrays of n + 1 entries
@@ -64,8 +70,12 @@ struct eb_ensemble_s {
       if (dmem[b]) cudaFree(dmem[b]);
       dmem[b] = nullptr;
     }
+    if (seg) cudaFree(seg);
+    if (off) cudaFree(off);
     if (units) cudaFree(units);
     if (pre) cudaFree(pre);
+    seg = nullptr;
+    off = nullptr;
     units = nullptr;
     pre = nullptr;
   }
@@ -92,17 +102,53 @@ struct eb_ensemble_s {
 
 namespace {
 
-// The persistent kernel's tables for the current work split and time
-// steps: per step direction every member's step and redistribution
-// arguments, the bulk work units of all members (one per CTA group of each
-// member's own split, longest first) and the prefix sums of every phase's
-// item counts.
+// The members' work splits and the persistent kernel's tables for the current
+// slab heights and time steps: per step direction every member's step and
+// redistribution arguments, the bulk work units of all members (one per CTA
+// group of each member's split, longest first) and the prefix sums of every
+// phase's item counts.
 template <typename T>
 eb_status build_tables(eb_ensemble e, EnsembleArgs<T> E[2]) {
   e->drop_tables();
   const int n = (int)e->m.size();
   e->gens.resize(n);
   for (int q = 0; q < n; ++q) e->gens[q] = e->m[q]->plan_gen;
+  // bulk units: CTA group u of member q marches the pieces of its split
+  struct Unit {
+    int q, g;
+    long long len;
+  };
+  std::vector<Unit> us;
+  std::vector<int> aseg, aoff;   // every member's split, one after another
+  e->split.assign(n, BulkSplit());
+  std::vector<size_t> seg0(n), off0(n);
+  for (int q = 0; q < n; ++q) {
+    eb_geom g = e->m[q];
+    if ((g->D.ny + g->tile_rows - 1) / g->tile_rows != (g->D.ny + 15) / 16)
+      return fail(EB_ERR_STATE, "a member's work split changed outside the ensemble; tune it again");
+    std::vector<int> seg, off;
+    CUDA_TRY(bulk_plan(g->D, g->kfast_host.data(), g->prec == EB_F64, g->slab_levels, 16, false, false, seg, off,
+                       e->split[q].rows),
+             "work split");
+    e->split[q].ctas = (int)off.size() - 1;
+    for (int u = 0; u + 1 < (int)off.size(); ++u) {
+      long long len = 0;
+      for (int p = off[u]; p < off[u + 1]; ++p) len += seg[4 * p + 2] - seg[4 * p + 1] + 3;
+      us.push_back({q, u, len});
+    }
+    seg0[q] = aseg.size() / 4;
+    off0[q] = aoff.size();
+    aseg.insert(aseg.end(), seg.begin(), seg.end());
+    aoff.insert(aoff.end(), off.begin(), off.end());
+  }
+  CUDA_TRY(cudaMalloc(&e->seg, sizeof(int) * std::max<size_t>(4, aseg.size())), "ensemble work splits");
+  CUDA_TRY(cudaMalloc(&e->off, sizeof(int) * aoff.size()), "ensemble work splits");
+  CUDA_TRY(cudaMemcpy(e->seg, aseg.data(), sizeof(int) * aseg.size(), cudaMemcpyHostToDevice), "ensemble work splits");
+  CUDA_TRY(cudaMemcpy(e->off, aoff.data(), sizeof(int) * aoff.size(), cudaMemcpyHostToDevice), "ensemble work splits");
+  for (int q = 0; q < n; ++q) {
+    e->split[q].seg = e->seg + seg0[q];
+    e->split[q].off = e->off + off0[q];
+  }
   std::vector<EnsMember<T>> host(n);
   for (int b = 0; b < 2; ++b) {
     for (int q = 0; q < n; ++q) {
@@ -111,32 +157,12 @@ eb_status build_tables(eb_ensemble e, EnsembleArgs<T> E[2]) {
         src[f] = e->field(b, q, f);
         dst[f] = e->field(1 - b, q, f);
       }
-      host[q].A = step_args<T>(e->m[q], src, src, dst, e->dt[q], 0);
+      host[q].A = step_args<T>(e->m[q], src, src, dst, e->dt[q], 0, &e->split[q]);
       host[q].S = wsrd_set<T>(e->m[q], dst);
     }
     CUDA_TRY(cudaMalloc(&e->dmem[b], sizeof(EnsMember<T>) * n), "ensemble tables");
     CUDA_TRY(cudaMemcpy(e->dmem[b], host.data(), sizeof(EnsMember<T>) * n, cudaMemcpyHostToDevice),
              "ensemble tables");
-  }
-  // bulk units: CTA group u of member q marches the pieces of its split
-  struct Unit {
-    int q, g;
-    long long len;
-  };
-  std::vector<Unit> us;
-  for (int q = 0; q < n; ++q) {
-    eb_geom g = e->m[q];
-    std::vector<int> seg, off;
-    int rows = 16;
-    CUDA_TRY(bulk_plan(g->D, g->kfast_host.data(), g->prec == EB_F64, g->slab_levels, 16, false, false, seg, off, rows),
-             "work split");
-    if ((int)off.size() - 1 != g->bctas)
-      return fail(EB_ERR_STATE, "a member's work split changed outside the ensemble; tune it again");
-    for (int u = 0; u + 1 < (int)off.size(); ++u) {
-      long long len = 0;
-      for (int p = off[u]; p < off[u + 1]; ++p) len += seg[4 * p + 2] - seg[4 * p + 1] + 3;
-      us.push_back({q, u, len});
-    }
   }
   std::stable_sort(us.begin(), us.end(), [](const Unit &a, const Unit &b) { return a.len > b.len; });
   std::vector<int2> hu(us.size());
@@ -188,7 +214,7 @@ void member_stage(eb_ensemble e, int q, int from, cudaStream_t s) {
     src[f] = e->field(from, q, f);
     dst[f] = e->field(1 - from, q, f);
   }
-  stage<T>(e->m[q], src, src, dst, e->dt[q], 0, s, false);
+  stage<T>(e->m[q], src, src, dst, e->dt[q], 0, s, false, &e->split[q]);
 }
 
 // One step of every member, buffer `from` to 1 - from, captured as a graph
@@ -226,8 +252,8 @@ eb_status capture(eb_ensemble e, int from, cudaGraphExec_t *out) {
 }
 
 eb_status run_steps(eb_ensemble e, int nsteps, cudaStream_t s) {
-  // a member's work split rebuilt since the tables were made (eb_geom_tune,
-  // eb_geom_set_slab_levels) moves its arrays: capture again
+  // a member's slab height set since the tables were made (eb_geom_tune,
+  // eb_geom_set_slab_levels): split and capture again
   for (size_t q = 0; q < e->gens.size(); ++q)
     if (e->gens[q] != e->m[q]->plan_gen) {
       e->drop_graphs();
@@ -265,14 +291,6 @@ eb_status eb_ensemble_create(const eb_geom *members, int n, eb_ensemble *out) {
     if (members[q]->src_flags)
       return fail(EB_ERR_STATE, "ensembles take no compressible sources: a member has them switched on");
   }
-  // the persistent kernel marches tiles of 16 rows: members keep that height
-  for (int q = 0; q < n; ++q)
-    if (members[q]->tile_rows != 16 || !members[q]->in_ensemble) {
-      members[q]->tile_rows = 16;
-      members[q]->in_ensemble = true;
-      const eb_status st = eb_replan_bulk(members[q], members[q]->slab_levels);
-      if (st != EB_OK) return st;
-    }
   for (int q = 1; q < n; ++q) {
     if (members[q]->prec != members[0]->prec) return fail(EB_ERR_INVALID_ARG, "members differ in precision");
     if (members[q]->device != members[0]->device) return fail(EB_ERR_INVALID_ARG, "members are on different devices");
@@ -321,6 +339,17 @@ eb_status eb_ensemble_create(const eb_geom *members, int n, eb_ensemble *out) {
     delete e;
     return cuda_fail(err, "ensemble buffers");
   }
+  // the persistent kernel marches tiles of 16 rows: members keep that height
+  for (int q = 0; q < n; ++q)
+    if (members[q]->tile_rows != 16) {
+      members[q]->tile_rows = 16;
+      const eb_status st = eb_replan_bulk(members[q], members[q]->slab_levels);
+      if (st != EB_OK) {
+        e->release();
+        delete e;
+        return st;
+      }
+    }
   *out = e;
   return EB_OK;
 }

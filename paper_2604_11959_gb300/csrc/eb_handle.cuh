@@ -95,7 +95,6 @@ struct eb_geom_s {
   int tile_rows = 16;     // rows of the bulk kernel's tiles (16, or 14 on the float path)
   bool rows_set = false;  // tile_rows was set by the caller: an automatic split keeps it
   int plan_rows = 16;     // rows of the tiles of the split in use (tile_rows, or 8: see bulk_plan)
-  bool in_ensemble = false;   // a member of an ensemble shares the GPU: its split is not fitted to an empty one
   int wsrd_side = 0;      // 1: the redistribution runs on the side stream (see stage)
   std::vector<int> kfast_host;
   int kcov_max = 0;
@@ -196,8 +195,17 @@ inline bool state_ok(const eb_state *U, size_t align) {
 
 inline void **state_ptrs(const eb_state *U) { return (void **)&U->rho; }
 
+// A work split of the bulk kernel on the device (see bulk_plan).
+struct BulkSplit {
+  const int4 *seg = nullptr;
+  const int *off = nullptr;
+  int ctas = 0, rows = 16;
+};
+
+// split: nullptr for the handle's own
 template <typename T>
-StepArgs<T> step_args(eb_geom g, void *const src[5], void *const base[5], void *const out[5], double dt, int copy) {
+StepArgs<T> step_args(eb_geom g, void *const src[5], void *const base[5], void *const out[5], double dt, int copy,
+                      const BulkSplit *split = nullptr) {
   StepArgs<T> A;
   A.D = g->D;
   for (int f = 0; f < 5; ++f) {
@@ -225,13 +233,13 @@ StepArgs<T> step_args(eb_geom g, void *const src[5], void *const base[5], void *
   A.dt = dt;
   A.dtT = (T)dt;
   A.kfast = g->kfast;
-  A.bseg = g->bseg;
-  A.boff = g->boff;
-  A.bctas = g->bctas;
+  A.bseg = split ? split->seg : g->bseg;
+  A.boff = split ? split->off : g->boff;
+  A.bctas = split ? split->ctas : g->bctas;
   for (int q = 0; q < 4; ++q) A.G[q] = g->G[q];
   A.status = g->status;
   A.copy_static = copy;
-  A.tile_rows = g->plan_rows;
+  A.tile_rows = split ? split->rows : g->plan_rows;
   A.kcov_max = g->kcov_max;
   return A;
 }
@@ -326,8 +334,8 @@ void wsrd_all(eb_geom g, void *const out[5], cudaStream_t s) {
 // covered CVs and the w wall levels of out are written too, from base.
 template <typename T>
 void stage(eb_geom g, void *const src[5], void *const base[5], void *const out[5], double dt, int copy,
-           cudaStream_t s, bool wsrd_beside = true) {
-  StepArgs<T> A = step_args<T>(g, src, base, out, dt, copy);
+           cudaStream_t s, bool wsrd_beside = true, const BulkSplit *split = nullptr) {
+  const StepArgs<T> A = step_args<T>(g, src, base, out, dt, copy, split);
   if (g->src_flags) {   // the sources follow the whole flux update; the redistribution follows them
     flux_update(g, A, s);
     const bool f64 = sizeof(T) == sizeof(double);

@@ -107,7 +107,7 @@ void launch_stage_marks(const Dims &D, const GridDev G[4], uint8_t *const marks[
 // slabs of slab_levels levels (0: chosen from the GPU's size); seg holds
 // (tile, first level, end level, 0) per piece, off[b] .. off[b+1] the pieces
 // of CTA b
-// alone: the kernel has the GPU to itself (not a member of an ensemble); rows_free: the caller has not set tile_rows;
+// alone: the kernel has the GPU to itself (not one member of an ensemble's step); rows_free: the caller has not set tile_rows;
 // plan_rows: rows of the split's tiles, tile_rows or 8 (16 x 8 tiles: double path, automatic height, free rows, small
 // domains)
 cudaError_t bulk_plan(const Dims &D, const int *kfast_host, bool f64, int slab_levels, int tile_rows, bool alone,

@@ -49,3 +49,65 @@ def test_reported_tile_rows_are_those_in_use(eb):
         eb.set_tile_rows(m, rows)
         assert m.info()["tile_rows"] == rows
     m.close()
+
+
+def test_an_ensemble_leaves_its_members_splits_alone(eb):
+    """A handle keeps its own split (16 x 8 tiles on a small FP64 domain)
+    through a rejected ensemble, a member's life in one and its end; the
+    ensemble's steps are the handle's bit for bit."""
+    w, refs, g = small(eb, "f64")
+    _, _, other = small(eb, "mixed")
+    U = to_device(w.state("sheltered", seed=3), "f64", refs)
+    want = eb.step(g, U, w.dt(), 2)
+    for members in ([g, other], [g, g]):
+        with pytest.raises(eb.EbError):
+            eb.Ensemble(members)
+        assert g.info()["tile_rows"] == 8
+    _, _, h = small(eb, "f64")
+    for schedule in ("persistent", "branches"):
+        ens = eb.Ensemble([g, h])
+        ens.set_schedule(schedule)
+        for q in range(2):
+            ens.set_state(q, U)
+        ens.step([w.dt()] * 2, 2)
+        assert g.info()["tile_rows"] == 8
+        for q in range(2):
+            got = ens.get_state(q)
+            for f in FIELDS:
+                assert torch.equal(got[f], want[f]), (schedule, q, f)
+        ens.close()
+    assert g.info()["tile_rows"] == 8
+    got = eb.step(g, U, w.dt(), 2)
+    for f in FIELDS:
+        assert torch.equal(got[f], want[f]), f
+
+
+@pytest.mark.parametrize("precision", ["f64", "mixed"])
+def test_captured_steps_outlive_an_ensemble(eb, precision):
+    """A graph of a handle's step replays right while the handle is a member
+    of an ensemble, and after: creating one frees nothing the graph reads."""
+    w, refs, g = small(eb, precision)
+    U = to_device(w.state("sheltered", seed=3), precision, refs)
+    out = g.empty_state()
+    want = {f: t.clone() for f, t in eb.step(g, U, w.dt(), out=out).items()}
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        eb.step(g, U, w.dt(), out=out)
+
+    def replay():
+        for f in FIELDS:
+            out[f].zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        for f in FIELDS:
+            assert torch.equal(out[f], want[f]), f
+
+    replay()
+    ens = eb.Ensemble([g])
+    replay()
+    ens.set_state(0, U)
+    ens.step([w.dt()], 1)
+    replay()
+    ens.close()
+    replay()
