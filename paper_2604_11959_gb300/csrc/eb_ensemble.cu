@@ -40,15 +40,11 @@ struct eb_ensemble_s {
   int ctas = 0;                 // CTAs of the persistent kernel (all resident at once)
   bool vec = true;              // every member's rows suit 16-byte copies
   // the members' work splits in an ensemble's step: 16-row tiles, each member's
-  // slab height, not fitted to an empty GPU; the handles keep their own.  Their
-  // arrays, and the device tables of the persistent kernel, are rebuilt with
-  // the graphs
+  // slab height, not fitted to an empty GPU; the handles keep their own
   std::vector<BulkSplit> split;
-  int4 *seg = nullptr;
-  int *off = nullptr;
-  void *dmem[2] = {nullptr, nullptr};   // EnsMember<T>[n] per step direction
-  int2 *units = nullptr;
-  long long *pre = nullptr;             // 5 prefix arrays of n + 1 entries
+  // one device block with the splits' arrays and the persistent kernel's tables
+  // (one allocation and one copy), rebuilt with the graphs
+  char *tables = nullptr;
   unsigned *ctl = nullptr;              // barrier and work counters
   int *fault = nullptr;                 // failure test: CTA + 1 that skips the first barrier
   int nunits = 0;
@@ -66,18 +62,8 @@ struct eb_ensemble_s {
       }
   }
   void drop_tables() {
-    for (int b = 0; b < 2; ++b) {
-      if (dmem[b]) cudaFree(dmem[b]);
-      dmem[b] = nullptr;
-    }
-    if (seg) cudaFree(seg);
-    if (off) cudaFree(off);
-    if (units) cudaFree(units);
-    if (pre) cudaFree(pre);
-    seg = nullptr;
-    off = nullptr;
-    units = nullptr;
-    pre = nullptr;
+    if (tables) cudaFree(tables);
+    tables = nullptr;
   }
   void release() {
     drop_graphs();
@@ -141,13 +127,25 @@ eb_status build_tables(eb_ensemble e, EnsembleArgs<T> E[2]) {
     aseg.insert(aseg.end(), seg.begin(), seg.end());
     aoff.insert(aoff.end(), off.begin(), off.end());
   }
-  CUDA_TRY(cudaMalloc(&e->seg, sizeof(int) * std::max<size_t>(4, aseg.size())), "ensemble work splits");
-  CUDA_TRY(cudaMalloc(&e->off, sizeof(int) * aoff.size()), "ensemble work splits");
-  CUDA_TRY(cudaMemcpy(e->seg, aseg.data(), sizeof(int) * aseg.size(), cudaMemcpyHostToDevice), "ensemble work splits");
-  CUDA_TRY(cudaMemcpy(e->off, aoff.data(), sizeof(int) * aoff.size(), cudaMemcpyHostToDevice), "ensemble work splits");
+  // the block: members per step direction, pieces, units, prefix sums (5 arrays
+  // of n + 1), offsets
+  size_t bytes = 0;
+  auto place = [&](size_t size) {
+    const size_t at = bytes;
+    bytes += (size + 255) / 256 * 256;
+    return at;
+  };
+  const size_t at_m[2] = {place(sizeof(EnsMember<T>) * n), place(sizeof(EnsMember<T>) * n)};
+  const size_t at_seg = place(sizeof(int) * aseg.size()), at_units = place(sizeof(int2) * us.size());
+  const size_t at_pre = place(sizeof(long long) * 5 * (n + 1)), at_off = place(sizeof(int) * aoff.size());
+  CUDA_TRY(cudaMalloc(&e->tables, bytes), "ensemble tables");
+  std::vector<char> block(bytes);
+  auto put = [&](size_t at, const auto &v) { std::copy_n((const char *)v.data(), sizeof(v[0]) * v.size(), &block[at]); };
+  put(at_seg, aseg);
+  put(at_off, aoff);
   for (int q = 0; q < n; ++q) {
-    e->split[q].seg = e->seg + seg0[q];
-    e->split[q].off = e->off + off0[q];
+    e->split[q].seg = (const int4 *)(e->tables + at_seg) + seg0[q];
+    e->split[q].off = (const int *)(e->tables + at_off) + off0[q];
   }
   std::vector<EnsMember<T>> host(n);
   for (int b = 0; b < 2; ++b) {
@@ -160,17 +158,13 @@ eb_status build_tables(eb_ensemble e, EnsembleArgs<T> E[2]) {
       host[q].A = step_args<T>(e->m[q], src, src, dst, e->dt[q], 0, &e->split[q]);
       host[q].S = wsrd_set<T>(e->m[q], dst);
     }
-    CUDA_TRY(cudaMalloc(&e->dmem[b], sizeof(EnsMember<T>) * n), "ensemble tables");
-    CUDA_TRY(cudaMemcpy(e->dmem[b], host.data(), sizeof(EnsMember<T>) * n, cudaMemcpyHostToDevice),
-             "ensemble tables");
+    put(at_m[b], host);
   }
   std::stable_sort(us.begin(), us.end(), [](const Unit &a, const Unit &b) { return a.len > b.len; });
   std::vector<int2> hu(us.size());
   for (size_t u = 0; u < us.size(); ++u) hu[u] = make_int2(us[u].q, us[u].g);
   e->nunits = (int)hu.size();
-  CUDA_TRY(cudaMalloc(&e->units, sizeof(int2) * std::max<size_t>(1, hu.size())), "ensemble units");
-  if (!hu.empty())
-    CUDA_TRY(cudaMemcpy(e->units, hu.data(), sizeof(int2) * hu.size(), cudaMemcpyHostToDevice), "ensemble units");
+  put(at_units, hu);
   // prefix sums: staged CVs, faces, near-EB CVs, small CVs of the four grids, affected CVs of the five fields
   std::vector<long long> pre(5 * (n + 1), 0);
   for (int q = 0; q < n; ++q) {
@@ -183,20 +177,20 @@ eb_status build_tables(eb_ensemble e, EnsembleArgs<T> E[2]) {
     }
     for (int k = 0; k < 5; ++k) pre[k * (n + 1) + q + 1] = pre[k * (n + 1) + q] + c[k];
   }
-  CUDA_TRY(cudaMalloc(&e->pre, sizeof(long long) * pre.size()), "ensemble prefixes");
-  CUDA_TRY(cudaMemcpy(e->pre, pre.data(), sizeof(long long) * pre.size(), cudaMemcpyHostToDevice),
-           "ensemble prefixes");
+  put(at_pre, pre);
+  CUDA_TRY(cudaMemcpy(e->tables, block.data(), bytes, cudaMemcpyHostToDevice), "ensemble tables");
+  const long long *dpre = (const long long *)(e->tables + at_pre);
   for (int b = 0; b < 2; ++b) {
     EnsembleArgs<T> &A = E[b];
-    A.m = (const EnsMember<T> *)e->dmem[b];
+    A.m = (const EnsMember<T> *)(e->tables + at_m[b]);
     A.nm = n;
-    A.units = e->units;
+    A.units = (const int2 *)(e->tables + at_units);
     A.nunits = e->nunits;
-    A.pre_stage = e->pre;
-    A.pre_face = e->pre + (n + 1);
-    A.pre_band = e->pre + 2 * (n + 1);
-    A.pre_small = e->pre + 3 * (n + 1);
-    A.pre_aff = e->pre + 4 * (n + 1);
+    A.pre_stage = dpre;
+    A.pre_face = dpre + (n + 1);
+    A.pre_band = dpre + 2 * (n + 1);
+    A.pre_small = dpre + 3 * (n + 1);
+    A.pre_aff = dpre + 4 * (n + 1);
     A.ctl = e->ctl;
     A.fault = e->fault;
     A.spin_limit = 1u << 20;   // about a second of polls a microsecond apart
@@ -214,7 +208,7 @@ void member_stage(eb_ensemble e, int q, int from, cudaStream_t s) {
     src[f] = e->field(from, q, f);
     dst[f] = e->field(1 - from, q, f);
   }
-  stage<T>(e->m[q], src, src, dst, e->dt[q], 0, s, false, &e->split[q]);
+  stage<T>(e->m[q], src, src, dst, e->dt[q], 0, s, &e->split[q]);
 }
 
 // One step of every member, buffer `from` to 1 - from, captured as a graph

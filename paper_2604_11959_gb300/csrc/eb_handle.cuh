@@ -271,18 +271,18 @@ void wsrd_field(eb_geom g, int field, T *u, cudaStream_t s) {
 // stage allows it); both streams are joined to the caller's stream at the
 // end.
 template <typename T, typename Side>
-void flux_update(eb_geom g, const StepArgs<T> &A, cudaStream_t s, Side &&after_band) {
+void flux_update(eb_geom g, const StepArgs<T> &A, cudaStream_t s, bool chain, Side &&after_band) {
   cudaEventRecord(g->ev_fork, s);
   cudaStreamWaitEvent(g->side, g->ev_fork, 0);
   if (g->bulk_high) {
     cudaStreamWaitEvent(g->bulk, g->ev_fork, 0);
     launch_flux_fast(A, g->bulk);
-    launch_flux_band(A, g->side);
+    launch_flux_band(A, g->side, chain);
     after_band(g->side);
     cudaEventRecord(g->ev_join_bulk, g->bulk);
     cudaStreamWaitEvent(s, g->ev_join_bulk, 0);
   } else {
-    launch_flux_band(A, g->side);
+    launch_flux_band(A, g->side, chain);
     after_band(g->side);
     launch_flux_fast(A, s);
   }
@@ -291,8 +291,8 @@ void flux_update(eb_geom g, const StepArgs<T> &A, cudaStream_t s, Side &&after_b
 }
 
 template <typename T>
-void flux_update(eb_geom g, const StepArgs<T> &A, cudaStream_t s) {
-  flux_update(g, A, s, [](cudaStream_t) {});
+void flux_update(eb_geom g, const StepArgs<T> &A, cudaStream_t s, bool chain = true) {
+  flux_update(g, A, s, chain, [](cudaStream_t) {});
 }
 
 // Arguments of the redistribution of all five fields of the state out[].
@@ -321,20 +321,24 @@ WsrdSet<T> wsrd_set(eb_geom g, void *const out[5]) {
 
 // Redistribution of all five fields of a state in one pass of three kernels.
 template <typename T>
-void wsrd_all(eb_geom g, void *const out[5], cudaStream_t s) {
-  launch_wsrd5(wsrd_set<T>(g, out), s);
+void wsrd_all(eb_geom g, void *const out[5], cudaStream_t s, bool chain = true) {
+  launch_wsrd5(wsrd_set<T>(g, out), s, chain);
 }
 
 // One stage: flux update, then redistribution.  When every CV the
-// redistribution reads or writes is a near-EB CV (checked at set-up) and the
-// caller allows it, it follows the near-EB kernels on the side stream, beside
-// the bulk kernel; otherwise it follows the join.  (Ensembles keep it after
-// the join: their members already fill the GPU side by side, and the longer
-// branches cost more than the shorter critical path gains.)  copy: the
-// covered CVs and the w wall levels of out are written too, from base.
+// redistribution reads or writes is a near-EB CV (checked at set-up), it
+// follows the near-EB kernels on the side stream, beside the bulk kernel;
+// otherwise it follows the join.  split: set for a member of an ensemble, its
+// split there.  Members keep the redistribution after the join (they already
+// fill the GPU side by side, and the longer branches cost more than the
+// shorter critical path gains) and launch plainly (ten steps of 12 hills 6985
+// us chained, 6947 plain; the first pass, which captures them, 8260 and 8145).
+// copy: the covered CVs and the w wall levels of out are written too, from
+// base.
 template <typename T>
 void stage(eb_geom g, void *const src[5], void *const base[5], void *const out[5], double dt, int copy,
-           cudaStream_t s, bool wsrd_beside = true, const BulkSplit *split = nullptr) {
+           cudaStream_t s, const BulkSplit *split = nullptr) {
+  const bool alone = split == nullptr;
   const StepArgs<T> A = step_args<T>(g, src, base, out, dt, copy, split);
   if (g->src_flags) {   // the sources follow the whole flux update; the redistribution follows them
     flux_update(g, A, s);
@@ -342,11 +346,11 @@ void stage(eb_geom g, void *const src[5], void *const base[5], void *const out[5
     launch_sources<T>(A, g->src_flags, f64 ? (const T *)g->src_d[0] : (const T *)g->src_f[0],
                       f64 ? (const T *)g->src_d[1] : (const T *)g->src_f[1], (T *)g->src_pp, s);
     wsrd_all<T>(g, out, s);
-  } else if (g->wsrd_side && wsrd_beside) {
-    flux_update(g, A, s, [&](cudaStream_t side) { wsrd_all<T>(g, out, side); });
+  } else if (g->wsrd_side && alone) {
+    flux_update(g, A, s, true, [&](cudaStream_t side) { wsrd_all<T>(g, out, side); });
   } else {
-    flux_update(g, A, s);
-    wsrd_all<T>(g, out, s);
+    flux_update(g, A, s, alone);
+    wsrd_all<T>(g, out, s, alone);
   }
 }
 

@@ -47,13 +47,15 @@ inline int ebk_sm_count() {
 // placed on the GPU while the kernel before it on the stream still runs, and
 // waits in chain_begin for that kernel's end (and its memory) before it
 // touches anything.  The 2-4 us between dependent launches shrink to about
-// one.  A chained kernel calls chain_begin first, in every thread.
+// one.  A chained kernel calls chain_begin first, in every thread; without
+// chain it is launched plainly.
 __device__ inline void chain_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 template <typename... P, typename... A>
-inline void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args) {
+inline void launch_chained_if(bool chain, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                              A &&...args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -63,8 +65,12 @@ inline void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t s
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = chain ? 1 : 0;
   cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+template <typename... P, typename... A>
+inline void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args) {
+  launch_chained_if(true, kernel, grid, block, smem, s, args...);
 }
 
 #define EBK_COVERED 0

@@ -1111,7 +1111,7 @@ cudaError_t launch_ensemble_v(const EnsembleArgs<T> &E, int ctas, cudaStream_t s
 // host wrappers
 // ---------------------------------------------------------------------------
 template <typename T>
-void launch_flux_band(const StepArgs<T> &A, cudaStream_t s) {
+void launch_flux_band(const StepArgs<T> &A, cudaStream_t s, bool chain) {
   long long nf = 0, nb = 0, nr = 0;
   for (int g = 0; g < 4; ++g) {
     nb += A.G[g].nband_rec;
@@ -1122,7 +1122,7 @@ void launch_flux_band(const StepArgs<T> &A, cudaStream_t s) {
   for (int g = 0; g < 4; ++g) ns += A.G[g].nstage;
   if (ns) k_stage<T><<<(unsigned)((ns + 255) / 256), 256, 0, s>>>(A);
   if (nf) k_face_flux<T><<<(unsigned)((nf + 255) / 256), 256, 0, s>>>(A);
-  if (nb + nr) launch_chained(k_band<T>, (unsigned)((nb + nr + 255) / 256), 256, 0, s, A);
+  if (nb + nr) launch_chained_if(chain, k_band<T>, (unsigned)((nb + nr + 255) / 256), 256, 0, s, A);
 }
 
 template <typename T>
@@ -1142,13 +1142,13 @@ void launch_wsrd(const WsrdArgs<T> &R, cudaStream_t s) {
 }
 
 template <typename T>
-void launch_wsrd5(const WsrdSet<T> &S, cudaStream_t s) {
+void launch_wsrd5(const WsrdSet<T> &S, cudaStream_t s, bool chain) {
   const unsigned ns = (unsigned)((S.off_small[4] + 127) / 128), na = (unsigned)((S.off_aff[5] + 127) / 128);
   if (ns) {
-    launch_chained(k_qhat5<T>, ns, 128, 0, s, S);
-    launch_chained(k_sigma5<T>, (unsigned)((S.off_small[4] * SIGMA_LANES + 127) / 128), 128, 0, s, S);
+    launch_chained_if(chain, k_qhat5<T>, ns, 128, 0, s, S);
+    launch_chained_if(chain, k_sigma5<T>, (unsigned)((S.off_small[4] * SIGMA_LANES + 127) / 128), 128, 0, s, S);
   }
-  if (na) launch_chained(k_final5<T>, na, 128, 0, s, S);
+  if (na) launch_chained_if(chain, k_final5<T>, na, 128, 0, s, S);
 }
 
 void launch_band_rows(const Dims &D, const GridDev G[4], int g, bool fill, long long *cnt, cudaStream_t s) {
@@ -1191,10 +1191,10 @@ void launch_rows_to_u32(const long long *src, long long n, unsigned *dst, cudaSt
 }
 
 template void launch_flux_update<double>(const StepArgs<double> &, cudaStream_t);
-template void launch_wsrd5<double>(const WsrdSet<double> &, cudaStream_t);
-template void launch_wsrd5<float>(const WsrdSet<float> &, cudaStream_t);
-template void launch_flux_band<double>(const StepArgs<double> &, cudaStream_t);
-template void launch_flux_band<float>(const StepArgs<float> &, cudaStream_t);
+template void launch_wsrd5<double>(const WsrdSet<double> &, cudaStream_t, bool);
+template void launch_wsrd5<float>(const WsrdSet<float> &, cudaStream_t, bool);
+template void launch_flux_band<double>(const StepArgs<double> &, cudaStream_t, bool);
+template void launch_flux_band<float>(const StepArgs<float> &, cudaStream_t, bool);
 template void launch_flux_update<float>(const StepArgs<float> &, cudaStream_t);
 template void launch_wsrd<double>(const WsrdArgs<double> &, cudaStream_t);
 template void launch_wsrd<float>(const WsrdArgs<float> &, cudaStream_t);

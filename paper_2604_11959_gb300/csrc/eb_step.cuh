@@ -61,12 +61,12 @@ void launch_static_copy(const StepArgs<T> &A, cudaStream_t s);
 template <typename T>
 void launch_flux_bulk(const StepArgs<T> &A, cudaStream_t s);
 template <typename T>
-void launch_flux_band(const StepArgs<T> &A, cudaStream_t s);
+void launch_flux_band(const StepArgs<T> &A, cudaStream_t s, bool chain = true);   // chain: see launch_chained_if
 
 template <typename T>
 void launch_wsrd(const WsrdArgs<T> &R, cudaStream_t s);
 template <typename T>
-void launch_wsrd5(const WsrdSet<T> &S, cudaStream_t s);
+void launch_wsrd5(const WsrdSet<T> &S, cudaStream_t s, bool chain = true);
 // sources of the compressible system (eb_sources.cu): flags EB_SOURCE_*,
 // per-level tables p0 and 1 / (rho0 theta0), scratch pp of one cell field
 template <typename T>
