@@ -53,8 +53,10 @@ struct Vol {
 // (tcgen05.mma, BF16 operands, FP32 accumulators in tensor memory).  A CTA
 // owns 8 x 16 voxels (x, y) on TZ consecutive z-levels.  Per z-level the
 // GEMM has M = 128 rows (row m = voxel (m % 8, m / 8) of the tile), N = the
-// output channels (NP: 16 ... 96) and K = the input channels, 16 per chunk;
-// the 27 taps add 27 products into the same accumulator.  Each tap's A
+// output channels (NP: 64 or 96; the layers with fewer, and with them those
+// that read a concatenation, take k_conv3_pipe) and K = the input channels,
+// 16 per chunk; the 27 taps add 27 products into the same accumulator.  Each
+// tap's A
 // operand is read in place from the chunk's halo: the halo holds, per group
 // of 8 channels, one 16-byte row per voxel (x fastest), so the 8 voxels of a
 // core matrix are 8 consecutive rows wherever the tap puts them, the next y
@@ -92,9 +94,10 @@ struct ConvIn {
 };
 
 // Where a convolution's output goes: channels below split to a, the others
-// to b (split a multiple of 16); with head set (the last layer, 16 channels)
-// the 1x1 head of the network is applied in the epilogue as well, y = hb + sum
-// of hw[c] times channel c, and a may be NULL (inference needs no more).
+// to b (split a multiple of 16); with y set (the last layer, 16 channels)
+// the 1x1 head of the network is applied in the epilogue of k_conv3_pipe as
+// well, y = hb + sum of hw[c] times channel c, and a may be NULL (inference
+// needs no more).
 struct ConvOut {
   float *a, *b;
   int split;
@@ -116,7 +119,7 @@ __device__ __forceinline__ void split_pair(float a, float b, uint32_t &hi, uint3
 }
 
 template <int NP, int TZ, bool MASK>
-__global__ void __launch_bounds__(256, 2) k_conv3_umma(ConvIn in, int cin, const __nv_bfloat16 *Wp,
+__global__ void __launch_bounds__(256, 2) k_conv3_umma(const float *in, int cin, const __nv_bfloat16 *Wp,
                                                        const float *bias, ConvOut out, int cout, Vol V, int relu,
                                                        const float *mask, int *err, int skip_commit) {
   using G = ConvTile<NP, TZ>;
@@ -147,10 +150,7 @@ __global__ void __launch_bounds__(256, 2) k_conv3_umma(ConvIn in, int cin, const
   auto load_step = [&](int i) {
     const int tile = tile_of(i), c0 = (i % nch) * 16;
     const int x0 = (tile % ntx) * 8, y0 = ((tile / ntx) % nty) * 16, z0 = (tile / (ntx * nty)) * TZ;
-    const bool up = c0 < in.cup;
-    const float *base = up ? in.a + (long long)c0 * (N / 8)
-                           : (in.cup ? in.b + (long long)(c0 - in.cup) * N : in.a + (long long)c0 * N);
-    const long long cs = up ? N / 8 : N;   // channel stride
+    const float *base = in + (long long)c0 * N;
 #pragma unroll
     for (int k = 0; k < IS; ++k) {
       const int q = tid + 256 * k;
@@ -158,12 +158,11 @@ __global__ void __launch_bounds__(256, 2) k_conv3_umma(ConvIn in, int cin, const
       const int hx = h % G::HX, hy = (h / G::HX) % G::HY, hz = h / (G::HX * G::HY);
       const int x = x0 + hx - 1, y = y0 + hy - 1, z = z0 + hz - 1;
       const bool inside = q < ITEMS && x >= 0 && x < V.nx && y >= 0 && y < V.ny && z >= 0 && z < V.nz;
-      const float *src = base + (up ? ((long long)(z >> 1) * (V.ny / 2) + (y >> 1)) * (V.nx / 2) + (x >> 1)
-                                    : ((long long)z * V.ny + y) * V.nx + x);
+      const float *src = base + ((long long)z * V.ny + y) * V.nx + x;
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const int c = kg * 8 + j;
-        pv[k][j] = inside && c0 + c < cin ? src[c * cs] : 0.f;
+        pv[k][j] = inside && c0 + c < cin ? src[c * N] : 0.f;
       }
     }
   };
@@ -204,7 +203,6 @@ __global__ void __launch_bounds__(256, 2) k_conv3_umma(ConvIn in, int cin, const
         umma::ld16(tm + ((uint32_t)(32 * quad) << 16) + (uint32_t)(rz * NP + cc), v);
         if (live) {
           float *dst = cc < out.split ? out.a + (long long)cc * N : out.b + (long long)(cc - out.split) * N;
-          float y = out.y ? out.hb[0] : 0.f;
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
             const int co = cc + j;
@@ -212,11 +210,9 @@ __global__ void __launch_bounds__(256, 2) k_conv3_umma(ConvIn in, int cin, const
               float o = v[j] + (bias ? bias[co] : 0.f);
               if (relu) o = fmaxf(o, 0.f);
               if (MASK && !(mk[j] > 0.f)) o = 0.f;   // ReLU backward of the input
-              if (out.y) y = fmaf(__bfloat162float(out.hw[co]), o, y);
-              if (out.a) dst[(long long)j * N + vox] = o;
+              dst[(long long)j * N + vox] = o;
             }
           }
-          if (out.y) out.y[vox] = y;
         }
       }
     }
@@ -964,7 +960,7 @@ namespace {
 long long packed_size(int cin, int cout) { return (long long)((cin + 15) / 16) * 27 * 2 * ((cout + 15) / 16 * 16) * 8; }
 
 template <int NP, int TZ, bool MASK>
-void conv3_umma_launch(const ConvIn &in, int cin, const __nv_bfloat16 *Wp, const float *bias, const ConvOut &out,
+void conv3_umma_launch(const float *in, int cin, const __nv_bfloat16 *Wp, const float *bias, const ConvOut &out,
                        int cout, const Vol &V, bool relu, const float *mask, int *err, int skip_commit, cudaStream_t s) {
   using G = ConvTile<NP, TZ>;
   static unsigned long long attr = 0;
@@ -1014,15 +1010,15 @@ void conv3_tc(eb_unet u, const ConvIn &in, int cin, const __nv_bfloat16 *Wp, con
     switch (NP) {
       case 16: conv3_pipe<16, true>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
       case 32: conv3_pipe<32, true>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
-      default: conv3_umma_launch<64, 2, true>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
+      default: conv3_umma_launch<64, 2, true>(in.a, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
     }
   } else {
     switch (NP) {
       case 16: conv3_pipe<16, false>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
       case 32: conv3_pipe<32, false>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
       case 48: conv3_pipe<48, false>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
-      case 64: conv3_umma_launch<64, 2, false>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
-      default: conv3_umma_launch<96, 2, false>(in, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
+      case 64: conv3_umma_launch<64, 2, false>(in.a, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
+      default: conv3_umma_launch<96, 2, false>(in.a, cin, Wp, bias, out, cout, V, relu, mask, u->err, skip, s); break;
     }
   }
 }
