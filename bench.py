@@ -179,15 +179,23 @@ def max_over_ranks(value, dist):
     return float(t.item())
 
 
+# Bytes per cell and iteration that the projection's kernels read and write
+# (each array once, above the terrain, where no coefficient is read).  Conjugate
+# gradients in FP64: operator p, q; update r, q, r and, with multigrid, r again in
+# float, with Jacobi 1 / diagonal; direction x, p, z, x, p and, with Jacobi,
+# 1 / diagonal.  V-cycle in FP32, finest level: first two sweeps b, t; sweep t, b,
+# x; residual and restriction x, b and 1/8 of a value; prolongation and sweep x,
+# 1/8, b, t; sweep t, b, x; last sweep x, b, and r and z in FP64.  A coarser level
+# has one double sweep, restriction, prolongation and sweep (41 bytes a cell, and
+# the levels together 1/7 of the finest's cells).
+PROJECTION_BYTES = {"mg": 16 + 28 + 40 + (8 + 12 + 8.5 + 12.5 + 12 + 24) + 41 / 7, "jacobi": 16 + 32 + 48}
+
+
 def run_anelastic(eb, steps, warmup, clk=None, dist=None):
     """Anelastic steps (Algorithm 2, two stages, projection to a relative
     residual of 1e-10 from a zero guess, multigrid-preconditioned) on the
     192x192x96 random terrain, mixed path; and one projection timed alone
-    with each preconditioner.  Algorithmic traffic per PCG iteration: 136
-    bytes per cell for the FP64 conjugate-gradient vectors (operator 48,
-    update 64, direction 24), plus 231 for the FP32 V-cycle (212 on the
-    finest level: six sweeps of about 28 bytes each, restriction and
-    prolongation; 19 more on the coarse levels)."""
+    with each preconditioner.  Its traffic: PROJECTION_BYTES."""
     import torch
     from paper_2604_11959_gb300 import inputs
     w = inputs.GRF_192
@@ -215,7 +223,7 @@ def run_anelastic(eb, steps, warmup, clk=None, dist=None):
     cells = w.cells()
     hbm, kind = peaks()
     proj = {}
-    for pc, bpc in (("mg", 136 + 231), ("jacobi", 136)):
+    for pc, bpc in PROJECTION_BYTES.items():
         eb.set_preconditioner(g, pc)
         eb.project(g, {f: U[f].clone() for f in U}, dt, rtol=1e-10)   # work space, warm-up
         W = {f: U[f].clone() for f in U}
