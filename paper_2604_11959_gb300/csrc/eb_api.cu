@@ -22,8 +22,10 @@ std::string &eb_error_slot() { return g_last_error; }
 eb_status eb_replan_bulk(eb_geom g, int slab_levels) {
   std::vector<int> seg, off;
   int rows = g->tile_rows;
+  long long near_cvs = 0;
+  for (int q = 0; q < 4; ++q) near_cvs += g->G[q].nband;
   CUDA_TRY(bulk_plan(g->D, g->kfast_host.data(), g->prec == EB_F64, slab_levels, g->tile_rows, true, !g->rows_set,
-                     seg, off, rows),
+                     near_cvs, seg, off, rows),
            "bulk work split");
   // the split arrays are small: the old ones are released right away
   for (void *p : {(void *)g->bseg, (void *)g->boff}) {

@@ -113,7 +113,7 @@ eb_status build_tables(eb_ensemble e, EnsembleArgs<T> E[2]) {
     if ((g->D.ny + g->tile_rows - 1) / g->tile_rows != (g->D.ny + 15) / 16)
       return fail(EB_ERR_STATE, "a member's work split changed outside the ensemble; tune it again");
     std::vector<int> seg, off;
-    CUDA_TRY(bulk_plan(g->D, g->kfast_host.data(), g->prec == EB_F64, g->slab_levels, 16, false, false, seg, off,
+    CUDA_TRY(bulk_plan(g->D, g->kfast_host.data(), g->prec == EB_F64, g->slab_levels, 16, false, false, 0, seg, off,
                        e->split[q].rows),
              "work split");
     e->split[q].ctas = (int)off.size() - 1;

@@ -3,8 +3,11 @@
 // launchers.
 #include "eb_bulk.cuh"
 
+#include <math.h>
+
 #include <algorithm>
 #include <functional>
+#include <queue>
 #include <vector>
 
 namespace {
@@ -150,10 +153,52 @@ double split_time(const Dims &D, const std::vector<int> &kb, long long Lc, int s
   return end;
 }
 
+// The float path's march with `per_sm` CTAs per SM, in units of the time a CTA
+// alone on its SM takes per level: a piece costs its levels and three of
+// prologue, and of n CTAs on an SM each runs 1 + 0.1 (n - 1) times slower.
+// end: when the last piece is done, the pieces starting in order; busy: the
+// SMs' time in it, per SM.
+struct MarchTime {
+  double end = 0.0, busy = 0.0;
+  long long pieces = 0;
+};
+MarchTime march_time(const Dims &D, const std::vector<int> &kb, long long Lc, int sms, int per_sm) {
+  auto slow = [](size_t n) { return 1.0 + 0.1 * ((double)n - 1.0); };
+  std::vector<double> cost;
+  for_pieces(D, kb, Lc, [&](int, int a, int b) { cost.push_back(3.0 + (b - a)); });
+  MarchTime M;
+  M.pieces = (long long)cost.size();
+  for (double c : cost) M.busy += c * slow((size_t)per_sm) / per_sm / sms;
+  std::vector<std::vector<double>> left(sms);   // of the CTAs on each SM, at time at[]
+  std::vector<double> at(sms, 0.0);
+  size_t next = 0;
+  for (int q = 0; q < per_sm; ++q)
+    for (int i = 0; i < sms && next < cost.size(); ++i) left[i].push_back(cost[next++]);
+  using Event = std::pair<double, int>;   // an SM's next finish
+  std::priority_queue<Event, std::vector<Event>, std::greater<Event>> events;
+  auto push = [&](int i) {
+    if (!left[i].empty())
+      events.push({at[i] + *std::min_element(left[i].begin(), left[i].end()) * slow(left[i].size()), i});
+  };
+  for (int i = 0; i < sms; ++i) push(i);
+  while (!events.empty()) {
+    const auto [t, i] = events.top();
+    events.pop();
+    std::vector<double> &L = left[i];
+    const double done = (t - at[i]) / slow(L.size());
+    at[i] = M.end = t;
+    for (double &c : L) c -= done;
+    L.erase(std::remove_if(L.begin(), L.end(), [](double c) { return c < 1e-9; }), L.end());
+    while ((int)L.size() < per_sm && next < cost.size()) L.push_back(cost[next++]);
+    push(i);
+  }
+  return M;
+}
+
 }  // namespace
 
 cudaError_t bulk_plan(const Dims &D, const int *kfast_host, bool f64, int slab_levels, int tile_rows, bool alone,
-                      bool rows_free, std::vector<int> &seg, std::vector<int> &off, int &plan_rows) {
+                      bool rows_free, long long near_cvs, std::vector<int> &seg, std::vector<int> &off, int &plan_rows) {
   plan_rows = tile_rows;
   std::vector<int> kb = tile_bottoms(D, kfast_host, 32, tile_rows);
   long long W = 0;
@@ -172,16 +217,38 @@ cudaError_t bulk_plan(const Dims &D, const int *kfast_host, bool f64, int slab_l
   // about three waves of CTAs.
   long long Lc = slab_levels > 0 ? (long long)slab_levels : std::max(16LL, (W + 3 * slots - 1) / (3 * slots));
   if (slab_levels == 0 && !f64 && alone) {
-    // Float path alone on the GPU: the near-EB kernels run beside the march
-    // and are as much of the step, so fewer, taller pieces (less prologue
-    // work in their way) win over full waves: about 1.5 CTAs per SM, one
-    // wave, of at least 16 levels; 8 where even those leave SMs idle and the
-    // longest piece counts.  Whole steps, slabs of three waves and this rule:
-    // 256x256x128 hill 248 and 228 us, 256x256x64 random terrain 348 and
-    // 328, 200x100x40 107 and 105, 64x64x64 49 and 43, 32x32x16 41 and 39.
-    const long long tiles = (long long)kb.size();
-    const long long nslab = std::max(1LL, std::min<long long>(D.nz / 16, (3LL * sms / 2 + tiles / 2) / tiles));
-    Lc = tiles * nslab < sms ? 8 : (D.nz + nslab - 1) / nslab;
+    // Float path alone on the GPU: the near-EB kernels run beside the march,
+    // so a step ends no sooner than the march by itself (short slabs fill
+    // every SM to the end) and than both kinds of work together take the whole
+    // GPU (tall slabs have fewer prologues).  The height, of at least eight
+    // levels, with the smallest eighth-power mean of the two.  The near-EB and
+    // redistribution kernels take 0.025 levels' time per 1000 near-EB CVs, a fifth
+    // more where the march has pieces waiting for SMs until late in the step.
+    // The constants are the best over 102 domains of 15 thousand to 34 million cells,
+    // hills and random terrain, one and three stages: steps take 0.66 to 1.16 times
+    // those of slabs of three waves, 0.90 in the mean, and 1.7 % more than with the
+    // best height of each.  (A rule of about 1.5 whole CTAs per SM in one wave, or
+    // eight levels where that left SMs idle, was 4.7 % above the best in the mean,
+    // up to 1.39 times slabs of three waves: 750 us instead of 570 on a 400x400x128
+    // hill, 127 instead of 110 on 320x200x30.)
+    constexpr int per_sm = 2;   // by registers and shared memory (the occupancy query counts tensor memory and says 1)
+    const double near = 2.5e-5 * (double)near_cvs / sms * 152;   // in levels, on this GPU's SMs
+    double best = 0.0;
+    long long last = 0;
+    auto consider = [&](long long L) {
+      const MarchTime M = march_time(D, kb, L, sms, per_sm);
+      const double both = M.busy + near * (M.pieces > (long long)per_sm * sms ? 1.2 : 1.0);
+      const double c = pow(M.end, 8) + pow(both, 8);
+      if (last == 0 || c < best) best = c, Lc = L;
+      last = L;
+    };
+    // heights of 1, 2, ... slabs, at least 15 % apart, and of 16 and 8 levels;
+    // splits of more than 16 waves are only taken whole
+    const long long tiles = (long long)kb.size(), most = 16LL * per_sm * sms;
+    for (long long n = 1; n == 1 || (D.nz / n >= 8 && tiles * n <= most); n = std::max(n + 1, n * 115 / 100))
+      consider((D.nz + n - 1) / n);
+    for (long long L : {16, 8})
+      if (L < D.nz && tiles * ((D.nz + L - 1) / L) <= most) consider(L);
   }
   if (slab_levels == 0 && f64 && alone) {
     // Double path alone on the GPU: the height (and for small domains the

@@ -108,10 +108,10 @@ void launch_stage_marks(const Dims &D, const GridDev G[4], uint8_t *const marks[
 // (tile, first level, end level, 0) per piece, off[b] .. off[b+1] the pieces
 // of CTA b
 // alone: the kernel has the GPU to itself (not one member of an ensemble's step); rows_free: the caller has not set tile_rows;
-// plan_rows: rows of the split's tiles, tile_rows or 8 (16 x 8 tiles: double path, automatic height, free rows, small
-// domains)
+// near_cvs: near-EB CVs of the four grids (the kernels beside the march); plan_rows: rows of the split's tiles, tile_rows
+// or 8 (16 x 8 tiles: double path, automatic height, free rows, small domains)
 cudaError_t bulk_plan(const Dims &D, const int *kfast_host, bool f64, int slab_levels, int tile_rows, bool alone,
-                      bool rows_free, std::vector<int> &seg, std::vector<int> &off, int &plan_rows);
+                      bool rows_free, long long near_cvs, std::vector<int> &seg, std::vector<int> &off, int &plan_rows);
 
 // eb_scan.cu: in-place exclusive scan of n values; total written to *total (device)
 void scan_exclusive(long long *data, long long n, long long *total, cudaStream_t s);

@@ -111,3 +111,36 @@ def test_captured_steps_outlive_an_ensemble(eb, precision):
     replay()
     ens.close()
     replay()
+
+
+@pytest.mark.parametrize("n", [(400, 400, 128), (320, 200, 30)])
+def test_the_automatic_split_is_no_slow_one(eb, n):
+    """An untuned mixed step of a hill takes no longer than the best of a few
+    explicit slab heights but for 15 %: about the spread of the heights near the
+    best one, and half of what a split whose last wave is nearly empty, or whose
+    pieces are mostly prologue, loses."""
+    w = inputs.Workload("split", *n, 1, terrain="gaussian", hmax=0.12)
+    refs = w.references("sheltered")
+    g = make_geometry(eb, w, w.heights(), "mixed", refs)
+    U = to_device(w.state("sheltered", seed=3), "mixed", refs)
+    out = g.empty_state()
+
+    def time():
+        best = float("inf")
+        for _ in range(12):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            eb.step(g, U, w.dt(), out=out)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        return best
+
+    time()
+    auto = time()
+    explicit = {}
+    for levels in (16, 32, 43, 64):
+        eb.set_slab_levels(g, levels)
+        explicit[levels] = time()
+    assert auto <= 1.15 * min(explicit.values()), (auto, explicit)
+    g.close()
