@@ -97,6 +97,34 @@ __device__ inline void grid_sum(double v, const Sum &S) {
   }
 }
 
+// The same for two sums of one kernel, with one count of its blocks (A's).
+__device__ inline void grid_sum2(double v, const Sum &A, double u, const Sum &B) {
+  __shared__ bool last;
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  const double a = block_sum(v), b = block_sum(u);
+  if (tid == 0) {
+    A.part[blockIdx.x] = a;
+    B.part[blockIdx.x] = b;
+    __threadfence();
+    last = atomicAdd(A.done, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double s = 0.0, t = 0.0;
+  for (unsigned q = tid; q < gridDim.x; q += PB) {
+    s += __ldcg(A.part + q);
+    t += __ldcg(B.part + q);
+  }
+  s = block_sum(s);
+  t = block_sum(t);
+  if (tid == 0) {
+    *A.total = s;
+    *B.total = t;
+    *A.done = 0;
+  }
+}
+
 // a float as a double, by integer instructions (FP64 conversions run at the
 // FP64 rate); subnormals, infinities and NaN take the conversion
 __device__ inline double widen(float f) {
@@ -241,6 +269,43 @@ __device__ inline Cols cols_of(const Dims &D, const Slabs &S) {
   return q;
 }
 
+// The operator's split: the column groups of a plane one after another, 256 to
+// a block (no lane idles at ragged rows: 16 x 16 tiles left a third of them
+// idle at 130x50), nbx blocks to a plane.  Its FP64 work is what an SM takes time
+// for, so the fullest SM decides: its blocks times their levels, and most of a
+// level more per block (the planes below and above, the sum); fewer than two
+// blocks per SM do not hide their own latency.
+inline Slabs apply_slabs(const Dims &D, int V, int sms) {
+  Slabs S;
+  S.nbx = (int)((D.nxy / V + PB - 1) / PB);
+  S.nby = S.nz = 1;
+  double best = 0.0;
+  for (int n = 1; n <= D.nz && (n == 1 || (long long)S.nbx * n <= 8LL * sms); ++n) {
+    const double c = (double)((S.nbx * (long long)n + sms - 1) / sms) * ((D.nz + n - 1) / n + 0.7);
+    const bool few = S.nbx * (long long)(n - 1) < 2LL * sms;
+    if (few || c <= 1.02 * best) S.nz = n;   // (more blocks where that costs next to nothing)
+    best = few ? c : std::min(best, c);
+  }
+  return S;
+}
+template <int V>
+__device__ inline Cols cols_flat(const Dims &D, const Slabs &S) {
+  Cols q;
+  const int sl = blockIdx.x / S.nbx, t = (blockIdx.x - sl * S.nbx) * PB + (int)threadIdx.x, g = D.nx / V;
+  q.in = t < g * D.ny;
+  q.j = q.in ? t / g : 0;
+  q.i = q.in ? V * (t - q.j * g) : 0;
+  const int row = D.nx * q.j;
+  q.c = q.i + row;
+  q.ym = q.i + (q.j == 0 ? D.nx * (D.ny - 1) : row - D.nx);
+  q.yp = q.i + (q.j == D.ny - 1 ? 0 : row + D.nx);
+  q.xl = row + (q.i == 0 ? D.nx - 1 : q.i - 1);
+  q.xr = row + (q.i + V == D.nx ? 0 : q.i + V);
+  q.k0 = (int)((long long)D.nz * sl / S.nz);
+  q.k1 = (int)((long long)D.nz * (sl + 1) / S.nz);
+  return q;
+}
+
 // rhs = D(m) / dt on the active cells; cx, cy, cz = 1 / (delta dt)
 template <typename T>
 __global__ void __launch_bounds__(PB) k_rhs(const __grid_constant__ Op O, const __grid_constant__ Slabs SL,
@@ -331,7 +396,7 @@ __global__ void __launch_bounds__(PB) k_apply(const __grid_constant__ Op O, cons
   chain_begin();
   if (finished(conv, it)) return;
   const Dims &D = O.D;
-  const Cols q = cols_of<V>(D, SL);
+  const Cols q = cols_flat<V>(D, SL);
   const double dreg = 2.0 * (O.ix2 + O.iy2 + O.iz2);
   double pq = 0.0;
   auto ld = [&](const double *s, double (&v)[V]) {
@@ -429,8 +494,8 @@ __global__ void __launch_bounds__(PB) k_update(const __grid_constant__ Op O, con
     r[N2] = v;
     if (!JAC) rf[N2] = (float)v;
   }
-  if (JAC) grid_sum(az, srz);
-  grid_sum(rr, srr);
+  if (JAC) grid_sum2(az, srz, rr, srr);
+  else grid_sum(rr, srr);
 }
 
 // x += alpha p; then, unless r.r meets the threshold (conv is set), p = z +
@@ -1022,7 +1087,8 @@ eb_status setup(eb_geom g, cudaStream_t s) {
   for (double **a : {&w.bx, &w.by, &w.bz, &w.ax, &w.ay, &w.az, &w.d, &w.id, &w.rhs, &w.r, &w.z, &w.p, &w.q, &w.x})
     CUDA_TRY(g->alloc(a, N), "alloc projection work space");
   w.ncols = D.nx % 2 == 0 ? 2 : 1;
-  w.npart = std::max({w.nb, slabs_of(D, 1, sms).blocks(), slabs_of(D, 2, sms).blocks(), slabs_of(D, 4, sms).blocks()});
+  w.npart = std::max({w.nb, slabs_of(D, 1, sms).blocks(), slabs_of(D, 2, sms).blocks(), slabs_of(D, 4, sms).blocks(),
+                      apply_slabs(D, w.ncols, sms).blocks()});
   CUDA_TRY(g->alloc(&w.part, (long long)S_SLOTS * w.npart), "alloc projection work space");
   CUDA_TRY(g->alloc(&w.scal, S_SLOTS), "alloc projection work space");
   CUDA_TRY(g->alloc(&w.done, S_SLOTS), "alloc projection work space");
@@ -1218,12 +1284,11 @@ void launch_correct(eb_geom g, void *const mom[3], double dt, cudaStream_t s) {
                                                        (T *)mom[0], (T *)mom[1], (T *)mom[2]);
 }
 
-void launch_apply(eb_geom g, const double *p, double *q, int it, cudaStream_t s) {
+void launch_apply(eb_geom g, const double *p, double *q, int it, bool chain, cudaStream_t s) {
   ProjWork &w = g->pw;
-  const Slabs S = slabs_of(g->D, w.ncols, ebk_sm_count());
-  const dim3 blk(MBX, MBY, 1);
-  if (w.ncols == 2) launch_chained(k_apply<2>, S.blocks(), blk, 0, s, make_op(g), S, p, q, sum_of(g, S_PQ), w.conv, it);
-  else launch_chained(k_apply<1>, S.blocks(), blk, 0, s, make_op(g), S, p, q, sum_of(g, S_PQ), w.conv, it);
+  const Slabs S = apply_slabs(g->D, w.ncols, ebk_sm_count());
+  if (w.ncols == 2) launch_chained_if(chain, k_apply<2>, S.blocks(), PB, 0, s, make_op(g), S, p, q, sum_of(g, S_PQ), w.conv, it);
+  else launch_chained_if(chain, k_apply<1>, S.blocks(), PB, 0, s, make_op(g), S, p, q, sum_of(g, S_PQ), w.conv, it);
 }
 
 }  // namespace
@@ -1277,19 +1342,26 @@ eb_status eb_project_impl(eb_geom g, void *const mom[3], double dt, double rtol,
   double rr = rr0;
   if (bb > 0.0 && rr0 > thr2) {
     int done = 0, next = mg ? 4 : 32;
+    const int nb = (int)std::max(1LL, std::min<long long>(w.nb, (N / 2 + PB - 1) / PB));   // two cells per thread
+    // Kernels of up to two blocks per SM are launched as a chain (launch_chained):
+    // 0.79 of the plain time per Jacobi iteration at 24x24x12, 0.90 at 64x64x32.
+    // Beside kernels that fill the GPU the waiting blocks cost more than the
+    // launches (1.08 at 130x50x26, 1.14 at 192x192x96), but not beside the many
+    // short kernels of a V-cycle.
+    const bool chain = mg || nb <= 2 * ebk_sm_count();
     for (it = 0; it < maxit; ++it) {
       const int rz = it % 2 ? S_RZ1 : S_RZ0, rz_next = it % 2 ? S_RZ0 : S_RZ1;
-      launch_apply(g, w.p, w.q, it, s);
+      launch_apply(g, w.p, w.q, it, chain, s);
       if (mg) {
-        launch_chained(k_update<false>, w.nb, PB, 0, s, O, w.q, w.r, rf, w.scal + rz, w.scal + S_PQ, sum_of(g, rz_next),
+        launch_chained(k_update<false>, nb, PB, 0, s, O, w.q, w.r, rf, w.scal + rz, w.scal + S_PQ, sum_of(g, rz_next),
                                             sum_of(g, S_RR), w.conv, it);
         vcycle(g, w.r, w.z, rz_next, s);
-        launch_chained(k_direction<false>, w.nb, PB, 0, s, O, w.x, w.p, w.z, w.scal + rz, w.scal + rz_next, w.scal + S_PQ,
+        launch_chained(k_direction<false>, nb, PB, 0, s, O, w.x, w.p, w.z, w.scal + rz, w.scal + rz_next, w.scal + S_PQ,
                                                w.scal + S_RR, thr2, it, w.conv);
       } else {
-        launch_chained(k_update<true>, w.nb, PB, 0, s, O, w.q, w.r, nullptr, w.scal + rz, w.scal + S_PQ, sum_of(g, rz_next),
+        launch_chained_if(chain, k_update<true>, nb, PB, 0, s, O, w.q, w.r, nullptr, w.scal + rz, w.scal + S_PQ, sum_of(g, rz_next),
                                            sum_of(g, S_RR), w.conv, it);
-        launch_chained(k_direction<true>, w.nb, PB, 0, s, O, w.x, w.p, w.r, w.scal + rz, w.scal + rz_next, w.scal + S_PQ,
+        launch_chained_if(chain, k_direction<true>, nb, PB, 0, s, O, w.x, w.p, w.r, w.scal + rz, w.scal + rz_next, w.scal + S_PQ,
                                               w.scal + S_RR, thr2, it, w.conv);
       }
       // The host reads the convergence flag after a first few iterations
