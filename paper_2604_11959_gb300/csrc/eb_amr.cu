@@ -233,9 +233,13 @@ struct LevelConst {
   double d;
   float hi, lo;
 };
-__device__ inline LevelConst level_const(double d) {
-  const float hi = (float)d;
-  return LevelConst{d, hi, (float)(d - (double)hi)};
+template <typename T>
+__device__ inline void level_const(double d, LevelConst &c) {
+  c.d = d;
+  if constexpr (sizeof(T) == sizeof(float)) {
+    c.hi = (float)d;
+    c.lo = (float)(d - (double)c.hi);
+  }
 }
 
 // the mean of N values (a power of two) plus a level constant, in double
@@ -257,25 +261,51 @@ __device__ inline double mean_double(const T (&v)[N], const LevelConst &c) {
 // value could be subnormal, sure becomes false, and the caller forms its
 // values by mean_double: all of a thread's after one test, so that their loads
 // stay together.
+// the sum of N floats as s + rest, up to bound; pairs first: a short chain
+struct PairSum {
+  float s, rest, bound;
+};
 template <int N>
+__device__ inline PairSum pair_sum(const float *v) {
+  if constexpr (N == 1) {
+    return PairSum{v[0], 0.f, 0.f};
+  } else {
+    const PairSum a = pair_sum<N / 2>(v), b = pair_sum<N / 2>(v + N / 2);
+    PairSum o{0.f, 0.f, 0.f};
+    if constexpr (N == 2) {
+      two_sum(a.s, b.s, o.s, o.rest);
+    } else {
+      float e, f, r1, r2;
+      two_sum(a.s, b.s, o.s, e);
+      two_sum(a.rest, b.rest, f, r1);
+      two_sum(f, e, o.rest, r2);
+      o.bound = __fadd_ru(__fadd_ru(a.bound, b.bound), __fadd_ru(fabsf(r1), fabsf(r2)));
+    }
+    return o;
+  }
+}
+template <bool CONST, int N>
 __device__ inline double mean_plus(const double (&v)[N], const LevelConst &c, bool &) {
   return mean_double(v, c);
 }
-template <int N>
+template <bool CONST, int N>   // CONST false: c is zero
 __device__ inline float mean_plus(const float (&v)[N], const LevelConst &c, bool &sure) {
-  float s = v[0], rest = 0.f, bound = 0.f, t, e, r;
-#pragma unroll
-  for (int q = 1; q < N; ++q) {
-    two_sum(s, v[q], s, e);
-    two_sum(rest, e, rest, r);
+  if (!CONST && N == 1) return v[0];
+  const PairSum p = pair_sum<N>(v);
+  float t = p.s, rest = p.rest, bound = p.bound;
+  if constexpr (CONST) {   // (products with N are exact)
+    float e, r;
+    two_sum(t, N * c.hi, t, e);
+    if constexpr (N > 1) {
+      two_sum(rest, e, rest, r);
+      bound = __fadd_ru(bound, fabsf(r));
+    } else {
+      rest = e;
+    }
+    two_sum(rest, N * c.lo, rest, r);
     bound = __fadd_ru(bound, fabsf(r));
+    bound = __fmaf_ru(fabsf(N * c.hi), 0x1p-47f, bound);
   }
-  two_sum(s, N * c.hi, t, e);   // (products with N are exact)
-  two_sum(rest, e, rest, r);
-  bound = __fadd_ru(bound, fabsf(r));
-  two_sum(rest, N * c.lo, rest, r);
-  bound = __fadd_ru(bound, fabsf(r));
-  bound = __fmaf_ru(fabsf(N * c.hi), 0x1p-47f, bound);
   const float a = __fadd_rn(t, __fsub_rd(rest, bound)), b = __fadd_rn(t, __fadd_ru(rest, bound));
   sure = sure && a == b && (fabsf(a) >= 0x1p-100f || a == 0.f);
   return a * (1.f / N);
@@ -348,7 +378,7 @@ __global__ void __launch_bounds__(256) k_restrict(const __grid_constant__ Restri
       double d = 0.0;
       if (R.pf[f]) d += 0.5 * (R.pf[f][2 * K] + R.pf[f][2 * K + 1]);
       if (R.pc[f]) d -= R.pc[f][K];
-      lc[f] = level_const(d);
+      level_const<T>(d, lc[f]);
     }
     __syncthreads();
     if (t >= n) continue;
@@ -371,8 +401,8 @@ __global__ void __launch_bounds__(256) k_restrict(const __grid_constant__ Restri
     const T vv[4] = {v[b0 + c00], v[b0 + c10], v[b1 + c00], v[b1 + c10]};
     const T vw[4] = {w[b0 + c00], w[b0 + c10], w[b0 + c01], w[b0 + c11]};
     bool sure = true;
-    T o[5] = {mean_plus(vr, lc[0], sure), mean_plus(vh, lc[1], sure), mean_plus(vu, lc[2], sure),
-              mean_plus(vv, lc[3], sure), mean_plus(vw, none, sure)};
+    T o[5] = {mean_plus<true>(vr, lc[0], sure), mean_plus<true>(vh, lc[1], sure), mean_plus<true>(vu, lc[2], sure),
+              mean_plus<true>(vv, lc[3], sure), mean_plus<false>(vw, none, sure)};
     if (!sure) {
       o[0] = (T)mean_double(vr, lc[0]);
       o[1] = (T)mean_double(vh, lc[1]);
@@ -424,37 +454,43 @@ __global__ void __launch_bounds__(256) k_prolong(const __grid_constant__ Prolong
       double d = 0.0;
       if (P.pc[f]) d += P.pc[f][K];
       if (P.pf[f]) d -= P.pf[f][k];
-      lc[f] = level_const(d);
+      level_const<T>(d, lc[f]);
     }
     __syncthreads();
     if (t >= cols * (unsigned)Df.ny) continue;
     const long long c = I + (long long)Dc.nx * J + Dc.nxy * K;
     const long long q = i + (long long)Df.nx * j + Df.nxy * k;
-    // one coarse value (twice the same), or the two coarse faces around an odd fine face
-    const bool cell = k < Df.nz;
-    const bool odd[5] = {false, false, (gi & 1) != 0, (j & 1) != 0, (k & 1) != 0};
-    const long long c2[5] = {c, c, odd[2] ? c - I + wrapi(I + 1, Dc.nx) : c,
-                             odd[3] ? c + (long long)Dc.nx * (wrapi(J + 1, Dc.ny) - J) : c, odd[4] ? c + Dc.nxy : c};
-    T v[5][2], o[5];
-#pragma unroll
-    for (int f = 0; f < 5; ++f) {
-      v[f][0] = cell || f == 4 ? P.uc[f][c] : T(0);
-      v[f][1] = f < 2 ? v[f][0] : cell || f == 4 ? P.uc[f][c2[f]] : T(0);
+    // one coarse value, or the two coarse faces around an odd fine face (else twice the same)
+    const bool cell = k < Df.nz, oddu = gi & 1, oddv = j & 1, oddw = k & 1;
+    T vr[1] = {T(0)}, vh[1] = {T(0)}, vu[2] = {T(0), T(0)}, vv[2] = {T(0), T(0)}, vw[2];
+    if (cell) {
+      vr[0] = P.uc[0][c];
+      vh[0] = P.uc[1][c];
+      vu[0] = vu[1] = P.uc[2][c];
+      vv[0] = vv[1] = P.uc[3][c];
+      if (oddu) vu[1] = P.uc[2][c - I + wrapi(I + 1, Dc.nx)];
+      if (oddv) vv[1] = P.uc[3][c + (long long)Dc.nx * (wrapi(J + 1, Dc.ny) - J)];
     }
+    vw[0] = vw[1] = P.uc[4][c];
+    if (oddw) vw[1] = P.uc[4][c + Dc.nxy];
+    T o[5];
     bool sure = sizeof(T) == sizeof(float);
     if (sure) {
-#pragma unroll
-      for (int f = 0; f < 5; ++f) {
-        const T (&two)[2] = v[f];
-        o[f] = mean_plus(two, f < 4 ? lc[f] : none, sure);
-      }
+      o[0] = mean_plus<true>(vr, lc[0], sure);
+      o[1] = mean_plus<true>(vh, lc[1], sure);
+      o[2] = mean_plus<true>(vu, lc[2], sure);
+      o[3] = mean_plus<true>(vv, lc[3], sure);
+      o[4] = mean_plus<false>(vw, none, sure);
     }
     if (!sure) {
-#pragma unroll
-      for (int f = 0; f < 5; ++f) {
-        const T one[1] = {v[f][0]};
-        o[f] = (T)(odd[f] ? mean_double(v[f], f < 4 ? lc[f] : none) : mean_double(one, f < 4 ? lc[f] : none));
-      }
+      auto one = [](const T (&v)[2], bool odd, const LevelConst &k) -> T {   // (twice a large value may overflow)
+        return (T)(odd ? mean_double(v, k) : (double)v[0] + k.d);
+      };
+      o[0] = (T)mean_double(vr, lc[0]);
+      o[1] = (T)mean_double(vh, lc[1]);
+      o[2] = one(vu, oddu, lc[2]);
+      o[3] = one(vv, oddv, lc[3]);
+      o[4] = one(vw, oddw, none);
     }
     if (k < Df.nz) {
 #pragma unroll
