@@ -138,26 +138,25 @@ cudaError_t update_background(eb_geom g) {
 template <typename T>
 cudaError_t update_rdiff_t(eb_geom g) {
   const int nz = g->D.nz;
+  const size_t n = (size_t)nz * WSRD_DK;   // entries per field
+  std::vector<double> r(nz);
+  std::vector<T> t(4 * n, T(0));
   for (int q = 0; q < 4; ++q) {
-    std::vector<double> r(nz);
-    cudaError_t e = cudaMemcpy(r.data(), g->ref_d[q], sizeof(double) * nz, cudaMemcpyDeviceToHost);
+    const cudaError_t e = cudaMemcpy(r.data(), g->ref_d[q], sizeof(double) * nz, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return e;
-    std::vector<T> t((size_t)nz * WSRD_DK, T(0));
     for (int k = 0; k < nz; ++k)
       for (int d = 0; d < WSRD_DK; ++d) {
         const int ka = k + d - WSRD_DK / 2;
-        if (ka >= 0 && ka < nz) t[(size_t)k * WSRD_DK + d] = (T)(r[ka] - r[k]);
+        if (ka >= 0 && ka < nz) t[q * n + (size_t)k * WSRD_DK + d] = (T)(r[ka] - r[k]);
       }
-    if (!g->rdiff[q]) {
-      T *p = nullptr;
-      e = g->alloc(&p, (long long)t.size());
-      if (e != cudaSuccess) return e;
-      g->rdiff[q] = p;
-    }
-    e = cudaMemcpy(g->rdiff[q], t.data(), sizeof(T) * t.size(), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return e;
   }
-  return cudaSuccess;
+  if (!g->rdiff[0]) {
+    T *p = nullptr;
+    const cudaError_t e = g->alloc(&p, (long long)(4 * n));
+    if (e != cudaSuccess) return e;
+    for (int q = 0; q < 4; ++q) g->rdiff[q] = p + q * n;
+  }
+  return cudaMemcpy(g->rdiff[0], t.data(), sizeof(T) * t.size(), cudaMemcpyHostToDevice);
 }
 cudaError_t update_rdiff(eb_geom g) { return g->prec == EB_F64 ? update_rdiff_t<double>(g) : update_rdiff_t<float>(g); }
 

@@ -153,46 +153,62 @@ double split_time(const Dims &D, const std::vector<int> &kb, long long Lc, int s
   return end;
 }
 
-// The float path's march with `per_sm` CTAs per SM, in units of the time a CTA
-// alone on its SM takes per level: a piece costs its levels and three of
-// prologue, and of n CTAs on an SM each runs 1 + 0.1 (n - 1) times slower.
-// end: when the last piece is done, the pieces starting in order; busy: the
-// SMs' time in it, per SM.
+// The float path's march with two CTAs per SM, in units of the time a CTA alone
+// on its SM takes per level: a piece costs its levels and three of prologue, and
+// of two CTAs on an SM each runs 1.1 times slower.  end: when the last piece is
+// done, the pieces starting in order; busy: the SMs' time in it, per SM.
 struct MarchTime {
   double end = 0.0, busy = 0.0;
   long long pieces = 0;
 };
-MarchTime march_time(const Dims &D, const std::vector<int> &kb, long long Lc, int sms, int per_sm) {
-  auto slow = [](size_t n) { return 1.0 + 0.1 * ((double)n - 1.0); };
+constexpr int kMarchCtas = 2;   // by registers and shared memory (the occupancy query counts tensor memory and says 1)
+constexpr double kMarchShared = 1.1;
+// pieces and busy
+MarchTime march_work(const Dims &D, const std::vector<int> &kb, long long Lc, int sms) {
+  MarchTime M;
+  long long levels = 0;
+  for_pieces(D, kb, Lc, [&](int, int a, int b) {
+    ++M.pieces;
+    levels += 3 + (b - a);
+  });
+  M.busy = (double)levels * kMarchShared / kMarchCtas / sms;
+  return M;
+}
+// end
+double march_end(const Dims &D, const std::vector<int> &kb, long long Lc, int sms) {
   std::vector<double> cost;
   for_pieces(D, kb, Lc, [&](int, int a, int b) { cost.push_back(3.0 + (b - a)); });
-  MarchTime M;
-  M.pieces = (long long)cost.size();
-  for (double c : cost) M.busy += c * slow((size_t)per_sm) / per_sm / sms;
-  std::vector<std::vector<double>> left(sms);   // of the CTAs on each SM, at time at[]
-  std::vector<double> at(sms, 0.0);
+  struct Sm {
+    double left[kMarchCtas], at;   // what its CTAs have left at time at
+    int n;
+  };
+  std::vector<Sm> sm(sms, Sm{{}, 0.0, 0});
   size_t next = 0;
-  for (int q = 0; q < per_sm; ++q)
-    for (int i = 0; i < sms && next < cost.size(); ++i) left[i].push_back(cost[next++]);
+  for (int q = 0; q < kMarchCtas; ++q)
+    for (int i = 0; i < sms && next < cost.size(); ++i) sm[i].left[sm[i].n++] = cost[next++];
   using Event = std::pair<double, int>;   // an SM's next finish
   std::priority_queue<Event, std::vector<Event>, std::greater<Event>> events;
+  auto slow = [](int n) { return n > 1 ? kMarchShared : 1.0; };
   auto push = [&](int i) {
-    if (!left[i].empty())
-      events.push({at[i] + *std::min_element(left[i].begin(), left[i].end()) * slow(left[i].size()), i});
+    const Sm &S = sm[i];
+    if (S.n) events.push({S.at + *std::min_element(S.left, S.left + S.n) * slow(S.n), i});
   };
   for (int i = 0; i < sms; ++i) push(i);
+  double end = 0.0;
   while (!events.empty()) {
     const auto [t, i] = events.top();
     events.pop();
-    std::vector<double> &L = left[i];
-    const double done = (t - at[i]) / slow(L.size());
-    at[i] = M.end = t;
-    for (double &c : L) c -= done;
-    L.erase(std::remove_if(L.begin(), L.end(), [](double c) { return c < 1e-9; }), L.end());
-    while ((int)L.size() < per_sm && next < cost.size()) L.push_back(cost[next++]);
+    Sm &S = sm[i];
+    const double done = (t - S.at) / slow(S.n);
+    S.at = end = t;
+    int n = 0;
+    for (int q = 0; q < S.n; ++q)
+      if (S.left[q] - done > 1e-9) S.left[n++] = S.left[q] - done;
+    while (n < kMarchCtas && next < cost.size()) S.left[n++] = cost[next++];
+    S.n = n;
     push(i);
   }
-  return M;
+  return end;
 }
 
 }  // namespace
@@ -231,20 +247,18 @@ cudaError_t bulk_plan(const Dims &D, const int *kfast_host, bool f64, int slab_l
     // eight levels where that left SMs idle, was 4.7 % above the best in the mean,
     // up to 1.39 times slabs of three waves: 750 us instead of 570 on a 400x400x128
     // hill, 127 instead of 110 on 320x200x30.)
-    constexpr int per_sm = 2;   // by registers and shared memory (the occupancy query counts tensor memory and says 1)
     const double near = 2.5e-5 * (double)near_cvs / sms * 152;   // in levels, on this GPU's SMs
     double best = 0.0;
-    long long last = 0;
     auto consider = [&](long long L) {
-      const MarchTime M = march_time(D, kb, L, sms, per_sm);
-      const double both = M.busy + near * (M.pieces > (long long)per_sm * sms ? 1.2 : 1.0);
-      const double c = pow(M.end, 8) + pow(both, 8);
-      if (last == 0 || c < best) best = c, Lc = L;
-      last = L;
+      const MarchTime M = march_work(D, kb, L, sms);
+      double c = pow(M.busy + near * (M.pieces > (long long)kMarchCtas * sms ? 1.2 : 1.0), 8);
+      if (best > 0.0 && c >= best) return;
+      c += pow(march_end(D, kb, L, sms), 8);
+      if (best == 0.0 || c < best) best = c, Lc = L;
     };
     // heights of 1, 2, ... slabs, at least 15 % apart, and of 16 and 8 levels;
     // splits of more than 16 waves are only taken whole
-    const long long tiles = (long long)kb.size(), most = 16LL * per_sm * sms;
+    const long long tiles = (long long)kb.size(), most = 16LL * kMarchCtas * sms;
     for (long long n = 1; n == 1 || (D.nz / n >= 8 && tiles * n <= most); n = std::max(n + 1, n * 115 / 100))
       consider((D.nz + n - 1) / n);
     for (long long L : {16, 8})

@@ -45,6 +45,7 @@ struct WsrdDev {
 struct WsrdTab {
   long long ns = 0, na = 0;       // small, affected CVs
   long long nl = 0, nw = 0;       // entries of the two lists
+  void *block = nullptr;          // the device memory of all arrays
   unsigned *plin = nullptr;       // [ns] state index of the pivot member
   uint8_t *nmem = nullptr;        // [ns] members incl. itself (<= 8) | pivot member << 4
   unsigned *mlin = nullptr;       // [8][ns] members' state indices

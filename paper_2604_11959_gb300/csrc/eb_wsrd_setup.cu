@@ -17,6 +17,9 @@
 
 #include <math.h>
 
+#include <algorithm>
+#include <type_traits>
+
 namespace {
 
 __constant__ int kPerm[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
@@ -645,24 +648,38 @@ cudaError_t pack_wsrd_t(const Dims &D, const WsrdDev &W, WsrdTab &P, cudaStream_
   P.na = na;
   P.nl = W.nlsq;
   P.nw = W.nw;
-  CK(dalloc(&P.loff, ns + 1));
-  CK(dalloc(&P.woff, na + 1));
+  // one block for all arrays (an allocation each took a tenth of a small
+  // handle's build)
+  size_t bytes = 0;
+  auto place = [&](auto *&p, long long n) {
+    const size_t at = bytes;
+    bytes += (std::max(1LL, n) * sizeof(*p) + 255) / 256 * 256;
+    if (P.block) p = reinterpret_cast<std::remove_reference_t<decltype(p)>>((char *)P.block + at);
+  };
+  T *mw = nullptr, *me = nullptr, *lc = nullptr, *es = nullptr, *wk = nullptr, *we = nullptr;
+  for (int pass = 0; pass < 2; ++pass) {   // sizes, then places
+    bytes = 0;
+    place(P.loff, ns + 1);
+    place(P.woff, na + 1);
+    place(P.plin, ns);
+    place(P.nmem, ns);
+    place(P.mlin, 8 * ns);
+    place(mw, 8 * ns);
+    place(me, 24 * ns);
+    place(P.lplin, P.nl);
+    place(P.ltag, P.nl);
+    place(lc, 3 * P.nl);
+    place(P.alin, na);
+    place(P.atag, na);
+    place(es, 3 * na);
+    place(P.wtag, P.nw);
+    place(wk, P.nw);
+    place(we, 3 * P.nw);
+    if (pass == 0) CK(cudaMalloc(&P.block, bytes));
+  }
+  P.mw = mw, P.me = me, P.lc = lc, P.es = es, P.wk = wk, P.we = we;
   CK(cudaMemcpyAsync(P.loff, W.s_loff, sizeof(long long) * (size_t)(ns + 1), cudaMemcpyDeviceToDevice, s));
   CK(cudaMemcpyAsync(P.woff, W.a_woff, sizeof(long long) * (size_t)(na + 1), cudaMemcpyDeviceToDevice, s));
-  CK(dalloc(&P.plin, ns));
-  CK(dalloc(&P.nmem, ns));
-  CK(dalloc(&P.mlin, 8 * ns));
-  CK(dalloc((T **)&P.mw, 8 * ns));
-  CK(dalloc((T **)&P.me, 24 * ns));
-  CK(dalloc(&P.lplin, P.nl));
-  CK(dalloc(&P.ltag, P.nl));
-  CK(dalloc((T **)&P.lc, 3 * P.nl));
-  CK(dalloc(&P.alin, na));
-  CK(dalloc(&P.atag, na));
-  CK(dalloc((T **)&P.es, 3 * na));
-  CK(dalloc(&P.wtag, P.nw));
-  CK(dalloc((T **)&P.wk, P.nw));
-  CK(dalloc((T **)&P.we, 3 * P.nw));
   if (ns) k_pack_small<T><<<lin_blocks(ns), 128, 0, s>>>(D, W, P);
   if (na) k_pack_aff<T><<<lin_blocks(na), 128, 0, s>>>(D, W, P);
   CK(cudaGetLastError());
@@ -677,10 +694,7 @@ cudaError_t pack_wsrd(const Dims &D, const WsrdDev &W, bool f64, WsrdTab &P, cud
 }
 
 void free_wsrd_tab(WsrdTab &P) {
-  void *ptrs[] = {P.plin, P.nmem, P.mlin, P.mw, P.me, P.loff, P.lplin, P.ltag, P.lc, P.alin, P.atag, P.es,
-                  P.woff, P.wtag, P.wk, P.we};
-  for (void *p : ptrs)
-    if (p) cudaFree(p);
+  if (P.block) cudaFree(P.block);
   P = WsrdTab();
 }
 
