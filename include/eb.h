@@ -386,9 +386,9 @@ eb_status eb_step_profile(eb_geom geom, const eb_state *Un, eb_state *Unp1, doub
  *   iters    host: iterations used (NULL allowed).
  *   relres   host: final relative residual (NULL allowed).
  * rho and rho*theta are not touched.  Synchronises the stream where the
- * reduction so far predicts convergence (at least every 64 iterations).  The first call on a handle allocates its
- * work space (about 10 doubles per cell), so it must not be inside a stream
- * capture.
+ * reduction so far predicts convergence (at least every 64 iterations).  The
+ * first call on a handle allocates its work space (about 14 doubles per cell),
+ * so it must not be inside a stream capture.
  */
 eb_status eb_project(eb_geom geom, eb_state *U, double dt, double rtol, int maxit, const double *phi0, double *phi,
                      int *iters, double *relres, void *stream);
@@ -614,11 +614,11 @@ eb_status eb_geom_set_slab_levels(eb_geom geom, int slab_levels);
 
 /* Rows of the bulk kernel's tiles of 32 columns: 16 (default; until this is
  * called, the automatic split of an FP64 handle may take tiles of 16 columns
- * and 8 rows on small domains) or, on the
- * mixed path, 14 (a 256-row domain then cuts into 19 tile rows, and two slabs
- * of its 152 tiles fill every SM with two CTAs).  Scheduling only: every
- * cell's arithmetic is the same.  eb_geom_tune tries both on the mixed path;
- * ensembles keep 16 for their members.  Waits for the device to be idle.
+ * and 8 rows on small domains) or, on the mixed path, 14 (a 256-row domain then
+ * cuts into 19 tile rows, and two slabs of its 152 tiles fill every SM with two
+ * CTAs).  Scheduling only: every cell's arithmetic is the same.  eb_geom_tune
+ * tries both on the mixed path; ensembles use 16 for their members.  Waits for
+ * the device to be idle.
  * EB_ERR_INVALID_ARG for other values, or 14 on an FP64 handle. */
 eb_status eb_geom_set_tile_rows(eb_geom geom, int rows);
 

@@ -357,11 +357,12 @@ __device__ inline void restrict_cut(const RestrictArgs<T> &R, const int cols[4],
 }
 
 // All five fields of one coarse level per blockIdx.y (the lid face above the
-// top level keeps its value).  HBM bounds it: where the four fine columns are
-// regular, every value is a plain mean of 8 (4) fine ones plus a constant of
-// the level, formed almost without FP64 on the float path.  64 x 256 x 128 fine cells
-// onto 32 x 128 x 64: 37 us, the FP64 sums over the cut cells most of it
-// (130 us for one launch per field with double sums over looked-up fractions).
+// top level keeps its value).  Where the four fine columns are regular, every
+// value is a plain mean of 8 (4) fine ones plus a constant of the level, formed
+// almost without FP64 on the float path.  Latency and the FP64 sums over the cut
+// cells bound it: 64 x 256 x 128 fine cells onto 32 x 128 x 64 take 36 us, their
+// 47 MB would take 7 (130 us for one launch per field with double sums over
+// looked-up fractions).
 template <typename T>
 __global__ void __launch_bounds__(256) k_restrict(const __grid_constant__ RestrictArgs<T> R) {
   const Dims &Dc = R.Dc, &Df = R.F.D;
@@ -419,7 +420,8 @@ __global__ void __launch_bounds__(256) k_restrict(const __grid_constant__ Restri
 // indices): every fine CV takes the value of the coarse CV it lies in; a fine
 // face of a face grid on a coarse face takes that face's value, one halfway
 // between two coarse faces (odd fine index along the face's axis) their mean;
-// full values (state plus profile) are interpolated, in double.
+// full values (state plus profile) are interpolated, with one rounding of the
+// double value.
 template <typename T>
 struct ProlongArgs {
   Dims Df, Dc;
@@ -430,10 +432,11 @@ struct ProlongArgs {
 };
 
 // One fine level per blockIdx.y, all five fields of the columns outside [lo,
-// hi) (the level above the top holds rho*w only).  HBM bounds it; a value
-// costs one addition of the level's profile difference (as on the
-// restriction's float path, almost without FP64).  24 of 88 columns x 256 x 128: 16
-// us (127 us for one launch per field over all columns).
+// hi) (the level above the top holds rho*w only).  A value costs one addition
+// of the level's profile difference (as on the restriction's float path, almost
+// without FP64).  24 of 88 columns x 256 x 128: 17 us, latency (127 us for one
+// launch per field over all columns); a whole level of 256 x 256 x 128: 101 us for
+// 189 MB, instructions.
 template <typename T>
 __global__ void __launch_bounds__(256) k_prolong(const __grid_constant__ ProlongArgs<T> P) {
   const Dims &Df = P.Df, &Dc = P.Dc;

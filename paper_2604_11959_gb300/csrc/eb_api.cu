@@ -986,7 +986,7 @@ eb_status eb_geom_set_sources(eb_geom geom, int flags) {
     }
   }
   if (flags && !geom->src_pp && geom->prec == EB_F64) {
-    double *pp = nullptr;   // p' of every cell (the float path keeps it in registers)
+    double *pp = nullptr;   // p' of every cell (the float path forms it in shared planes)
     CUDA_TRY(geom->alloc(&pp, geom->D.nxy * geom->D.nz), "alloc source scratch");
     geom->src_pp = pp;
   }

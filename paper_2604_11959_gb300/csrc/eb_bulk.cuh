@@ -163,9 +163,9 @@ __device__ inline double2 psub(double2 a, double2 b) { return make_double2(__dsu
 __device__ inline float2 prcp(float2 a) { return make_float2(__fdividef(1.f, a.x), __fdividef(1.f, a.y)); }
 // The double path's are correctly rounded.  A cubic iteration from the
 // hardware's approximate reciprocal (three FP64 instructions, 256x256x128 hill
-// step 3017 us against 3207) was an ulp off in 0.03 % of the values and
-// could flush to zero just below 2^1022; its rounding corrected by two more (3220)
-// it gained nothing over the division.
+// step 3017 us against 3207) was an ulp off in 0.03 % of the values and could
+// flush to zero just below 2^1022; its rounding corrected by two more (3220) it
+// gained nothing over the division.
 __device__ inline double2 prcp(double2 a) { return make_double2(1.0 / a.x, 1.0 / a.y); }
 template <typename P>
 __device__ inline P psel_pos(P m, P a, P b) {   // a where m > 0, else b

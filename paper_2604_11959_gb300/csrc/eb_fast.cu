@@ -240,10 +240,10 @@ cudaError_t bulk_plan(const Dims &D, const int *kfast_host, bool f64, int slab_l
     // levels, with the smallest eighth-power mean of the two.  The near-EB and
     // redistribution kernels take 0.025 levels' time per 1000 near-EB CVs, a fifth
     // more where the march has pieces waiting for SMs until late in the step.
-    // The constants are the best over 102 domains of 15 thousand to 34 million cells,
-    // hills and random terrain, one and three stages: steps take 0.66 to 1.16 times
-    // those of slabs of three waves, 0.90 in the mean, and 1.7 % more than with the
-    // best height of each.  (A rule of about 1.5 whole CTAs per SM in one wave, or
+    // The constants are the best over 102 domains of 15 thousand to 34 million
+    // cells, hills and random terrain, one and three stages: steps take 0.66 to
+    // 1.16 times those of slabs of three waves, 0.90 in the mean, and 1.7 % more
+    // than with the best height of each.  (A rule of about 1.5 whole CTAs per SM in one wave, or
     // eight levels where that left SMs idle, was 4.7 % above the best in the mean,
     // up to 1.39 times slabs of three waves: 750 us instead of 570 on a 400x400x128
     // hill, 127 instead of 110 on 320x200x30.)
@@ -266,15 +266,16 @@ cudaError_t bulk_plan(const Dims &D, const int *kfast_host, bool f64, int slab_l
   }
   if (slab_levels == 0 && f64 && alone) {
     // Double path alone on the GPU: the height (and for small domains the
-    // 16 x 8 tile) of the shortest estimated time, in microseconds as
-    // measured for one CTA per SM: 39 + 23.7 per level for a 32 x 16 tile; 28
-    // + 13.7 per level for a 16 x 8 tile (four of them per 32 x 16 tile,
-    // each cheaper in time but not in FP64 instructions: more halo), which
-    // is taken only while every piece has an SM of its own, and not where the
-    // caller set the rows.  32x32x16 ridge:
-    // 337 us with one slab of 32 x 16 tiles, 63 with one level per piece, 42
-    // with 16 x 8 tiles; 64x64x32: 407 -> 87; 256x256x128: 3084 -> 2816
-    // (slabs of 35 and 16 levels).
+    // 16 x 8 tile) of the shortest estimated time for one CTA per SM: 39 us +
+    // 23.7 per level for a 32 x 16 tile; 28 + 13.7 per level for a 16 x 8 tile
+    // (four of them per 32 x 16 tile, each cheaper in time but not in FP64
+    // instructions: more halo), which is taken only while every piece has an
+    // SM of its own, and not where the caller set the rows.  (The constants
+    // were measured with a reciprocal that made all four about 6 % shorter.)
+    // The kernel alone, 32x32x16 ridge: 364 us with one slab of 32 x 16 tiles,
+    // 71 with one level per piece, 46 with 16 x 8 tiles; 64x64x32 hill: 439 in
+    // slabs of 16 levels, 97 of two; 256x256x128 hill: 3273 in slabs of 32, 3056
+    // of 16.
     double best = split_time(D, kb, Lc, sms, 39.0, 23.7);
     const std::vector<int> ks = tile_bottoms(D, kfast_host, 16, 8);
     for (long long L : {1, 2, 3, 4, 6, 8, 12, 16, 24, 32}) {

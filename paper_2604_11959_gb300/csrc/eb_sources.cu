@@ -60,16 +60,15 @@ __global__ void k_pressure(const __grid_constant__ SourceArgs<T> S) {
 }
 
 // The sources of the u and v CVs of levels 0 .. nz - 1 and the w CVs of face
-// levels 1 .. nz - 1.  HBM bounds it (rho', (rho theta)' and the three momenta
-// read, the momenta written: 32 bytes per cell in float), so one pass does
-// all: a block marches a tile of 32 x SR columns up a slab of levels, one
+// levels 1 .. nz - 1.  It reads rho', (rho theta)' and the three momenta and
+// writes the momenta, 32 bytes per cell in float, so one pass does all: a block marches a tile of 32 x SR columns up a slab of levels, one
 // column per thread.  Each level's p' is formed once per cell into a shared
 // plane (two planes, one barrier per level) with the cells beside the tile's
 // low x and y sides; the level below stays in registers.  From a column's
 // kfast up no flag is read.  Every load of a level precedes its stores, which
 // might alias them for all the compiler knows.  256x256x128, float: 80 us (a
-// pass that stored p' and one that read it took 40 + 126); the logarithms and
-// exponentials keep it from the 40 us of its 268 MB.
+// pass that stored p' and one that read it took 40 + 126).  The logarithms and
+// exponentials bound it on the float path too: its 268 MB are 40 us.
 constexpr int SR = 8;
 
 template <typename T, bool STORED>

@@ -472,7 +472,9 @@ __global__ void k_aff_fill(Dims D, int g, GridDev G, const long long *aff_id, Ws
 }
 
 // ---- the step's tables (WsrdTab) ------------------------------------------
-constexpr unsigned kMaxSmall = 1u << 28;   // a tag's room for small ids
+// a tag's room for small ids.  (The set-up's tables take about 1.5 KB per small
+// CV: 2^28 of them would be 400 GB, beyond the GPU's memory.)
+constexpr unsigned kMaxSmall = 1u << 28;
 
 __device__ inline unsigned make_tag(long long sid, int dk) { return (unsigned)(sid + 1) | (unsigned)(dk + 8) << 28; }
 
