@@ -591,9 +591,9 @@ eb_status eb_ensemble_destroy(eb_ensemble e);
  * higher stream priority than the near-EB kernels (eb_geom_set_bulk_priority)
  * and, on the mixed path, with tiles of 16 and of 14 rows
  * (eb_geom_set_tile_rows), and keeps the fastest combination; *slab_levels
- * (NULL allowed) receives the height (0 = automatic), eb_geom_info the rest.  Results of later steps do not
- * depend on either.  Synchronises the stream; allocates and frees the
- * temporary state. */
+ * (NULL allowed) receives the height (0 = automatic), eb_geom_info the rest.
+ * Results of later steps do not depend on either.  Synchronises the stream;
+ * allocates and frees the temporary state. */
 eb_status eb_geom_tune(eb_geom geom, const eb_state *U, double dt, int reps, int *slab_levels, void *stream);
 
 /* Stream priority of the bulk kernel within a step (scheduling only: results

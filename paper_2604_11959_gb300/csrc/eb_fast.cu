@@ -243,10 +243,10 @@ cudaError_t bulk_plan(const Dims &D, const int *kfast_host, bool f64, int slab_l
     // The constants are the best over 102 domains of 15 thousand to 34 million
     // cells, hills and random terrain, one and three stages: steps take 0.66 to
     // 1.16 times those of slabs of three waves, 0.90 in the mean, and 1.7 % more
-    // than with the best height of each.  (A rule of about 1.5 whole CTAs per SM in one wave, or
-    // eight levels where that left SMs idle, was 4.7 % above the best in the mean,
-    // up to 1.39 times slabs of three waves: 750 us instead of 570 on a 400x400x128
-    // hill, 127 instead of 110 on 320x200x30.)
+    // than with the best height of each.  (A rule of about 1.5 whole CTAs per
+    // SM in one wave, or eight levels where that left SMs idle, was 4.7 % above
+    // the best in the mean and up to 1.39 times slabs of three waves: 750 us
+    // instead of 570 on a 400x400x128 hill, 127 instead of 110 on 320x200x30.)
     const double near = 2.5e-5 * (double)near_cvs / sms * 152;   // in levels, on this GPU's SMs
     double best = 0.0;
     auto consider = [&](long long L) {
