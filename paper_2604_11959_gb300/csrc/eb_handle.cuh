@@ -67,6 +67,7 @@ struct ProjWork {
   double *id = nullptr;        // its reciprocal (0 off the active cells): the Jacobi preconditioner
   double *rhs = nullptr, *r = nullptr, *z = nullptr, *p = nullptr, *q = nullptr, *x = nullptr;
   int npart = 0, ncols = 1;    // partial sums per slot; columns per thread of the operator kernel
+  int aslabs = 1;              // slabs of the operator kernel
   double *part = nullptr;      // partial sums of the solver's dot products, npart per slot
   double *scal = nullptr;      // their totals, one per slot
   unsigned *done = nullptr;    // blocks that have added theirs, per slot

@@ -275,10 +275,9 @@ __device__ inline Cols cols_of(const Dims &D, const Slabs &S) {
 // for, so the fullest SM decides: its blocks times their levels, and most of a
 // level more per block (the planes below and above, the sum); fewer than two
 // blocks per SM do not hide their own latency.
+inline int apply_blocks(const Dims &D, int V) { return (int)((D.nxy / V + PB - 1) / PB); }
 inline Slabs apply_slabs(const Dims &D, int V, int sms) {
-  Slabs S;
-  S.nbx = (int)((D.nxy / V + PB - 1) / PB);
-  S.nby = S.nz = 1;
+  Slabs S{apply_blocks(D, V), 1, 1};
   double best = 0.0;
   for (int n = 1; n <= D.nz && (n == 1 || (long long)S.nbx * n <= 8LL * sms); ++n) {
     const double c = (double)((S.nbx * (long long)n + sms - 1) / sms) * ((D.nz + n - 1) / n + 0.7);
@@ -1089,6 +1088,7 @@ eb_status setup(eb_geom g, cudaStream_t s) {
   w.ncols = D.nx % 2 == 0 ? 2 : 1;
   w.npart = std::max({w.nb, slabs_of(D, 1, sms).blocks(), slabs_of(D, 2, sms).blocks(), slabs_of(D, 4, sms).blocks(),
                       apply_slabs(D, w.ncols, sms).blocks()});
+  w.aslabs = apply_slabs(D, w.ncols, sms).nz;
   CUDA_TRY(g->alloc(&w.part, (long long)S_SLOTS * w.npart), "alloc projection work space");
   CUDA_TRY(g->alloc(&w.scal, S_SLOTS), "alloc projection work space");
   CUDA_TRY(g->alloc(&w.done, S_SLOTS), "alloc projection work space");
@@ -1286,7 +1286,7 @@ void launch_correct(eb_geom g, void *const mom[3], double dt, cudaStream_t s) {
 
 void launch_apply(eb_geom g, const double *p, double *q, int it, bool chain, cudaStream_t s) {
   ProjWork &w = g->pw;
-  const Slabs S = apply_slabs(g->D, w.ncols, ebk_sm_count());
+  const Slabs S{apply_blocks(g->D, w.ncols), 1, w.aslabs};
   if (w.ncols == 2) launch_chained_if(chain, k_apply<2>, S.blocks(), PB, 0, s, make_op(g), S, p, q, sum_of(g, S_PQ), w.conv, it);
   else launch_chained_if(chain, k_apply<1>, S.blocks(), PB, 0, s, make_op(g), S, p, q, sum_of(g, S_PQ), w.conv, it);
 }
