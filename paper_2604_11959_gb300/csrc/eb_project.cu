@@ -27,9 +27,10 @@
 // terrain are formed from sums of opposite neighbours, x is updated with the
 // direction (p is read once), floats are widened by integer instructions, and
 // nothing is computed for the mask of inactive cells (their r, p and q are
-// zero).  192x192x96: operator 63 -> 64 us (its floor is about 47), update 47 ->
-// 27 (x moved out), direction 24 -> 22 (x moved in), right-hand side 116 -> 70,
-// correction 114 -> 74, start of the solve 95 -> 30, centring 34 -> 25.
+// zero).  192x192x96: a Jacobi iteration 172 -> 147 us (the operator's floor is
+// about 47; update and direction 47 and 24 before, 27 and 22 with x moved),
+// right-hand side 116 -> 70, correction 114 -> 74, start of the solve 95 -> 30,
+// centring 34 -> 25.
 #include "eb_handle.cuh"
 
 #include <math.h>
